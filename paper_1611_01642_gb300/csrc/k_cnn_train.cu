@@ -2,73 +2,265 @@
 // activations, BCE-with-logits loss, backward, Adam), all on CUDA cores with
 // fp32 accumulation. Activations a1, a2 are stored in bf16 exactly as the
 // inference kernel stores them; a3 and h stay fp32. Every reduction runs in
-// a fixed order (no floating-point atomics), so a training step is
-// deterministic and resuming from a checkpoint reproduces the same run.
+// a fixed order (no floating-point atomics, a fixed number of blocks), so a
+// training step is deterministic and resuming from a checkpoint reproduces
+// the same run.
 //
 // Layout: for each pyramid level of the batch, planar activation maps
-// a1[16][H1][W1], a2[32][H2][W2] (bf16), a3[32][H3][W3] (fp32) at offsets of
-// a TrainLevel table; h, dh on the cell atlas (row cell_row + cy, pitch P);
-// logits, labels and dz at the score-map offsets of the level.
+// a1[16][H1][P1], a2[32][H2][P2] (bf16), a3[32][H3][P3] (fp32) and
+// dz2[32][H2][P2] (fp32) at offsets of a TrainLevel table, rows padded to a
+// multiple of 8 elements so that four of them move per access; h, dh on the
+// cell atlas (row cell_row + cy, pitch P); logits, labels and dz at the
+// score-map offsets of the level.
+//
+// What bounds them: the convolutions are 3 x 468 multiply-adds per pyramid
+// pixel, and dz is fp32, so they run on the FP32 pipe, two multiply-adds per
+// instruction (fma.rn.f32x2 over pairs of channels). Every kernel walks a
+// contiguous share of the batch's tiles with persistent blocks; the operands
+// of a tile sit in shared memory, columns split by parity so that a stride-2
+// window is unit stride, and a thread holds 4 to 8 positions times 8 to 16
+// channels, so that one broadcast weight load feeds 4 to 8 instructions.
+// Weight gradients stay in registers over a block's whole share and leave as
+// one partial per block, summed in block order by the last kernel.
+// 4 x 1280x720 frames (38 M pyramid pixels, 36 levels each), one step:
+// 74.4 -> 6.67 ms against one thread per position with all levels of a weight's
+// gradient in one block (weight gradient of layer 1 and data gradient of layer 2
+// 49.8 -> 2.05, weight gradients of layers 2 and 3 9.2 -> 1.31 and 6.6 -> 0.75,
+// data gradient of layer 3 6.1 -> 0.55, forward convolutions 2.5 -> 1.65 ms).
 #include "pd_internal.h"
 
 #include <cuda_bf16.h>
 
+#include "f32x2.cuh"
+
 namespace pd {
 namespace {
 
-__device__ __forceinline__ float bf(const __nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
 
-// ---- forward: 3x3 stride-2 pad-1 conv + bias + relu, one thread per output
-// position, all output channels. IN: planar input (bf16, or the u8 level with
-// the input table when CIN == 1).
-template <int CIN, int COUT, bool FROM_IMAGE, bool OUT_BF16>
-__global__ void __launch_bounds__(256) t_conv_fwd(const TrainLevel *__restrict__ tl, const LevelDesc *__restrict__ levels,
-                                                  const uint8_t *__restrict__ pyr, const float *__restrict__ in_tab,
-                                                  const __nv_bfloat16 *__restrict__ in_act, int layer,
-                                                  const float *__restrict__ w, const float *__restrict__ b,
-                                                  void *out_act) {
-    const TrainLevel T = tl[blockIdx.y];
-    const LevelDesc L = levels[T.level];
-    int Hi, Wi, Ho, Wo;
-    int64_t in_off, out_off;
-    if (layer == 1) { Hi = L.Hk; Wi = L.Wk; Ho = T.H1; Wo = T.W1; in_off = 0; out_off = T.a1; }
-    else if (layer == 2) { Hi = T.H1; Wi = T.W1; Ho = T.H2; Wo = T.W2; in_off = T.a1; out_off = T.a2; }
-    else { Hi = T.H2; Wi = T.W2; Ho = T.H3; Wo = T.W3; in_off = T.a2; out_off = T.a3; }
-    __shared__ float ws[COUT * CIN * 9];
-    __shared__ float bs[COUT];
-    for (int i = threadIdx.x; i < COUT * CIN * 9; i += blockDim.x) ws[i] = w[i];
-    for (int i = threadIdx.x; i < COUT; i += blockDim.x) bs[i] = b[i];
-    __syncthreads();
-    const int n = Ho * Wo;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const int i = p / Wo, j = p - i * Wo;
-        float acc[COUT];
+// A block's contiguous share [t, end) of a tile grid over all levels
+// (TrainLevel::g[GRID] is a level's first tile; the grids are listed there).
+template <int GRID>
+struct Walk {
+    const TrainLevel *tl;
+    int n, t, end, k, next;
+    __device__ Walk(const TrainLevel *levels, int n_levels, int total) : tl(levels), n(n_levels) {
+        t = (int)((int64_t)total * blockIdx.x / gridDim.x);
+        end = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
+        int lo = 0, hi = n - 1;  // the last level whose first tile is <= t
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (tl[mid].g[GRID] <= t) lo = mid;
+            else hi = mid - 1;
+        }
+        k = lo;
+        next = k + 1 < n ? tl[k + 1].g[GRID] : total;
+    }
+    __device__ bool valid() const { return t < end; }
+    __device__ int local() const { return t - tl[k].g[GRID]; }
+    __device__ void step(int total) {
+        ++t;
+        while (t >= next && k + 1 < n) {
+            ++k;
+            next = k + 1 < n ? tl[k + 1].g[GRID] : total;
+        }
+    }
+};
+
+constexpr int kXE = 64, kXO = 68;  // input tile row pitches: even columns, odd columns (from -1)
+
+// Input pixels of the 64 x 16 layer-1 positions from (i0, j0): E[r][j] = x at
+// column 2 (j0 + j), O[r][j] = x at column 2 (j0 + j) - 1, row 2 i0 + r - 1;
+// zero outside the level. Level rows are 4-byte aligned (pitch a multiple of 16).
+__device__ __forceinline__ void stage_pixels(const uint8_t *img, int pitch, int Wk, int Hk, const float *lut, int i0,
+                                             int j0, float *E, float *O) {
+    for (int i = threadIdx.x; i < 33 * 33; i += 256) {
+        const int r = i / 33, w = i - 33 * r;
+        const int y = 2 * i0 + r - 1, c = 2 * j0 - 4 + 4 * w;
+        uint32_t v = 0u;
+        const bool in = y >= 0 && y < Hk && c >= 0 && c < pitch;
+        if (in) v = *reinterpret_cast<const uint32_t *>(img + (int64_t)y * pitch + c);
+        const int m = 2 * w - 2;
+        if (m >= 0) {
+            E[r * kXE + m] = in && c < Wk ? lut[v & 255u] : 0.f;
+            O[r * kXO + m + 1] = in && c + 1 < Wk ? lut[(v >> 8) & 255u] : 0.f;
+            E[r * kXE + m + 1] = in && c + 2 < Wk ? lut[(v >> 16) & 255u] : 0.f;
+        }
+        O[r * kXO + m + 2] = in && c + 3 < Wk ? lut[v >> 24] : 0.f;
+    }
+}
+
+// ---- layer 1: 64 x 16 positions per tile, 4 positions x 16 channels per
+// thread. The sum of a channel runs over (dy, dx) in order, as everywhere.
+// Bound by its stores (a1 is 32 bytes per position) and the staging.
+__global__ void __launch_bounds__(256) t_conv1(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
+                                               const LevelDesc *__restrict__ levels, const uint8_t *__restrict__ pyr,
+                                               const float *__restrict__ in_tab, const float *__restrict__ w,
+                                               const float *__restrict__ b, __nv_bfloat16 *__restrict__ act) {
+    __shared__ __align__(16) float E[33 * kXE], O[33 * kXO], ws[9 * 16], bs[16], lut[256];
+    const int tid = threadIdx.x;
+    lut[tid] = in_tab[tid];
+    if (tid < 144) ws[(tid % 9) * 16 + tid / 9] = w[tid];
+    if (tid < 16) bs[tid] = b[tid];
+    const int g = tid & 15, ir = tid >> 4;
+    for (Walk<0> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+        const TrainLevel &T = tl[wk.k];
+        const LevelDesc &L = levels[T.level];
+        const int ntx = (T.W2 + 31) / 32, lt = wk.local();
+        const int i0 = 16 * (lt / ntx), j0 = 64 * (lt % ntx);
+        __syncthreads();
+        stage_pixels(pyr + L.img_off, L.img_pitch, L.Wk, L.Hk, lut, i0, j0, E, O);
+        __syncthreads();
+        f32x2 acc[4][8];
 #pragma unroll
-        for (int o = 0; o < COUT; ++o) acc[o] = bs[o];
-        for (int c = 0; c < CIN; ++c) {
+        for (int o = 0; o < 8; ++o) {
+            const f32x2 bb = pack2(bs[2 * o], bs[2 * o + 1]);
 #pragma unroll
-            for (int dy = 0; dy < 3; ++dy) {
-                const int y = 2 * i + dy - 1;
+            for (int p = 0; p < 4; ++p) acc[p][o] = bb;
+        }
 #pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    const int x = 2 * j + dx - 1;
-                    float v = 0.f;
-                    if (y >= 0 && y < Hi && x >= 0 && x < Wi) {
-                        if (FROM_IMAGE) v = in_tab[pyr[L.img_off + (int64_t)y * L.img_pitch + x]];
-                        else v = bf(in_act[in_off + ((int64_t)c * Hi + y) * Wi + x]);
+        for (int dy = 0; dy < 3; ++dy) {
+            const int r = 2 * ir + dy;
+            const float4 e = *reinterpret_cast<const float4 *>(E + r * kXE + 4 * g);
+            const float4 o4 = *reinterpret_cast<const float4 *>(O + r * kXO + 4 * g);
+            const float ol = O[r * kXO + 4 * g + 4];
+            const f32x2 v0[4] = {dup2(o4.x), dup2(o4.y), dup2(o4.z), dup2(o4.w)};
+            const f32x2 v1[4] = {dup2(e.x), dup2(e.y), dup2(e.z), dup2(e.w)};
+            const f32x2 v2[4] = {v0[1], v0[2], v0[3], dup2(ol)};
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+                const f32x2 *v = dx == 0 ? v0 : dx == 1 ? v1 : v2;
+#pragma unroll
+                for (int o = 0; o < 8; o += 2) {
+                    const ulonglong2 ww = *reinterpret_cast<const ulonglong2 *>(ws + (dy * 3 + dx) * 16 + 2 * o);
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        acc[p][o] = fma2(ww.x, v[p], acc[p][o]);
+                        acc[p][o + 1] = fma2(ww.y, v[p], acc[p][o + 1]);
                     }
-#pragma unroll
-                    for (int o = 0; o < COUT; ++o) acc[o] = fmaf(ws[(o * CIN + c) * 9 + dy * 3 + dx], v, acc[o]);
                 }
             }
         }
+        const int i = i0 + ir, j = j0 + 4 * g;
+        if (i < T.H1 && j < T.P1) {
+            __nv_bfloat16 *dst = act + T.a1 + (int64_t)i * T.P1 + j;
 #pragma unroll
-        for (int o = 0; o < COUT; ++o) {
-            const float a = fmaxf(acc[o], 0.f);
-            if (OUT_BF16)
-                reinterpret_cast<__nv_bfloat16 *>(out_act)[out_off + ((int64_t)o * Ho + i) * Wo + j] = __float2bfloat16_rn(a);
-            else
-                reinterpret_cast<float *>(out_act)[out_off + ((int64_t)o * Ho + i) * Wo + j] = a;
+            for (int o = 0; o < 16; ++o) {
+                float v[4];
+#pragma unroll
+                for (int p = 0; p < 4; ++p) v[p] = fmaxf(o & 1 ? hi2(acc[p][o >> 1]) : lo2(acc[p][o >> 1]), 0.f);
+                const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), c = __floats2bfloat162_rn(v[2], v[3]);
+                uint2 u;
+                u.x = *reinterpret_cast<const uint32_t *>(&a);
+                u.y = *reinterpret_cast<const uint32_t *>(&c);
+                *reinterpret_cast<uint2 *>(dst + (int64_t)o * T.H1 * T.P1) = u;
+            }
+        }
+    }
+}
+
+constexpr int kAP = 36;  // bf16 row pitch of a staged activation tile (32 even columns, 33 odd ones)
+
+// ---- layers 2 and 3: 32 x 8 positions per tile, 4 positions x 16 output
+// channels per thread, 16 input channels staged at a time. Per input channel
+// and window row: 3 activation loads and 12 broadcast weight loads for 96
+// packed multiply-adds.
+template <int CIN, bool LAST>
+__global__ void __launch_bounds__(128) t_conv23(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
+                                                const __nv_bfloat16 *__restrict__ act, const float *__restrict__ w,
+                                                const float *__restrict__ b, __nv_bfloat16 *__restrict__ out16,
+                                                float *__restrict__ out32) {
+    extern __shared__ __align__(16) float smem_f[];
+    float *ws = smem_f;                                                      // [CIN][9][32]
+    __nv_bfloat16 *E = reinterpret_cast<__nv_bfloat16 *>(ws + CIN * 9 * 32);  // [16][17][kAP]
+    __nv_bfloat16 *O = E + 16 * 17 * kAP;
+    __shared__ float bs[32];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < CIN * 9 * 32; i += 128) {
+        const int o = i & 31, ct = i >> 5;
+        ws[i] = w[o * CIN * 9 + ct];
+    }
+    if (tid < 32) bs[tid] = b[tid];
+    const int o0 = 16 * (tid >> 6), g = tid & 7, ir = (tid >> 3) & 7;
+    constexpr int GRID = LAST ? 2 : 0;
+    for (Walk<GRID> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+        const TrainLevel &T = tl[wk.k];
+        const int Hi = LAST ? T.H2 : T.H1, Wi = LAST ? T.W2 : T.W1, Pi = LAST ? T.P2 : T.P1;
+        const int Ho = LAST ? T.H3 : T.H2, Wo = LAST ? T.W3 : T.W2, Po = LAST ? T.P3 : T.P2;
+        const int64_t in_off = LAST ? T.a2 : T.a1;
+        const int ntx = (Wo + 31) / 32, lt = wk.local();
+        const int i0 = 8 * (lt / ntx), j0 = 32 * (lt % ntx);
+        f32x2 acc[4][8];
+        for (int c0 = 0; c0 < CIN; c0 += 16) {
+            __syncthreads();
+            for (int i = tid; i < 16 * 17 * 33; i += 128) {
+                const int cr = i / 33, m = i - 33 * cr - 1;
+                const int cc = cr / 17, r = cr - 17 * cc;
+                const int y = 2 * i0 + r - 1, x = 2 * (j0 + m);
+                uint32_t v = 0u;
+                if (y >= 0 && y < Hi && x >= 0 && x < Wi) {
+                    v = *reinterpret_cast<const uint32_t *>(act + in_off + ((int64_t)(c0 + cc) * Hi + y) * Pi + x);
+                    if (x + 1 >= Wi) v &= 0xffffu;
+                }
+                if (m >= 0) reinterpret_cast<uint16_t *>(E)[cr * kAP + m] = (uint16_t)v;
+                reinterpret_cast<uint16_t *>(O)[cr * kAP + m + 1] = (uint16_t)(v >> 16);
+            }
+            __syncthreads();
+            if (c0 == 0) {
+#pragma unroll
+                for (int o = 0; o < 8; ++o) {
+                    const f32x2 bb = pack2(bs[o0 + 2 * o], bs[o0 + 2 * o + 1]);
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) acc[p][o] = bb;
+                }
+            }
+#pragma unroll 1
+            for (int c = 0; c < 16; ++c) {
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy) {
+                    const int row = (c * 17 + 2 * ir + dy) * kAP + 4 * g;
+                    const uint2 e = *reinterpret_cast<const uint2 *>(E + row);
+                    const uint2 od = *reinterpret_cast<const uint2 *>(O + row);
+                    const uint32_t ol = reinterpret_cast<const uint16_t *>(O)[row + 4];
+                    const f32x2 v0[4] = {dup2(bf_lo(od.x)), dup2(bf_hi(od.x)), dup2(bf_lo(od.y)), dup2(bf_hi(od.y))};
+                    const f32x2 v1[4] = {dup2(bf_lo(e.x)), dup2(bf_hi(e.x)), dup2(bf_lo(e.y)), dup2(bf_hi(e.y))};
+                    const f32x2 v2[4] = {v0[1], v0[2], v0[3], dup2(bf_lo(ol))};
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx) {
+                        const f32x2 *v = dx == 0 ? v0 : dx == 1 ? v1 : v2;
+                        const float *wp = ws + ((c0 + c) * 9 + dy * 3 + dx) * 32 + o0;
+#pragma unroll
+                        for (int o = 0; o < 8; o += 2) {
+                            const ulonglong2 ww = *reinterpret_cast<const ulonglong2 *>(wp + 2 * o);
+#pragma unroll
+                            for (int p = 0; p < 4; ++p) {
+                                acc[p][o] = fma2(ww.x, v[p], acc[p][o]);
+                                acc[p][o + 1] = fma2(ww.y, v[p], acc[p][o + 1]);
+                            }
+                        }
+                    }
+                }
+            }
+        }
+        const int i = i0 + ir, j = j0 + 4 * g;
+        if (i < Ho && j < Po) {
+#pragma unroll
+            for (int o = 0; o < 16; ++o) {
+                float v[4];
+#pragma unroll
+                for (int p = 0; p < 4; ++p) v[p] = fmaxf(o & 1 ? hi2(acc[p][o >> 1]) : lo2(acc[p][o >> 1]), 0.f);
+                const int64_t at = (LAST ? T.a3 : T.a2) + ((int64_t)(o0 + o) * Ho + i) * Po + j;
+                if (LAST) {
+                    *reinterpret_cast<float4 *>(out32 + at) = make_float4(v[0], v[1], v[2], v[3]);
+                } else {
+                    const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), c = __floats2bfloat162_rn(v[2], v[3]);
+                    uint2 u;
+                    u.x = *reinterpret_cast<const uint32_t *>(&a);
+                    u.y = *reinterpret_cast<const uint32_t *>(&c);
+                    *reinterpret_cast<uint2 *>(out16 + at) = u;
+                }
+            }
         }
     }
 }
@@ -77,27 +269,30 @@ __global__ void __launch_bounds__(256) t_conv_fwd(const TrainLevel *__restrict__
 __global__ void t_head_fwd(const TrainLevel *__restrict__ tl, const LevelDesc *__restrict__ levels,
                            const float *__restrict__ a3, const float *__restrict__ wh,
                            const float *__restrict__ bh, float *__restrict__ hmap, int32_t hp) {
-    const TrainLevel T = tl[blockIdx.y];
-    const LevelDesc L = levels[T.level];
+    const TrainLevel &T = tl[blockIdx.y];
+    const LevelDesc &L = levels[T.level];
     const int n = L.Hc * L.Wc;
+    const int64_t plane = (int64_t)T.H3 * T.P3;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
         const int cy = p / L.Wc, cx = p - cy * L.Wc;
+        const float *src = a3 + T.a3 + (int64_t)cy * T.P3 + cx;
         float h = bh[0];
-        for (int c = 0; c < 32; ++c) h = fmaf(wh[c], a3[T.a3 + ((int64_t)c * T.H3 + cy) * T.W3 + cx], h);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) h = fmaf(__ldg(wh + c), src[c * plane], h);
         hmap[(int64_t)(L.cell_row + cy) * hp + cx] = h;
     }
 }
 
 // ---- BCE with logits: per window dz = (p y (s - 1) + (1 - y) s) / N, loss
-// terms; labels y = score > thr. One block per level, fixed-order sums.
-__global__ void t_loss(const TrainLevel *__restrict__ tl, const LevelDesc *__restrict__ levels,
-                       const float *__restrict__ logits, const float *__restrict__ scores, float thr,
-                       float pos_weight, float inv_n, float *__restrict__ dz, float *__restrict__ level_loss) {
-    const TrainLevel T = tl[blockIdx.x];
-    const LevelDesc L = levels[T.level];
+// terms; labels y = score > thr. kLossParts blocks per level, fixed-order sums.
+__global__ void __launch_bounds__(256) t_loss(const TrainLevel *__restrict__ tl, const LevelDesc *__restrict__ levels,
+                                              const float *__restrict__ logits, const float *__restrict__ scores,
+                                              float thr, float pos_weight, float inv_n, float *__restrict__ dz,
+                                              float *__restrict__ level_loss) {
+    const LevelDesc &L = levels[tl[blockIdx.y].level];
     const int n = L.rows * L.cols;
     float part = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += kLossParts * 256) {
         const float z = logits[L.score_off + i];
         const float y = scores[L.score_off + i] > thr ? 1.f : 0.f;
         // log sigmoid(z) = -softplus(-z), log(1 - sigmoid(z)) = -softplus(z)
@@ -110,11 +305,11 @@ __global__ void t_loss(const TrainLevel *__restrict__ tl, const LevelDesc *__res
     __shared__ float red[256];
     red[threadIdx.x] = part;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    for (int o = 128; o > 0; o >>= 1) {
         if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) level_loss[blockIdx.x] = red[0] * inv_n;
+    if (threadIdx.x == 0) level_loss[blockIdx.y * kLossParts + blockIdx.x] = red[0] * inv_n;
 }
 
 // ---- pooling backward into h: dh[c] = sum over the windows that see cell c
@@ -122,8 +317,7 @@ __global__ void t_loss(const TrainLevel *__restrict__ tl, const LevelDesc *__res
 __global__ void t_pool_bwd_h(const TrainLevel *__restrict__ tl, const LevelDesc *__restrict__ levels,
                              const float *__restrict__ dz, const float *__restrict__ v,
                              float *__restrict__ dh, int32_t hp) {
-    const TrainLevel T = tl[blockIdx.y];
-    const LevelDesc L = levels[T.level];
+    const LevelDesc &L = levels[tl[blockIdx.y].level];
     const int n = L.Hc * L.Wc;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
         const int cy = p / L.Wc, cx = p - cy * L.Wc;
@@ -141,213 +335,510 @@ __global__ void t_pool_bwd_h(const TrainLevel *__restrict__ tl, const LevelDesc 
     }
 }
 
-// Block-wide sum of `v` in a fixed order (256 threads).
-__device__ __forceinline__ float block_sum(float v, float *red) {
-    red[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    const float r = red[0];
-    __syncthreads();
-    return r;
+// Sum over a warp in a fixed order (every lane gets it).
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
-// ---- gradients of V, bv, wh, bh: one block per parameter, looping over the
-// levels in order. Block q: 0..127 V, 128 bv, 129..160 wh, 161 bh; results go
-// to their places in the flat parameter order.
-__global__ void __launch_bounds__(256) t_small_grads(const TrainLevel *__restrict__ tl, int n_tl,
-                                                     const LevelDesc *__restrict__ levels,
+// ---- gradients of V, bv (32 x 16 windows per tile in shared memory, one
+// thread per template position and half of the rows) and of wh, bh (32 x 8
+// cells per tile, a warp per 4 channels). Partial p of a block: 0..127 V,
+// 128 bv, 129..160 wh, 161 bh.
+constexpr int kSmallParts = 162;
+__global__ void __launch_bounds__(256) t_small_grads(const TrainLevel *__restrict__ tl, int n_tl, int n_win_tiles,
+                                                     int n_cell_tiles, const LevelDesc *__restrict__ levels,
                                                      const float *__restrict__ dz, const float *__restrict__ hmap,
                                                      const float *__restrict__ dh, int32_t hp,
-                                                     const float *__restrict__ a3, float *__restrict__ grad_out) {
-    __shared__ float red[256];
-    const int q = blockIdx.x;
-    float acc = 0.f;
-    for (int k = 0; k < n_tl; ++k) {
-        const TrainLevel T = tl[k];
-        const LevelDesc L = levels[T.level];
-        float part = 0.f;
-        if (q < 129) {
-            const int n = L.rows * L.cols;
-            const int r = q / 8, s = q % 8;
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                const int wy = i / L.cols, wx = i - wy * L.cols;
-                const float d = dz[L.score_off + i];
-                part += q == 128 ? d : d * hmap[(int64_t)(L.cell_row + wy + r) * hp + wx + s];
-            }
-        } else {
-            const int n = L.Hc * L.Wc;
-            const int c = q - 129;
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                const int cy = i / L.Wc, cx = i - cy * L.Wc;
-                const float d = dh[(int64_t)(L.cell_row + cy) * hp + cx];
-                part += q == 161 ? d : d * a3[T.a3 + ((int64_t)c * T.H3 + cy) * T.W3 + cx];
+                                                     const float *__restrict__ a3, float *__restrict__ part) {
+    __shared__ float sd[16 * 32], sh[31 * 40], red[256 + 8];
+    const int tid = threadIdx.x, q = tid & 127, half = tid >> 7, lane = tid & 31, warp = tid >> 5;
+    const int r = q >> 3, s = q & 7;
+    float acc = 0.f, accd = 0.f;
+    for (Walk<4> wk(tl, n_tl, n_win_tiles); wk.valid(); wk.step(n_win_tiles)) {
+        const LevelDesc &L = levels[tl[wk.k].level];
+        const int ntx = (L.cols + 31) / 32, lt = wk.local();
+        const int y0 = 16 * (lt / ntx), x0 = 32 * (lt % ntx);
+        __syncthreads();
+        for (int i = tid; i < 16 * 32; i += 256) {
+            const int y = y0 + (i >> 5), x = x0 + (i & 31);
+            sd[i] = y < L.rows && x < L.cols ? dz[L.score_off + (int64_t)y * L.cols + x] : 0.f;
+        }
+        for (int i = tid; i < 31 * 39; i += 256) {
+            const int yy = i / 39, xx = i - 39 * yy;
+            const int y = y0 + yy, x = x0 + xx;
+            sh[yy * 40 + xx] = y < L.Hc && x < L.Wc ? hmap[(int64_t)(L.cell_row + y) * hp + x] : 0.f;
+        }
+        __syncthreads();
+        for (int y = 8 * half; y < 8 * half + 8; ++y) {
+#pragma unroll 8
+            for (int x = 0; x < 32; ++x) {
+                const float d = sd[y * 32 + x];
+                acc = fmaf(d, sh[(y + r) * 40 + x + s], acc);
+                accd += d;
             }
         }
-        acc += block_sum(part, red);
     }
-    if (threadIdx.x == 0) {
-        const int at = q < 128 ? kOffV + q : q == 128 ? kOffBv : q < 161 ? kOffWh + (q - 129) : kOffBh;
-        grad_out[at] = acc;
+    float aw[4] = {0.f, 0.f, 0.f, 0.f}, ab = 0.f;
+    for (Walk<2> wk(tl, n_tl, n_cell_tiles); wk.valid(); wk.step(n_cell_tiles)) {
+        const TrainLevel &T = tl[wk.k];
+        const LevelDesc &L = levels[T.level];
+        const int ntx = (T.W3 + 31) / 32, lt = wk.local();
+        const int y0 = 8 * (lt / ntx), x = 32 * (lt % ntx) + lane;
+        const int64_t plane = (int64_t)T.H3 * T.P3;
+#pragma unroll
+        for (int yy = 0; yy < 8; ++yy) {
+            const int y = y0 + yy;
+            if (y < L.Hc && x < L.Wc) {
+                const float d = dh[(int64_t)(L.cell_row + y) * hp + x];
+                const float *src = a3 + T.a3 + 4 * warp * plane + (int64_t)y * T.P3 + x;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) aw[c] = fmaf(d, src[c * plane], aw[c]);
+                ab += d;
+            }
+        }
     }
-}
-
-// ---- dz3[c][cell] = wh[c] dh[cell] (a3 > 0), zero outside the cells used
-__global__ void t_head_bwd(const TrainLevel *__restrict__ tl, const LevelDesc *__restrict__ levels,
-                           const float *__restrict__ dh, int32_t hp, const float *__restrict__ wh,
-                           const float *__restrict__ a3, float *__restrict__ dz3) {
-    const TrainLevel T = tl[blockIdx.y];
-    const LevelDesc L = levels[T.level];
-    const int n = 32 * T.H3 * T.W3;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const int c = p / (T.H3 * T.W3), r = p - c * T.H3 * T.W3;
-        const int cy = r / T.W3, cx = r - cy * T.W3;
-        float g = 0.f;
-        if (cy < L.Hc && cx < L.Wc && a3[T.a3 + p] > 0.f) g = wh[c] * dh[(int64_t)(L.cell_row + cy) * hp + cx];
-        dz3[T.a3 + p] = g;
-    }
-}
-
-// ---- data gradient of a 3x3 stride-2 conv, times the relu mask of its input:
-// dz_in[c][y][x] = (a_in > 0) * sum_{o,dy,dx} w[o][c][dy][dx] dz_out[o][(y+1-dy)/2][(x+1-dx)/2]
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(256) t_conv_bwd_data(const TrainLevel *__restrict__ tl, int layer,
-                                                       const float *__restrict__ w,
-                                                       const float *__restrict__ dz_out,
-                                                       const __nv_bfloat16 *__restrict__ a_in,
-                                                       float *__restrict__ dz_in) {
-    const TrainLevel T = tl[blockIdx.y];
-    int Hi, Wi, Ho, Wo;
-    int64_t in_off, out_off;
-    if (layer == 3) { Hi = T.H2; Wi = T.W2; Ho = T.H3; Wo = T.W3; in_off = T.a2; out_off = T.a3; }
-    else { Hi = T.H1; Wi = T.W1; Ho = T.H2; Wo = T.W2; in_off = T.a1; out_off = T.a2; }
-    __shared__ float ws[COUT * CIN * 9];
-    for (int i = threadIdx.x; i < COUT * CIN * 9; i += blockDim.x) ws[i] = w[i];
+    float *out = part + (int64_t)blockIdx.x * kSmallParts;
+    red[tid] = acc;
+    if (q == 0) red[256 + half] = accd;
     __syncthreads();
-    const int n = CIN * Hi * Wi;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const int c = p / (Hi * Wi), r = p - c * Hi * Wi;
-        const int y = r / Wi, x = r - y * Wi;
-        float g = 0.f;
-        if (bf(a_in[in_off + p]) > 0.f) {
+    if (tid < 128) out[tid] = red[tid] + red[tid + 128];
+    if (tid == 0) out[128] = red[256] + red[257];
 #pragma unroll
-            for (int dy = 0; dy < 3; ++dy) {
-                const int ty = y + 1 - dy;
-                if (ty < 0 || (ty & 1) || (ty >> 1) >= Ho) continue;
+    for (int c = 0; c < 4; ++c) {
+        const float v = warp_sum(aw[c]);
+        if (lane == 0) out[129 + 4 * warp + c] = v;
+    }
+    ab = warp_sum(ab);
+    if (tid == 0) out[161] = ab;
+}
+
+// dz3[o] of layer-3 position (i, j): wh[o] dh (a3 > 0) on the cells, else 0.
+__device__ __forceinline__ float dz3_at(const TrainLevel &T, const LevelDesc &L, const float *a3, const float *dh,
+                                        int32_t hp, float who, int o, int i, int j) {
+    if (i >= L.Hc || j >= L.Wc) return 0.f;
+    const float a = a3[T.a3 + ((int64_t)o * T.H3 + i) * T.P3 + j];
+    return a > 0.f ? who * dh[(int64_t)(L.cell_row + i) * hp + j] : 0.f;
+}
+
+// Data gradient of a stride-2 layer for two horizontally adjacent quads of
+// input positions (2i, 2i+1) x (4 columns) and 8 input channels: a quad takes
+// 9 products per (output channel, input channel) from the 2 x 2 output
+// positions it reaches. d: the tile's output gradients [32][dplane], row pitch
+// DP, at (i, j); ws: [32 o][9 taps][CIN] weights at the thread's channels.
+// acc[quad][2 * row + column][channel pair].
+template <int CIN, int DP>
+__device__ __forceinline__ void quad_pair(const float *d, int dplane, const float *ws, f32x2 (&acc)[2][4][4]) {
 #pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    const int tx = x + 1 - dx;
-                    if (tx < 0 || (tx & 1) || (tx >> 1) >= Wo) continue;
-                    const int64_t base = out_off + (int64_t)(ty >> 1) * Wo + (tx >> 1);
-                    for (int o = 0; o < COUT; ++o)
-                        g = fmaf(ws[(o * CIN + c) * 9 + dy * 3 + dx], dz_out[base + (int64_t)o * Ho * Wo], g);
-                }
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[q][p][c] = 0ull;
+#pragma unroll 1
+    for (int o = 0; o < 32; ++o) {
+        const float *dp = d + o * dplane;
+        const float2 t = *reinterpret_cast<const float2 *>(dp), u = *reinterpret_cast<const float2 *>(dp + DP);
+        const f32x2 top[3] = {dup2(t.x), dup2(t.y), dup2(dp[2])};
+        const f32x2 bot[3] = {dup2(u.x), dup2(u.y), dup2(dp[DP + 2])};
+        const float *wo = ws + o * 9 * CIN;
+        // tap, input position (2 * row + column), output position (row, column)
+        constexpr int kTap[9] = {4, 3, 5, 1, 7, 0, 2, 6, 8};
+        constexpr int kPos[9] = {0, 1, 1, 2, 2, 3, 3, 3, 3};
+        constexpr int kRow[9] = {0, 0, 0, 1, 0, 1, 1, 0, 0};
+        constexpr int kCol[9] = {0, 1, 0, 0, 0, 1, 0, 1, 0};
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(wo + kTap[k] * CIN);
+            const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(wo + kTap[k] * CIN + 4);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const f32x2 v = kRow[k] ? bot[q + kCol[k]] : top[q + kCol[k]];
+                f32x2(&a)[4] = acc[q][kPos[k]];
+                a[0] = fma2(w0.x, v, a[0]);
+                a[1] = fma2(w0.y, v, a[1]);
+                a[2] = fma2(w1.x, v, a[2]);
+                a[3] = fma2(w1.y, v, a[3]);
             }
         }
-        dz_in[in_off + p] = g;
     }
 }
 
-// ---- weight gradient of a 3x3 stride-2 conv: one block per (o, c) pair,
-// 9 taps (+ the bias when c == 0), fixed-order sums over levels and positions.
-template <int CIN, int COUT, bool FROM_IMAGE>
-__global__ void __launch_bounds__(256) t_conv_bwd_weight(const TrainLevel *__restrict__ tl, int n_tl,
-                                                         const LevelDesc *__restrict__ levels, int layer,
-                                                         const uint8_t *__restrict__ pyr,
-                                                         const float *__restrict__ in_tab,
-                                                         const __nv_bfloat16 *__restrict__ a_in,
-                                                         const float *__restrict__ dz_out,
-                                                         float *__restrict__ gw, float *__restrict__ gb) {
-    __shared__ float red[256];
-    const int o = blockIdx.x / CIN, c = blockIdx.x % CIN;
-    float acc[10];
+// ---- dz2 = (a2 > 0) * data gradient of layer 3: a tile is 16 x 8 quads
+// (32 x 16 layer-2 positions), 64 quad pairs x 4 groups of 8 channels.
+constexpr int kD3P = 18;  // staged dz3 row pitch (17 columns)
+__global__ void __launch_bounds__(256) t_dz2(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
+                                             const LevelDesc *__restrict__ levels, const float *__restrict__ a3,
+                                             const float *__restrict__ dh, int32_t hp, const float *__restrict__ wh,
+                                             const float *__restrict__ w, const __nv_bfloat16 *__restrict__ act,
+                                             float *__restrict__ dz2) {
+    extern __shared__ __align__(16) float smem_f[];
+    float *ws = smem_f;               // [32 o][9][32 c]
+    float *ds = smem_f + 32 * 9 * 32;  // [32 o][9][kD3P]
+    __shared__ float whs[32];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < 32 * 9 * 32; i += 256) {
+        const int c = i & 31, ot = i >> 5, o = ot / 9;
+        ws[i] = w[(o * 32 + c) * 9 + ot - 9 * o];
+    }
+    if (tid < 32) whs[tid] = wh[tid];
+    const int c0 = 8 * (tid >> 6), qx = tid & 7, qr = (tid >> 3) & 7;
+    for (Walk<3> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+        const TrainLevel &T = tl[wk.k];
+        const LevelDesc &L = levels[T.level];
+        const int ntx = (T.W3 + 15) / 16, lt = wk.local();
+        const int i0 = 8 * (lt / ntx), j0 = 16 * (lt % ntx);
+        __syncthreads();
+        for (int e = tid; e < 32 * 9 * 17; e += 256) {
+            const int oi = e / 17, j = e - 17 * oi, o = oi / 9, i = oi - 9 * o;
+            ds[oi * kD3P + j] = dz3_at(T, L, a3, dh, hp, whs[o], o, i0 + i, j0 + j);
+        }
+        __syncthreads();
+        f32x2 acc[2][4][4];
+        quad_pair<32, kD3P>(ds + qr * kD3P + 2 * qx, 9 * kD3P, ws + c0, acc);
+        const int x = 2 * j0 + 4 * qx;
 #pragma unroll
-    for (int k = 0; k < 10; ++k) acc[k] = 0.f;
-    for (int lv = 0; lv < n_tl; ++lv) {
-        const TrainLevel T = tl[lv];
-        const LevelDesc L = levels[T.level];
-        int Hi, Wi, Ho, Wo;
-        int64_t in_off, out_off;
-        if (layer == 1) { Hi = L.Hk; Wi = L.Wk; Ho = T.H1; Wo = T.W1; in_off = 0; out_off = T.a1; }
-        else if (layer == 2) { Hi = T.H1; Wi = T.W1; Ho = T.H2; Wo = T.W2; in_off = T.a1; out_off = T.a2; }
-        else { Hi = T.H2; Wi = T.W2; Ho = T.H3; Wo = T.W3; in_off = T.a2; out_off = T.a3; }
-        float part[10];
+        for (int a = 0; a < 2; ++a) {
+            const int y = 2 * (i0 + qr) + a;
+            if (y >= T.H2 || x >= T.P2) continue;
 #pragma unroll
-        for (int k = 0; k < 10; ++k) part[k] = 0.f;
-        const int n = Ho * Wo;
-        for (int p = threadIdx.x; p < n; p += blockDim.x) {
-            const int i = p / Wo, j = p - i * Wo;
-            const float d = dz_out[out_off + (int64_t)o * n + p];
-            if (d == 0.f) continue;
+            for (int c = 0; c < 8; ++c) {
+                const int64_t at = ((int64_t)(c0 + c) * T.H2 + y) * T.P2 + x;
+                const uint2 m = *reinterpret_cast<const uint2 *>(act + T.a2 + at);
+                float v[4];
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const f32x2 s = acc[p >> 1][2 * a + (p & 1)][c >> 1];
+                    v[p] = c & 1 ? hi2(s) : lo2(s);
+                }
+                *reinterpret_cast<float4 *>(dz2 + T.d2 + at) =
+                    make_float4(bf_lo(m.x) > 0.f ? v[0] : 0.f, bf_hi(m.x) > 0.f ? v[1] : 0.f,
+                                bf_lo(m.y) > 0.f ? v[2] : 0.f, bf_hi(m.y) > 0.f ? v[3] : 0.f);
+            }
+        }
+    }
+}
+
+// ---- layer 1's weight gradient. dz1 = (a1 > 0) * data gradient of layer 2 is
+// only needed for it, so a thread keeps its 8 positions x 8 channels of dz1 in
+// registers and adds their products with the input pixels to its own sums;
+// dz1 is never written (it would be 2 x 64 bytes per position of traffic). A
+// tile is 32 x 8 quads (64 x 16 layer-1 positions): 128 quad pairs x 2 channel groups.
+constexpr int kD2P = 34;  // staged dz2 row pitch (33 columns)
+constexpr int kW1Parts = 160;
+__global__ void __launch_bounds__(256, 1) t_dw1(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
+                                                const LevelDesc *__restrict__ levels,
+                                                const uint8_t *__restrict__ pyr, const float *__restrict__ in_tab,
+                                                const float *__restrict__ w, const __nv_bfloat16 *__restrict__ act,
+                                                const float *__restrict__ dz2, float *__restrict__ part) {
+    extern __shared__ __align__(16) float smem_f[];
+    float *ws = smem_f;                  // [32 o][9][16 c]
+    float *ds = ws + 32 * 9 * 16;        // [32 o][9][kD2P]
+    float *E = ds + 32 * 9 * kD2P;       // [33][kXE]
+    float *O = E + 33 * kXE;             // [33][kXO]
+    __shared__ float lut[256], red[8 * 80];
+    const int tid = threadIdx.x;
+    lut[tid] = in_tab[tid];
+    for (int i = tid; i < 32 * 9 * 16; i += 256) {
+        const int c = i & 15, ot = i >> 4, o = ot / 9;
+        ws[i] = w[(o * 16 + c) * 9 + ot - 9 * o];
+    }
+    const int c0 = 8 * (tid >> 7), qx = tid & 15, qr = (tid >> 4) & 7;
+    f32x2 sum[10][4];
+#pragma unroll
+    for (int k = 0; k < 10; ++k)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) sum[k][c] = 0ull;
+    for (Walk<0> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+        const TrainLevel &T = tl[wk.k];
+        const LevelDesc &L = levels[T.level];
+        const int ntx = (T.W2 + 31) / 32, lt = wk.local();
+        const int i0 = 8 * (lt / ntx), j0 = 32 * (lt % ntx);
+        __syncthreads();
+        stage_pixels(pyr + L.img_off, L.img_pitch, L.Wk, L.Hk, lut, 2 * i0, 2 * j0, E, O);
+        for (int e = tid; e < 32 * 9 * 33; e += 256) {
+            const int oi = e / 33, j = e - 33 * oi, o = oi / 9, i = oi - 9 * o;
+            ds[oi * kD2P + j] = i0 + i < T.H2 && j0 + j < T.W2
+                                    ? dz2[T.d2 + ((int64_t)o * T.H2 + i0 + i) * T.P2 + j0 + j]
+                                    : 0.f;
+        }
+        __syncthreads();
+        f32x2 acc[2][4][4];
+        quad_pair<16, kD2P>(ds + qr * kD2P + 2 * qx, 9 * kD2P, ws + c0, acc);
+        // relu mask of a1 (and the layer's edge)
+        const int x = 2 * j0 + 4 * qx;
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const int y = 2 * (i0 + qr) + a;
+            const bool in = y < T.H1 && x < T.P1;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint2 m0 = make_uint2(0u, 0u), m1 = m0;
+                if (in) {
+                    const __nv_bfloat16 *src = act + T.a1 + ((int64_t)(c0 + 2 * c) * T.H1 + y) * T.P1 + x;
+                    m0 = *reinterpret_cast<const uint2 *>(src);
+                    m1 = *reinterpret_cast<const uint2 *>(src + (int64_t)T.H1 * T.P1);
+                }
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const uint32_t u0 = p < 2 ? m0.x : m0.y, u1 = p < 2 ? m1.x : m1.y;
+                    const bool ok = x + p < T.W1;
+                    const bool k0 = ok && (p & 1 ? bf_hi(u0) : bf_lo(u0)) > 0.f;
+                    const bool k1 = ok && (p & 1 ? bf_hi(u1) : bf_lo(u1)) > 0.f;
+                    f32x2 &s = acc[p >> 1][2 * a + (p & 1)][c];
+                    s = pack2(k0 ? lo2(s) : 0.f, k1 ? hi2(s) : 0.f);
+                }
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
 #pragma unroll
             for (int dy = 0; dy < 3; ++dy) {
-                const int y = 2 * i + dy - 1;
+                const int r = 2 * (2 * qr + a) + dy;
+                const float4 e = *reinterpret_cast<const float4 *>(E + r * kXE + 4 * qx);
+                const float4 o4 = *reinterpret_cast<const float4 *>(O + r * kXO + 4 * qx);
+                const f32x2 ev[4] = {dup2(e.x), dup2(e.y), dup2(e.z), dup2(e.w)};
+                const f32x2 ov[5] = {dup2(o4.x), dup2(o4.y), dup2(o4.z), dup2(o4.w), dup2(O[r * kXO + 4 * qx + 4])};
 #pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    const int x = 2 * j + dx - 1;
-                    float v = 0.f;
-                    if (y >= 0 && y < Hi && x >= 0 && x < Wi) {
-                        if (FROM_IMAGE) v = in_tab[pyr[L.img_off + (int64_t)y * L.img_pitch + x]];
-                        else v = bf(a_in[in_off + ((int64_t)c * Hi + y) * Wi + x]);
+                for (int p = 0; p < 4; ++p)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const f32x2 d = acc[p >> 1][2 * a + (p & 1)][c];
+                        sum[3 * dy][c] = fma2(d, ov[p], sum[3 * dy][c]);
+                        sum[3 * dy + 1][c] = fma2(d, ev[p], sum[3 * dy + 1][c]);
+                        sum[3 * dy + 2][c] = fma2(d, ov[p + 1], sum[3 * dy + 2][c]);
+                        if (dy == 0) sum[9][c] = add2(sum[9][c], d);
                     }
-                    part[dy * 3 + dx] = fmaf(d, v, part[dy * 3 + dx]);
+            }
+        }
+    }
+    const int warp = tid >> 5, lane = tid & 31;
+#pragma unroll
+    for (int k = 0; k < 10; ++k)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const float v = warp_sum(c & 1 ? hi2(sum[k][c >> 1]) : lo2(sum[k][c >> 1]));
+            if (lane == 0) red[warp * 80 + k * 8 + c] = v;
+        }
+    __syncthreads();
+    if (tid < kW1Parts) {  // order: 144 weights [c][tap], 16 biases
+        const int c = tid < 144 ? tid / 9 : tid - 144, k = tid < 144 ? tid % 9 : 9;
+        const int at = (c >> 3) * 4 * 80 + k * 8 + (c & 7);
+        part[(int64_t)blockIdx.x * kW1Parts + tid] = ((red[at] + red[at + 80]) + red[at + 160]) + red[at + 240];
+    }
+}
+
+// ---- weight gradients of layers 2 and 3: dW[o][c][tap] = sum over positions
+// of dz[o] a[c at the tap]. A tile is 16 x 8 positions; a thread holds one
+// input channel x 4 output channels x 9 taps (CIN = 16: the two halves of the
+// block take half of the rows each). Lanes are channels: the activation planes
+// are an odd number of words apart (no bank conflict), dz is a broadcast.
+constexpr int kWAP = 33, kWAC = 17 * kWAP;  // staged activation row pitch (16 even, 17 odd columns), plane
+constexpr int kWDP = 36;                    // staged dz: words per position
+static_assert(kWAC % 2 == 1, "planes an odd number of words apart");
+template <int CIN>
+__global__ void __launch_bounds__(256) t_dw23(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
+                                              const LevelDesc *__restrict__ levels, const float *__restrict__ a3,
+                                              const float *__restrict__ dh, int32_t hp, const float *__restrict__ wh,
+                                              const __nv_bfloat16 *__restrict__ act, const float *__restrict__ dz2,
+                                              float *__restrict__ part) {
+    constexpr bool LAST = CIN == 32;
+    constexpr int kRows = LAST ? 8 : 4;
+    extern __shared__ __align__(16) float smem_f[];
+    float *ds = smem_f;                // [128 positions][kWDP]
+    float *as = smem_f + 128 * kWDP;   // [CIN][17][16 even | 17 odd columns]
+    __shared__ float whs[32];
+    const int tid = threadIdx.x;
+    if (LAST && tid < 32) whs[tid] = wh[tid];
+    const int c = tid % CIN, og = (tid / CIN) & 7, r0 = LAST ? 0 : 4 * (tid >> 7);
+    f32x2 acc[9][2], accb[2] = {0ull, 0ull};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) acc[k][0] = acc[k][1] = 0ull;
+    constexpr int GRID = LAST ? 3 : 1;
+    for (Walk<GRID> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+        const TrainLevel &T = tl[wk.k];
+        const LevelDesc &L = levels[T.level];
+        const int Hi = LAST ? T.H2 : T.H1, Wi = LAST ? T.W2 : T.W1, Pi = LAST ? T.P2 : T.P1;
+        const int Wo = LAST ? T.W3 : T.W2;
+        const int64_t in_off = LAST ? T.a2 : T.a1;
+        const int ntx = (Wo + 15) / 16, lt = wk.local();
+        const int i0 = 8 * (lt / ntx), j0 = 16 * (lt % ntx);
+        __syncthreads();
+        for (int e = tid; e < 32 * 128; e += 256) {
+            const int o = e >> 7, p = e & 127, i = i0 + (p >> 4), j = j0 + (p & 15);
+            float v;
+            if (LAST) v = dz3_at(T, L, a3, dh, hp, whs[o], o, i, j);
+            else v = i < T.H2 && j < T.W2 ? dz2[T.d2 + ((int64_t)o * T.H2 + i) * T.P2 + j] : 0.f;
+            ds[p * kWDP + o] = v;
+        }
+        for (int e = tid; e < CIN * 17 * 17; e += 256) {
+            const int cr = e / 17, m = e - 17 * cr - 1, cc = cr / 17, r = cr - 17 * cc;
+            const int y = 2 * i0 + r - 1, x = 2 * (j0 + m);
+            uint32_t v = 0u;
+            if (y >= 0 && y < Hi && x >= 0 && x < Wi) {
+                v = *reinterpret_cast<const uint32_t *>(act + in_off + ((int64_t)cc * Hi + y) * Pi + x);
+                if (x + 1 >= Wi) v &= 0xffffu;
+            }
+            float *row = as + cc * kWAC + r * kWAP;
+            if (m >= 0) row[m] = bf_lo(v);
+            row[16 + m + 1] = bf_hi(v);
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int i = r0; i < r0 + kRows; ++i) {
+            const float *ap = as + c * kWAC + 2 * i * kWAP;
+            const float *dp = ds + i * 16 * kWDP + 4 * og;
+            f32x2 od[3];
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) od[dy] = dup2(ap[dy * kWAP + 16]);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const ulonglong2 d = *reinterpret_cast<const ulonglong2 *>(dp + j * kWDP);
+                accb[0] = add2(accb[0], d.x);
+                accb[1] = add2(accb[1], d.y);
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy) {
+                    const f32x2 e = dup2(ap[dy * kWAP + j]), on = dup2(ap[dy * kWAP + 17 + j]);
+                    acc[3 * dy][0] = fma2(d.x, od[dy], acc[3 * dy][0]);
+                    acc[3 * dy][1] = fma2(d.y, od[dy], acc[3 * dy][1]);
+                    acc[3 * dy + 1][0] = fma2(d.x, e, acc[3 * dy + 1][0]);
+                    acc[3 * dy + 1][1] = fma2(d.y, e, acc[3 * dy + 1][1]);
+                    acc[3 * dy + 2][0] = fma2(d.x, on, acc[3 * dy + 2][0]);
+                    acc[3 * dy + 2][1] = fma2(d.y, on, acc[3 * dy + 2][1]);
+                    od[dy] = on;
                 }
             }
-            part[9] += d;
         }
-#pragma unroll
-        for (int k = 0; k < 10; ++k) acc[k] += block_sum(part[k], red);
     }
-    if (threadIdx.x == 0) {
+    float v[10][4];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) gw[(o * CIN + c) * 9 + k] = acc[k];
-        if (c == 0) gb[o] = acc[9];
+    for (int k = 0; k < 10; ++k) {
+        unpack2(k < 9 ? acc[k][0] : accb[0], v[k][0], v[k][1]);
+        unpack2(k < 9 ? acc[k][1] : accb[1], v[k][2], v[k][3]);
+    }
+    if (!LAST) {  // add the second half's sums to the first's
+        __syncthreads();
+        if (tid >= 128) {
+#pragma unroll
+            for (int k = 0; k < 10; ++k)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) smem_f[(k * 4 + u) * 128 + tid - 128] = v[k][u];
+        }
+        __syncthreads();
+        if (tid >= 128) return;
+#pragma unroll
+        for (int k = 0; k < 10; ++k)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[k][u] += smem_f[(k * 4 + u) * 128 + tid];
+    }
+    float *out = part + (int64_t)blockIdx.x * (32 * CIN * 9 + 32);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int o = 4 * og + u;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) out[(o * CIN + c) * 9 + k] = v[k][u];
+        if (c == 0) out[32 * CIN * 9 + o] = v[9][u];
     }
 }
 
-// dz of a stored relu layer output: dz = (a > 0) * g, where g came from the
-// data gradient of the next layer (already masked there), so layer-2 and
-// layer-1 dz are the outputs of t_conv_bwd_data.
-
-// ---- the working copy the forward pass uses: conv weights rounded to bf16
+// Conv weights are rounded to bf16 in the working copy the forward pass uses.
+__device__ __forceinline__ float working_value(int i, float master) {
+    const bool conv_w = i < kOffB1 || (i >= kOffW2 && i < kOffB2) || (i >= kOffW3 && i < kOffB3);
+    return conv_w ? __bfloat162float(__float2bfloat16_rn(master)) : master;
+}
 __global__ void t_round(const float *__restrict__ master, float *__restrict__ wr, int n) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const bool conv_w = i < kOffB1 || (i >= kOffW2 && i < kOffB2) || (i >= kOffW3 && i < kOffB3);
-        wr[i] = conv_w ? __bfloat162float(__float2bfloat16_rn(master[i])) : master[i];
-    }
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        wr[i] = working_value(i, master[i]);
 }
 
-// ---- Adam on the fp32 master parameters
-__global__ void t_adam(float *__restrict__ p, float *__restrict__ m, float *__restrict__ v,
-                       const float *__restrict__ g, int n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float gi = g[i];
+// ---- the gradient from the blocks' partials (8 warps of a block take every
+// 8th partial of 32 parameters, then add up in order), Adam on the fp32 master
+// parameters (lr > 0) and their working copy.
+__global__ void __launch_bounds__(256) t_finish(const float *__restrict__ p1, int n1, const float *__restrict__ p2,
+                                                int n2, const float *__restrict__ p3, int n3,
+                                                const float *__restrict__ ps, int ns, float *__restrict__ grad,
+                                                float *__restrict__ p, float *__restrict__ m, float *__restrict__ v,
+                                                float *__restrict__ wr, float lr, float b1, float b2, float eps,
+                                                float c1, float c2) {
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    const float *src = nullptr;
+    int n = 0, stride = 0;
+    if (i < kOffW2) {  // w1, b1
+        src = p1 + i; n = n1; stride = kW1Parts;
+    } else if (i < kOffW3) {  // w2, b2
+        src = p2 + (i - kOffW2); n = n2; stride = kOffW3 - kOffW2;
+    } else if (i < kOffWh) {  // w3, b3
+        src = p3 + (i - kOffW3); n = n3; stride = kOffWh - kOffW3;
+    } else if (i < kCnnParams) {  // wh, bh, V, bv
+        const int k = i < kOffV ? 129 + (i - kOffWh) : i - kOffV;
+        src = ps + k; n = ns; stride = kSmallParts;
+    }
+    float s = 0.f;
+#pragma unroll 4
+    for (int b = warp; b < n; b += 8) s += src[(int64_t)b * stride];
+    red[warp][lane] = s;
+    __syncthreads();
+    if (warp || i >= kCnnParams) return;
+    float gi = red[0][lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) gi += red[k][lane];
+    grad[i] = gi;
+    if (lr > 0.f) {
         const float mi = b1 * m[i] + (1.f - b1) * gi;
         const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
         m[i] = mi;
         v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        const float pn = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        p[i] = pn;
+        wr[i] = working_value(i, pn);
     }
 }
 
+constexpr size_t conv23_smem(int cin) { return (size_t)cin * 9 * 32 * 4 + 2 * 16 * 17 * kAP * 2; }
+constexpr size_t kDz2Smem = (size_t)(32 * 9 * 32 + 32 * 9 * kD3P) * 4;
+constexpr size_t kDw1Smem = (size_t)(32 * 9 * 16 + 32 * 9 * kD2P + 33 * (kXE + kXO)) * 4;
+constexpr size_t dw23_smem(int cin) { return (size_t)(128 * kWDP + cin * kWAC) * 4; }
+static_assert(dw23_smem(16) >= 40 * 128 * 4, "the halves' exchange fits");
+
 }  // namespace
+
+cudaError_t init_train() {
+    cudaError_t e = cudaFuncSetAttribute(t_conv23<16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)conv23_smem(16));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(t_conv23<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)conv23_smem(32));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(t_dz2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDz2Smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(t_dw1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDw1Smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(t_dw23<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dw23_smem(16));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(t_dw23<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dw23_smem(32));
+    return e;
+}
+
+size_t train_partial_floats() {
+    return (size_t)kTrainBlocks * (kW1Parts + (kOffW3 - kOffW2) + (kOffWh - kOffW3) + kSmallParts);
+}
 
 cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a) {
     const dim3 blk(256);
-    const int gx = 48;
     const int nl = a.n_levels;
     if (nl <= 0) return cudaSuccess;
-    const dim3 g2(gx, nl);
+    const dim3 g2(8, nl);
+    // persistent blocks: a fixed number, so that the sums' order does not depend on the device
+    constexpr int G = kTrainBlocks;
+    float *p1 = a.part, *p2 = p1 + (size_t)G * kW1Parts, *p3 = p2 + (size_t)G * (kOffW3 - kOffW2),
+          *ps = p3 + (size_t)G * (kOffWh - kOffW3);
     // forward
-    t_conv_fwd<1, 16, true, true><<<g2, blk, 0, s>>>(a.tl, a.levels, a.pyr, a.w.in_tab, nullptr, 1, a.wr + kOffW1,
-                                                     a.wr + kOffB1, a.act16);
-    t_conv_fwd<16, 32, false, true><<<g2, blk, 0, s>>>(a.tl, a.levels, a.pyr, a.w.in_tab, a.act16, 2, a.wr + kOffW2,
-                                                       a.wr + kOffB2, a.act16);
-    t_conv_fwd<32, 32, false, false><<<g2, blk, 0, s>>>(a.tl, a.levels, a.pyr, a.w.in_tab, a.act16, 3, a.wr + kOffW3,
-                                                        a.wr + kOffB3, a.act32);
+    t_conv1<<<4 * G, blk, 0, s>>>(a.tl, nl, a.tiles[0], a.levels, a.pyr, a.w.in_tab, a.wr + kOffW1, a.wr + kOffB1,
+                                  a.act16);
+    t_conv23<16, false><<<3 * G, 128, conv23_smem(16), s>>>(a.tl, nl, a.tiles[0], a.act16, a.wr + kOffW2,
+                                                            a.wr + kOffB2, a.act16, nullptr);
+    t_conv23<32, true><<<2 * G, 128, conv23_smem(32), s>>>(a.tl, nl, a.tiles[2], a.act16, a.wr + kOffW3,
+                                                           a.wr + kOffB3, nullptr, a.act32);
     t_head_fwd<<<g2, blk, 0, s>>>(a.tl, a.levels, a.act32, a.wr + kOffWh, a.wr + kOffBh, a.hmap, a.hp);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -359,27 +850,21 @@ cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a) {
     e = launch_cnn(s, a.levels, nl, nullptr, nullptr, 0, pw, a.hmap, a.hp, a.logits, a.pool_tiles, nullptr);  // pooling only
     if (e != cudaSuccess) return e;
     // loss and backward
-    t_loss<<<nl, 256, 0, s>>>(a.tl, a.levels, a.logits, a.scores, a.label_thr, a.pos_weight, a.inv_n, a.dz,
-                              a.level_loss);
-    t_pool_bwd_h<<<g2, blk, 0, s>>>(a.tl, a.levels, a.dz, a.wr + kOffV, a.dh, a.hp);
-    t_small_grads<<<162, 256, 0, s>>>(a.tl, nl, a.levels, a.dz, a.hmap, a.dh, a.hp, a.act32, a.grad);
-    t_head_bwd<<<g2, blk, 0, s>>>(a.tl, a.levels, a.dh, a.hp, a.wr + kOffWh, a.act32, a.dz32);
-    t_conv_bwd_weight<32, 32, false><<<32 * 32, 256, 0, s>>>(a.tl, nl, a.levels, 3, a.pyr, a.w.in_tab, a.act16,
-                                                             a.dz32, a.grad + kOffW3, a.grad + kOffB3);
-    t_conv_bwd_data<32, 32><<<g2, blk, 0, s>>>(a.tl, 3, a.wr + kOffW3, a.dz32, a.act16, a.dz16);
-    t_conv_bwd_weight<16, 32, false><<<32 * 16, 256, 0, s>>>(a.tl, nl, a.levels, 2, a.pyr, a.w.in_tab, a.act16,
-                                                             a.dz16, a.grad + kOffW2, a.grad + kOffB2);
-    t_conv_bwd_data<16, 32><<<g2, blk, 0, s>>>(a.tl, 2, a.wr + kOffW2, a.dz16, a.act16, a.dz16);
-    t_conv_bwd_weight<1, 16, true><<<16, 256, 0, s>>>(a.tl, nl, a.levels, 1, a.pyr, a.w.in_tab, nullptr, a.dz16,
-                                                      a.grad + kOffW1, a.grad + kOffB1);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (a.lr > 0.f) {
-        t_adam<<<64, 256, 0, s>>>(a.master, a.m, a.v, a.grad, kCnnParams, a.lr, a.beta1, a.beta2, a.eps, a.c1, a.c2);
-        t_round<<<64, 256, 0, s>>>(a.master, a.wr, kCnnParams);
-        e = cudaGetLastError();
-    }
-    return e;
+    t_loss<<<dim3(kLossParts, nl), 256, 0, s>>>(a.tl, a.levels, a.logits, a.scores, a.label_thr, a.pos_weight, a.inv_n,
+                                                a.dz, a.level_loss);
+    t_pool_bwd_h<<<dim3(48, nl), blk, 0, s>>>(a.tl, a.levels, a.dz, a.wr + kOffV, a.dh, a.hp);
+    t_small_grads<<<G, blk, 0, s>>>(a.tl, nl, a.tiles[4], a.tiles[2], a.levels, a.dz, a.hmap, a.dh, a.hp, a.act32, ps);
+    t_dw23<32><<<G, blk, dw23_smem(32), s>>>(a.tl, nl, a.tiles[3], a.levels, a.act32, a.dh, a.hp, a.wr + kOffWh,
+                                             a.act16, nullptr, p3);
+    t_dz2<<<G, blk, kDz2Smem, s>>>(a.tl, nl, a.tiles[3], a.levels, a.act32, a.dh, a.hp, a.wr + kOffWh, a.wr + kOffW3,
+                                   a.act16, a.dz2);
+    t_dw23<16><<<G, blk, dw23_smem(16), s>>>(a.tl, nl, a.tiles[1], a.levels, nullptr, nullptr, 0, nullptr, a.act16,
+                                             a.dz2, p2);
+    t_dw1<<<G, blk, kDw1Smem, s>>>(a.tl, nl, a.tiles[0], a.levels, a.pyr, a.w.in_tab, a.wr + kOffW2, a.act16, a.dz2,
+                                   p1);
+    t_finish<<<(kCnnParams + 31) / 32, blk, 0, s>>>(p1, G, p2, G, p3, G, ps, G, a.grad, a.master, a.m, a.v, a.wr, a.lr,
+                                                    a.beta1, a.beta2, a.eps, a.c1, a.c2);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_round_params(cudaStream_t s, const float *master, float *wr) {

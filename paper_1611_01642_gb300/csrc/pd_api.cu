@@ -287,7 +287,7 @@ struct pd_handle {
     unsigned char *scheme_ws = nullptr;  // scratch of the paper's kernel schemes (grown on demand)
     size_t scheme_ws_bytes = 0;
     size_t train_ws_bytes = 0;
-    int train_levels = 0;
+    int train_losses = 0;
     float *train_loss_ptr = nullptr;
     // tensor maps over the atlases, one pair per K4 tile shape
     CUtensorMap hog_map[kSvmShapes]{}, lbp_map[kSvmShapes]{};
@@ -921,7 +921,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     if (cudaGetDevice(&h->device) != cudaSuccess) return bail(PD_ECUDA);
     if (init_resize() != cudaSuccess || init_cells() != cudaSuccess || init_cells_warp() != cudaSuccess ||
         init_svm() != cudaSuccess || init_svm_tc() != cudaSuccess ||
-        init_nms() != cudaSuccess ||
+        init_nms() != cudaSuccess || init_train() != cudaSuccess ||
         init_cnn() != cudaSuccess)
         return bail(PD_ECUDA);
 
@@ -1385,7 +1385,9 @@ int pd_cnn_train_step(pd_handle *h, void *stream, float pos_weight, float label_
     const Plan &p = h->plan;
     const int nl = (int)p.levels.size();
     std::vector<TrainLevel> tl(nl);
-    int64_t n16 = 0, n32 = 0, nwin = 0;
+    int64_t n16 = 0, n32 = 0, nd2 = 0, nwin = 0;
+    int32_t tiles[kTrainGrids] = {};
+    auto ceil_div = [](int a, int b) { return (a + b - 1) / b; };
     for (int k = 0; k < nl; ++k) {
         const LevelDesc &L = p.levels[k];
         TrainLevel &T = tl[k];
@@ -1393,18 +1395,31 @@ int pd_cnn_train_step(pd_handle *h, void *stream, float pos_weight, float label_
         T.H1 = (L.Hk + 1) / 2; T.W1 = (L.Wk + 1) / 2;
         T.H2 = (T.H1 + 1) / 2; T.W2 = (T.W1 + 1) / 2;
         T.H3 = (T.H2 + 1) / 2; T.W3 = (T.W2 + 1) / 2;
+        T.P1 = (int32_t)round_up(T.W1, 8);
+        T.P2 = (int32_t)round_up(T.W2, 8);
+        T.P3 = (int32_t)round_up(T.W3, 8);
         T.pad = 0;
-        T.a1 = n16; n16 += (int64_t)16 * T.H1 * T.W1;
-        T.a2 = n16; n16 += (int64_t)32 * T.H2 * T.W2;
-        T.a3 = n32; n32 += (int64_t)32 * T.H3 * T.W3;
+        const int n[kTrainGrids] = {ceil_div(T.W2, 32) * ceil_div(T.H2, 8), ceil_div(T.W2, 16) * ceil_div(T.H2, 8),
+                                    ceil_div(T.W3, 32) * ceil_div(T.H3, 8), ceil_div(T.W3, 16) * ceil_div(T.H3, 8),
+                                    ceil_div(L.cols, 32) * ceil_div(L.rows, 16)};
+        for (int g = 0; g < kTrainGrids; ++g) {
+            T.g[g] = tiles[g];
+            tiles[g] += n[g];
+        }
+        T.a1 = n16; n16 += (int64_t)16 * T.H1 * T.P1;
+        T.a2 = n16; n16 += (int64_t)32 * T.H2 * T.P2;
+        T.d2 = nd2; nd2 += (int64_t)32 * T.H2 * T.P2;
+        T.a3 = n32; n32 += (int64_t)32 * T.H3 * T.P3;
         nwin += (int64_t)L.rows * L.cols;
     }
     if (nwin == 0) return fail(h, PD_EINVAL, "batch has no window");
-    // workspace: tl | act16 (bf16) | act32 | dz16 | dz32 | dh plane | dz | level losses
+    // workspace: tl | act16 (bf16) | act32 | dz2 | dh plane | dz | partial losses | partial gradients
     const int64_t rows = h->atlas.rows, P = h->atlas.pitch;
+    const int64_t n_loss = (int64_t)nl * kLossParts, n_part = (int64_t)train_partial_floats();
     const size_t need = round_up((int64_t)nl * sizeof(TrainLevel), 256) + round_up(n16 * 2, 256) +
-                        round_up(n32 * 4, 256) + round_up(n16 * 4, 256) + round_up(n32 * 4, 256) +
-                        round_up(rows * P * 4, 256) + round_up(h->score_cap * 4, 256) + round_up((int64_t)nl * 4, 256);
+                        round_up(n32 * 4, 256) + round_up(nd2 * 4, 256) +
+                        round_up(rows * P * 4, 256) + round_up(h->score_cap * 4, 256) + round_up(n_loss * 4, 256) +
+                        round_up(n_part * 4, 256);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (need > h->train_ws_bytes) {
         PD_CUDA(h, cudaStreamSynchronize(s));
@@ -1424,11 +1439,12 @@ int pd_cnn_train_step(pd_handle *h, void *stream, float pos_weight, float label_
     a.tl = reinterpret_cast<TrainLevel *>(take((int64_t)nl * sizeof(TrainLevel)));
     a.act16 = reinterpret_cast<__nv_bfloat16 *>(take(n16 * 2));
     a.act32 = reinterpret_cast<float *>(take(n32 * 4));
-    a.dz16 = reinterpret_cast<float *>(take(n16 * 4));
-    a.dz32 = reinterpret_cast<float *>(take(n32 * 4));
+    a.dz2 = reinterpret_cast<float *>(take(nd2 * 4));
     a.dh = reinterpret_cast<float *>(take(rows * P * 4));
     a.dz = reinterpret_cast<float *>(take(h->score_cap * 4));
-    a.level_loss = reinterpret_cast<float *>(take((int64_t)nl * 4));
+    a.level_loss = reinterpret_cast<float *>(take(n_loss * 4));
+    a.part = reinterpret_cast<float *>(take(n_part * 4));
+    for (int g = 0; g < kTrainGrids; ++g) a.tiles[g] = tiles[g];
     PD_CUDA(h, cudaMemcpyAsync((void *)a.tl, tl.data(), tl.size() * sizeof(TrainLevel), cudaMemcpyHostToDevice, s));
     PD_CUDA(h, cudaStreamSynchronize(s));  // the host vector goes out of scope
     a.n_levels = nl;
@@ -1458,7 +1474,7 @@ int pd_cnn_train_step(pd_handle *h, void *stream, float pos_weight, float label_
         a.c2 = 1.0f - (float)std::pow(0.999, h->adam_t);
         h->frag_stale = true;
     }
-    h->train_levels = nl;
+    h->train_losses = (int)n_loss;
     h->train_loss_ptr = a.level_loss;
     PD_CUDA(h, launch_train_step(s, a));
     return PD_OK;
@@ -1466,11 +1482,11 @@ int pd_cnn_train_step(pd_handle *h, void *stream, float pos_weight, float label_
 
 int pd_cnn_train_loss(pd_handle *h, void *stream, float *loss) {
     if (!h || !loss) return PD_EINVAL;
-    if (!h->train_ws || h->train_levels <= 0) return fail(h, PD_ESTATE, "no training step yet");
+    if (!h->train_ws || h->train_losses <= 0) return fail(h, PD_ESTATE, "no training step yet");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     PD_CUDA(h, cudaStreamSynchronize(s));
-    // one partial loss per level (already weighted by its share of the windows)
-    std::vector<float> ll(h->train_levels);
+    // partial losses of every level (already weighted by their share of the windows)
+    std::vector<float> ll(h->train_losses);
     PD_CUDA(h, cudaMemcpy(ll.data(), h->train_loss_ptr, ll.size() * 4, cudaMemcpyDeviceToHost));
     double sum = 0;
     for (float v : ll) sum += v;

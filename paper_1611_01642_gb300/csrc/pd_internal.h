@@ -204,12 +204,20 @@ struct CnnWeights {
     const float *v, *bv;      // [16][8], [1]
 };
 
+// One level of a training batch. Tile grids (first tile of the level in each; row
+// pitches P are widths rounded up to 8 elements):
+//   g[0] 32 x 8 layer-2 positions, g[1] 16 x 8 of them, g[2] 32 x 8 layer-3
+//   positions, g[3] 16 x 8 of them, g[4] 32 x 16 windows.
+constexpr int kTrainGrids = 5;
 struct TrainLevel {
     int32_t level;            // index in the LevelDesc table
-    int32_t H1, W1, H2, W2, H3, W3;
+    int32_t H1, W1, P1, H2, W2, P2, H3, W3, P3;
+    int32_t g[kTrainGrids];
     int32_t pad;
-    int64_t a1, a2, a3;       // element offsets: a1, a2 in the bf16 buffer, a3 in the f32 buffer
+    int64_t a1, a2, a3, d2;   // element offsets: a1, a2 in the bf16 buffer, a3 and d2 in f32 buffers
 };
+constexpr int kTrainBlocks = 304;  // persistent blocks of the training kernels (partials per weight)
+constexpr int kLossParts = 8;      // partial losses per level
 
 struct TrainArgs {
     const TrainLevel *tl;
@@ -220,7 +228,9 @@ struct TrainArgs {
     float *wr;                // rounded working copy [kCnnParams]
     float *master, *m, *v, *grad;
     __nv_bfloat16 *act16;
-    float *act32, *dz16, *dz32;
+    float *act32, *dz2;
+    float *part;              // train_partial_floats() of weight-gradient partials
+    int32_t tiles[kTrainGrids];
     float *hmap, *dh;
     int32_t hp;
     float *logits;
@@ -245,6 +255,8 @@ constexpr int kCnnBoxW = 96, kCnnBoxH = 72;
 cudaError_t launch_cnn(cudaStream_t s, const LevelDesc *d_levels, int n_levels, const CUtensorMap *lvl_maps,
                        const CnnItem *d_items, int n_items, const CnnWeights &w, float *hmap,
                        int32_t hmap_pitch, float *logits, int pool_tiles, unsigned *err);
+cudaError_t init_train();
+size_t train_partial_floats();
 cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a);
 cudaError_t launch_round_params(cudaStream_t s, const float *master, float *wr);
 
