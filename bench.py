@@ -202,9 +202,10 @@ def cells_per_frame() -> int:
     return sum((wk // 8) * (hk // 8) for wk, hk in pd_pyramid(WIDTH, HEIGHT, FACTOR))
 
 
-def tc_units_per_frame() -> int:
-    """Block rows the tensor-core K4 walks per frame: strips of 104 window columns, each cut into
-    pieces of at most 64 window rows, each piece also walking the 14 block rows below it."""
+def tc_units_per_frame() -> float:
+    """MMA steps of the tensor-core K4 per frame: strips of 26 window columns, each cut into pieces of
+    at most 64 window rows; a piece of n rows walks n + 15 cell rows, and a step takes one cell row of
+    four pieces."""
     from paper_1611_01642_gb300 import pd_pyramid
     n = 0
     for wk, hk in pd_pyramid(WIDTH, HEIGHT, FACTOR):
@@ -212,8 +213,8 @@ def tc_units_per_frame() -> int:
         if rows <= 0 or cols <= 0:
             continue
         pieces = -(-rows // 64)
-        n += -(-cols // 104) * (rows + 14 * pieces)
-    return n
+        n += -(-cols // 26) * (rows + 15 * pieces)
+    return n / 4
 
 
 def windows_per_frame(upscale: int = 0) -> int:

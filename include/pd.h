@@ -206,9 +206,10 @@ int pd_last_launch_count(const pd_handle *h);
  *                 pyramid kernel: 4, 8 or 16; a warp's 32 lanes are
  *                 k1_groups groups x 32 / k1_groups row slices (default 8);
  *   tc_item_rows  window rows per work item of the tensor-core score kernel,
- *                 8 .. 64: a 104-window strip is cut into near-equal pieces
+ *                 8 .. 64: a 26-window strip is cut into near-equal pieces
  *                 of at most this many rows, each piece also reading the 14
- *                 block rows below its last window row (default 64).
+ *                 block rows below its last window row (default 64). Plans too
+ *                 small to give every SM work are cut finer than this.
  * Results do not depend on them: every output is the same sum in the same
  * order. Errors: PD_EINVAL. Affects the next pd_detect. */
 typedef struct pd_tuning {

@@ -386,6 +386,11 @@ __global__ void __launch_bounds__(kThreads) k_cells(const LevelDesc *__restrict_
                 const uint32_t v = S.cnt[cyl & 1][cxo][wd];
                 S.cnt[cyl & 1][cxo][wd] = 0u;  // recycled for cell row cyl + 2
                 if (cx >= Wc) continue;
+                if (atlas.lbp_cells) {  // two bins of the cell's 64 bytes
+                    reinterpret_cast<uint16_t *>(atlas.lbp + (row + cx) * kLbpCellBytes)[wd] =
+                        (uint16_t)((v & 0xffu) | ((v >> 8) & 0xff00u));
+                    continue;
+                }
                 atlas.lbp[(int64_t)(2 * wd) * atlas.lbp_plane + row + cx] = (uint8_t)(v & 0xffffu);
                 if (2 * wd + 1 < kLbpBins)
                     atlas.lbp[(int64_t)(2 * wd + 1) * atlas.lbp_plane + row + cx] = (uint8_t)(v >> 16);

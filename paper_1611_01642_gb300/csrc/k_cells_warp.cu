@@ -58,8 +58,9 @@
 // HOG epilogue of cell row r: each lane forms, per bin, the weighted sums of
 // its 4 columns for its own cell and for the neighbouring cell they reach;
 // three shuffles add the 4 lanes that reach a cell (fixed order:
-// deterministic). The LBP counts go out bin-plane by bin-plane, one byte per
-// cell, lanes on consecutive cells (coalesced). At the top and bottom of a
+// deterministic). The LBP counts of a cell go out as 64 bytes, two 16-byte
+// stores per lane (the counter words are already four bins each), or, for
+// callers that ask for planes, bin-plane by bin-plane. At the top and bottom of a
 // level the votes of the clamped cell row (Algorithm 5's interpolation
 // clamped into the grid) are added into the first and last row before they
 // are written. The result does not depend on the strip height: every cell
@@ -154,7 +155,7 @@ __device__ __forceinline__ uint32_t ge4(uint32_t n, uint32_t c_lo, uint32_t c_no
     return (n7 & c_not7) | (t & (n7 | c_not7));
 }
 
-template <int FEAT>
+template <int FEAT, bool CELLS>  // CELLS: cell-major LBP counts
 __global__ void __launch_bounds__(kWarps * 32, 4)
     k_cells_warp(const LevelDesc *__restrict__ levels, const uint8_t *__restrict__ pyr, CellAtlas atlas,
                  const StripItem *__restrict__ items, int n_items, int *__restrict__ queue,
@@ -315,7 +316,20 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
             __syncwarp();  // every lane's counts of row r are in
             const int r = band - 1;
             const int c = lane & 15, half = lane >> 4;
-            if (walked && need(r) && c < kCellTW && cx0 + c < Wc) {
+            if (CELLS) {
+                // words 8 half .. 8 half + 7 of cell c: 32 bytes (the last word is padding)
+                if (walked && need(r) && c < kCellTW && cx0 + c < Wc) {
+                    const uint32_t *cw = Wm.cnt + half * 8 * 32 + 2 * c + 1;
+                    uint32_t v[8];
+#pragma unroll
+                    for (int i = 0; i < 7; ++i) v[i] = cw[i * 32] + cw[i * 32 + 1];  // counts <= 32 each: no carry
+                    v[7] = half ? 0u : cw[7 * 32] + cw[7 * 32 + 1];
+                    uint4 *dst = reinterpret_cast<uint4 *>(
+                        atlas.lbp + ((int64_t)(L.cell_row + cy0 + r) * atlas.pitch + cx0 + c) * kLbpCellBytes + 32 * half);
+                    dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
+                    dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
+                }
+            } else if (walked && need(r) && c < kCellTW && cx0 + c < Wc) {
                 const int64_t pl = atlas.lbp_plane;
                 // bin planes 32 half .. 32 half + 31 of cell c
                 uint8_t *dst = atlas.lbp + (int64_t)(L.cell_row + cy0 + r) * atlas.pitch + cx0 + c + 32 * half * pl;
@@ -468,8 +482,10 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
 
 using StripFn = void (*)(const LevelDesc *, const uint8_t *, CellAtlas, const StripItem *, int, int *,
                          const uint8_t *, const uint32_t *);
-const StripFn kStripFns[3] = {k_cells_warp<kFeatHog | kFeatLbp>, k_cells_warp<kFeatHog>,
-                              k_cells_warp<kFeatLbp>};
+// [feature set][cell-major LBP counts]; without LBP the layout does not matter
+const StripFn kStripFns[3][2] = {{k_cells_warp<kFeatHog | kFeatLbp, false>, k_cells_warp<kFeatHog | kFeatLbp, true>},
+                                 {k_cells_warp<kFeatHog, false>, k_cells_warp<kFeatHog, false>},
+                                 {k_cells_warp<kFeatLbp, false>, k_cells_warp<kFeatLbp, true>}};
 
 int strip_fn_index(int feat) {
     if (feat == kFeatHog) return 1;
@@ -480,9 +496,9 @@ int strip_fn_index(int feat) {
 }  // namespace
 
 cudaError_t init_cells_warp() {
-    for (int i = 0; i < 3; ++i) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(kStripFns[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StripSmem));
+    for (int i = 0; i < 6; ++i) {
+        const cudaError_t e = cudaFuncSetAttribute(kStripFns[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)sizeof(StripSmem));
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -496,8 +512,8 @@ cudaError_t launch_cells_warp(cudaStream_t s, const LevelDesc *d_levels, const u
     // small plan gets one CTA per strip, so that its warps spread over the SMs.
     static_assert(kWarps * 4 == kStripWarpsPerSm, "resident warps per SM");
     const int grid = std::min(n_items, 4 * sm_count);
-    kStripFns[strip_fn_index(feat)]<<<grid, kWarps * 32, sizeof(StripSmem), s>>>(d_levels, pyr, atlas, d_items,
-                                                                                 n_items, d_queue, d_lbp_map, c_flag);
+    kStripFns[strip_fn_index(feat)][atlas.lbp_cells != 0]<<<grid, kWarps * 32, sizeof(StripSmem), s>>>(
+        d_levels, pyr, atlas, d_items, n_items, d_queue, d_lbp_map, c_flag);
     return cudaGetLastError();
 }
 

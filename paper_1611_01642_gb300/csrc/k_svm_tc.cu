@@ -5,110 +5,134 @@
 // with f[by][bx] the 95-value block feature (36 L2-Hys HOG values of the 2x2
 // cells, then the 59 L1-sqrt LBP values of their summed counts).
 //
-// Per block row r of a level this is one GEMM: P[bx][(i, j)] =
-// < f[r][bx], w[i][j] > for all 105 template positions (M = blocks of the
-// row, N = 105 padded to 112, K = 95 padded to 96). Window (wy, wx) then
-// collects P_{wy+i}[wx+j][(i, j)] over its 15 x 7 positions: the j terms
-// come from the 7 neighbouring blocks of one block row, the i terms from 15
-// consecutive block rows. The GEMM runs on tcgen05 (bf16 operands, fp32
-// accumulators in tensor memory); fp32 accuracy is kept by splitting both
-// operands into bf16 high and low parts, x = xh + xl and w = wh + wl, and
-// summing xh.wh + xl.wh + xh.wl (K = 3 x 96; the dropped xl.wl and the
-// rounding of the low parts are below 2^-16 of |x w| per term).
+// Per block row r this is one GEMM: P[bx][(i, j)] = < f[r][bx], w[i][j] > for
+// all 105 template positions (M = blocks, N = 105 padded to 112, K = 95 padded
+// to 96). Window (wy, wx) then collects P_{wy+i}[wx+j][(i, j)] over its 15 x 7
+// positions: the j terms come from the 7 neighbouring blocks of one block row,
+// the i terms from 15 consecutive block rows. The GEMM runs on tcgen05 (bf16
+// operands, fp32 accumulators in tensor memory); fp32 accuracy is kept by
+// splitting both operands into bf16 high and low parts, x = xh + xl and
+// w = wh + wl, and summing xh.wh + xl.wh + xh.wl (K = 3 x 96; the dropped
+// xl.wl and the rounding of the low parts are below 2^-16 of |x w| per term).
 //
-// One persistent CTA per SM takes items from a queue: an item is a strip of
-// up to 104 window columns and up to 64 window rows of one level, walked one
-// block row at a time by a warp-specialised pipeline (mbarriers between the
-// roles, bounded waits):
-//  * 8 producer warps: first all of them replace a staged row's LBP counts
-//    by sums of horizontally adjacent cells (in place); then they write the
-//    A operand straight into tensor memory (tcgen05.st: row m = lane m, two
-//    bf16 per column), row m holding block wx0 + 26 (m / 32) + m % 32: warps
-//    0-3 the 36 values of its 2x2 HOG cells (L2-Hys, bf16 split) and LBP
-//    bins 0..9, warps 4-7 LBP bins 10..58 (the 2 x 2 count sums, L1-sqrt
-//    and its bf16 split from a 512-entry table; the split balances the two
-//    groups' work per row). Every group of 32 rows
-//    covers 26 windows and the 6 blocks to their right, so the j terms of a
-//    window stay inside one warp of the epilogue;
-//  * one thread (lane 0 of the first epilogue warp, between its epilogue
-//    rows) issues the TMA (cp.async.bulk.tensor.3d) of cell rows into a ring
-//    of four slots (the 9 HOG planes, f32, and the 59 LBP count planes, u8,
-//    of the strip's 112 + 16 cells) and the 18 MMAs of every block row (A in
-//    tensor memory, the template's B operand K-major no-swizzle canonical in
-//    shared memory, D in one of two 128-column TMEM buffers), committed to
-//    the A-free and D-full barriers;
-//  * 4 epilogue warps (warp e reads TMEM lanes 32 e .. 32 e + 31): lane l adds
-//    P[l + j][(i, j)] (a shuffle by j) to the running score of window row
-//    r - i, for all 105 positions, in the fixed order (i, j) = (0,0), (0,1),
-//    ..., so every score is b plus its terms in one order whatever the item
-//    cut; window row r - 14 is complete and stored.
-// The A operand (two 96-column TMEM stages) and the accumulators are double
-// buffered, so the producers build row r + 1 and the epilogue reads row
-// r - 1 while row r's MMAs run.
+// One persistent CTA per SM. Its 128 MMA rows are four groups of 32 (a TMEM
+// lane quarter each), and every group walks its own items: up to 26 window
+// columns (32 blocks, 33 cells) and up to 64 window rows of one level, one
+// cell row per step. The groups share a step's MMAs and nothing else, so a
+// level's width is padded to 26 columns and not to 104 (23 levels of a
+// 1242x375 frame: 89 groups of work instead of 4 x 30), and items of any
+// level or frame run side by side. The roles (mbarriers between them, bounded
+// waits):
+//  * warp 13, lane g: the items of group g (the first by its place in the
+//    grid, the next ones from a queue), its TMA (cp.async.bulk.tensor.3d) of
+//    one cell row per step into a ring of slots (9 HOG planes, f32, of 36
+//    cells from a 4-cell boundary; 33 cells x 64 LBP count bytes, 64-byte
+//    swizzle), and the step's description for the other roles;
+//  * warps 0-3 (group = warp): 36 L2-Hys HOG values per block, warps 4-7 its
+//    59 LBP values, written as bf16 high and low parts straight into the A
+//    operand in tensor memory (tcgen05.st: row m = lane m, two bf16 per
+//    column). A block needs two cell rows; the upper one stays in registers
+//    from the step before, so every cell is read from shared memory once. LBP
+//    counts are cell-major: a lane reads its cell's bins 16 at a time and adds
+//    four at once, and a 512-entry table gives the bf16 split of the L1-sqrt;
+//  * warp 12, one thread: the 18 MMAs of every step (A in tensor memory, the
+//    template's B operand K-major no-swizzle canonical in shared memory, D in
+//    one of two 128-column TMEM buffers), committed to the A-free and D-full
+//    barriers;
+//  * warps 8-11 (group = warp - 8): lane l adds P[l + j][(i, j)] (a shuffle by
+//    j) to the running score of window row r - i, for all 105 positions, in
+//    the fixed order (i, j) = (0,0), (0,1), ..., so every score is b plus its
+//    terms in one order whatever the item cut; window row r - 14 is complete
+//    and stored.
+// A and D are double buffered: the producers build step s + 1 and the epilogue
+// reads step s - 1 while step s's MMAs run.
+// What bounds it: a step takes about 2,350 cycles, its MMAs 1,010 of them; the
+// schedulers issue on 53% of cycles and the shared-memory pipe is 51% busy, so
+// it is the latency of the hand-offs between the roles, with 3.5 warps per
+// scheduler. 64 x 1242x375 frames: 0.352 ms; 0.661 ms with one strip of 104
+// columns per CTA, LBP planes read a byte per bin and summed in place, and a
+// single warp issuing the MMAs between its epilogue rows (3,400 cycles per
+// row, 901 rows per frame; now 693 steps). One 1242x375 frame: 84 -> 31 us,
+// with items cut until every SM has work (see the planner). 14 warps leave 128
+// registers per thread (4 warps on a scheduler), which the epilogue's loads
+// are staged for.
 // Per-block HOG (Algorithm 5 read per block): each staged cell row holds 36
 // HOG planes, the cell's 4 block-restricted histograms (plane 9 q + bin, q =
-// its place in the block); a block takes q = 0, 1 from row r and q = 2, 3
-// from row r + 1, and nothing else changes.
-// Sparse path: a window is scored when every cell tile under it was
-// computed; block rows that no such window needs are skipped, other windows
-// get -inf. A wait that gives up (1 s) sets the error word and a CTA flag
-// that ends every role's waits; the CTA then drains its copies and MMAs,
-// frees its tensor memory and leaves.
+// its place in the block); a block takes q = 0, 1 from its upper row and
+// q = 2, 3 from its lower one, and nothing else changes.
+// Sparse path: a window is scored when every cell tile under it was computed;
+// cell rows that no such window of the item needs are skipped, other windows
+// get -inf. A wait that gives up (1 s) sets the error word and a CTA flag that
+// ends every role's waits; the CTA then drains its copies and MMAs, frees its
+// tensor memory and leaves.
 #include "pd_internal.h"
 
 #include <cuda_bf16.h>
 
+#include <cstring>
+#include <vector>
+
+#include "f32x2.cuh"
+
 namespace pd {
 namespace {
 
-constexpr int kWarps = 12;            // 4 HOG, 4 LBP, 4 epilogue (one thread of which also issues)
-constexpr int kProducers = 8;         // producer warps
+constexpr int kWarps = 14;            // 4 HOG, 4 LBP, 4 epilogue, MMA issue, items and TMA
 constexpr int kThreads = 32 * kWarps;
+constexpr int kGroups = 4;            // lane quarters of the A operand
 constexpr int kM = 128;               // A rows = TMEM lanes
 constexpr int kN = 112;               // 105 template positions, padded
-constexpr int kWinPerWarp = 26;
 constexpr int kChunks = 24;           // 16-byte K chunks per operand row: 12 high + 12 low
 constexpr int kSBO = kChunks * 128;   // bytes per 8-row group
-constexpr int kHogX = 112;            // HOG cells per staged row (TMA box width)
-constexpr int kLbpX = 128;            // LBP cells per staged row (box width, from a 16-cell boundary)
-constexpr int kSlots = 4;
+constexpr int kHogX = 36;             // HOG cells per staged row of a group (from a 4-cell boundary)
+constexpr int kLbpX = 33;             // LBP cells per staged row of a group
+constexpr int kTileRows = (kTcChunk - 1 + kWinBH) / kCellTH + 2;  // cell-tile rows under an item at most
+static_assert(kTileRows <= 32 && kWinBW < kCellTW && kWinBH < 2 * kCellTH, "sparse masks");
+constexpr int kMeta = 16;             // step descriptions in flight (more than any role can lag behind)
 constexpr uint32_t kTmemCols = 512;   // two accumulator buffers of 128 columns, two A stages of 96
 constexpr uint32_t kTmemA = 256;      // first A stage column (bf16 pairs: high parts 0..47, low 48..95)
 constexpr uint64_t kWaitNs = 1000000000ull;
-constexpr int kProducerBarrier = 1;   // named barrier of the producer warps
-constexpr int kHogLbpPairs = 5;       // LBP bin pairs built by the HOG warps (the LBP warps take the rest)
-static_assert(4 * kWinPerWarp == kTcStrip, "strip width");
-static_assert(kWinPerWarp + kWinBW - 1 <= 32, "window blocks inside a warp");
+constexpr int kBBytes = 14 * kSBO;    // B operand: template high | low parts
+constexpr int kTabBytes = 512 * 4;    // sum of 4 cell counts -> bf16 high | low << 16 of sqrt(S / 256)
+static_assert(kTcStrip + kWinBW - 1 <= 32, "a window's blocks inside a group");
+static_assert(kBBytes + kTabBytes == kTcConstBytes, "constant block");
 
 template <int HP>  // HOG planes per cell row: 9, or 36 for per-block HOG
 struct SlotT {
-    static constexpr int kPlanes = HP;
-    float hog[HP][kHogX];                       // 4032 B (16128 B per-block)
-    alignas(128) uint8_t lbp[kLbpBins][kLbpX];  // 7552 B
-    uint8_t pad1[128];
+    static constexpr int kHogBytes = (HP * kHogX * 4 + 127) / 128 * 128;
+    uint8_t lbp[kGroups][2560];            // 33 cells x 64 bytes, swizzled; a 512-byte multiple per group
+    uint8_t hog[kGroups][kHogBytes];       // [HP][36] floats
 };
-static_assert(sizeof(SlotT<9>) == 11776 && offsetof(SlotT<9>, lbp) == 4096, "slot layout");
-static_assert(sizeof(SlotT<36>) % 128 == 0 && offsetof(SlotT<36>, lbp) % 128 == 0, "TMA destinations");
+static_assert(sizeof(SlotT<9>) % 512 == 0 && sizeof(SlotT<36>) % 512 == 0, "TMA destinations");
+
+// What a step is for one group. kind: 0 idle, 1 an item's (or run's) first
+// cell row (no block row yet), 2 a block row, 3 no more steps.
+struct StepMeta {
+    uint32_t flags;  // kind | store << 2 | HOG x offset << 4 | window columns << 8
+    uint32_t keep;   // windows of the stored row that are scored (others: -inf)
+    int64_t out;     // score index of the stored row's first window
+};
 
 template <int HP>
 struct TcSmemT {
-    uint8_t b[14 * kSBO];             // B operand: template high | low parts
-    SlotT<HP> slot[kSlots];           // staged cell rows
-    uint32_t tab[512];                // sum of 4 cell counts -> bf16 high | low << 16 of sqrt(S / 256)
-    uint32_t win_ok[kTcChunk][4];     // sparse: window of the strip is scored
-    uint8_t row_ok[kTcChunk];         // sparse: window row holds a scored window
-    uint8_t tflag[16][16];            // sparse: cell-tile flags of the item's region
-    unsigned long long cfull[kSlots];   // cell row arrived (TMA transaction count)
-    unsigned long long cempty[kSlots];  // cell row no longer read (8 producer warps)
-    unsigned long long afull[2];        // A operand written (8 producer warps)
-    unsigned long long aempty[2];       // A operand read by the MMAs (commit)
-    unsigned long long dfull[2];        // accumulators written (commit)
-    unsigned long long dempty[2];       // accumulators read (4 epilogue warps)
+    static constexpr int kSlots = HP == 9 ? 6 : 4;
+    uint8_t b[kBBytes];
+    uint32_t tab[512];
+    SlotT<HP> slot[kSlots];               // staged cell rows
+    StepMeta meta[kMeta][kGroups];
+    uint32_t keep[kGroups][kTcChunk];     // sparse: scored windows of an item's rows
+    unsigned long long bfull;             // constants arrived
+    unsigned long long cfull[kSlots];     // cell row arrived (TMA transaction count)
+    unsigned long long cempty[kSlots];    // cell row no longer read (8 producer warps)
+    unsigned long long mready[kMeta];     // step description written
+    unsigned long long afull[2];          // A operand written (8 producer warps)
+    unsigned long long aempty[2];         // A operand read by the MMAs (commit)
+    unsigned long long dfull[2];          // accumulators written (commit)
+    unsigned long long dempty[2];         // accumulators read (4 epilogue warps)
     uint32_t tmem;
-    int item;
     volatile int failed;
 };
-static_assert(offsetof(TcSmemT<9>, slot) % 128 == 0 && offsetof(TcSmemT<36>, slot) % 128 == 0, "alignment");
+static_assert(offsetof(TcSmemT<9>, slot) % 512 == 0 && offsetof(TcSmemT<36>, slot) % 512 == 0, "alignment");
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -152,6 +176,9 @@ __device__ __forceinline__ void drain_wait(unsigned long long *bar, uint32_t par
 __device__ __forceinline__ void arrive(unsigned long long *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+__device__ __forceinline__ void arrive_tx(unsigned long long *bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void tma_3d(void *dst, const CUtensorMap *map, unsigned long long *bar, int x, int y,
                                        int z) {
     asm volatile(
@@ -183,17 +210,25 @@ __device__ __forceinline__ void umma_commit(unsigned long long *bar) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-#define PD_LD_X16(taddr, v, o)                                                                             \
+#define PD_LD_X16(taddr, v)                                                                                \
     asm volatile(                                                                                          \
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "  \
         "[%16];"                                                                                           \
-        : "=f"(v[o + 0]), "=f"(v[o + 1]), "=f"(v[o + 2]), "=f"(v[o + 3]), "=f"(v[o + 4]), "=f"(v[o + 5]),   \
-          "=f"(v[o + 6]), "=f"(v[o + 7]), "=f"(v[o + 8]), "=f"(v[o + 9]), "=f"(v[o + 10]), "=f"(v[o + 11]), \
-          "=f"(v[o + 12]), "=f"(v[o + 13]), "=f"(v[o + 14]), "=f"(v[o + 15])                                \
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),   \
+          "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]),          \
+          "=f"(v[15])                                                                                      \
         : "r"(taddr))
+// waits for the loads so far; names the registers so that nothing reads them earlier
+#define PD_WAIT_X16(v)                                                                                     \
+    asm volatile("tcgen05.wait::ld.sync.aligned;"                                                          \
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]),      \
+                   "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), \
+                   "+f"(v[14]), "+f"(v[15])::"memory")
 
-// bf16 high and low parts of two floats, packed (first float in the low half)
-__device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t &lo) {
+// bf16 high and low parts of a pair of floats, packed (first float in the low half)
+__device__ __forceinline__ void split2(f32x2 x, uint32_t &hi, uint32_t &lo) {
+    float a, b;
+    unpack2(x, a, b);
     uint32_t h, l;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(b), "f"(a));
     const float ah = __uint_as_float(h << 16), bh = __uint_as_float(h & 0xffff0000u);
@@ -201,10 +236,7 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t 
     hi = h;
     lo = l;
 }
-// this thread's TMEM lane: 4, 8 or 16 consecutive 32-bit columns from taddr
-__device__ __forceinline__ void tst1(uint32_t t, const uint32_t *v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(t), "r"(v[0]) : "memory");
-}
+// this thread's TMEM lane: 2, 4, 8 or 16 consecutive 32-bit columns from taddr
 __device__ __forceinline__ void tst2(uint32_t t, const uint32_t *v) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};" ::"r"(t), "r"(v[0]), "r"(v[1]) : "memory");
 }
@@ -226,126 +258,85 @@ __device__ __forceinline__ void tst16(uint32_t t, const uint32_t *v) {
         : "memory");
 }
 
-// LBP features of A row m for bins [T0, T0 + 2 NP) (bin 59 is the zero pad):
-// the staged rows hold sums of horizontally adjacent cells, so cells
-// (r, c..c+1) + (r+1, c..c+1) are two loads; the table gives the bf16 split
-// of sqrt(S / 256), packed two bins per word.
-template <int T0, int NP, class Slot>
-__device__ __forceinline__ void lbp_pairs(const Slot &s0, const Slot &s1, const uint32_t *tab, int c, uint32_t *hi,
-                                          uint32_t *lo) {
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        const int t = T0 + 2 * p;
-        const uint32_t e0 = tab[(uint32_t)s0.lbp[t][c] + (uint32_t)s1.lbp[t][c]];
-        const uint32_t e1 = t + 1 < kLbpBins ? tab[(uint32_t)s0.lbp[t + 1][c] + (uint32_t)s1.lbp[t + 1][c]] : 0u;
-        hi[p] = __byte_perm(e0, e1, 0x5410);
-        lo[p] = __byte_perm(e0, e1, 0x7632);
-    }
-}
-
-// Features 0..45 of A row m into its TMEM lane (columns a + f / 2 for the high
-// parts, a + 48 + f / 2 for the low parts): the 36 HOG values of its cells
-// (r, c), (r, c+1), (r+1, c), (r+1, c+1) (slots s0 = row r, s1 = row r + 1) in
-// the template's order (cells TL, TR, BL, BR, 9 bins each), L2-Hys, bf16
-// split; then LBP bins 0..9 (LBP column cl).
-template <class Slot>
-__device__ __forceinline__ void build_hog(const Slot &s0, const Slot &s1, const uint32_t *tab, int c, int cl,
-                                          float clip, uint32_t a) {
-    constexpr int pq = Slot::kPlanes == 36 ? kHogBins : 0;  // per-block: plane set of the cell's place
-    float v[36];
-#pragma unroll
-    for (int b = 0; b < kHogBins; ++b) {
-        v[b] = s0.hog[b][c];
-        v[9 + b] = s0.hog[pq + b][c + 1];
-        v[18 + b] = s1.hog[2 * pq + b][c];
-        v[27 + b] = s1.hog[3 * pq + b][c + 1];
-    }
+// The 36 HOG values of A row m into its TMEM lane (columns a + f / 2 for the
+// high parts, a + 48 + f / 2 for the low parts): cells (r, c), (r, c+1),
+// (r+1, c), (r+1, c+1) in the template's order (TL, TR, BL, BR, 9 bins each),
+// L2-Hys, bf16 split.
+__device__ __forceinline__ void build_hog(const float (&x)[36], float clip, uint32_t a) {
     // sums of squares in four interleaved partial sums (independent chains)
-    float q[4] = {0.f, 0.f, 0.f, 0.f};
+    f32x2 v[18], q01 = 0ull, q23 = 0ull;
 #pragma unroll
-    for (int t = 0; t < 36; ++t) q[t & 3] = fmaf(v[t], v[t], q[t & 3]);
-    const float i1 = rsqrtf((q[0] + q[1]) + (q[2] + q[3]) + 1.0f);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) q[k] = 0.f;
-#pragma unroll
-    for (int t = 0; t < 36; ++t) {
-        v[t] = fminf(v[t] * i1, clip);
-        q[t & 3] = fmaf(v[t], v[t], q[t & 3]);
+    for (int t = 0; t < 18; ++t) {
+        v[t] = pack2(x[2 * t], x[2 * t + 1]);
+        f32x2 &q = t & 1 ? q23 : q01;
+        q = fma2(v[t], v[t], q);
     }
-    const float i2 = rsqrtf((q[0] + q[1]) + (q[2] + q[3]) + 1e-6f);
-    uint32_t hi[16], lo[16];
+    const float i1 = rsqrtf((lo2(q01) + hi2(q01)) + (lo2(q23) + hi2(q23)) + 1.0f);
+    const f32x2 i11 = dup2(i1);
+    q01 = q23 = 0ull;
 #pragma unroll
-    for (int p = 0; p < 16; ++p) split2(v[2 * p] * i2, v[2 * p + 1] * i2, hi[p], lo[p]);
-    tst16(a, hi);        // features 0..31
+    for (int t = 0; t < 18; ++t) {
+        float p, r;
+        unpack2(mul2(v[t], i11), p, r);
+        v[t] = pack2(fminf(p, clip), fminf(r, clip));
+        f32x2 &q = t & 1 ? q23 : q01;
+        q = fma2(v[t], v[t], q);
+    }
+    const float i2 = rsqrtf((lo2(q01) + hi2(q01)) + (lo2(q23) + hi2(q23)) + 1e-6f);
+    const f32x2 i22 = dup2(i2);
+    uint32_t hi[18], lo[18];
+#pragma unroll
+    for (int t = 0; t < 18; ++t) split2(mul2(v[t], i22), hi[t], lo[t]);
+    tst16(a, hi);
+    tst2(a + 16, hi + 16);
     tst16(a + 48, lo);
-    // features 32..35 (HOG) and the first kHogLbpPairs LBP bin pairs
-    split2(v[32] * i2, v[33] * i2, hi[0], lo[0]);
-    split2(v[34] * i2, v[35] * i2, hi[1], lo[1]);
-    static_assert(kHogLbpPairs == 5, "TMEM column split");
-    lbp_pairs<0, kHogLbpPairs>(s0, s1, tab, cl, hi + 2, lo + 2);  // columns 16..22
-    tst4(a + 16, hi);
-    tst2(a + 20, hi + 4);
-    tst1(a + 22, hi + 6);
-    tst4(a + 64, lo);
-    tst2(a + 68, lo + 4);
-    tst1(a + 70, lo + 6);
+    tst2(a + 64, lo + 16);
 }
 
-// Features 46..95 of A row m (LBP bins 10..58 and the zero pad): columns
-// a + 23 .. a + 47 and a + 71 .. a + 95.
-template <class Slot>
-__device__ __forceinline__ void build_lbp(const Slot &s0, const Slot &s1, const uint32_t *tab, int cl, uint32_t a) {
-    uint32_t hi[25], lo[25];
-    lbp_pairs<2 * kHogLbpPairs, 30 - kHogLbpPairs>(s0, s1, tab, cl, hi, lo);  // bins 10..59: columns 23..47
-    tst1(a + 23, hi);
-    tst8(a + 24, hi + 1);
-    tst16(a + 32, hi + 9);
-    tst1(a + 71, lo);
-    tst8(a + 72, lo + 1);
-    tst16(a + 80, lo + 9);
-}
-
-// In place, by the 256 producer threads: LBP count c[t][x] -> c[t][x] +
-// c[t][x + 1] (x < 127) of a staged row. A warp takes whole plane rows (word
-// k of the row per lane), all its loads first; counts are at most 64, and
-// the 7-bit mask keeps bytes that hold no valid count from carrying into a
-// neighbour.
-constexpr int kPairIters = (kLbpBins * 32 + 255) / 256;  // 8
-template <class Slot>
-__device__ __forceinline__ void pair_sums(Slot &s, int pt) {
-    uint32_t x[kPairIters], y[kPairIters];
-    const int k = pt & 31;
+// Horizontal sums of the LBP counts of a cell and its right neighbour, times 4
+// (table byte offsets), two 16-bit counts per word: even[w] bins 4w, 4w+2,
+// odd[w] bins 4w+1, 4w+3. Cells are 64 bytes, 16-byte chunks swizzled by the
+// cell's bits 1, 2. Counts are at most 64, so byte sums do not carry (larger
+// ones would only give another entry of the 512-entry table).
+__device__ __forceinline__ void lbp_row(const uint8_t *base, int cell, uint32_t (&even)[15], uint32_t (&odd)[15]) {
 #pragma unroll
-    for (int n = 0; n < kPairIters; ++n) {
-        const int w = pt + 256 * n;
-        if (w < kLbpBins * 32) {
-            const uint32_t *row = reinterpret_cast<const uint32_t *>(s.lbp[w >> 5]);
-            x[n] = row[k] & 0x7f7f7f7fu;
-            y[n] = k < 31 ? row[k + 1] & 0x7f7f7f7fu : 0u;
-        }
-    }
-    __syncwarp();
+    for (int k = 0; k < 4; ++k) {
+        const uint4 x = *reinterpret_cast<const uint4 *>(base + cell * 64 + ((k ^ ((cell >> 1) & 3)) << 4));
+        const uint4 y =
+            *reinterpret_cast<const uint4 *>(base + (cell + 1) * 64 + ((k ^ (((cell + 1) >> 1) & 3)) << 4));
+        const uint32_t h[4] = {x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w};
 #pragma unroll
-    for (int n = 0; n < kPairIters; ++n) {
-        const int w = pt + 256 * n;
-        if (w < kLbpBins * 32) reinterpret_cast<uint32_t *>(s.lbp[w >> 5])[k] = x[n] + __funnelshift_r(x[n], y[n], 8);
+        for (int u = 0; u < 4; ++u)
+            if (4 * k + u < 15) {
+                even[4 * k + u] = (h[u] << 2) & 0x03fc03fcu;
+                odd[4 * k + u] = (h[u] >> 6) & 0x03fc03fcu;
+            }
     }
 }
 
-// named barrier of the producer warps
-__device__ __forceinline__ void producer_barrier() {
-    asm volatile("bar.sync %0, %1;" ::"n"(kProducerBarrier), "n"(32 * kProducers) : "memory");
+// bf16 split pairs of four bins from the table: columns 2 w, 2 w + 1 of the LBP part
+__device__ __forceinline__ void lbp_word(const uint32_t *tab, uint32_t e, uint32_t o, uint32_t *hi, uint32_t *lo) {
+    const uint8_t *t = reinterpret_cast<const uint8_t *>(tab);
+    const uint32_t v0 = *reinterpret_cast<const uint32_t *>(t + (e & 0xffffu));
+    const uint32_t v1 = *reinterpret_cast<const uint32_t *>(t + (o & 0xffffu));
+    const uint32_t v2 = *reinterpret_cast<const uint32_t *>(t + (e >> 16));
+    const uint32_t v3 = *reinterpret_cast<const uint32_t *>(t + (o >> 16));
+    hi[0] = __byte_perm(v0, v1, 0x5410);
+    lo[0] = __byte_perm(v0, v1, 0x7632);
+    hi[1] = __byte_perm(v2, v3, 0x5410);
+    lo[1] = __byte_perm(v2, v3, 0x7632);
 }
 
 template <int HP>
 __global__ void __launch_bounds__(kThreads, 1)
     k_svm_tc(const __grid_constant__ CUtensorMap hog_map, const __grid_constant__ CUtensorMap lbp_map,
              const LevelDesc *__restrict__ levels, const TcItem *__restrict__ items, int n_items,
-             int *__restrict__ queue, const float *__restrict__ wt, float bias, float clip,
+             int *__restrict__ queue, const unsigned char *__restrict__ consts, float bias, float clip,
              float *__restrict__ scores, const uint32_t *__restrict__ c_flag, unsigned *__restrict__ err,
              const CUtensorMap *__restrict__ level_maps) {
     using Slot = SlotT<HP>;
     using TcSmem = TcSmemT<HP>;
+    constexpr int kSlots = TcSmem::kSlots;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     TcSmem &S = *reinterpret_cast<TcSmem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -357,281 +348,369 @@ __global__ void __launch_bounds__(kThreads, 1)
         auto init = [](unsigned long long *bar, uint32_t count) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
         };
+        init(&S.bfull, 1);
         for (int s = 0; s < kSlots; ++s) {
             init(&S.cfull[s], 1);
-            init(&S.cempty[s], kProducers);
+            init(&S.cempty[s], 2 * kGroups);
         }
+        for (int s = 0; s < kMeta; ++s) init(&S.mready[s], 1);
         for (int s = 0; s < 2; ++s) {
-            init(&S.afull[s], kProducers);
+            init(&S.afull[s], 2 * kGroups);
             init(&S.aempty[s], 1);
             init(&S.dfull[s], 1);
-            init(&S.dempty[s], 4);
+            init(&S.dempty[s], kGroups);
         }
         S.failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // the template's B operand and the LBP table, laid out by the host
+        arrive_tx(&S.bfull, kTcConstBytes);
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                smem_u32(S.b)),
+            "l"(reinterpret_cast<uint64_t>(consts)), "r"(kTcConstBytes), "r"(smem_u32(&S.bfull))
+            : "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem)),
                      "r"(kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    // B operand: template position n = 7 i + j (rows), feature t (K); high
-    // parts in chunks 0..11, low parts in chunks 12..23
-    for (int e = tid; e < kN * 96; e += kThreads) {
-        const int n = e / 96, t = e - 96 * (e / 96);
-        const int i = n / kWinBW, j = n - kWinBW * (n / kWinBW);
-        const float w = (n < kWinBH * kWinBW && t < kFeat) ? wt[((size_t)t * kWinBH + i) * kWPad + j] : 0.f;
-        const __nv_bfloat16 h = __float2bfloat16_rn(w);
-        const __nv_bfloat16 l = __float2bfloat16_rn(w - __bfloat162float(h));
-        const uint32_t off = (n >> 3) * kSBO + (t >> 3) * 128 + (n & 7) * 16 + (t & 7) * 2;
-        *reinterpret_cast<__nv_bfloat16 *>(S.b + off) = h;
-        *reinterpret_cast<__nv_bfloat16 *>(S.b + off + 12 * 128) = l;
-    }
-    for (int s = tid; s < 512; s += kThreads) {
-        uint32_t e = 0u;
-        if (s <= 256) {
-            const float f = sqrtf((float)s * (1.0f / 256.0f));
-            const __nv_bfloat16 h = __float2bfloat16_rn(f);
-            const __nv_bfloat16 l = __float2bfloat16_rn(f - __bfloat162float(h));
-            e = (uint32_t)__bfloat16_as_ushort(h) | ((uint32_t)__bfloat16_as_ushort(l) << 16);
-        }
-        S.tab[s] = e;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // B -> tensor cores
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = S.tmem;
-    const uint32_t b_base = smem_u32(S.b);
+    // bounded wait by every lane of a warp, decided for the whole warp
+    auto warp_wait = [&](unsigned long long *bar, uint32_t parity) {
+        return __all_sync(0xffffffffu, bar_wait(S, bar, parity, err)) != 0;
+    };
+    uint32_t loads = 0, committed = 0;  // cell-row steps sent (warp 13), MMA steps committed (warp 12)
 
-    // pipeline counters, advanced identically by every role
-    uint32_t nrow = 0;      // block rows (A buffer, D buffer, their barrier phases)
-    uint32_t ncell = 0;     // cell rows loaded (slot and its barrier phases)
-    uint32_t issued = 0, committed = 0;  // control thread: loads issued, MMA rows committed
-
-    for (;;) {
-        if (tid == 0) S.item = atomicAdd(queue, 1);
-        __syncthreads();
-        const int item = S.item;
-        if (item >= n_items || S.failed) break;
-        const TcItem it = items[item];
-        const LevelDesc L = levels[it.level];
-        const int wend = min(it.wx0 + kTcStrip, L.cols);
-        const int nrows = it.wy1 - it.wy0;
-        const bool sparse = c_flag != nullptr;
-        const int xl = it.wx0 & ~15;   // LBP box origin (16-byte boundary)
-
-        // ---- sparse: which windows of the item are scored (all threads)
-        if (sparse) {
-            const int ty0 = it.wy0 / kCellTH, ty1 = (it.wy1 - 1 + kWinBH) / kCellTH;
-            const int tx0 = it.wx0 / kCellTW, tx1 = (wend - 1 + kWinBW) / kCellTW;
-            const int ntx = tx1 - tx0 + 1, nt = (ty1 - ty0 + 1) * ntx;
-            for (int i = tid; i < nt; i += kThreads) {
-                const int ty = ty0 + i / ntx, tx = tx0 + i % ntx;
-                S.tflag[ty - ty0][tx - tx0] = c_flag[L.citem0 + ty * L.ctx + tx] != 0u;
-            }
-            __syncthreads();
-            for (int row = warp; row < nrows; row += kWarps) {
-                const int wy = it.wy0 + row;
-                const int a0 = wy / kCellTH - ty0, a1 = (wy + kWinBH) / kCellTH - ty0;
-                uint32_t any = 0u;
+    if (warp < 8) {
+        // ---- producers: warps 0-3 the HOG part of group `warp`, warps 4-7 the
+        // LBP part of group warp - 4; lane m = block m of the group
+        const int g = warp & 3;
+        const bool is_lbp = warp >= 4;
+        const uint32_t lanes = tmem + ((uint32_t)(32 * g) << 16) + kTmemA;
+        bool ok = !is_lbp || warp_wait(&S.bfull, 0);
+        auto stage_free = [&](uint32_t s) { return s < 2 || warp_wait(&S.aempty[s & 1], ((s >> 1) - 1) & 1u); };
+        auto publish = [&](uint32_t s) {
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive(&S.afull[s & 1]);
+        };
+        if (!is_lbp) {
+            constexpr int pq = HP == 36 ? kHogBins : 0;  // per-block: plane set of the cell's place
+            float up[18];                                // the upper cell row: cells c, c + 1
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int wx = it.wx0 + 32 * k + lane;
-                    bool ok = wx < wend && 32 * k + lane < kTcStrip;
-                    if (ok) {
-                        const int c0 = wx / kCellTW - tx0, c1 = (wx + kWinBW) / kCellTW - tx0;
-                        for (int a = a0; a <= a1; ++a)
-                            for (int c = c0; c <= c1; ++c) ok = ok && S.tflag[a][c];
-                    }
-                    const uint32_t bits = __ballot_sync(0xffffffffu, ok);
-                    if (lane == 0) S.win_ok[row][k] = bits;
-                    any |= bits;
+            for (int t = 0; t < 18; ++t) up[t] = 0.f;
+            for (uint32_t s = 0; ok; ++s) {
+                if (!(ok = warp_wait(&S.cfull[s % kSlots], (s / kSlots) & 1u))) break;
+                const uint32_t fl = S.meta[s % kMeta][g].flags, kind = fl & 3u;
+                if (kind == 3u) break;
+                const float *hs = reinterpret_cast<const float *>(S.slot[s % kSlots].hog[g]) + lane + ((fl >> 4) & 3u);
+                float x[36], nxt[18];
+#pragma unroll
+                for (int t = 0; t < 18; ++t) x[t] = up[t];
+#pragma unroll
+                for (int t = 0; t < kHogBins; ++t) {
+                    x[18 + t] = hs[(2 * pq + t) * kHogX];
+                    x[27 + t] = hs[(3 * pq + t) * kHogX + 1];
+                    nxt[t] = pq ? hs[t * kHogX] : x[18 + t];
+                    nxt[9 + t] = pq ? hs[(pq + t) * kHogX + 1] : x[27 + t];
                 }
-                if (lane == 0) S.row_ok[row] = any != 0u;
-                if (!any)  // no scored window in this row: it is never stored below
-                    for (int wx = it.wx0 + lane; wx < wend; wx += 32)
-                        scores[L.score_off + (int64_t)wy * L.cols + wx] = -INFINITY;
-            }
-            __syncthreads();
-        }
-
-        // ---- runs of block rows [ra, rb]; every role walks the same runs
-        int r_next = it.wy0;
-        const int r_last = it.wy1 - 1 + kWinBH - 1;
-        while (r_next <= r_last) {
-            int ra, rb;
-            if (!sparse) {
-                ra = it.wy0;
-                rb = r_last;
-            } else {
-                int wy = max(r_next - (kWinBH - 1), it.wy0);
-                while (wy < it.wy1 && !S.row_ok[wy - it.wy0]) ++wy;
-                if (wy >= it.wy1) break;
-                ra = wy;
-                rb = wy + kWinBH - 1;
-                for (int w2 = wy + 1; w2 < it.wy1 && w2 <= rb; ++w2)
-                    if (S.row_ok[w2 - it.wy0]) rb = w2 + kWinBH - 1;
-            }
-            const int n_cell = rb - ra + 2;  // cell rows ra .. rb + 1
-            const int n_blk = rb - ra + 1;
-            auto slot_of = [&](int u) -> Slot & { return S.slot[(ncell + u) % kSlots]; };
-            // bounded wait by every lane of a warp, decided for the whole warp
-            auto warp_wait = [&](unsigned long long *bar, uint32_t parity) {
-                return __all_sync(0xffffffffu, bar_wait(S, bar, parity, err));
-            };
-            auto cell_wait = [&](int u) {  // cell row ra + u has arrived
-                const uint32_t idx = ncell + u;
-                return warp_wait(&S.cfull[idx % kSlots], (idx / kSlots) & 1u);
-            };
-
-            if (warp < kProducers) {
-                // ---- producers: warps 0-3 HOG and LBP bins 0..9, warps 4-7
-                // LBP bins 10..58, for rows 32 (w % 4) + lane
-                const bool is_lbp = warp >= 4;
-                const int m = 32 * (warp & 3) + lane;
-                const int c = kWinPerWarp * (m >> 5) + (m & 31);
-                const int cl = c + it.wx0 - xl;
-                // (a row whose block lies past the level's last block holds whatever
-                // the staged cells give: its products only reach windows past the
-                // score map, which are never stored)
-                bool ok = cell_wait(0);
-                if (ok) pair_sums(slot_of(0), tid);
-                for (int u = 0; u < n_blk; ++u) {
-                    const uint32_t k = nrow + u;
-                    ok = ok && cell_wait(u) && cell_wait(u + 1);
-                    if (ok) pair_sums(slot_of(u + 1), tid);
-                    producer_barrier();  // every producer warp, also after a failed wait
-                    if (ok && k >= 2) ok = warp_wait(&S.aempty[k & 1], ((k >> 1) - 1) & 1u);
-                    if (ok) {
-                        tc_fence_after();
-                        // this warp's TMEM lanes 32 (w % 4) .., A stage k % 2
-                        const uint32_t a = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + kTmemA + (k & 1) * 96;
-                        const Slot &s0 = slot_of(u), &s1 = slot_of(u + 1);
-                        if (!is_lbp)
-                            build_hog(s0, s1, S.tab, c, cl, clip, a);
-                        else
-                            build_lbp(s0, s1, S.tab, cl, a);
-                        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                        tc_fence_before();
-                    }
-                    __syncwarp();
-                    if (ok && lane == 0) {
-                        arrive(&S.afull[k & 1]);
-                        arrive(&S.cempty[(ncell + u) % kSlots]);
-                        if (u == n_blk - 1) arrive(&S.cempty[(ncell + u + 1) % kSlots]);
-                    }
-                }
-            } else {
-                // ---- epilogue warps 8-11 (TMEM lanes 32 q .. 32 q + 31); lane 0 of
-                // warp 8 also issues the cell loads and the MMAs of each row
-                // before the epilogue of the row above it
-                const int q = warp & 3;
-                const bool ctrl = warp == kProducers && lane == 0;
-                const int wl = kWinPerWarp * q + lane;
-                const int wx = it.wx0 + wl;
-                bool ok = true, cok = true;  // epilogue / control progress
-                float acc[kWinBH];           // running scores of window rows r - i (a run starts afresh)
 #pragma unroll
-                for (int i = 0; i < kWinBH; ++i) acc[i] = 0.f;
-                auto issue = [&](int u) {  // control: load cell row ra + u into its slot once free
-                    const uint32_t idx = ncell + u;
-                    if (idx >= kSlots)
-                        cok = cok && bar_wait(S, &S.cempty[idx % kSlots], (idx / kSlots - 1) & 1u, err);
-                    if (!cok) return;
-                    Slot &sl = S.slot[idx % kSlots];
-                    unsigned long long *bar = &S.cfull[idx % kSlots];
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                                 "r"((uint32_t)(sizeof(float) * HP * kHogX + kLbpBins * kLbpX))
-                                 : "memory");
-                    tma_3d(&sl.hog[0][0], level_maps ? level_maps + 2 * L.tc_map : &hog_map, bar, it.wx0,
-                           L.cell_row + ra + u, 0);
-                    tma_3d(&sl.lbp[0][0], level_maps ? level_maps + 2 * L.tc_map + 1 : &lbp_map, bar, xl,
-                           L.cell_row + ra + u, 0);
-                    issued = idx + 1;
-                };
-                if (ctrl)
-                    for (int u = 0; u < min(kSlots, n_cell); ++u) issue(u);
-                for (int u = 0; u <= n_blk; ++u) {
-                    if (ctrl && u < n_blk && cok) {
-                        const uint32_t k = nrow + u;
-                        cok = bar_wait(S, &S.afull[k & 1], (k >> 1) & 1u, err);
-                        if (cok && k >= 2) cok = bar_wait(S, &S.dempty[k & 1], ((k >> 1) - 1) & 1u, err);
-                        if (cok) {
-                            tc_fence_after();
-                            const uint32_t d = tmem + (k & 1) * 128;
-                            const uint32_t a0 = tmem + kTmemA + (k & 1) * 96;  // 8 columns per K step
-#pragma unroll
-                            for (int s = 0; s < 6; ++s)
-                                umma_ts(d, a0 + 8 * s, umma_desc(b_base + 256 * s), s > 0);
-#pragma unroll
-                            for (int s = 0; s < 6; ++s)
-                                umma_ts(d, a0 + 48 + 8 * s, umma_desc(b_base + 256 * s), 1);
-#pragma unroll
-                            for (int s = 0; s < 6; ++s)
-                                umma_ts(d, a0 + 8 * s, umma_desc(b_base + 12 * 128 + 256 * s), 1);
-                            umma_commit(&S.aempty[k & 1]);
-                            umma_commit(&S.dfull[k & 1]);
-                            committed = k + 1;
-                            // cell row ra + u is released after this block row: its slot takes ra + u + 4
-                            if (u + kSlots < n_cell) issue(u + kSlots);
-                        }
-                    }
-                    __syncwarp();
-                    if (u == 0) continue;
-                    // epilogue of block row ra + u - 1
-                    const uint32_t k = nrow + u - 1;
-                    const int r = ra + u - 1;
-                    ok = ok && warp_wait(&S.dfull[k & 1], (k >> 1) & 1u);
-                    if (!ok) continue;
+                for (int t = 0; t < 18; ++t) up[t] = nxt[t];
+                __syncwarp();
+                if (lane == 0) arrive(&S.cempty[s % kSlots]);
+                if (!(ok = stage_free(s))) break;
+                if (kind == 2u) {
                     tc_fence_after();
-                    const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + (k & 1) * 128;
-                    // 105 columns in seven groups of 16
-                    acc[0] = bias;
+                    build_hog(x, clip, lanes + (s & 1) * 96);
+                }
+                publish(s);
+            }
+        } else {
+            uint32_t ue[15], uo[15];  // the upper cell row's sums
 #pragma unroll
-                    for (int g = 0; g < 7; ++g) {
-                        float v[16];
-                        PD_LD_X16(t0 + 16 * g, v, 0);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                        if (g == 6) {
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) arrive(&S.dempty[k & 1]);  // the accumulators may be overwritten
-                        }
+            for (int t = 0; t < 15; ++t) ue[t] = uo[t] = 0u;
+            for (uint32_t s = 0; ok; ++s) {
+                if (!(ok = warp_wait(&S.cfull[s % kSlots], (s / kSlots) & 1u))) break;
+                const uint32_t kind = S.meta[s % kMeta][g].flags & 3u;
+                if (kind == 3u) break;
+                uint32_t e[15], o[15];
+                lbp_row(S.slot[s % kSlots].lbp[g], lane, e, o);
+                __syncwarp();
+                if (lane == 0) arrive(&S.cempty[s % kSlots]);
+                uint32_t hi[30], lo[30];
+                if (kind == 2u) {
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            const int n = 16 * g + e;  // (i, j) = (n / 7, n % 7)
-                            if (n < kWinBH * kWinBW) {
-                                const int i = n / kWinBW, j = n % kWinBW;
-                                acc[i] += j ? __shfl_down_sync(0xffffffffu, v[e], j) : v[e];
-                            }
-                        }
+                    for (int w = 0; w < 15; ++w) lbp_word(S.tab, ue[w] + e[w], uo[w] + o[w], hi + 2 * w, lo + 2 * w);
+                }
+#pragma unroll
+                for (int w = 0; w < 15; ++w) {
+                    ue[w] = e[w];
+                    uo[w] = o[w];
+                }
+                if (!(ok = stage_free(s))) break;
+                if (kind == 2u) {
+                    tc_fence_after();
+                    const uint32_t a = lanes + (s & 1) * 96;
+                    tst2(a + 18, hi);
+                    tst4(a + 20, hi + 2);
+                    tst8(a + 24, hi + 6);
+                    tst16(a + 32, hi + 14);
+                    tst2(a + 66, lo);
+                    tst4(a + 68, lo + 2);
+                    tst8(a + 72, lo + 6);
+                    tst16(a + 80, lo + 14);
+                }
+                publish(s);
+            }
+        }
+    } else if (warp < 12) {
+        // ---- epilogue of group g
+        const int g = warp - 8;
+        float acc[kWinBH];  // running scores of window rows r - i (an item's first rows start afresh)
+#pragma unroll
+        for (int i = 0; i < kWinBH; ++i) acc[i] = 0.f;
+        for (uint32_t s = 0;; ++s) {
+            if (!warp_wait(&S.mready[s % kMeta], (s / kMeta) & 1u)) break;
+            const StepMeta m = S.meta[s % kMeta][g];
+            const uint32_t kind = m.flags & 3u;
+            if (kind == 3u) break;
+            if (!warp_wait(&S.dfull[s & 1], (s >> 1) & 1u)) break;
+            if (kind != 2u) {
+                if (lane == 0) arrive(&S.dempty[s & 1]);
+                continue;
+            }
+            tc_fence_after();
+            const uint32_t t0 = tmem + ((uint32_t)(32 * g) << 16) + (s & 1) * 128;
+            // Columns from the last template row up, so that acc[i] = acc[i - 1] + the terms
+            // of row i moves the running scores on by one row without copies. The 7 terms of
+            // a row are added in order of j; rows i, i + 1 (i odd) are packed.
+            // The next 16 columns load while the current ones are added (three in flight fit
+            // the 128 registers that 14 warps leave a thread).
+            float v[7][16];
+            auto term = [&](int i, int j) {
+                const int n = i * kWinBW + j;
+                return j ? __shfl_down_sync(0xffffffffu, v[n >> 4][n & 15], j) : v[n >> 4][n & 15];
+            };
+            auto rows = [&](int i) {  // rows i, i - 1
+                f32x2 t = pack2(acc[i - 2] + term(i - 1, 0), acc[i - 1] + term(i, 0));
+#pragma unroll
+                for (int j = 1; j < kWinBW; ++j) t = add2(t, pack2(term(i - 1, j), term(i, j)));
+                unpack2(t, acc[i - 1], acc[i]);
+            };
+            PD_LD_X16(t0 + 96, v[6]);
+            PD_LD_X16(t0 + 80, v[5]);
+            PD_WAIT_X16(v[6]);
+            PD_WAIT_X16(v[5]);
+            PD_LD_X16(t0 + 64, v[4]);
+            rows(14);
+            PD_WAIT_X16(v[4]);
+            PD_LD_X16(t0 + 48, v[3]);
+            rows(12);
+            PD_WAIT_X16(v[3]);
+            PD_LD_X16(t0 + 32, v[2]);
+            rows(10);
+            rows(8);
+            PD_WAIT_X16(v[2]);
+            PD_LD_X16(t0 + 16, v[1]);
+            rows(6);
+            PD_WAIT_X16(v[1]);
+            PD_LD_X16(t0, v[0]);
+            rows(4);
+            PD_WAIT_X16(v[0]);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive(&S.dempty[s & 1]);  // the accumulators may be overwritten
+            rows(2);
+            acc[0] = bias;
+#pragma unroll
+            for (int j = 0; j < kWinBW; ++j) acc[0] += term(0, j);
+            if ((m.flags & 4u) && lane < (int)(m.flags >> 8))
+                scores[m.out + lane] = (m.keep >> lane) & 1u ? acc[kWinBH - 1] : -INFINITY;
+        }
+    } else if (warp == 12) {
+        // ---- MMA issue
+        if (lane == 0 && bar_wait(S, &S.bfull, 0, err)) {
+            const uint32_t b_base = smem_u32(S.b);
+            for (uint32_t s = 0;; ++s) {
+                if (!bar_wait(S, &S.mready[s % kMeta], (s / kMeta) & 1u, err)) break;
+                if ((S.meta[s % kMeta][0].flags & 3u) == 3u) break;
+                if (!bar_wait(S, &S.afull[s & 1], (s >> 1) & 1u, err)) break;
+                if (s >= 2 && !bar_wait(S, &S.dempty[s & 1], ((s >> 1) - 1) & 1u, err)) break;
+                tc_fence_after();
+                const uint32_t d = tmem + (s & 1) * 128;
+                const uint32_t a0 = tmem + kTmemA + (s & 1) * 96;  // 8 columns per K step
+#pragma unroll
+                for (int k = 0; k < 6; ++k) umma_ts(d, a0 + 8 * k, umma_desc(b_base + 256 * k), k > 0);
+#pragma unroll
+                for (int k = 0; k < 6; ++k) umma_ts(d, a0 + 48 + 8 * k, umma_desc(b_base + 256 * k), 1);
+#pragma unroll
+                for (int k = 0; k < 6; ++k) umma_ts(d, a0 + 8 * k, umma_desc(b_base + 12 * 128 + 256 * k), 1);
+                umma_commit(&S.aempty[s & 1]);
+                umma_commit(&S.dfull[s & 1]);
+                committed = s + 1;
+            }
+        }
+        __syncwarp();
+    } else {
+        // ---- items and cell rows; lane g < 4 serves group g
+        const bool sparse = c_flag != nullptr;
+        const bool mine = lane < kGroups;
+        int next = mine ? (int)blockIdx.x + lane * (int)gridDim.x : n_items;  // next item of the group
+        TcItem nit{};
+        if (next < n_items) nit = items[next];
+        // the item being walked
+        bool active = false;
+        const CUtensorMap *hm = &hog_map, *lm = &lbp_map;
+        int wx0 = 0, ncols = 0, wy0 = 0, cols = 0, cell_row = 0;
+        int r = 0, r0 = 0, r_end = -1;  // next cell row, first and last one of the run
+        bool first = false;
+        int64_t score_off = 0;
+        unsigned long long rows64 = 0;  // sparse: window rows (from wy0) with a scored window
+        auto next_run = [&]() {         // sparse: the next run of cell rows, if any
+            if (!rows64) return false;
+            const int a = __ffsll((long long)rows64) - 1;
+            int b = a;  // last kept row of the run: rows whose walks overlap
+            rows64 &= rows64 - 1ull;
+            while (rows64) {
+                const int n = __ffsll((long long)rows64) - 1;
+                if (n > b + kWinBH) break;
+                b = n;
+                rows64 &= rows64 - 1ull;
+            }
+            r = r0 = wy0 + a;
+            r_end = wy0 + b + kWinBH;
+            first = true;
+            return true;
+        };
+        for (uint32_t s = 0;; ++s) {
+            // groups whose item (or run) is done take the next
+            if (active && r > r_end) active = sparse && next_run();
+            for (;;) {
+                const bool want = mine && !active && next < n_items;
+                const unsigned who = __ballot_sync(0xffffffffu, want);
+                if (!who) break;
+                int n_rows = 0, lv = 0;
+                if (want) {
+                    const TcItem it = nit;
+                    next = 4 * (int)gridDim.x + atomicAdd(queue, 1);
+                    if (next < n_items) nit = items[next];  // in flight while this item is walked
+                    lv = it.level;
+                    const LevelDesc &L = levels[lv];
+                    wx0 = it.wx0;
+                    wy0 = it.wy0;
+                    n_rows = it.wy1 - it.wy0;
+                    cols = L.cols;
+                    ncols = min(kTcStrip, cols - wx0);
+                    cell_row = L.cell_row;
+                    score_off = L.score_off;
+                    if (level_maps) {
+                        hm = level_maps + 2 * L.tc_map;
+                        lm = hm + 1;
                     }
-                    const int wy = r - (kWinBH - 1);
-                    if (wy >= it.wy0 && lane < kWinPerWarp && wx < wend) {
-                        const bool keep = !sparse || ((S.win_ok[wy - it.wy0][wl >> 5] >> (wl & 31)) & 1u);
-                        scores[L.score_off + (int64_t)wy * L.cols + wx] = keep ? acc[kWinBH - 1] : -INFINITY;
-                    }
+                    r = r0 = wy0;
+                    r_end = it.wy1 - 1 + kWinBH;
+                    first = active = true;
+                }
+                if (!sparse) break;
+                // sparse: the scored windows of each new item, by the whole warp
+                for (unsigned left = who; left; left &= left - 1u) {
+                    const int g = __ffs((int)left) - 1;
+                    const int y0 = __shfl_sync(0xffffffffu, wy0, g), x0 = __shfl_sync(0xffffffffu, wx0, g);
+                    const int n = __shfl_sync(0xffffffffu, n_rows, g), nc = __shfl_sync(0xffffffffu, ncols, g);
+                    const int width = __shfl_sync(0xffffffffu, cols, g);
+                    const int64_t so = __shfl_sync(0xffffffffu, (long long)score_off, g);
+                    const LevelDesc &L = levels[__shfl_sync(0xffffffffu, lv, g)];
+                    // lane = window column: a window lies in one or two cell tiles across; the
+                    // ballot of tile row t (at most 11 of them) stays with lane t
+                    const int ty0 = y0 / kCellTH, nt = (y0 + n - 1 + kWinBH) / kCellTH - ty0 + 1;
+                    const int wx = x0 + lane;
+                    const int cl = lane < nc ? wx / kCellTW : 0, cr = lane < nc ? (wx + kWinBW) / kCellTW : 0;
+                    uint32_t f[kTileRows][2];
 #pragma unroll
-                    for (int i = kWinBH - 1; i > 0; --i) acc[i] = acc[i - 1];
+                    for (int t = 0; t < kTileRows; ++t) {
+                        const uint32_t *row = c_flag + L.citem0 + (ty0 + min(t, nt - 1)) * L.ctx;
+                        f[t][0] = __ldg(row + cl);
+                        f[t][1] = __ldg(row + cr);
+                    }
+                    uint32_t bits = 0;
+#pragma unroll
+                    for (int t = 0; t < kTileRows; ++t) {
+                        const uint32_t b = __ballot_sync(0xffffffffu, lane < nc && f[t][0] && f[t][1]);
+                        if (lane == t) bits = b;
+                    }
+                    // lane = window row: its 16 cell rows lie in two or three tile rows
+                    unsigned long long kept = 0;
+#pragma unroll
+                    for (int h = 0; h < kTcChunk / 32; ++h) {
+                        const int row = 32 * h + lane, y = y0 + min(row, n - 1);
+                        const int a0 = y / kCellTH - ty0, a1 = (y + kWinBH) / kCellTH - ty0;
+                        const uint32_t k = __shfl_sync(0xffffffffu, bits, a0) & __shfl_sync(0xffffffffu, bits, a0 + 1) &
+                                           __shfl_sync(0xffffffffu, bits, a1);
+                        const bool any = row < n && k;
+                        if (row < n) S.keep[g][row] = k;
+                        kept |= (unsigned long long)__ballot_sync(0xffffffffu, any) << (32 * h);
+                    }
+                    for (unsigned long long none = ~kept & (n == 64 ? ~0ull : (1ull << n) - 1ull); none; none &= none - 1ull) {
+                        const int row = __ffsll((long long)none) - 1;
+                        if (lane < nc) scores[so + (int64_t)(y0 + row) * width + wx] = -INFINITY;
+                    }
+                    __syncwarp();
+                    if (lane == g) {
+                        rows64 = kept;
+                        active = next_run();
+                    }
                 }
             }
-            nrow += n_blk;
-            ncell += n_cell;
-            r_next = rb + 1;
+            const uint32_t slot = s % kSlots;
+            if (s >= kSlots && !warp_wait(&S.cempty[slot], (s / kSlots - 1) & 1u)) break;
+            const unsigned act = __ballot_sync(0xffffffffu, active);
+            if (mine) {
+                StepMeta m{};
+                if (!act) m.flags = 3u;
+                if (active) {
+                    const int wy = r - kWinBH;  // the window row that this cell row completes
+                    const bool store = wy >= r0;
+                    m.flags = (first ? 1u : 2u) | (store ? 4u : 0u) | ((uint32_t)(wx0 & 3) << 4) | ((uint32_t)ncols << 8);
+                    m.keep = sparse && store ? S.keep[lane][wy - wy0] : 0xffffffffu;
+                    m.out = score_off + (int64_t)wy * cols + wx0;
+                }
+                S.meta[s % kMeta][lane] = m;
+            }
+            __syncwarp();
+            if (lane == 0) {
+                arrive_tx(&S.cfull[slot], __popc(act) * (uint32_t)(HP * kHogX * 4 + kLbpX * 64));
+                arrive(&S.mready[s % kMeta]);
+            }
+            __syncwarp();
+            if (!act) break;
+            if (active) {
+                Slot &sl = S.slot[slot];
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                tma_3d(sl.hog[lane], hm, &S.cfull[slot], wx0 & ~3, cell_row + r, 0);
+                tma_3d(sl.lbp[lane], lm, &S.cfull[slot], 0, wx0, cell_row + r);
+                first = false;
+                ++r;
+            }
+            loads = s + 1;
         }
-        __syncthreads();  // the item is done by every role (nothing in flight unless a wait failed)
-        if (S.failed) break;
     }
 
     __syncthreads();
-    if (S.failed && warp == kProducers && lane == 0) {
-        // drain this CTA's copies and MMAs (bounded) before the tensor memory
-        // is freed: the last load of every slot, the last commit
-        for (uint32_t idx = issued > kSlots ? issued - kSlots : 0u; idx < issued; ++idx)
-            drain_wait(&S.cfull[idx % kSlots], (idx / kSlots) & 1u);
-        if (committed > 0) drain_wait(&S.dfull[(committed - 1) & 1], ((committed - 1) >> 1) & 1u);
+    if (S.failed) {
+        // drain this CTA's copies and MMAs (bounded) before the tensor memory is
+        // freed: the constants, the last load of every slot, the last commit
+        if (warp == 13 && lane == 0) {
+            drain_wait(&S.bfull, 0);
+            for (uint32_t i = loads > kSlots ? loads - kSlots : 0u; i < loads; ++i)
+                drain_wait(&S.cfull[i % kSlots], (i / kSlots) & 1u);
+        }
+        if (warp == 12 && lane == 0 && committed > 0)
+            drain_wait(&S.dfull[(committed - 1) & 1], ((committed - 1) >> 1) & 1u);
     }
     tc_fence_before();
     __syncthreads();
@@ -640,6 +719,28 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 #undef PD_LD_X16
+#undef PD_WAIT_X16
+
+// LBP count planes [59][rows][pitch] -> 64 bytes per cell, [rows][width][64]
+// (bins 59..63 zero): one thread per 16 bins of a cell. For callers' planes;
+// the detector's own cells are written that way.
+__global__ void __launch_bounds__(128) k_lbp_cells(const uint8_t *__restrict__ planes, int64_t plane, int pitch,
+                                                   int width, uint8_t *__restrict__ out) {
+    const int x = blockIdx.x * 32 + (threadIdx.x & 31), k = threadIdx.x >> 5, y = blockIdx.y;
+    if (x >= width) return;
+    const uint8_t *src = planes + (int64_t)y * pitch + x;
+    uint32_t w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        w[u] = 0u;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int t = 16 * k + 4 * u + b;
+            if (t < kLbpBins) w[u] |= (uint32_t)__ldg(src + t * plane) << (8 * b);
+        }
+    }
+    reinterpret_cast<uint4 *>(out)[((int64_t)y * width + x) * 4 + k] = make_uint4(w[0], w[1], w[2], w[3]);
+}
 
 }  // namespace
 
@@ -651,24 +752,59 @@ cudaError_t init_svm_tc() {
                                 (int)sizeof(TcSmemT<4 * kHogBins>));
 }
 
-int svm_tc_smem_bytes(int hog_planes) {
-    return hog_planes == 4 * kHogBins ? (int)sizeof(TcSmemT<4 * kHogBins>) : (int)sizeof(TcSmemT<kHogBins>);
+void build_tc_consts(const float *wt, unsigned char *out) {
+    std::memset(out, 0, kTcConstBytes);
+    // B operand: template position n = 7 i + j (rows), feature t (K); high
+    // parts in chunks 0..11, low parts in chunks 12..23
+    for (int n = 0; n < kWinBH * kWinBW; ++n)
+        for (int t = 0; t < kFeat; ++t) {
+            const float w = wt[((size_t)t * kWinBH + n / kWinBW) * kWPad + n % kWinBW];
+            const __nv_bfloat16 h = __float2bfloat16_rn(w);
+            const __nv_bfloat16 l = __float2bfloat16_rn(w - __bfloat162float(h));
+            const size_t off = (size_t)(n >> 3) * kSBO + (t >> 3) * 128 + (n & 7) * 16 + (t & 7) * 2;
+            std::memcpy(out + off, &h, 2);
+            std::memcpy(out + off + 12 * 128, &l, 2);
+        }
+    for (int s = 0; s <= 256; ++s) {
+        const float f = sqrtf((float)s * (1.0f / 256.0f));
+        const __nv_bfloat16 h = __float2bfloat16_rn(f);
+        const __nv_bfloat16 l = __float2bfloat16_rn(f - __bfloat162float(h));
+        std::memcpy(out + kBBytes + 4 * s, &h, 2);
+        std::memcpy(out + kBBytes + 4 * s + 2, &l, 2);
+    }
+}
+
+int encode_tc_maps(CUtensorMap *hog_map, CUtensorMap *lbp_map, const float *hog, int64_t hog_pitch, int64_t hog_plane,
+                   int hog_planes, const uint8_t *lbp, int64_t lbp_pitch, int64_t rows, int64_t width) {
+    // 36 cells of one row of every HOG plane; 33 cells x 64 bytes of one row
+    if (encode_plane_map(hog_map, const_cast<float *>(hog), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, hog_pitch, rows,
+                         hog_planes, hog_plane, kHogX, 1, hog_planes, width) != PD_OK)
+        return PD_ECUDA;
+    return encode_cell_map(lbp_map, const_cast<uint8_t *>(lbp), lbp_pitch, rows, width, kLbpX);
+}
+
+cudaError_t launch_lbp_cells(cudaStream_t s, const uint8_t *planes, int64_t plane, int pitch, int width, int rows,
+                             uint8_t *out) {
+    if (width <= 0 || rows <= 0) return cudaSuccess;
+    k_lbp_cells<<<dim3((width + 31) / 32, rows), 128, 0, s>>>(planes, plane, pitch, width, out);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_svm_tc(cudaStream_t s, const CUtensorMap &hog_map, const CUtensorMap &lbp_map,
                           const LevelDesc *d_levels, const TcItem *d_items, int n_items, int *d_queue, int grid,
-                          const float *d_w, float bias, float clip, float *scores, const uint32_t *c_flag,
-                          unsigned *d_err, int hog_planes, const CUtensorMap *level_maps) {
+                          const unsigned char *d_consts, float bias, float clip, float *scores,
+                          const uint32_t *c_flag, unsigned *d_err, int hog_planes, const CUtensorMap *level_maps) {
     if (n_items <= 0) return cudaSuccess;
-    if (reinterpret_cast<uintptr_t>(level_maps) & 63) return cudaErrorInvalidValue;
+    if ((reinterpret_cast<uintptr_t>(level_maps) & 63) || (reinterpret_cast<uintptr_t>(d_consts) & 15))
+        return cudaErrorInvalidValue;
     grid = grid < n_items ? grid : n_items;
     if (hog_planes == 4 * kHogBins)
         k_svm_tc<4 * kHogBins><<<grid, kThreads, sizeof(TcSmemT<4 * kHogBins>), s>>>(
-            hog_map, lbp_map, d_levels, d_items, n_items, d_queue, d_w, bias, clip, scores, c_flag, d_err,
+            hog_map, lbp_map, d_levels, d_items, n_items, d_queue, d_consts, bias, clip, scores, c_flag, d_err,
             level_maps);
     else
         k_svm_tc<kHogBins><<<grid, kThreads, sizeof(TcSmemT<kHogBins>), s>>>(
-            hog_map, lbp_map, d_levels, d_items, n_items, d_queue, d_w, bias, clip, scores, c_flag, d_err,
+            hog_map, lbp_map, d_levels, d_items, n_items, d_queue, d_consts, bias, clip, scores, c_flag, d_err,
             level_maps);
     return cudaGetLastError();
 }

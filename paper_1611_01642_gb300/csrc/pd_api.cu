@@ -68,7 +68,6 @@ struct Plan {
     std::vector<CnnItem> cnn_items;
     std::vector<int32_t> tabs;
     std::vector<int32_t> tc_widths;  // tensor-core K4: level widths (cells) with a pair of maps
-    int tc_rows = kTcChunk;  // tensor-core K4 window rows per item (tuning; kept by clear())
     int64_t pyr_bytes = 0;
     int64_t score_floats = 0;
     int32_t atlas_rows = 0;
@@ -217,6 +216,19 @@ int encode_plane_map(CUtensorMap *map, void *base, CUtensorMapDataType dtype, in
     return r == CUDA_SUCCESS ? PD_OK : PD_ECUDA;
 }
 
+int encode_cell_map(CUtensorMap *map, uint8_t *base, int64_t pitch, int64_t rows, int64_t width, uint32_t box_cells) {
+    auto fn = get_encode();
+    if (!fn) return PD_ECUDA;
+    cuuint64_t dims[3] = {kLbpCellBytes, (cuuint64_t)width, (cuuint64_t)rows};
+    cuuint64_t strides[2] = {kLbpCellBytes, (cuuint64_t)(pitch * kLbpCellBytes)};
+    cuuint32_t box[3] = {kLbpCellBytes, box_cells, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? PD_OK : PD_ECUDA;
+}
+
 // 2D map over one pyramid level (u8 [Hk][pitch]) for the proposal network's
 // input tiles.
 int encode_level_map(CUtensorMap *map, const uint8_t *base, int Wk, int Hk, int pitch) {
@@ -284,14 +296,14 @@ struct pd_handle {
     int adam_t = 0;
     // training workspace (allocated on first use, grown with the batch)
     unsigned char *train_ws = nullptr;
-    unsigned char *scheme_ws = nullptr;  // scratch of the paper's kernel schemes (grown on demand)
+    unsigned char *scheme_ws = nullptr;  // scratch of the stage and scheme entries (grown on demand)
     size_t scheme_ws_bytes = 0;
     size_t train_ws_bytes = 0;
     int train_losses = 0;
     float *train_loss_ptr = nullptr;
-    // tensor maps over the atlases, one pair per K4 tile shape
+    // tensor maps over the atlases, one pair per tile shape of the FP32 K4
     CUtensorMap hog_map[kSvmShapes]{}, lbp_map[kSvmShapes]{};
-    CUtensorMap tc_hog_map{}, tc_lbp_map{};  // the same planes for the tensor-core K4
+    unsigned char *d_tc_consts = nullptr;    // tensor-core K4: B operand and LBP table
     int *d_queue = nullptr;                  // [2]: K4's and K2+K3's item counters (zeroed before each launch)
     int *d_nms_sched = nullptr;              // NMS ticket counter, frame order and candidate counts
     int sm_count = 1;
@@ -397,15 +409,85 @@ void plan_windows(std::vector<SvmItem> &out, int li, int rows, int cols, const f
     }
 }
 
-// Tensor-core K4 items of a rows x cols score map: strips of kTcStrip window
-// columns, each cut into near-equal pieces of at most `chunk` window rows
-// (a piece also reads the 14 block rows below its last window row).
-void plan_tc(std::vector<TcItem> &out, int li, int rows, int cols, int chunk) {
-    if (rows <= 0 || cols <= 0) return;
-    const int pieces = (rows + chunk - 1) / chunk;
-    for (int x = 0; x < cols; x += kTcStrip)
-        for (int k = 0; k < pieces; ++k)
-            out.push_back({li, x, (int)((int64_t)rows * k / pieces), (int)((int64_t)rows * (k + 1) / pieces)});
+// End of a greedy longest-first schedule of n[r] jobs of r rows (r <= max_rows,
+// each costing r + extra) on `workers` workers, from the histogram: workers are
+// counted per integer time, jobs of one length go to the free ones in bulk.
+int64_t makespan(const int64_t *n, int max_rows, int extra, int64_t workers) {
+    std::vector<int64_t> free_at(1, workers);  // free_at[t]: workers that become free at time t
+    size_t t = 0, end = 0;
+    for (int r = max_rows; r >= 1; --r) {
+        for (int64_t left = n[r]; left > 0;) {
+            while (free_at[t] == 0) ++t;
+            const int64_t k = std::min(free_at[t], left);
+            const size_t e = t + (size_t)(r + extra);
+            if (e >= free_at.size()) free_at.resize(e + 1, 0);
+            free_at[t] -= k;
+            free_at[e] += k;
+            left -= k;
+            end = std::max(end, e);
+        }
+    }
+    return (int64_t)end;
+}
+
+// Tensor-core K4 items of every level: strips of kTcStrip window columns, cut
+// into near-equal pieces of at most `chunk` window rows, most rows first (a
+// stable counting sort), so that the persistent CTAs' queue ends with the small
+// ones. A piece of n rows walks n + kWinBH cell rows and about two more steps of
+// fill, and an SM walks kTcWalkers pieces at a time. With many rounds of pieces
+// per walker the largest chunk walks the fewest rows; a small plan would leave
+// most SMs idle while a few walk long pieces (a 320x240 frame: 7 pieces of up to
+// 30 cell rows), so of max_rows, 48, 32, ..., 1 rows the one whose schedule ends
+// first is taken, a smaller one only if it ends at least 3% sooner. Below
+// kTcMinChunk rows only plans of at most kTcFineItems pieces are cut.
+// The chunk does not change the result.
+void plan_tc(Plan &p, int max_rows, int sm_count) {
+    const int64_t workers = (int64_t)kTcWalkers * std::max(sm_count, 1);
+    int64_t n[kTcChunk + 1];
+    auto histogram = [&](int chunk) {
+        int64_t total = 0;
+        std::fill(n, n + kTcChunk + 1, 0);
+        for (const LevelDesc &L : p.levels) {
+            if (L.rows <= 0) continue;
+            const int pieces = (L.rows + chunk - 1) / chunk, strips = (L.cols + kTcStrip - 1) / kTcStrip;
+            const int lo = L.rows / pieces, more = L.rows % pieces;
+            n[lo] += (int64_t)(pieces - more) * strips;
+            if (more) n[lo + 1] += (int64_t)more * strips;
+            total += (int64_t)pieces * strips;
+        }
+        return total;
+    };
+    constexpr int kExtra = kWinBH + 2;
+    int chunk = max_rows;
+    if (histogram(max_rows) < 16 * workers) {
+        int64_t best = makespan(n, kTcChunk, kExtra, workers);
+        static const int kRows[] = {48, 32, 24, 16, 12, 8, 6, 4, 3, 2, 1};
+        for (int c : kRows) {
+            if (c >= max_rows) continue;
+            if (histogram(c) > kTcFineItems && c < kTcMinChunk) break;
+            const int64_t t = makespan(n, kTcChunk, kExtra, workers);
+            if (100 * t <= 97 * best) {
+                best = t;
+                chunk = c;
+            }
+        }
+    }
+    const int64_t total = histogram(chunk);
+    int64_t at[kTcChunk + 1], sum = 0;
+    for (int r = kTcChunk; r >= 0; --r) {
+        at[r] = sum;
+        sum += n[r];
+    }
+    p.t_items.resize((size_t)total);
+    for (int li = 0; li < (int)p.levels.size(); ++li) {
+        const LevelDesc &L = p.levels[li];
+        if (L.rows <= 0) continue;
+        const int pieces = (L.rows + chunk - 1) / chunk;
+        for (int k = 0; k < pieces; ++k) {
+            const int y0 = (int)((int64_t)L.rows * k / pieces), y1 = (int)((int64_t)L.rows * (k + 1) / pieces);
+            for (int x = 0; x < L.cols; x += kTcStrip) p.t_items[(size_t)at[y1 - y0]++] = {li, x, y0, y1};
+        }
+    }
 }
 
 // K2+K3 strips of every level of a plan, tallest first (the warps take them
@@ -437,31 +519,17 @@ void plan_strips(Plan &p, int resident_warps) {
         }
         return total;
     };
-    auto makespan = [&](int rows) {
+    auto schedule = [&](int rows) {
         int64_t n[kMaxRows + 1];
         histogram(rows, n);
-        std::vector<int64_t> free_at(1, R);  // free_at[t]: warps that become free at time t
-        size_t t = 0, end = 0;
-        for (int r = kMaxRows; r >= 1; --r) {
-            for (int64_t left = n[r]; left > 0;) {
-                while (free_at[t] == 0) ++t;
-                const int64_t k = std::min(free_at[t], left);
-                const size_t e = t + (size_t)r + 1;
-                if (e >= free_at.size()) free_at.resize(e + 1, 0);
-                free_at[t] -= k;
-                free_at[e] += k;
-                left -= k;
-                end = std::max(end, e);
-            }
-        }
-        return (int64_t)end;
+        return makespan(n, kMaxRows, 1, R);
     };
     int rows = kMaxRows;
     int64_t n32[kMaxRows + 1];
     if (histogram(rows, n32) < 16 * R) {
-        int64_t best = makespan(rows);
+        int64_t best = schedule(rows);
         for (int r = rows / 2; r >= 2; r /= 2) {
-            const int64_t t = makespan(r);
+            const int64_t t = schedule(r);
             if (100 * t <= 97 * best) {
                 best = t;
                 rows = r;
@@ -476,13 +544,6 @@ void plan_strips(Plan &p, int resident_warps) {
     }
     std::stable_sort(p.strips.begin(), p.strips.end(),
                      [](const StripItem &a, const StripItem &b) { return a.cy1 - a.cy0 > b.cy1 - b.cy0; });
-}
-
-// Largest items first (block rows walked: window rows + 14), so that the
-// persistent CTAs' queue ends with the small ones.
-void order_tc(std::vector<TcItem> &t) {
-    std::stable_sort(t.begin(), t.end(),
-                     [](const TcItem &a, const TcItem &b) { return a.wy1 - a.wy0 > b.wy1 - b.wy0; });
 }
 
 // K1 tables of one level (Section 4.4 resample, reading Q).
@@ -601,7 +662,6 @@ void plan_level(Plan &p, int frame, int level, int W, int H, int Wk, int Hk, int
     for (int cy = 0; cy < L.Hc; cy += kCellTH)
         for (int cx = 0; cx < L.Wc; cx += kCellTW) p.c_items.push_back({li, cx, cy, 0});
     plan_windows(p.s_items, li, L.rows, L.cols, tile_cost);
-    plan_tc(p.t_items, li, L.rows, L.cols, p.tc_rows);
     p.atlas_rows += L.Hc;
     p.score_floats += (int64_t)L.rows * L.cols;
     p.max_wc = std::max(p.max_wc, L.Wc);
@@ -670,17 +730,6 @@ bool params_ok(const pd_params *p) {
            !((p->flags & PD_FLAG_HOG_PER_BLOCK) && (p->flags & (PD_FLAG_SVM_FP32 | PD_FLAG_LBP_ONLY)));
 }
 
-int encode_tc_maps(CUtensorMap *hog_map, CUtensorMap *lbp_map, const float *hog, const uint8_t *lbp, int64_t pitch,
-                   int64_t rows, int64_t hog_plane, int64_t lbp_plane, int hog_planes = kHogBins,
-                   int64_t width = 0) {
-    if (encode_plane_map(hog_map, const_cast<float *>(hog), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, pitch, rows,
-                         hog_planes, hog_plane, 112, 1, hog_planes, width) != PD_OK ||
-        encode_plane_map(lbp_map, const_cast<uint8_t *>(lbp), CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, pitch, rows,
-                         kLbpBins, lbp_plane, 128, 1, kLbpBins, width) != PD_OK)
-        return PD_ECUDA;
-    return PD_OK;
-}
-
 // Tensor-core K4: one pair of cell-plane maps per distinct level width, so
 // that a box reaching past a level's right edge reads zeros (TMA fill) and
 // not the atlas row's padding from memory (the windows that use those cells
@@ -717,8 +766,9 @@ int upload_plan(pd_handle *h, cudaStream_t s, const Plan &p, Packed &o, const ui
     put(o.tabs, p.tabs.data(), p.tabs.size() * sizeof(int32_t));
     for (size_t k = 0; k < p.tc_widths.size(); ++k) {
         CUtensorMap *maps = reinterpret_cast<CUtensorMap *>(h->h_desc + o.tc_maps) + 2 * k;
-        if (encode_tc_maps(&maps[0], &maps[1], h->atlas.hog, h->atlas.lbp, h->atlas.pitch, h->atlas.rows,
-                           h->atlas.hog_plane, h->atlas.lbp_plane, hog_planes_of(h->p.flags), p.tc_widths[k]) != PD_OK)
+        if (encode_tc_maps(&maps[0], &maps[1], h->atlas.hog, h->atlas.pitch, h->atlas.hog_plane,
+                           hog_planes_of(h->p.flags), h->atlas.lbp, h->atlas.pitch, h->atlas.rows,
+                           p.tc_widths[k]) != PD_OK)
             return fail(h, PD_ECUDA, "cell-plane tensor map");
     }
     if (!p.cnn_items.empty()) {
@@ -750,8 +800,6 @@ int encode_svm_maps(CUtensorMap *hog_maps, CUtensorMap *lbp_maps, const float *h
     return PD_OK;
 }
 
-// The tensor-core K4's maps: one cell row of a 112-cell strip of the 9 (or,
-// per-block HOG, 36) HOG planes, and of a 128-cell strip of the 59 LBP planes.
 // Round to the nearest bfloat16 (ties to even): 8 significant bits of the
 // exact value, as a float.
 float bf16_round_host(double a) {
@@ -855,6 +903,21 @@ int refresh_fragments(pd_handle *h) {
 
 }  // namespace
 
+namespace {
+// Scratch of the stage and kernel-scheme entries, grown on demand (the stream is
+// synchronised first: earlier work on it may still use the old buffer).
+int scheme_scratch(pd_handle *h, cudaStream_t s, size_t need) {
+    if (need <= h->scheme_ws_bytes) return PD_OK;
+    PD_CUDA(h, cudaStreamSynchronize(s));
+    if (h->scheme_ws) cudaFree(h->scheme_ws);
+    h->scheme_ws = nullptr;
+    h->scheme_ws_bytes = 0;
+    if (cudaMalloc(&h->scheme_ws, need) != cudaSuccess) return fail(h, PD_ENOMEM, "scheme scratch");
+    h->scheme_ws_bytes = need;
+    return PD_OK;
+}
+}  // namespace
+
 extern "C" {
 
 int pd_params_default(pd_params *p) {
@@ -940,7 +1003,6 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     // tables (frames of different sizes do not share them).
     {
         Plan one;
-        one.tc_rows = kTcMinChunk;  // the most tensor-core K4 items any tuning can ask for
         plan_frame(one, *params, nullptr, params->max_width, params->max_height, params->max_width);
         int64_t s_bound = 0;
         for (const LevelDesc &L : one.levels) {
@@ -956,6 +1018,9 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
             s_bound += most;
         }
         const int64_t F = params->max_frames;
+        int64_t t_bound = 0;  // tensor-core K4 items at the fewest rows any plan of many items has
+        for (const LevelDesc &L : one.levels)
+            t_bound += (int64_t)((L.cols + kTcStrip - 1) / kTcStrip) * ((L.rows + kTcMinChunk - 1) / kTcMinChunk);
         int64_t cnn_bound = 0;
         for (const LevelDesc &L : one.levels)
             cnn_bound += (int64_t)((L.Hc + kCnnTile - 1) / kCnnTile) * ((L.Wc + kCnnTile - 1) / kCnnTile);
@@ -969,7 +1034,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
                       round_up(F * (int64_t)one.c_items.size() * (int64_t)sizeof(CellItem), 16) +
                       round_up(4 * F * (int64_t)one.c_items.size() * (int64_t)sizeof(StripItem), 16) +  // 2-row strips
                       round_up(F * s_bound * (int64_t)sizeof(SvmItem), 16) +
-                      round_up(F * (int64_t)one.t_items.size() * (int64_t)sizeof(TcItem), 16) +
+                      round_up((F * t_bound + 4 * kTcFineItems) * (int64_t)sizeof(TcItem), 16) +
                       round_up(F * (int64_t)one.tabs.size() * 4, 16) + 4096;
         h->desc_cap = round_up(h->desc_cap, kAlign);
     }
@@ -980,6 +1045,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     h->atlas.rows = rows;
     h->atlas.hog_plane = (int64_t)rows * P;
     h->atlas.lbp_plane = (int64_t)rows * P;
+    h->atlas.lbp_cells = (params->flags & PD_FLAG_SVM_FP32) ? 0 : 1;
     h->score_cap = std::max<int64_t>(worst.score_floats, 1);
     h->frames_cap = (int64_t)params->max_frames * round_up(params->max_width, 16) * params->max_height;
 
@@ -993,7 +1059,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
         {h->desc_cap, 0},                                          // 2 descriptors
         {h->pyr_cap, 0},                                           // 3 pyramid
         {(int64_t)hog_planes_of(params->flags) * h->atlas.hog_plane * 4, 0},  // 4 hog atlas
-        {(int64_t)kLbpBins * h->atlas.lbp_plane, 0},               // 5 lbp atlas
+        {(h->atlas.lbp_cells ? kLbpCellBytes : kLbpBins) * h->atlas.lbp_plane, 0},  // 5 lbp atlas
         {h->score_cap * 4, 0},                                     // 6 scores
         {(int64_t)params->max_frames * params->max_boxes_per_frame * (int64_t)sizeof(pd_box), 0},  // 7
         {(int64_t)params->max_frames * 2 * 4 + 16, 0},             // 8 counts + error word + item counters
@@ -1005,6 +1071,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
         {h->score_cap * 4, 0},                                                      // 13 window logits
         {2 * h->flag_cap * 4, 0},                                                   // 14 tile flags
         {(int64_t)nms_sched_ints(params->max_frames) * 4, 0},                       // 15 NMS frame order
+        {kTcConstBytes, 0},                                                         // 16 tensor-core K4 constants
     };
     int64_t total = 0;
     for (auto &pt : parts) {
@@ -1025,6 +1092,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     h->d_counts = reinterpret_cast<int32_t *>(h->arena + parts[8].off);
     h->d_err = reinterpret_cast<unsigned *>(h->d_counts + 2 * params->max_frames);
     h->d_queue = reinterpret_cast<int *>(h->d_err + 1);
+    h->d_tc_consts = h->arena + parts[16].off;
     h->d_frames = h->arena + parts[9].off;
     h->d_nms_scratch = reinterpret_cast<float4 *>(h->arena + parts[10].off);
     h->cnn = reinterpret_cast<float *>(h->arena + parts[11].off);
@@ -1080,10 +1148,13 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     if (cudaMemcpy(h->d_w, wt.data(), wt.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_lbp_map, map, 256, cudaMemcpyHostToDevice) != cudaSuccess)
         return bail(PD_ECUDA);
-    if (encode_svm_maps(h->hog_map, h->lbp_map, h->atlas.hog, h->atlas.lbp, P, rows, h->atlas.hog_plane,
-                        h->atlas.lbp_plane) != PD_OK ||
-        encode_tc_maps(&h->tc_hog_map, &h->tc_lbp_map, h->atlas.hog, h->atlas.lbp, P, rows, h->atlas.hog_plane,
-                       h->atlas.lbp_plane, hog_planes_of(params->flags)) != PD_OK)
+    std::vector<unsigned char> consts(kTcConstBytes);
+    build_tc_consts(wt.data(), consts.data());
+    if (cudaMemcpy(h->d_tc_consts, consts.data(), consts.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        return bail(PD_ECUDA);
+    if ((params->flags & PD_FLAG_SVM_FP32) &&
+        encode_svm_maps(h->hog_map, h->lbp_map, h->atlas.hog, h->atlas.lbp, P, rows, h->atlas.hog_plane,
+                        h->atlas.lbp_plane) != PD_OK)
         return bail(PD_ECUDA);
     if (cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
         return bail(PD_ECUDA);
@@ -1123,13 +1194,12 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
     if (!reuse) {
         invalidate_cache(h);
         p.clear();
-        p.tc_rows = h->tuning.tc_item_rows;
         for (int f = 0; f < n_frames; ++f) {
             int r = plan_frame(p, h->p, d_frames[f], widths[f], heights[f], pitches[f],
                                h->proposal ? kSparseTileCost : h->tile_cost, h->proposal);
             if (r != PD_OK) return fail(h, r, "frame %d: planning failed", f);
         }
-        order_tc(p.t_items);
+        plan_tc(p, h->tuning.tc_item_rows, h->sm_count);
         plan_strips(p, h->sm_count * kStripWarpsPerSm);
         if (!(h->p.flags & PD_FLAG_SVM_FP32)) assign_tc_maps(p);
         if (p.atlas_rows > h->atlas.rows || p.pyr_bytes > h->pyr_cap || p.score_floats > h->score_cap ||
@@ -1186,10 +1256,10 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
                                   dptr<SvmItem>(h, o.s_items), (int)p.s_items.size(), h->d_err, sf));
         } else {
             PD_CUDA(h, cudaMemsetAsync(h->d_queue, 0, sizeof(int), q));
-            PD_CUDA(h, launch_svm_tc(q, h->tc_hog_map, h->tc_lbp_map, dl, dptr<TcItem>(h, o.t_items),
-                                     (int)p.t_items.size(), h->d_queue, h->sm_count, h->d_w, h->bias,
+            PD_CUDA(h, launch_svm_tc(q, CUtensorMap{}, CUtensorMap{}, dl, dptr<TcItem>(h, o.t_items),
+                                     (int)p.t_items.size(), h->d_queue, h->sm_count, h->d_tc_consts, h->bias,
                                      h->p.l2hys_clip, h->d_scores, cf, h->d_err, hog_planes_of(h->p.flags),
-                                     p.tc_widths.empty() ? nullptr : dptr<CUtensorMap>(h, o.tc_maps)));
+                                     dptr<CUtensorMap>(h, o.tc_maps)));
         }
         if (timed) PD_CUDA(h, record(h->stage_ev[3], q));
         PD_CUDA(h, launch_nms(q, df, dl, n_frames, h->d_scores, h->p.threshold, h->p.nms_iou,
@@ -1663,7 +1733,6 @@ int pd_window_scores(pd_handle *h, void *stream, const float *d_hog, int64_t hog
         (reinterpret_cast<uintptr_t>(d_hog) & 15) || (reinterpret_cast<uintptr_t>(d_lbp) & 15))
         return fail(h, PD_EINVAL, "pd_window_scores: bad argument");
     Plan p;
-    p.tc_rows = h->tuning.tc_item_rows;
     plan_level(p, 0, 0, 8 * cells_x, 8 * cells_y, 8 * cells_x, 8 * cells_y, 0, 8 * cells_x, nullptr,
                h->tile_cost);
     p.c_items.clear();
@@ -1671,18 +1740,24 @@ int pd_window_scores(pd_handle *h, void *stream, const float *d_hog, int64_t hog
     p.tabs.clear();
     if (p.s_items.empty()) return PD_OK;
     const bool fp32 = (h->p.flags & PD_FLAG_SVM_FP32) != 0;
-    if (fp32)
-        p.t_items.clear();
-    else
-        p.s_items.clear();
-    order_tc(p.t_items);
     CUtensorMap hm[kSvmShapes], lm[kSvmShapes], th, tl;
-    const int64_t rows = std::max(cells_y, 1);
-    if (encode_svm_maps(hm, lm, d_hog, d_lbp, cell_pitch, rows, hog_plane, lbp_plane) != PD_OK ||
-        encode_tc_maps(&th, &tl, d_hog, d_lbp, cell_pitch, rows, hog_plane, lbp_plane,
-                       hog_planes_of(h->p.flags)) != PD_OK)
-        return fail(h, PD_ECUDA, "pd_window_scores: tensor map encoding failed");
+    uint8_t *cells = h->atlas.lbp;  // tensor cores: the planes' counts, cell-major
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    if (fp32) {
+        if (encode_svm_maps(hm, lm, d_hog, d_lbp, cell_pitch, cells_y, hog_plane, lbp_plane) != PD_OK)
+            return fail(h, PD_ECUDA, "pd_window_scores: tensor map encoding failed");
+    } else {
+        p.s_items.clear();
+        plan_tc(p, h->tuning.tc_item_rows, h->sm_count);
+        if ((int64_t)cells_x * cells_y > h->atlas.lbp_plane) {  // a level larger than the handle's own
+            const int r = scheme_scratch(h, s, (size_t)cells_x * cells_y * kLbpCellBytes);
+            if (r != PD_OK) return r;
+            cells = h->scheme_ws;
+        }
+        if (encode_tc_maps(&th, &tl, d_hog, cell_pitch, hog_plane, hog_planes_of(h->p.flags), cells, cells_x, cells_y,
+                           cells_x) != PD_OK)
+            return fail(h, PD_ECUDA, "pd_window_scores: tensor map encoding failed");
+    }
     Packed o;
     int r = upload_plan(h, s, p, o);
     if (r != PD_OK) return r;
@@ -1692,8 +1767,9 @@ int pd_window_scores(pd_handle *h, void *stream, const float *d_hog, int64_t hog
                               d_scores, dptr<SvmItem>(h, o.s_items), (int)p.s_items.size(), h->d_err));
     } else {
         PD_CUDA(h, cudaMemsetAsync(h->d_queue, 0, sizeof(int), s));
+        PD_CUDA(h, launch_lbp_cells(s, d_lbp, lbp_plane, cell_pitch, cells_x, cells_y, cells));
         PD_CUDA(h, launch_svm_tc(s, th, tl, dptr<LevelDesc>(h, o.levels), dptr<TcItem>(h, o.t_items),
-                                 (int)p.t_items.size(), h->d_queue, h->sm_count, h->d_w, h->bias,
+                                 (int)p.t_items.size(), h->d_queue, h->sm_count, h->d_tc_consts, h->bias,
                                  h->p.l2hys_clip, d_scores, nullptr, h->d_err, hog_planes_of(h->p.flags)));
     }
     return PD_OK;
@@ -1740,20 +1816,6 @@ int pd_nms_maps(pd_handle *h, void *stream, const float *d_scores, int n_levels,
     return PD_OK;
 }
 
-namespace {
-// Scratch of the kernel-scheme entries, grown on demand (the stream is
-// synchronised first: earlier work on it may still use the old buffer).
-int scheme_scratch(pd_handle *h, cudaStream_t s, size_t need) {
-    if (need <= h->scheme_ws_bytes) return PD_OK;
-    PD_CUDA(h, cudaStreamSynchronize(s));
-    if (h->scheme_ws) cudaFree(h->scheme_ws);
-    h->scheme_ws = nullptr;
-    h->scheme_ws_bytes = 0;
-    if (cudaMalloc(&h->scheme_ws, need) != cudaSuccess) return fail(h, PD_ENOMEM, "scheme scratch");
-    h->scheme_ws_bytes = need;
-    return PD_OK;
-}
-}  // namespace
 
 int pd_scheme_cells(pd_handle *h, void *stream, int scheme, const uint8_t *d_level, int Wk, int Hk, int pitch,
                     float *d_hog, int64_t hog_plane, uint8_t *d_lbp, int64_t lbp_plane, int cell_pitch) {

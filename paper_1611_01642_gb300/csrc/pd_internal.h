@@ -63,7 +63,7 @@ struct LevelDesc {
 struct ResizeItem { int32_t frame, x0, y0, pad; };   // source tile of a frame
 struct CellItem { int32_t level, cx0, cy0, pad; };   // cell tile of a level
 struct SvmItem { int32_t level, wx0, wy0, shape; };  // window tile of a level, tile shape index
-struct TcItem { int32_t level, wx0, wy0, wy1; };     // tensor-core K4: window columns [wx0, wx0 + 104), rows [wy0, wy1)
+struct TcItem { int32_t level, wx0, wy0, wy1; };     // tensor-core K4: window columns [wx0, wx0 + 26), rows [wy0, wy1)
 struct StripItem { int32_t level, cx0, cy0, cy1; };  // K2+K3 warp: cells [cx0, cx0 + 15) x rows [cy0, cy1)
 
 // Tiles.
@@ -80,9 +80,13 @@ constexpr int kCellTH = 8;      // cells per cell tile along y
 constexpr int kStripTiles = 4;  // cell tiles per K2+K3 strip (one warp each), top to bottom, at most
 constexpr int kStripWarpsPerSm = 16;  // K2+K3 warps resident per SM (4 CTAs of 4)
 constexpr int kSvmShapes = 7;   // K4 tile shapes: 32x16, 64x8, 32x8, 64x4, 64x2, 32x12, 32x4 windows
-constexpr int kTcStrip = 104;   // tensor-core K4: window columns per item
+constexpr int kTcStrip = 26;    // tensor-core K4: window columns per item (32 blocks, a lane quarter of the MMA)
 constexpr int kTcChunk = 64;    // tensor-core K4: window rows per item at most (tunable down to kTcMinChunk)
 constexpr int kTcMinChunk = 8;
+constexpr int kTcWalkers = 4;   // tensor-core K4: items walked at a time by a CTA (one CTA per SM)
+constexpr int kTcFineItems = 4096;  // plans of at most this many items may cut them below kTcMinChunk rows
+constexpr int kTcConstBytes = 45056;  // tensor-core K4: B operand (43,008 bytes) and LBP table (2,048)
+constexpr int kLbpCellBytes = 64;     // LBP counts of a cell in the cell-major atlas (59 bins, zeros)
 
 struct SvmShapeInfo {
     int tw, th;     // windows per tile along x / y
@@ -93,7 +97,10 @@ struct SvmShapeInfo {
 SvmShapeInfo svm_shape(int s);
 int svm_lbp_chunk();  // LBP planes per TMA box
 
-// Cell atlas: plane-major [plane][atlas_rows][pitch]; pitch in elements.
+// Cell atlas: plane-major [plane][atlas_rows][pitch]; pitch in elements. The LBP
+// counts are cell-major, [atlas_rows][pitch][64 bytes], when lbp_cells is set:
+// the tensor-core K4 then reads 16 bins of a cell per load, and the cells
+// kernel writes a cell's counts with 16-byte stores instead of 59 byte planes.
 struct CellAtlas {
     float *hog;        // 9 planes (36 for per-block HOG)
     uint8_t *lbp;      // 59 planes
@@ -101,6 +108,7 @@ struct CellAtlas {
     int64_t lbp_plane; // elements per LBP plane
     int32_t pitch;     // elements per row (multiple of 16)
     int32_t rows;      // rows per plane
+    int32_t lbp_cells; // 1: cell-major LBP counts
 };
 
 // One-time per-device kernel attribute set-up (dynamic shared memory opt-in).
@@ -137,17 +145,25 @@ cudaError_t launch_svm(cudaStream_t s, const CUtensorMap *hog_maps, const CUtens
                        const uint32_t *s_flag = nullptr);
 // Tensor-core K4: persistent CTAs (grid at most one per SM) over an item
 // queue (*d_queue must be 0 at launch); c_flag non-null selects the sparse
-// path. hog_map / lbp_map: 3-D maps over the cell planes with boxes of
-// 112 x 1 x hog_planes (f32; 9, or 36 for per-block HOG) and 128 x 1 x 59 (u8).
+// path. The maps are encode_tc_maps pairs; d_consts: build_tc_consts.
 cudaError_t init_svm_tc();
-int svm_tc_smem_bytes(int hog_planes = kHogBins);
+// Constants of the tensor-core K4 from the template [95][15][8]: kTcConstBytes bytes.
+void build_tc_consts(const float *wt, unsigned char *out);
+// HOG planes (x extent: width) and cell-major LBP counts, one cell row per box;
+// boxes reaching past the width read zeros.
+int encode_tc_maps(CUtensorMap *hog_map, CUtensorMap *lbp_map, const float *hog, int64_t hog_pitch, int64_t hog_plane,
+                   int hog_planes, const uint8_t *lbp, int64_t lbp_pitch, int64_t rows, int64_t width);
+// LBP planes -> cell-major counts [rows][width][64].
+cudaError_t launch_lbp_cells(cudaStream_t s, const uint8_t *planes, int64_t plane, int pitch, int width, int rows,
+                             uint8_t *out);
 // level_maps: null, or 2 maps per entry of LevelDesc::tc_map (HOG, LBP) in device
 // memory (64-byte aligned) whose x extent is the level's width, so that a box
 // reaching past it reads zeros instead of the atlas row's padding.
 cudaError_t launch_svm_tc(cudaStream_t s, const CUtensorMap &hog_map, const CUtensorMap &lbp_map,
                           const LevelDesc *d_levels, const TcItem *d_items, int n_items, int *d_queue, int grid,
-                          const float *d_w, float bias, float clip, float *scores, const uint32_t *c_flag,
-                          unsigned *d_err, int hog_planes = kHogBins, const CUtensorMap *level_maps = nullptr);
+                          const unsigned char *d_consts, float bias, float clip, float *scores,
+                          const uint32_t *c_flag, unsigned *d_err, int hog_planes = kHogBins,
+                          const CUtensorMap *level_maps = nullptr);
 // Per-frame NMS scratch (float4 units) for a candidate cap: the decoded
 // boxes, plus the sort keys when the cap is above 16,384 (shared memory
 // holds them below).
@@ -265,6 +281,8 @@ cudaError_t launch_round_params(cudaStream_t s, const float *master, float *wr);
 int encode_plane_map(CUtensorMap *map, void *base, CUtensorMapDataType dtype, int elem_bytes,
                      int64_t pitch, int64_t rows, int64_t planes, int64_t plane_stride_elems,
                      uint32_t box_x, uint32_t box_y, uint32_t box_planes, int64_t width = 0);
+// Cell-major LBP counts [rows][pitch][64 bytes]: boxes of box_cells cells of one row, 64-byte swizzle.
+int encode_cell_map(CUtensorMap *map, uint8_t *base, int64_t pitch, int64_t rows, int64_t width, uint32_t box_cells);
 
 // Host-side tables.
 void build_lbp_bin_table(uint8_t table[256]);
