@@ -623,8 +623,16 @@ void k1_tables(Plan &p, LevelDesc &L, int W, int H, int Wk, int Hk) {
     }
 }
 
-// Adds one level to the plan (tables, descriptor, work items).
-void plan_level(Plan &p, int frame, int level, int W, int H, int Wk, int Hk, int64_t img_off,
+// What a plan is for: only the tables and items that its kernels read are made.
+// (The Q11 tables and the FP32 tiles' dynamic programming are most of a level's
+// planning time: a pd_cell_features call on a 1920x1080 level planned for 50 us
+// what it never launched.)
+constexpr unsigned kPlanResize = 1;   // K1 tables
+constexpr unsigned kPlanTiles = 2;    // cell tiles (per-block HOG, sparse flags)
+constexpr unsigned kPlanWindows = 4;  // FP32 K4 window tiles (also the proposal's keep granularity)
+
+// Adds one level to the plan (descriptor, and the tables and items of `what`).
+void plan_level(Plan &p, unsigned what, int frame, int level, int W, int H, int Wk, int Hk, int64_t img_off,
                 int32_t img_pitch, const LevelDesc *share = nullptr,
                 const float *tile_cost = kDefaultTileCost) {
     LevelDesc L{};
@@ -652,16 +660,17 @@ void plan_level(Plan &p, int frame, int level, int W, int H, int Wk, int Hk, int
         L.rgroup = share->rgroup;
         L.rspan = share->rspan;
         L.xq_off = share->xq_off;
-    } else {
+    } else if (what & kPlanResize) {
         k1_tables(p, L, W, H, Wk, Hk);
     }
     const int li = (int)p.levels.size();
     L.hsrc = li;
     L.citem0 = (int32_t)p.c_items.size();
     L.ctx = (L.Wc + kCellTW - 1) / kCellTW;
-    for (int cy = 0; cy < L.Hc; cy += kCellTH)
-        for (int cx = 0; cx < L.Wc; cx += kCellTW) p.c_items.push_back({li, cx, cy, 0});
-    plan_windows(p.s_items, li, L.rows, L.cols, tile_cost);
+    if (what & kPlanTiles)
+        for (int cy = 0; cy < L.Hc; cy += kCellTH)
+            for (int cx = 0; cx < L.Wc; cx += kCellTW) p.c_items.push_back({li, cx, cy, 0});
+    if (what & kPlanWindows) plan_windows(p.s_items, li, L.rows, L.cols, tile_cost);
     p.atlas_rows += L.Hc;
     p.score_floats += (int64_t)L.rows * L.cols;
     p.max_wc = std::max(p.max_wc, L.Wc);
@@ -676,7 +685,7 @@ int32_t staged_bytes(const Plan &p, const FrameDesc &fd) {
 }
 
 // Plans one frame with the pyramid rule; returns PD_OK or an error.
-int plan_frame(Plan &p, const pd_params &prm, const uint8_t *ptr, int W, int H, int pitch,
+int plan_frame(Plan &p, unsigned what, const pd_params &prm, const uint8_t *ptr, int W, int H, int pitch,
                const float *tile_cost = kDefaultTileCost, bool proposal = false) {
     int32_t Wk[PD_MAX_LEVELS], Hk[PD_MAX_LEVELS];
     int n = level_sizes(W, H, prm.pyr_factor, prm.upscale_levels, PD_MAX_LEVELS, Wk, Hk);
@@ -695,7 +704,7 @@ int plan_frame(Plan &p, const pd_params &prm, const uint8_t *ptr, int W, int H, 
     for (int k = 0; k < n; ++k) {
         const int32_t lp = (int32_t)round_up(Wk[k], 16);
         const LevelDesc share = first_shared >= 0 ? p.levels[first_shared + k] : LevelDesc{};
-        plan_level(p, f, k, W, H, Wk[k], Hk[k], p.pyr_bytes, lp, first_shared >= 0 ? &share : nullptr,
+        plan_level(p, what, f, k, W, H, Wk[k], Hk[k], p.pyr_bytes, lp, first_shared >= 0 ? &share : nullptr,
                    tile_cost);
         p.pyr_bytes += (int64_t)lp * Hk[k];
         if (proposal) {
@@ -991,7 +1000,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     // Worst-case plan: max_frames frames of max_width x max_height.
     Plan worst;
     for (int f = 0; f < params->max_frames; ++f)
-        if (plan_frame(worst, *params, nullptr, params->max_width, params->max_height,
+        if (plan_frame(worst, 0, *params, nullptr, params->max_width, params->max_height,
                        params->max_width) != PD_OK)
             return bail(PD_EINVAL);
     if (worst.levels.empty()) {
@@ -1003,7 +1012,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     // tables (frames of different sizes do not share them).
     {
         Plan one;
-        plan_frame(one, *params, nullptr, params->max_width, params->max_height, params->max_width);
+        plan_frame(one, kPlanResize | kPlanTiles, *params, nullptr, params->max_width, params->max_height, params->max_width);
         int64_t s_bound = 0;
         for (const LevelDesc &L : one.levels) {
             int64_t most = 0;
@@ -1194,14 +1203,20 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
     if (!reuse) {
         invalidate_cache(h);
         p.clear();
+        const bool fp32 = (h->p.flags & PD_FLAG_SVM_FP32) != 0;
+        const unsigned what = kPlanResize |
+                              (h->proposal || (h->p.flags & PD_FLAG_HOG_PER_BLOCK) ? kPlanTiles : 0u) |
+                              (h->proposal || fp32 ? kPlanWindows : 0u);
         for (int f = 0; f < n_frames; ++f) {
-            int r = plan_frame(p, h->p, d_frames[f], widths[f], heights[f], pitches[f],
+            int r = plan_frame(p, what, h->p, d_frames[f], widths[f], heights[f], pitches[f],
                                h->proposal ? kSparseTileCost : h->tile_cost, h->proposal);
             if (r != PD_OK) return fail(h, r, "frame %d: planning failed", f);
         }
-        plan_tc(p, h->tuning.tc_item_rows, h->sm_count);
+        if (!fp32) {
+            plan_tc(p, h->tuning.tc_item_rows, h->sm_count);
+            assign_tc_maps(p);
+        }
         plan_strips(p, h->sm_count * kStripWarpsPerSm);
-        if (!(h->p.flags & PD_FLAG_SVM_FP32)) assign_tc_maps(p);
         if (p.atlas_rows > h->atlas.rows || p.pyr_bytes > h->pyr_cap || p.score_floats > h->score_cap ||
             (int64_t)p.s_items.size() > h->flag_cap || (int64_t)p.c_items.size() > h->flag_cap)
             return fail(h, PD_EINVAL, "batch exceeds the arena");
@@ -1297,8 +1312,8 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         if (r != PD_OK) return r;
     }
     PD_CUDA(h, cudaEventRecord(h->graph_done, s));
-    h->last_launches = (p.r_items.empty() ? 0 : 1) + (p.c_items.empty() ? 0 : 1) +
-                       (p.s_items.empty() ? 0 : 1) +
+    h->last_launches = (p.r_items.empty() ? 0 : 1) + (p.strips.empty() ? 0 : 1) +
+                       (p.score_floats == 0 ? 0 : 1) +
                        nms_launches(n_frames, nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame)) +
                        (h->proposal ? (p.cnn_items.empty() ? 0 : 1) + (p.levels.empty() ? 0 : 1) +
                                           (p.s_items.empty() ? 0 : 1)
@@ -1429,12 +1444,7 @@ int pd_cnn_forward(pd_handle *h, void *stream, const uint8_t *d_level, int Wk, i
         pitch = lp;
     }
     Plan p;
-    plan_level(p, 0, 0, Wk, Hk, Wk, Hk, 0, pitch);
-    p.c_items.clear();
-    p.strips.clear();
-    p.s_items.clear();
-    p.t_items.clear();
-    p.tabs.clear();
+    plan_level(p, 0, 0, 0, Wk, Hk, Wk, Hk, 0, pitch);
     for (int cy = 0; cy < Hc; cy += kCnnTile)
         for (int cx = 0; cx < Wc; cx += kCnnTile) p.cnn_items.push_back({0, cy, cx, 0});
     Packed o;
@@ -1672,16 +1682,12 @@ int pd_resize_levels(pd_handle *h, void *stream, const uint8_t *d_frame, int W, 
     for (int k = 0; k < n_levels; ++k) {
         if (Wk[k] < 1 || Hk[k] < 1 || Wk[k] > 4 * W || Hk[k] > 4 * H || level_pitches[k] < Wk[k])
             return fail(h, PD_EINVAL, "pd_resize_levels: level %d size %dx%d", k, Wk[k], Hk[k]);
-        plan_level(p, 0, k, W, H, Wk[k], Hk[k], level_offsets[k], level_pitches[k]);
+        plan_level(p, kPlanResize, 0, k, W, H, Wk[k], Hk[k], level_offsets[k], level_pitches[k]);
     }
     fd.rbw = staged_bytes(p, fd);
     for (int y = 0; y < H; y += kResizeTH)
         for (int x = 0; x < W; x += kResizeTW) p.r_items.push_back({0, x, y, 0});
     p.frames.push_back(fd);
-    p.c_items.clear();
-    p.strips.clear();
-    p.s_items.clear();
-    p.t_items.clear();
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     Packed o;
     int r = upload_plan(h, s, p, o);
@@ -1701,11 +1707,9 @@ int pd_cell_features(pd_handle *h, void *stream, const uint8_t *d_level, int Wk,
         cell_pitch % 16 != 0 || hog_plane < (int64_t)Hc * cell_pitch || lbp_plane < (int64_t)Hc * cell_pitch)
         return fail(h, PD_EINVAL, "pd_cell_features: bad argument");
     Plan p;
-    plan_level(p, 0, 0, Wk, Hk, Wk, Hk, 0, pitch);
-    plan_strips(p, h->sm_count * kStripWarpsPerSm);
-    p.s_items.clear();
-    p.t_items.clear();
-    p.tabs.clear();
+    const bool per_block = (features_of(h->p.flags) & kFeatHogBlock) != 0;
+    plan_level(p, per_block ? kPlanTiles : 0u, 0, 0, Wk, Hk, Wk, Hk, 0, pitch);
+    if (!per_block) plan_strips(p, h->sm_count * kStripWarpsPerSm);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     Packed o;
     int r = upload_plan(h, s, p, o);
@@ -1733,13 +1737,10 @@ int pd_window_scores(pd_handle *h, void *stream, const float *d_hog, int64_t hog
         (reinterpret_cast<uintptr_t>(d_hog) & 15) || (reinterpret_cast<uintptr_t>(d_lbp) & 15))
         return fail(h, PD_EINVAL, "pd_window_scores: bad argument");
     Plan p;
-    plan_level(p, 0, 0, 8 * cells_x, 8 * cells_y, 8 * cells_x, 8 * cells_y, 0, 8 * cells_x, nullptr,
-               h->tile_cost);
-    p.c_items.clear();
-    p.strips.clear();
-    p.tabs.clear();
-    if (p.s_items.empty()) return PD_OK;
     const bool fp32 = (h->p.flags & PD_FLAG_SVM_FP32) != 0;
+    plan_level(p, fp32 ? kPlanWindows : 0u, 0, 0, 8 * cells_x, 8 * cells_y, 8 * cells_x, 8 * cells_y, 0, 8 * cells_x,
+               nullptr, h->tile_cost);
+    if (p.score_floats == 0) return PD_OK;
     CUtensorMap hm[kSvmShapes], lm[kSvmShapes], th, tl;
     uint8_t *cells = h->atlas.lbp;  // tensor cores: the planes' counts, cell-major
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -1747,7 +1748,6 @@ int pd_window_scores(pd_handle *h, void *stream, const float *d_hog, int64_t hog
         if (encode_svm_maps(hm, lm, d_hog, d_lbp, cell_pitch, cells_y, hog_plane, lbp_plane) != PD_OK)
             return fail(h, PD_ECUDA, "pd_window_scores: tensor map encoding failed");
     } else {
-        p.s_items.clear();
         plan_tc(p, h->tuning.tc_item_rows, h->sm_count);
         if ((int64_t)cells_x * cells_y > h->atlas.lbp_plane) {  // a level larger than the handle's own
             const int r = scheme_scratch(h, s, (size_t)cells_x * cells_y * kLbpCellBytes);
