@@ -61,8 +61,8 @@
 // its place in the block); a block takes q = 0, 1 from its upper row and
 // q = 2, 3 from its lower one, and nothing else changes.
 // Sparse path: a window is scored when every cell tile under it was computed;
-// cell rows that no such window of the item needs are skipped, other windows
-// get -inf. A wait that gives up (1 s) sets the error word and a CTA flag that
+// cell rows that no such window of the item needs are skipped. The caller has
+// filled the score maps with -inf; a walked row's other windows get it again. A wait that gives up (1 s) sets the error word and a CTA flag that
 // ends every role's waits; the CTA then drains its copies and MMAs, frees its
 // tensor memory and leaves.
 #include "pd_internal.h"
@@ -86,8 +86,9 @@ constexpr int kChunks = 24;           // 16-byte K chunks per operand row: 12 hi
 constexpr int kSBO = kChunks * 128;   // bytes per 8-row group
 constexpr int kHogX = 36;             // HOG cells per staged row of a group (from a 4-cell boundary)
 constexpr int kLbpX = 33;             // LBP cells per staged row of a group
-constexpr int kTileRows = (kTcChunk - 1 + kWinBH) / kCellTH + 2;  // cell-tile rows under an item at most
-static_assert(kTileRows <= 32 && kWinBW < kCellTW && kWinBH < 2 * kCellTH, "sparse masks");
+constexpr int kTileRows = (kTcSparseRows - 1 + kWinBH) / kCellTH + 2;  // cell-tile rows under an item at most
+static_assert(kTileRows <= 32 && kWinBW < kCellTW && kWinBH < 2 * kCellTH && kTcSparseRows + kWinBH <= 64 &&
+                  kTcSparseRows > 32, "sparse masks");
 constexpr int kMeta = 16;             // step descriptions in flight (more than any role can lag behind)
 constexpr uint32_t kTmemCols = 512;   // two accumulator buffers of 128 columns, two A stages of 96
 constexpr uint32_t kTmemA = 256;      // first A stage column (bf16 pairs: high parts 0..47, low 48..95)
@@ -120,7 +121,7 @@ struct TcSmemT {
     uint32_t tab[512];
     SlotT<HP> slot[kSlots];               // staged cell rows
     StepMeta meta[kMeta][kGroups];
-    uint32_t keep[kGroups][kTcChunk];     // sparse: scored windows of an item's rows
+    uint32_t keep[kGroups][2][kTcSparseRows];  // sparse: scored windows of the rows of the current and next items
     unsigned long long bfull;             // constants arrived
     unsigned long long cfull[kSlots];     // cell row arrived (TMA transaction count)
     unsigned long long cempty[kSlots];    // cell row no longer read (8 producer warps)
@@ -557,12 +558,84 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         __syncwarp();
     } else {
-        // ---- items and cell rows; lane g < 4 serves group g
+        // ---- items and cell rows; lane g < 4 serves group g. The group's next item is
+        // fetched a stage per step (queue ticket, item, level), so that no step waits for
+        // a chain of global loads; on the sparse path the warp then works out its windows.
         const bool sparse = c_flag != nullptr;
         const bool mine = lane < kGroups;
-        int next = mine ? (int)blockIdx.x + lane * (int)gridDim.x : n_items;  // next item of the group
+        enum : int { kTicket = 1, kItem, kLevel, kReady, kNone };  // what of the next item is in flight or here
+        int stage = mine ? kTicket : kNone;
+        int ticket = (int)blockIdx.x + lane * (int)gridDim.x;
         TcItem nit{};
-        if (next < n_items) nit = items[next];
+        int n_cell_row = 0, n_cols = 0, n_map = 0, n_citem0 = 0, n_ctx = 0;
+        int64_t n_score = 0;
+        unsigned long long n_walk = 0;  // sparse: cell rows (from the item's first) to walk
+        auto advance = [&]() {
+            if (stage == kTicket) {
+                stage = kNone;
+                if (ticket < n_items) {
+                    nit = items[ticket];
+                    stage = kItem;
+                }
+            } else if (stage == kItem) {
+                const LevelDesc &L = levels[nit.level];
+                n_cell_row = L.cell_row;
+                n_cols = L.cols;
+                n_map = L.tc_map;
+                n_citem0 = L.citem0;
+                n_ctx = L.ctx;
+                n_score = L.score_off;
+                stage = sparse ? kLevel : kReady;
+            }
+        };
+        int buf = 0;  // sparse: the buffer of S.keep that the group's current item uses
+        // Sparse, whole warp: the scored windows of group g's next item, and the cell rows
+        // they need (a window row needs 16 of them).
+        auto prepare = [&](int g) {
+            const int y0 = __shfl_sync(0xffffffffu, nit.wy0, g), x0 = __shfl_sync(0xffffffffu, nit.wx0, g);
+            const int n = __shfl_sync(0xffffffffu, nit.wy1, g) - y0;
+            const int nc = min(kTcStrip, __shfl_sync(0xffffffffu, n_cols, g) - x0);
+            const int ctx = __shfl_sync(0xffffffffu, n_ctx, g), other = __shfl_sync(0xffffffffu, buf, g) ^ 1;
+            // lane = window column: a window lies in one or two cell tiles across; the
+            // ballot of tile row t stays with lane t
+            const int ty0 = y0 / kCellTH, nt = (y0 + n - 1 + kWinBH) / kCellTH - ty0 + 1;
+            const int wx = x0 + lane;
+            const int cl = lane < nc ? wx / kCellTW : 0, cr = lane < nc ? (wx + kWinBW) / kCellTW : 0;
+            const uint32_t *flags = c_flag + __shfl_sync(0xffffffffu, n_citem0, g) + ty0 * ctx;
+            uint32_t f[kTileRows][2];
+#pragma unroll
+            for (int t = 0; t < kTileRows; ++t) {
+                const uint32_t *row = flags + min(t, nt - 1) * ctx;
+                f[t][0] = __ldg(row + cl);
+                f[t][1] = __ldg(row + cr);
+            }
+            uint32_t bits = 0;
+#pragma unroll
+            for (int t = 0; t < kTileRows; ++t) {
+                const uint32_t b = __ballot_sync(0xffffffffu, lane < nc && f[t][0] && f[t][1]);
+                if (lane == t) bits = b;
+            }
+            // lane = window row: its 16 cell rows lie in two or three tile rows
+            unsigned long long kept = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int row = 32 * h + lane, y = y0 + min(row, n - 1);
+                const int a0 = y / kCellTH - ty0, a1 = (y + kWinBH) / kCellTH - ty0;
+                const uint32_t k = __shfl_sync(0xffffffffu, bits, a0) & __shfl_sync(0xffffffffu, bits, a0 + 1) &
+                                   __shfl_sync(0xffffffffu, bits, a1);
+                if (row < n) S.keep[g][other][row] = k;
+                kept |= (unsigned long long)__ballot_sync(0xffffffffu, row < n && k) << (32 * h);
+            }
+            __syncwarp();
+            if (lane == g) {
+                kept |= kept << 1;  // 16 wide: kTcSparseRows + 15 bits
+                kept |= kept << 2;
+                kept |= kept << 4;
+                kept |= kept << 8;
+                n_walk = kept;
+                stage = kReady;
+            }
+        };
         // the item being walked
         bool active = false;
         const CUtensorMap *hm = &hog_map, *lm = &lbp_map;
@@ -570,20 +643,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         int r = 0, r0 = 0, r_end = -1;  // next cell row, first and last one of the run
         bool first = false;
         int64_t score_off = 0;
-        unsigned long long rows64 = 0;  // sparse: window rows (from wy0) with a scored window
-        auto next_run = [&]() {         // sparse: the next run of cell rows, if any
-            if (!rows64) return false;
-            const int a = __ffsll((long long)rows64) - 1;
-            int b = a;  // last kept row of the run: rows whose walks overlap
-            rows64 &= rows64 - 1ull;
-            while (rows64) {
-                const int n = __ffsll((long long)rows64) - 1;
-                if (n > b + kWinBH) break;
-                b = n;
-                rows64 &= rows64 - 1ull;
-            }
+        unsigned long long walk = 0;  // sparse: cell rows of the later runs
+        auto next_run = [&]() {
+            if (!walk) return false;
+            const int a = __ffsll((long long)walk) - 1;
+            const unsigned long long after = ~(walk >> a);  // its lowest bit ends the run
+            const int len = after ? __ffsll((long long)after) - 1 : 64 - a;
+            walk = a + len < 64 ? walk >> (a + len) << (a + len) : 0ull;
             r = r0 = wy0 + a;
-            r_end = wy0 + b + kWinBH;
+            r_end = r + len - 1;
             first = true;
             return true;
         };
@@ -591,79 +659,41 @@ __global__ void __launch_bounds__(kThreads, 1)
             // groups whose item (or run) is done take the next
             if (active && r > r_end) active = sparse && next_run();
             for (;;) {
-                const bool want = mine && !active && next < n_items;
-                const unsigned who = __ballot_sync(0xffffffffu, want);
-                if (!who) break;
-                int n_rows = 0, lv = 0;
-                if (want) {
-                    const TcItem it = nit;
-                    next = 4 * (int)gridDim.x + atomicAdd(queue, 1);
-                    if (next < n_items) nit = items[next];  // in flight while this item is walked
-                    lv = it.level;
-                    const LevelDesc &L = levels[lv];
-                    wx0 = it.wx0;
-                    wy0 = it.wy0;
-                    n_rows = it.wy1 - it.wy0;
-                    cols = L.cols;
+                const bool want = mine && !active && stage != kNone;
+                if (!__any_sync(0xffffffffu, want)) break;
+                if (want)
+                    while (stage == kTicket || stage == kItem) advance();
+                if (sparse)
+                    for (unsigned left = __ballot_sync(0xffffffffu, want && stage == kLevel); left; left &= left - 1u)
+                        prepare(__ffs((int)left) - 1);
+                if (want && stage == kReady) {
+                    wx0 = nit.wx0;
+                    wy0 = nit.wy0;
+                    cols = n_cols;
                     ncols = min(kTcStrip, cols - wx0);
-                    cell_row = L.cell_row;
-                    score_off = L.score_off;
+                    cell_row = n_cell_row;
+                    score_off = n_score;
                     if (level_maps) {
-                        hm = level_maps + 2 * L.tc_map;
+                        hm = level_maps + 2 * n_map;
                         lm = hm + 1;
                     }
                     r = r0 = wy0;
-                    r_end = it.wy1 - 1 + kWinBH;
+                    r_end = nit.wy1 - 1 + kWinBH;
                     first = active = true;
-                }
-                if (!sparse) break;
-                // sparse: the scored windows of each new item, by the whole warp
-                for (unsigned left = who; left; left &= left - 1u) {
-                    const int g = __ffs((int)left) - 1;
-                    const int y0 = __shfl_sync(0xffffffffu, wy0, g), x0 = __shfl_sync(0xffffffffu, wx0, g);
-                    const int n = __shfl_sync(0xffffffffu, n_rows, g), nc = __shfl_sync(0xffffffffu, ncols, g);
-                    const int width = __shfl_sync(0xffffffffu, cols, g);
-                    const int64_t so = __shfl_sync(0xffffffffu, (long long)score_off, g);
-                    const LevelDesc &L = levels[__shfl_sync(0xffffffffu, lv, g)];
-                    // lane = window column: a window lies in one or two cell tiles across; the
-                    // ballot of tile row t (at most 11 of them) stays with lane t
-                    const int ty0 = y0 / kCellTH, nt = (y0 + n - 1 + kWinBH) / kCellTH - ty0 + 1;
-                    const int wx = x0 + lane;
-                    const int cl = lane < nc ? wx / kCellTW : 0, cr = lane < nc ? (wx + kWinBW) / kCellTW : 0;
-                    uint32_t f[kTileRows][2];
-#pragma unroll
-                    for (int t = 0; t < kTileRows; ++t) {
-                        const uint32_t *row = c_flag + L.citem0 + (ty0 + min(t, nt - 1)) * L.ctx;
-                        f[t][0] = __ldg(row + cl);
-                        f[t][1] = __ldg(row + cr);
-                    }
-                    uint32_t bits = 0;
-#pragma unroll
-                    for (int t = 0; t < kTileRows; ++t) {
-                        const uint32_t b = __ballot_sync(0xffffffffu, lane < nc && f[t][0] && f[t][1]);
-                        if (lane == t) bits = b;
-                    }
-                    // lane = window row: its 16 cell rows lie in two or three tile rows
-                    unsigned long long kept = 0;
-#pragma unroll
-                    for (int h = 0; h < kTcChunk / 32; ++h) {
-                        const int row = 32 * h + lane, y = y0 + min(row, n - 1);
-                        const int a0 = y / kCellTH - ty0, a1 = (y + kWinBH) / kCellTH - ty0;
-                        const uint32_t k = __shfl_sync(0xffffffffu, bits, a0) & __shfl_sync(0xffffffffu, bits, a0 + 1) &
-                                           __shfl_sync(0xffffffffu, bits, a1);
-                        const bool any = row < n && k;
-                        if (row < n) S.keep[g][row] = k;
-                        kept |= (unsigned long long)__ballot_sync(0xffffffffu, any) << (32 * h);
-                    }
-                    for (unsigned long long none = ~kept & (n == 64 ? ~0ull : (1ull << n) - 1ull); none; none &= none - 1ull) {
-                        const int row = __ffsll((long long)none) - 1;
-                        if (lane < nc) scores[so + (int64_t)(y0 + row) * width + wx] = -INFINITY;
-                    }
-                    __syncwarp();
-                    if (lane == g) {
-                        rows64 = kept;
+                    if (sparse) {
+                        buf ^= 1;
+                        walk = n_walk;
                         active = next_run();
                     }
+                    ticket = 4 * (int)gridDim.x + atomicAdd(queue, 1);
+                    stage = kTicket;
+                }
+            }
+            if (s & 1) {  // the next items, a stage at a time
+                advance();
+                if (sparse) {
+                    const unsigned ready = __ballot_sync(0xffffffffu, stage == kLevel);
+                    if (ready) prepare(__ffs((int)ready) - 1);
                 }
             }
             const uint32_t slot = s % kSlots;
@@ -676,7 +706,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int wy = r - kWinBH;  // the window row that this cell row completes
                     const bool store = wy >= r0;
                     m.flags = (first ? 1u : 2u) | (store ? 4u : 0u) | ((uint32_t)(wx0 & 3) << 4) | ((uint32_t)ncols << 8);
-                    m.keep = sparse && store ? S.keep[lane][wy - wy0] : 0xffffffffu;
+                    m.keep = sparse && store ? S.keep[lane][buf][wy - wy0] : 0xffffffffu;
                     m.out = score_off + (int64_t)wy * cols + wx0;
                 }
                 S.meta[s % kMeta][lane] = m;

@@ -629,7 +629,7 @@ void k1_tables(Plan &p, LevelDesc &L, int W, int H, int Wk, int Hk) {
 // what it never launched.)
 constexpr unsigned kPlanResize = 1;   // K1 tables
 constexpr unsigned kPlanTiles = 2;    // cell tiles (per-block HOG, sparse flags)
-constexpr unsigned kPlanWindows = 4;  // FP32 K4 window tiles (also the proposal's keep granularity)
+constexpr unsigned kPlanWindows = 4;  // FP32 K4 window tiles
 
 // Adds one level to the plan (descriptor, and the tables and items of `what`).
 void plan_level(Plan &p, unsigned what, int frame, int level, int W, int H, int Wk, int Hk, int64_t img_off,
@@ -848,6 +848,12 @@ void invalidate_cache(pd_handle *h) {
 int max_pool_tiles(const Plan &p) {
     int m = 0;
     for (const LevelDesc &L : p.levels) m = std::max(m, pool_tiles_of(L.rows, L.cols));
+    return m;
+}
+
+int max_windows(const Plan &p) {
+    int m = 0;
+    for (const LevelDesc &L : p.levels) m = std::max(m, L.rows * L.cols);
     return m;
 }
 
@@ -1206,14 +1212,15 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         const bool fp32 = (h->p.flags & PD_FLAG_SVM_FP32) != 0;
         const unsigned what = kPlanResize |
                               (h->proposal || (h->p.flags & PD_FLAG_HOG_PER_BLOCK) ? kPlanTiles : 0u) |
-                              (h->proposal || fp32 ? kPlanWindows : 0u);
+                              (fp32 ? kPlanWindows : 0u);
         for (int f = 0; f < n_frames; ++f) {
             int r = plan_frame(p, what, h->p, d_frames[f], widths[f], heights[f], pitches[f],
                                h->proposal ? kSparseTileCost : h->tile_cost, h->proposal);
             if (r != PD_OK) return fail(h, r, "frame %d: planning failed", f);
         }
         if (!fp32) {
-            plan_tc(p, h->tuning.tc_item_rows, h->sm_count);
+            plan_tc(p, h->proposal ? std::min(h->tuning.tc_item_rows, kTcSparseRows) : h->tuning.tc_item_rows,
+                    h->sm_count);
             assign_tc_maps(p);
         }
         plan_strips(p, h->sm_count * kStripWarpsPerSm);
@@ -1258,8 +1265,12 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
                                   (int)p.cnn_items.size(), cnn_weights(h), h->hmap, h->atlas.pitch, h->logits,
                                   max_pool_tiles(p), h->d_err));
             PD_CUDA(h, cudaMemsetAsync(h->c_flag, 0, p.c_items.size() * 4 + 4, q));
-            PD_CUDA(h, launch_proposal_flags(q, dl, dptr<SvmItem>(h, o.s_items), (int)p.s_items.size(), h->logits,
-                                             h->tau, h->s_flag, h->c_flag, !(h->p.flags & PD_FLAG_SVM_FP32)));
+            if (h->p.flags & PD_FLAG_SVM_FP32)
+                PD_CUDA(h, launch_proposal_flags(q, dl, dptr<SvmItem>(h, o.s_items), (int)p.s_items.size(),
+                                                 h->logits, h->tau, h->s_flag, h->c_flag));
+            else
+                PD_CUDA(h, launch_window_flags(q, dl, (int)p.levels.size(), max_windows(p), h->logits, h->tau,
+                                               h->c_flag, h->d_scores));
             cf = h->c_flag;
             sf = h->s_flag;
         }
@@ -1316,7 +1327,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
                        (p.score_floats == 0 ? 0 : 1) +
                        nms_launches(n_frames, nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame)) +
                        (h->proposal ? (p.cnn_items.empty() ? 0 : 1) + (p.levels.empty() ? 0 : 1) +
-                                          (p.s_items.empty() ? 0 : 1)
+                                          (p.score_floats == 0 ? 0 : 1)
                                     : 0);
     h->detected = true;
     h->ran_proposal = h->proposal;

@@ -83,6 +83,7 @@ constexpr int kSvmShapes = 7;   // K4 tile shapes: 32x16, 64x8, 32x8, 64x4, 64x2
 constexpr int kTcStrip = 26;    // tensor-core K4: window columns per item (32 blocks, a lane quarter of the MMA)
 constexpr int kTcChunk = 64;    // tensor-core K4: window rows per item at most (tunable down to kTcMinChunk)
 constexpr int kTcMinChunk = 8;
+constexpr int kTcSparseRows = 48;  // window rows per item at most on the sparse path (+ 15: bits of a 64-bit mask)
 constexpr int kTcWalkers = 4;   // tensor-core K4: items walked at a time by a CTA (one CTA per SM)
 constexpr int kTcFineItems = 4096;  // plans of at most this many items may cut them below kTcMinChunk rows
 constexpr int kTcConstBytes = 45056;  // tensor-core K4: B operand (43,008 bytes) and LBP table (2,048)
@@ -137,15 +138,18 @@ cudaError_t launch_cells_warp(cudaStream_t s, const LevelDesc *d_levels, const u
                               const StripItem *d_items, int n_items, int *d_queue, int sm_count,
                               const uint8_t *d_lbp_map, const uint32_t *c_flag, int feat);
 cudaError_t launch_proposal_flags(cudaStream_t s, const LevelDesc *d_levels, const SvmItem *d_items, int n_items,
-                                  const float *logits, float tau, uint32_t *s_flag, uint32_t *c_flag,
-                                  bool per_window);
+                                  const float *logits, float tau, uint32_t *s_flag, uint32_t *c_flag);
+// Tensor-core K4: cell tiles under every kept window, and -inf in every score.
+cudaError_t launch_window_flags(cudaStream_t s, const LevelDesc *d_levels, int n_levels, int max_windows,
+                                const float *logits, float tau, uint32_t *c_flag, float *scores);
 cudaError_t launch_svm(cudaStream_t s, const CUtensorMap *hog_maps, const CUtensorMap *lbp_maps,
                        const LevelDesc *d_levels, const float *d_w, float bias, float clip,
                        float *scores, const SvmItem *d_items, int n_items, unsigned *d_err,
                        const uint32_t *s_flag = nullptr);
 // Tensor-core K4: persistent CTAs (grid at most one per SM) over an item
 // queue (*d_queue must be 0 at launch); c_flag non-null selects the sparse
-// path. The maps are encode_tc_maps pairs; d_consts: build_tc_consts.
+// path (items of at most kTcSparseRows rows, scores filled with -inf before).
+// The maps are encode_tc_maps pairs; d_consts: build_tc_consts.
 cudaError_t init_svm_tc();
 // Constants of the tensor-core K4 from the template [95][15][8]: kTcConstBytes bytes.
 void build_tc_consts(const float *wt, unsigned char *out);
