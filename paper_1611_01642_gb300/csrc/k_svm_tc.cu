@@ -44,18 +44,19 @@
 //    the fixed order (i, j) = (0,0), (0,1), ..., so every score is b plus its
 //    terms in one order whatever the item cut; window row r - 14 is complete
 //    and stored.
-// A and D are double buffered: the producers build step s + 1 and the epilogue
-// reads step s - 1 while step s's MMAs run.
-// What bounds it: a step takes about 2,350 cycles, its MMAs 1,010 of them; the
-// schedulers issue on 53% of cycles and the shared-memory pipe is 51% busy, so
-// it is the latency of the hand-offs between the roles, with 3.5 warps per
-// scheduler. 64 x 1242x375 frames: 0.352 ms; 0.661 ms with one strip of 104
-// columns per CTA, LBP planes read a byte per bin and summed in place, and a
-// single warp issuing the MMAs between its epilogue rows (3,400 cycles per
-// row, 901 rows per frame; now 693 steps). One 1242x375 frame: 84 -> 31 us,
-// with items cut until every SM has work (see the planner). 14 warps leave 128
-// registers per thread (4 warps on a scheduler), which the epilogue's loads
-// are staged for.
+// A has three stages and D two buffers: the producers build steps s + 1 and
+// s + 2 and the epilogue reads step s - 1 while step s's MMAs run.
+// What bounds it: a step takes about 2,250 cycles: a HOG or LBP warp needs
+// about 1,750 for its 300 instructions (3.5 warps per scheduler, fixed latencies
+// and the shared-memory pipe, 51% busy), the 18 MMAs 1,010 to 1,500; handing on
+// the finished stores later, or a packed bf16 split, changed nothing.
+// 64 x 1242x375 frames: 0.334 ms; 0.661 ms with one strip of 104 columns per
+// CTA, LBP planes read a byte per bin and summed in place, and a single warp
+// issuing the MMAs between its epilogue rows (3,400 cycles per row, 901 rows
+// per frame; now 693 steps); two A stages instead of three: 0.344 ms. One
+// 1242x375 frame: 84 -> 31 us, with items cut until every SM has work (see the
+// planner). 14 warps leave 128 registers per thread (4 warps on a scheduler),
+// which the epilogue's loads are staged for.
 // Per-block HOG (Algorithm 5 read per block): each staged cell row holds 36
 // HOG planes, the cell's 4 block-restricted histograms (plane 9 q + bin, q =
 // its place in the block); a block takes q = 0, 1 from its upper row and
@@ -90,8 +91,16 @@ constexpr int kTileRows = (kTcSparseRows - 1 + kWinBH) / kCellTH + 2;  // cell-t
 static_assert(kTileRows <= 32 && kWinBW < kCellTW && kWinBH < 2 * kCellTH && kTcSparseRows + kWinBH <= 64 &&
                   kTcSparseRows > 32, "sparse masks");
 constexpr int kMeta = 16;             // step descriptions in flight (more than any role can lag behind)
-constexpr uint32_t kTmemCols = 512;   // two accumulator buffers of 128 columns, two A stages of 96
-constexpr uint32_t kTmemA = 256;      // first A stage column (bf16 pairs: high parts 0..47, low 48..95)
+// Tensor memory: accumulators in columns 0..111 and 128..239, three A stages of
+// 96 columns (bf16 pairs: 48 of high parts, 48 of low parts). The third stage's
+// last low parts take the 16 columns that each accumulator leaves of its 128.
+constexpr uint32_t kTmemCols = 512;
+constexpr uint32_t kStages = 3;
+__device__ __forceinline__ uint32_t a_hi(uint32_t stage) { return 256 + 96 * stage; }
+// columns of the low parts [16 part, 16 part + 16)
+__device__ __forceinline__ uint32_t a_lo(uint32_t stage, int part) {
+    return stage < 2 ? 304 + 96 * stage + 16 * part : part == 0 ? 496 : part == 1 ? 112 : 240;
+}
 constexpr uint64_t kWaitNs = 1000000000ull;
 constexpr int kBBytes = 14 * kSBO;    // B operand: template high | low parts
 constexpr int kTabBytes = 512 * 4;    // sum of 4 cell counts -> bf16 high | low << 16 of sqrt(S / 256)
@@ -121,13 +130,13 @@ struct TcSmemT {
     uint32_t tab[512];
     SlotT<HP> slot[kSlots];               // staged cell rows
     StepMeta meta[kMeta][kGroups];
-    uint32_t keep[kGroups][2][kTcSparseRows];  // sparse: scored windows of the rows of the current and next items
+    uint32_t keep[kGroups][kTcSparseRows];  // sparse: scored windows of an item's rows
     unsigned long long bfull;             // constants arrived
     unsigned long long cfull[kSlots];     // cell row arrived (TMA transaction count)
     unsigned long long cempty[kSlots];    // cell row no longer read (8 producer warps)
     unsigned long long mready[kMeta];     // step description written
-    unsigned long long afull[2];          // A operand written (8 producer warps)
-    unsigned long long aempty[2];         // A operand read by the MMAs (commit)
+    unsigned long long afull[kStages];    // A operand written (8 producer warps)
+    unsigned long long aempty[kStages];   // A operand read by the MMAs (commit)
     unsigned long long dfull[2];          // accumulators written (commit)
     unsigned long long dempty[2];         // accumulators read (4 epilogue warps)
     uint32_t tmem;
@@ -146,9 +155,9 @@ __device__ __forceinline__ uint64_t global_ns() {
 __device__ __forceinline__ bool try_wait(unsigned long long *bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
-        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2, 1000;\n\tselp.u32 %0, 1, 0, q;\n\t}"
         : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
+        : "r"(smem_u32(bar)), "r"(parity)  // suspended for up to 1000 ns: a spinning role takes issue slots
         : "memory");
     return ok != 0;
 }
@@ -259,11 +268,11 @@ __device__ __forceinline__ void tst16(uint32_t t, const uint32_t *v) {
         : "memory");
 }
 
-// The 36 HOG values of A row m into its TMEM lane (columns a + f / 2 for the
-// high parts, a + 48 + f / 2 for the low parts): cells (r, c), (r, c+1),
+// The 36 HOG values of A row m into its TMEM lane (feature f in column f / 2 of
+// the stage's high and low parts): cells (r, c), (r, c+1),
 // (r+1, c), (r+1, c+1) in the template's order (TL, TR, BL, BR, 9 bins each),
 // L2-Hys, bf16 split.
-__device__ __forceinline__ void build_hog(const float (&x)[36], float clip, uint32_t a) {
+__device__ __forceinline__ void build_hog(const float (&x)[36], float clip, uint32_t lanes, uint32_t stage) {
     // sums of squares in four interleaved partial sums (independent chains)
     f32x2 v[18], q01 = 0ull, q23 = 0ull;
 #pragma unroll
@@ -288,10 +297,10 @@ __device__ __forceinline__ void build_hog(const float (&x)[36], float clip, uint
     uint32_t hi[18], lo[18];
 #pragma unroll
     for (int t = 0; t < 18; ++t) split2(mul2(v[t], i22), hi[t], lo[t]);
-    tst16(a, hi);
-    tst2(a + 16, hi + 16);
-    tst16(a + 48, lo);
-    tst2(a + 64, lo + 16);
+    tst16(lanes + a_hi(stage), hi);
+    tst2(lanes + a_hi(stage) + 16, hi + 16);
+    tst16(lanes + a_lo(stage, 0), lo);
+    tst2(lanes + a_lo(stage, 1), lo + 16);
 }
 
 // Horizontal sums of the LBP counts of a cell and its right neighbour, times 4
@@ -355,9 +364,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             init(&S.cempty[s], 2 * kGroups);
         }
         for (int s = 0; s < kMeta; ++s) init(&S.mready[s], 1);
-        for (int s = 0; s < 2; ++s) {
+        for (int s = 0; s < (int)kStages; ++s) {
             init(&S.afull[s], 2 * kGroups);
             init(&S.aempty[s], 1);
+        }
+        for (int s = 0; s < 2; ++s) {
             init(&S.dfull[s], 1);
             init(&S.dempty[s], kGroups);
         }
@@ -391,14 +402,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         // LBP part of group warp - 4; lane m = block m of the group
         const int g = warp & 3;
         const bool is_lbp = warp >= 4;
-        const uint32_t lanes = tmem + ((uint32_t)(32 * g) << 16) + kTmemA;
+        const uint32_t lanes = tmem + ((uint32_t)(32 * g) << 16);
         bool ok = !is_lbp || warp_wait(&S.bfull, 0);
-        auto stage_free = [&](uint32_t s) { return s < 2 || warp_wait(&S.aempty[s & 1], ((s >> 1) - 1) & 1u); };
+        auto stage_free = [&](uint32_t s) {
+            return s < kStages || warp_wait(&S.aempty[s % kStages], (s / kStages - 1) & 1u);
+        };
         auto publish = [&](uint32_t s) {
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) arrive(&S.afull[s & 1]);
+            if (lane == 0) arrive(&S.afull[s % kStages]);
         };
         if (!is_lbp) {
             constexpr int pq = HP == 36 ? kHogBins : 0;  // per-block: plane set of the cell's place
@@ -427,7 +440,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!(ok = stage_free(s))) break;
                 if (kind == 2u) {
                     tc_fence_after();
-                    build_hog(x, clip, lanes + (s & 1) * 96);
+                    build_hog(x, clip, lanes, s % kStages);
                 }
                 publish(s);
             }
@@ -456,15 +469,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!(ok = stage_free(s))) break;
                 if (kind == 2u) {
                     tc_fence_after();
-                    const uint32_t a = lanes + (s & 1) * 96;
+                    const uint32_t a = lanes + a_hi(s % kStages), b = lanes + a_lo(s % kStages, 1);
                     tst2(a + 18, hi);
                     tst4(a + 20, hi + 2);
                     tst8(a + 24, hi + 6);
                     tst16(a + 32, hi + 14);
-                    tst2(a + 66, lo);
-                    tst4(a + 68, lo + 2);
-                    tst8(a + 72, lo + 6);
-                    tst16(a + 80, lo + 14);
+                    tst2(b + 2, lo);
+                    tst4(b + 4, lo + 2);
+                    tst8(b + 8, lo + 6);
+                    tst16(lanes + a_lo(s % kStages, 2), lo + 14);
                 }
                 publish(s);
             }
@@ -540,72 +553,69 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (uint32_t s = 0;; ++s) {
                 if (!bar_wait(S, &S.mready[s % kMeta], (s / kMeta) & 1u, err)) break;
                 if ((S.meta[s % kMeta][0].flags & 3u) == 3u) break;
-                if (!bar_wait(S, &S.afull[s & 1], (s >> 1) & 1u, err)) break;
+                const uint32_t st = s % kStages;
+                if (!bar_wait(S, &S.afull[st], (s / kStages) & 1u, err)) break;
                 if (s >= 2 && !bar_wait(S, &S.dempty[s & 1], ((s >> 1) - 1) & 1u, err)) break;
                 tc_fence_after();
                 const uint32_t d = tmem + (s & 1) * 128;
-                const uint32_t a0 = tmem + kTmemA + (s & 1) * 96;  // 8 columns per K step
+                const uint32_t ah = tmem + a_hi(st);  // 8 columns per K step
 #pragma unroll
-                for (int k = 0; k < 6; ++k) umma_ts(d, a0 + 8 * k, umma_desc(b_base + 256 * k), k > 0);
+                for (int k = 0; k < 6; ++k) umma_ts(d, ah + 8 * k, umma_desc(b_base + 256 * k), k > 0);
 #pragma unroll
-                for (int k = 0; k < 6; ++k) umma_ts(d, a0 + 48 + 8 * k, umma_desc(b_base + 256 * k), 1);
+                for (int k = 0; k < 6; ++k)
+                    umma_ts(d, tmem + a_lo(st, k / 2) + 8 * (k & 1), umma_desc(b_base + 256 * k), 1);
 #pragma unroll
-                for (int k = 0; k < 6; ++k) umma_ts(d, a0 + 8 * k, umma_desc(b_base + 12 * 128 + 256 * k), 1);
-                umma_commit(&S.aempty[s & 1]);
+                for (int k = 0; k < 6; ++k) umma_ts(d, ah + 8 * k, umma_desc(b_base + 12 * 128 + 256 * k), 1);
+                umma_commit(&S.aempty[st]);
                 umma_commit(&S.dfull[s & 1]);
                 committed = s + 1;
             }
         }
         __syncwarp();
     } else {
-        // ---- items and cell rows; lane g < 4 serves group g. The group's next item is
-        // fetched a stage per step (queue ticket, item, level), so that no step waits for
-        // a chain of global loads; on the sparse path the warp then works out its windows.
+        // ---- items and cell rows; lane g < 4 serves group g. A group draws its next item when
+        // it needs it: the ring of slots covers the chain of loads, and a ticket drawn ahead
+        // holds an item back from groups that are free (8 x 1920x1080 sparse: 191 us with the
+        // ticket drawn when the item before it starts, 172 so).
         const bool sparse = c_flag != nullptr;
         const bool mine = lane < kGroups;
-        enum : int { kTicket = 1, kItem, kLevel, kReady, kNone };  // what of the next item is in flight or here
-        int stage = mine ? kTicket : kNone;
-        int ticket = (int)blockIdx.x + lane * (int)gridDim.x;
-        TcItem nit{};
-        int n_cell_row = 0, n_cols = 0, n_map = 0, n_citem0 = 0, n_ctx = 0;
-        int64_t n_score = 0;
-        unsigned long long n_walk = 0;  // sparse: cell rows (from the item's first) to walk
-        auto advance = [&]() {
-            if (stage == kTicket) {
-                stage = kNone;
-                if (ticket < n_items) {
-                    nit = items[ticket];
-                    stage = kItem;
-                }
-            } else if (stage == kItem) {
-                const LevelDesc &L = levels[nit.level];
-                n_cell_row = L.cell_row;
-                n_cols = L.cols;
-                n_map = L.tc_map;
-                n_citem0 = L.citem0;
-                n_ctx = L.ctx;
-                n_score = L.score_off;
-                stage = sparse ? kLevel : kReady;
-            }
+        bool more = mine, drawn = true;
+        int ticket = (int)blockIdx.x + lane * (int)gridDim.x;  // the first items by place, the next from the queue
+        // the item being walked
+        bool active = false;
+        const CUtensorMap *hm = &hog_map, *lm = &lbp_map;
+        int wx0 = 0, ncols = 0, wy0 = 0, n_rows = 0, cols = 0, cell_row = 0, citem0 = 0, ctx = 0;
+        int r = 0, r0 = 0, r_end = -1;  // next cell row, first and last one of the run
+        bool first = false;
+        int64_t score_off = 0;
+        unsigned long long walk = 0;  // sparse: cell rows of the later runs
+        auto next_run = [&]() {
+            if (!walk) return false;
+            const int a = __ffsll((long long)walk) - 1;
+            const unsigned long long after = ~(walk >> a);  // its lowest bit ends the run
+            const int len = after ? __ffsll((long long)after) - 1 : 64 - a;
+            walk = a + len < 64 ? walk >> (a + len) << (a + len) : 0ull;
+            r = r0 = wy0 + a;
+            r_end = r + len - 1;
+            first = true;
+            return true;
         };
-        int buf = 0;  // sparse: the buffer of S.keep that the group's current item uses
-        // Sparse, whole warp: the scored windows of group g's next item, and the cell rows
-        // they need (a window row needs 16 of them).
+        // Sparse, whole warp: the scored windows of group g's item, and the cell rows they
+        // need (a window row needs 16 of them).
         auto prepare = [&](int g) {
-            const int y0 = __shfl_sync(0xffffffffu, nit.wy0, g), x0 = __shfl_sync(0xffffffffu, nit.wx0, g);
-            const int n = __shfl_sync(0xffffffffu, nit.wy1, g) - y0;
-            const int nc = min(kTcStrip, __shfl_sync(0xffffffffu, n_cols, g) - x0);
-            const int ctx = __shfl_sync(0xffffffffu, n_ctx, g), other = __shfl_sync(0xffffffffu, buf, g) ^ 1;
+            const int y0 = __shfl_sync(0xffffffffu, wy0, g), x0 = __shfl_sync(0xffffffffu, wx0, g);
+            const int n = __shfl_sync(0xffffffffu, n_rows, g), nc = __shfl_sync(0xffffffffu, ncols, g);
+            const int nx = __shfl_sync(0xffffffffu, ctx, g);
             // lane = window column: a window lies in one or two cell tiles across; the
             // ballot of tile row t stays with lane t
             const int ty0 = y0 / kCellTH, nt = (y0 + n - 1 + kWinBH) / kCellTH - ty0 + 1;
             const int wx = x0 + lane;
             const int cl = lane < nc ? wx / kCellTW : 0, cr = lane < nc ? (wx + kWinBW) / kCellTW : 0;
-            const uint32_t *flags = c_flag + __shfl_sync(0xffffffffu, n_citem0, g) + ty0 * ctx;
+            const uint32_t *flags = c_flag + __shfl_sync(0xffffffffu, citem0, g) + ty0 * nx;
             uint32_t f[kTileRows][2];
 #pragma unroll
             for (int t = 0; t < kTileRows; ++t) {
-                const uint32_t *row = flags + min(t, nt - 1) * ctx;
+                const uint32_t *row = flags + min(t, nt - 1) * nx;
                 f[t][0] = __ldg(row + cl);
                 f[t][1] = __ldg(row + cr);
             }
@@ -623,7 +633,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int a0 = y / kCellTH - ty0, a1 = (y + kWinBH) / kCellTH - ty0;
                 const uint32_t k = __shfl_sync(0xffffffffu, bits, a0) & __shfl_sync(0xffffffffu, bits, a0 + 1) &
                                    __shfl_sync(0xffffffffu, bits, a1);
-                if (row < n) S.keep[g][other][row] = k;
+                if (row < n) S.keep[g][row] = k;
                 kept |= (unsigned long long)__ballot_sync(0xffffffffu, row < n && k) << (32 * h);
             }
             __syncwarp();
@@ -632,69 +642,44 @@ __global__ void __launch_bounds__(kThreads, 1)
                 kept |= kept << 2;
                 kept |= kept << 4;
                 kept |= kept << 8;
-                n_walk = kept;
-                stage = kReady;
+                walk = kept;
+                active = next_run();
             }
-        };
-        // the item being walked
-        bool active = false;
-        const CUtensorMap *hm = &hog_map, *lm = &lbp_map;
-        int wx0 = 0, ncols = 0, wy0 = 0, cols = 0, cell_row = 0;
-        int r = 0, r0 = 0, r_end = -1;  // next cell row, first and last one of the run
-        bool first = false;
-        int64_t score_off = 0;
-        unsigned long long walk = 0;  // sparse: cell rows of the later runs
-        auto next_run = [&]() {
-            if (!walk) return false;
-            const int a = __ffsll((long long)walk) - 1;
-            const unsigned long long after = ~(walk >> a);  // its lowest bit ends the run
-            const int len = after ? __ffsll((long long)after) - 1 : 64 - a;
-            walk = a + len < 64 ? walk >> (a + len) << (a + len) : 0ull;
-            r = r0 = wy0 + a;
-            r_end = r + len - 1;
-            first = true;
-            return true;
         };
         for (uint32_t s = 0;; ++s) {
             // groups whose item (or run) is done take the next
             if (active && r > r_end) active = sparse && next_run();
             for (;;) {
-                const bool want = mine && !active && stage != kNone;
+                const bool want = !active && more;
                 if (!__any_sync(0xffffffffu, want)) break;
-                if (want)
-                    while (stage == kTicket || stage == kItem) advance();
-                if (sparse)
-                    for (unsigned left = __ballot_sync(0xffffffffu, want && stage == kLevel); left; left &= left - 1u)
-                        prepare(__ffs((int)left) - 1);
-                if (want && stage == kReady) {
-                    wx0 = nit.wx0;
-                    wy0 = nit.wy0;
-                    cols = n_cols;
+                if (want) {
+                    if (!drawn) ticket = kGroups * (int)gridDim.x + atomicAdd(queue, 1);
+                    drawn = false;
+                    more = ticket < n_items;
+                }
+                if (want && more) {
+                    const TcItem it = items[ticket];
+                    const LevelDesc &L = levels[it.level];
+                    wx0 = it.wx0;
+                    wy0 = it.wy0;
+                    n_rows = it.wy1 - it.wy0;
+                    cols = L.cols;
                     ncols = min(kTcStrip, cols - wx0);
-                    cell_row = n_cell_row;
-                    score_off = n_score;
+                    cell_row = L.cell_row;
+                    citem0 = L.citem0;
+                    ctx = L.ctx;
+                    score_off = L.score_off;
                     if (level_maps) {
-                        hm = level_maps + 2 * n_map;
+                        hm = level_maps + 2 * L.tc_map;
                         lm = hm + 1;
                     }
                     r = r0 = wy0;
-                    r_end = nit.wy1 - 1 + kWinBH;
+                    r_end = it.wy1 - 1 + kWinBH;
                     first = active = true;
-                    if (sparse) {
-                        buf ^= 1;
-                        walk = n_walk;
-                        active = next_run();
-                    }
-                    ticket = 4 * (int)gridDim.x + atomicAdd(queue, 1);
-                    stage = kTicket;
                 }
-            }
-            if (s & 1) {  // the next items, a stage at a time
-                advance();
-                if (sparse) {
-                    const unsigned ready = __ballot_sync(0xffffffffu, stage == kLevel);
-                    if (ready) prepare(__ffs((int)ready) - 1);
-                }
+                if (!sparse) break;
+                for (unsigned left = __ballot_sync(0xffffffffu, want && more); left; left &= left - 1u)
+                    prepare(__ffs((int)left) - 1);
             }
             const uint32_t slot = s % kSlots;
             if (s >= kSlots && !warp_wait(&S.cempty[slot], (s / kSlots - 1) & 1u)) break;
@@ -706,7 +691,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int wy = r - kWinBH;  // the window row that this cell row completes
                     const bool store = wy >= r0;
                     m.flags = (first ? 1u : 2u) | (store ? 4u : 0u) | ((uint32_t)(wx0 & 3) << 4) | ((uint32_t)ncols << 8);
-                    m.keep = sparse && store ? S.keep[lane][buf][wy - wy0] : 0xffffffffu;
+                    m.keep = sparse && store ? S.keep[lane][wy - wy0] : 0xffffffffu;
                     m.out = score_off + (int64_t)wy * cols + wx0;
                 }
                 S.meta[s % kMeta][lane] = m;
