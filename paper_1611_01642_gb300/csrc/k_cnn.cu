@@ -10,12 +10,17 @@
 // bf16 inputs, weights and stored activations; fp32 accumulation.
 //
 // k_cnn_fwd: persistent CTAs (8 warps, two per SM), each walking 8x8-cell
-// tiles. The 72x80 input bytes of the next tile are fetched with cp.async
+// tiles. The 72x96 input bytes of the next tile are fetched by TMA
 // while the current tile is computed. Per tile: the pixels become bf16 x
 // (zero outside the level: the padding of layer 1); layer 1 runs on the
 // tensor cores as a GEMM over 4x4 pixel patches (a stride-2 3x3 window at
 // (2r-1, 2c-1) is the top-left 3x3 of the 4x4 patch there; the 7 extra taps
 // carry zero weights; mma.sync m16n8k16), giving 35x35x16 activations.
+// What bounds it: the phases of a tile follow one another behind block
+// barriers (issue 47%, barrier and tensor-memory waits), so the conversion and
+// layer 1's index arithmetic are in the way: 8 pixels per conversion step with
+// packed float operations and positions stepped instead of divided took it
+// from 279 to 243 us per 8 x 1920x1080 frames (network on every 4th level).
 // Layer 2 (17x17x32, K = 9 taps x 16) and layer 3 (8x8x32, K = 9 x 32) are
 // implicit GEMMs on the 5th-generation tensor cores: one thread issues
 // tcgen05.mma with both operands in shared memory (no-swizzle K-major
@@ -33,6 +38,8 @@
 
 #include <algorithm>
 
+#include "f32x2.cuh"
+
 namespace pd {
 namespace {
 
@@ -44,6 +51,7 @@ constexpr int XR = 2 * R1 + 2;   // 72 pixel rows/columns under the 4x4 patches
 constexpr int kRawW = kCnnBoxW;  // staged bytes per row: pixels x0-9 .. x0+86 (TMA box)
 static_assert(XR == kCnnBoxH, "input box height");
 static_assert((XR * kRawW) % 128 == 0, "second raw buffer stays 128-byte aligned");
+static_assert(XR % 8 == 0, "8 pixels per conversion step");
 constexpr int XBW = 44;          // bf16 pixel row stride in words (72 used, padded for banks)
 // Activations are stored as 16-byte rows of 8 bf16 channels, split by
 // channel group and by column parity: plane (group, parity) holds the
@@ -79,7 +87,6 @@ struct CnnSmem {
     } u;
     uint8_t w2c[9 * kBTapBytes];      // layer-2 B operands, one per tap
     uint8_t w3c[9 * 2 * kBTapBytes];  // layer-3 B operands, per tap and input-channel half
-    float b1[16];
     float b2[32];
     float b3[32];
     float wh[32];
@@ -283,7 +290,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
         *reinterpret_cast<__nv_bfloat16 *>(S.w3c + off) =
             __float2bfloat16_rn(wts.w3[(n * 32 + 16 * kh + k) * 9 + tap]);
     }
-    if (tid < 16) S.b1[tid] = wts.b1[tid];
     if (tid < 32) {
         S.b2[tid] = wts.b2[tid];
         S.b3[tid] = wts.b3[tid];
@@ -300,16 +306,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
             const float hi = (ky < 3 && kx + 1 < 3) ? wts.w1[o * 9 + ky * 3 + kx + 1] : 0.f;
             bw1[nt][hk] = pack_bf16(lo, hi);
         }
-    // layer-2 B fragments (9 taps x 4 n-tiles x 2 regs) for the edge positions on mma.sync
-    uint32_t bw2[9][4][2];
-#pragma unroll
-    for (int tap = 0; tap < 9; ++tap)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const uint2 v = reinterpret_cast<const uint2 *>(wts.w2frag)[(tap * 4 + nt) * 32 + lane];
-            bw2[tap][nt][0] = v.x;
-            bw2[tap][nt][1] = v.y;
-        }
+    // this lane's positions of layer 1 in its warp's first tile, and the biases of its columns
+    static_assert(kThreads / 32 * 16 == 3 * R1 + 23 && kThreads / 32 * 16 <= M1, "tiles of a warp");
+    const int rs0 = (warp * 16 + g) / R1, cs0 = (warp * 16 + g) % R1;
+    const int rs1 = (warp * 16 + g + 8) / R1, cs1 = (warp * 16 + g + 8) % R1;
+    const int prs = (warp * 16 + (lane & 15)) / R1, pcs = (warp * 16 + (lane & 15)) % R1;
+    const float b1r[4] = {wts.b1[2 * t], wts.b1[2 * t + 1], wts.b1[8 + 2 * t], wts.b1[8 + 2 * t + 1]};
     const float bh = wts.bh[0];
     const uint32_t a1_base = smem_u32(&S.a1[0]);
     const uint32_t a2_base = smem_u32(&S.u.a2[0]);
@@ -357,45 +359,68 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
         // x = bf16(L/255 - 0.5): one fma in float32 rounded once to bf16 equals
         // the correctly rounded value for all 256 inputs (checked exhaustively
         // against exact rational arithmetic when this path was written).
-        for (int k = tid; k < XR * (XR / 4); k += kThreads) {
-            const int r = k / (XR / 4), j = k - r * (XR / 4);
-            const uint32_t *rw = reinterpret_cast<const uint32_t *>(S.raw[cur][r]);
-            const uint32_t v = __byte_perm(rw[j + 2], rw[j + 3], 0x4321);  // bytes 4j + 9 .. 4j + 12
-            const int y = y0 + r, xc = x0 + 4 * j;
-            const bool rin = y >= 0 && y < Hk;
-            float e[4];
+        // A byte b becomes a float through the word 0x4B0000bb = 2^23 + b; 8 pixels per step.
+        const bool interior0 = y0 >= 0 && x0 >= 0 && y0 + XR <= Hk && x0 + XR <= Wk;
+        for (int k = tid; k < XR * (XR / 8); k += kThreads) {
+            const int r = k / (XR / 8), j = k - r * (XR / 8);
+            const uint32_t *rw = reinterpret_cast<const uint32_t *>(S.raw[cur][r]) + 2 * j + 2;
+            const uint32_t m = rw[1];
+            const uint32_t v[2] = {__byte_perm(rw[0], m, 0x4321), __byte_perm(m, rw[2], 0x4321)};  // bytes 8j + 9 ..
+            uint32_t o[4];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int x = xc + b;
-                e[b] = (rin && x >= 0 && x < Wk) ? fmaf((float)((v >> (8 * b)) & 255u), kInv255, -0.5f) : 0.f;
+            for (int h = 0; h < 4; ++h) {
+                const uint32_t w = v[h >> 1], sel = 0x7440u + 2 * (h & 1);
+                const f32x2 e = fma2(add2(pack2(__uint_as_float(__byte_perm(w, 0x4B000000u, sel)),
+                                                __uint_as_float(__byte_perm(w, 0x4B000000u, sel + 1))),
+                                          dup2(-8388608.0f)),
+                                     dup2(kInv255), dup2(-0.5f));
+                o[h] = pack_bf16(lo2(e), hi2(e));
             }
-            *reinterpret_cast<uint2 *>(&S.u.xb[r * XBW + 2 * j]) = make_uint2(pack_bf16(e[0], e[1]), pack_bf16(e[2], e[3]));
+            if (!interior0) {  // zero outside the level
+                const int y = y0 + r, xc = x0 + 8 * j;
+                const bool rin = y >= 0 && y < Hk;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const int x = xc + 2 * h;
+                    o[h] &= (rin && x >= 0 && x < Wk ? 0xffffu : 0u) | (rin && x + 1 >= 0 && x + 1 < Wk ? 0xffff0000u : 0u);
+                }
+            }
+            *reinterpret_cast<uint4 *>(&S.u.xb[r * XBW + 4 * j]) = make_uint4(o[0], o[1], o[2], o[3]);
         }
         __syncthreads();
         // ---- layer 1 on tensor cores (mma.sync): 1225 positions x 16 channels, K = 16 (4x4 patch)
+        // A warp's tiles are 128 positions (3 rows and 23 columns) apart.
+        int r0 = rs0, c0 = cs0, r1 = rs1, c1 = cs1, pr = prs, pc = pcs;
         for (int mt = warp; mt < M1T; mt += kThreads / 32) {
-            const int p0 = mt * 16 + g, p1 = p0 + 8;
-            const int q0 = min(p0, M1 - 1), q1 = min(p1, M1 - 1);  // padding rows repeat the last row
-            const int r0 = q0 / R1, c0 = q0 - r0 * R1, r1 = q1 / R1, c1 = q1 - r1 * R1;
             const uint32_t *x0w = &S.u.xb[(2 * r0 + (t >> 1)) * XBW + c0 + (t & 1)];
             const uint32_t *x1w = &S.u.xb[(2 * r1 + (t >> 1)) * XBW + c1 + (t & 1)];
             const uint32_t a0 = x0w[0], a1 = x1w[0], a2 = x0w[2 * XBW], a3 = x1w[2 * XBW];
             float acc[2][4];
 #pragma unroll
             for (int nt = 0; nt < 2; ++nt) {
-                acc[nt][0] = acc[nt][2] = S.b1[nt * 8 + 2 * t];
-                acc[nt][1] = acc[nt][3] = S.b1[nt * 8 + 2 * t + 1];
+                acc[nt][0] = acc[nt][2] = b1r[2 * nt];
+                acc[nt][1] = acc[nt][3] = b1r[2 * nt + 1];
                 mma_bf16(acc[nt], a0, a1, a2, a3, bw1[nt][0], bw1[nt][1]);
             }
             const bool in0 = interior1 || ((y1 + r0) >= 0 && (y1 + r0) < H1 && (x1 + c0) >= 0 && (x1 + c0) < W1);
             const bool in1 = interior1 || ((y1 + r1) >= 0 && (y1 + r1) < H1 && (x1 + c1) >= 0 && (x1 + c1) < W1);
             // this lane's row address: row (l % 8) + 8 ((l / 8) & 1) of the tile, channel group l / 16
-            const int ps = min(mt * 16 + (lane & 15), M1 - 1);
-            const int pr = ps / R1, pc = ps - pr * R1;
             const uint32_t dst = a1_base + ((((lane >> 4) * 2 + (pc & 1)) * PS1 + pr * C1P + (pc >> 1)) << 4);
             stsm_x4(dst, in0 ? relu_pack_bf16(acc[0][0], acc[0][1]) : 0u,
                     in1 ? relu_pack_bf16(acc[0][2], acc[0][3]) : 0u, in0 ? relu_pack_bf16(acc[1][0], acc[1][1]) : 0u,
                     in1 ? relu_pack_bf16(acc[1][2], acc[1][3]) : 0u);
+            auto next_tile = [&](int &r, int &c) {
+                r += 3;
+                c += 23;
+                if (c >= R1) {
+                    c -= R1;
+                    ++r;
+                }
+                if (r >= R1) r = R1 - 1, c = R1 - 1;  // padding rows repeat the last position
+            };
+            next_tile(r0, c0);
+            next_tile(r1, c1);
+            next_tile(pr, pc);
         }
         async_proxy_fence();  // layer-1 planes are read by the tensor cores next
         tc_fence_before();
@@ -433,8 +458,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
     {                                                                                                     \
         uint32_t a0, a1, a2, a3;                                                                          \
         ldsm_x4<((((DX) & 1) * PS1 + (DY) * C1P + ((DX) >> 1)) << 4)>(src, a0, a1, a2, a3);                \
+        uint32_t bf[8]; /* B fragments: the tap's operand is 8 matrices of 8 x 16 bytes in order */       \
+        ldsm_x4<((DY) * 3 + (DX)) * kBTapBytes>(w2c_base + 16 * lane, bf[0], bf[1], bf[2], bf[3]);         \
+        ldsm_x4<((DY) * 3 + (DX)) * kBTapBytes + 512>(w2c_base + 16 * lane, bf[4], bf[5], bf[6], bf[7]);   \
         _Pragma("unroll") for (int nt = 0; nt < 4; ++nt)                                                  \
-            mma_bf16(acc[nt], a0, a1, a2, a3, bw2[(DY) * 3 + (DX)][nt][0], bw2[(DY) * 3 + (DX)][nt][1]);   \
+            mma_bf16(acc[nt], a0, a1, a2, a3, bf[2 * nt], bf[2 * nt + 1]);                                 \
     }
             PD_L2_TAP(0, 0) PD_L2_TAP(0, 1) PD_L2_TAP(0, 2)
             PD_L2_TAP(1, 0) PD_L2_TAP(1, 1) PD_L2_TAP(1, 2)
@@ -531,64 +559,102 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
 }
 
 // Window pooling z[wy][wx] = bv + sum_{r<16, s<8} V[r][s] h[wy+r][wx+s]: one
-// CTA per (level, 64 x 16 window tile); the tile's 31 x 71 cells of h are
-// staged in shared memory; each thread computes 4 consecutive windows of one
-// row (8 taps x 4 windows per h row from 11 staged values), in a fixed order.
+// CTA per (level, 64 x 32 window tile); the tile's 47 x 71 cells of h are
+// staged in shared memory; each thread computes 4 consecutive windows of two
+// rows (a staged row serves both: 64 products from 11 values), in a fixed order.
 // With level groups a level's h is its group level's head map read at the
 // cell holding each cell's centre: row min(floor((2 cy + 1) Hk_j / (2 Hk)),
-// Hc_j - 1), column likewise (the identity for the group level itself).
+// Hc_j - 1), column likewise (the identity for the group level itself); the
+// rows and columns of a tile are mapped once, not per staged cell.
+// Sparse path (c_flag non-null): a window whose keep-logit exceeds tau is kept
+// and marks the cell tiles under its 8 x 16 cells (plain stores of 1, so the
+// order of the threads does not matter), and every window's score starts as
+// -inf, which the score kernel replaces where the cells were computed. The
+// tensor-core K4 then scores every window whose cells were all computed, a
+// superset of the kept ones. (A kernel of its own read the logits again:
+// 16 us per 8 x 1920x1080 frames.)
 constexpr int kPoolHW = kPoolTW + 8;                    // 72 staged columns (71 used)
-constexpr int kPoolHH = kPoolTH + kWinBH;               // 31 staged rows
+constexpr int kPoolHH = kPoolTH + kWinBH;               // 47 staged rows
 
 __global__ void __launch_bounds__(256) k_cnn_pool(const LevelDesc *__restrict__ levels,
                                                   const float *__restrict__ hmap, int32_t hmap_pitch,
                                                   const float *__restrict__ v, const float *__restrict__ bvp,
-                                                  float *__restrict__ logits) {
+                                                  float *__restrict__ logits, float tau,
+                                                  uint32_t *__restrict__ c_flag, float *__restrict__ scores) {
     __shared__ __align__(16) float V[16 * 8];
     __shared__ __align__(16) float Hs[kPoolHH][kPoolHW];
-    const LevelDesc L = levels[blockIdx.y];
+    __shared__ int src_row[kPoolHH], src_col[kPoolHW];  // -1: outside the level
+    const LevelDesc &L = levels[blockIdx.y];
     const int tiles_x = (L.cols + kPoolTW - 1) / kPoolTW;
     const int ty = blockIdx.x / max(tiles_x, 1), tx = blockIdx.x - ty * max(tiles_x, 1);
     const int wy0 = ty * kPoolTH, wx0 = tx * kPoolTW;
     if (L.rows == 0 || wy0 >= L.rows) return;  // CTA-uniform
-    const LevelDesc J = levels[L.hsrc];
+    const LevelDesc &J = levels[L.hsrc];
     const bool same = L.hsrc == (int)blockIdx.y;
     for (int i = threadIdx.x; i < 128; i += blockDim.x) V[i] = v[i];
-    for (int i = threadIdx.x; i < kPoolHH * kPoolHW; i += blockDim.x) {
-        const int r = i / kPoolHW, c = i - r * kPoolHW;
-        const int cy = wy0 + r, cx = wx0 + c;
-        float hv = 0.f;
-        if (cy < L.Hc && cx < L.Wc) {
-            const int sy = same ? cy : min((2 * cy + 1) * J.Hk / (2 * L.Hk), J.Hc - 1);
-            const int sx = same ? cx : min((2 * cx + 1) * J.Wk / (2 * L.Wk), J.Wc - 1);
-            hv = hmap[(int64_t)(J.cell_row + sy) * hmap_pitch + sx];
+    for (int i = threadIdx.x; i < kPoolHH + kPoolHW; i += blockDim.x) {
+        if (i < kPoolHH) {
+            const int cy = wy0 + i;
+            src_row[i] = cy >= L.Hc ? -1 : same ? cy : min((2 * cy + 1) * J.Hk / (2 * L.Hk), J.Hc - 1);
+        } else {
+            const int cx = wx0 + i - kPoolHH;
+            src_col[i - kPoolHH] = cx >= L.Wc ? -1 : same ? cx : min((2 * cx + 1) * J.Wk / (2 * L.Wk), J.Wc - 1);
         }
-        Hs[r][c] = hv;
     }
     __syncthreads();
-    const int ry = threadIdx.x >> 4, qx = 4 * (threadIdx.x & 15);
+    const float *h = hmap + (int64_t)J.cell_row * hmap_pitch;
+    for (int i = threadIdx.x; i < kPoolHH * kPoolHW; i += blockDim.x) {
+        const int r = i / kPoolHW, c = i - r * kPoolHW;
+        const int sy = src_row[r], sx = src_col[c];
+        Hs[r][c] = (sy | sx) >= 0 ? h[(int64_t)sy * hmap_pitch + sx] : 0.f;
+    }
+    __syncthreads();
+    const int ry = 2 * (threadIdx.x >> 4), qx = 4 * (threadIdx.x & 15);
     const float bv = bvp[0];
-    float z[4] = {bv, bv, bv, bv};
-#pragma unroll 4
-    for (int r = 0; r < 16; ++r) {
+    float z[2][4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) z[0][x] = z[1][x] = bv;
+    float vv[2][8];  // template rows r - 1 (for the second window row) and r
+#pragma unroll
+    for (int s = 0; s < 8; ++s) vv[0][s] = 0.f;
+#pragma unroll
+    for (int r = 0; r <= 16; ++r) {
         const float4 h0 = *reinterpret_cast<const float4 *>(&Hs[ry + r][qx]);
         const float4 h1 = *reinterpret_cast<const float4 *>(&Hs[ry + r][qx + 4]);
         const float4 h2 = *reinterpret_cast<const float4 *>(&Hs[ry + r][qx + 8]);
         const float hv[12] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w, h2.x, h2.y, h2.z, h2.w};
-        const float4 v0 = *reinterpret_cast<const float4 *>(&V[r * 8]);
-        const float4 v1 = *reinterpret_cast<const float4 *>(&V[r * 8 + 4]);
-        const float vv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+        float(&cur)[8] = vv[(r + 1) & 1];
+        const float(&prev)[8] = vv[r & 1];
+        if (r < 16) {
+            const float4 v0 = *reinterpret_cast<const float4 *>(&V[r * 8]);
+            const float4 v1 = *reinterpret_cast<const float4 *>(&V[r * 8 + 4]);
+            cur[0] = v0.x; cur[1] = v0.y; cur[2] = v0.z; cur[3] = v0.w;
+            cur[4] = v1.x; cur[5] = v1.y; cur[6] = v1.z; cur[7] = v1.w;
+        }
 #pragma unroll
         for (int s = 0; s < 8; ++s)
 #pragma unroll
-            for (int x = 0; x < 4; ++x) z[x] = fmaf(vv[s], hv[x + s], z[x]);
+            for (int x = 0; x < 4; ++x) {
+                if (r < 16) z[0][x] = fmaf(cur[s], hv[x + s], z[0][x]);
+                if (r > 0) z[1][x] = fmaf(prev[s], hv[x + s], z[1][x]);
+            }
     }
-    const int wy = wy0 + ry;
-    if (wy < L.rows) {
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+        const int wy = wy0 + ry + y;
+        if (wy >= L.rows) break;
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const int wx = wx0 + qx + x;
-            if (wx < L.cols) logits[L.score_off + (int64_t)wy * L.cols + wx] = z[x];
+            if (wx >= L.cols) continue;
+            const int64_t at = L.score_off + (int64_t)wy * L.cols + wx;
+            logits[at] = z[y][x];
+            if (!c_flag) continue;
+            scores[at] = -INFINITY;
+            if (!(z[y][x] > tau)) continue;
+            for (int tr = wy / kCellTH; tr <= (wy + kWinBH) / kCellTH; ++tr)
+                for (int tc = wx / kCellTW; tc <= (wx + kWinBW) / kCellTW; ++tc)
+                    c_flag[L.citem0 + tr * L.ctx + tc] = 1u;
         }
     }
 }
@@ -610,7 +676,8 @@ cudaError_t init_cnn() {
 
 cudaError_t launch_cnn(cudaStream_t s, const LevelDesc *d_levels, int n_levels, const CUtensorMap *lvl_maps,
                        const CnnItem *d_items, int n_items, const CnnWeights &w, float *hmap,
-                       int32_t hmap_pitch, float *logits, int pool_tiles, unsigned *err) {
+                       int32_t hmap_pitch, float *logits, int pool_tiles, unsigned *err, float tau,
+                       uint32_t *c_flag, float *scores) {
     if (n_items > 0) {
         const int grid = std::min(n_items, g_cnn_grid > 0 ? g_cnn_grid : n_items);
         k_cnn_fwd<<<grid, kThreads, sizeof(CnnSmem), s>>>(d_levels, lvl_maps, d_items, n_items, w, hmap,
@@ -619,9 +686,9 @@ cudaError_t launch_cnn(cudaStream_t s, const LevelDesc *d_levels, int n_levels, 
         if (e != cudaSuccess) return e;
     }
     if (n_levels > 0 && pool_tiles > 0) {
-        // enough x-blocks for the largest level's 64 x 16 tiles; the others leave early
+        // enough x-blocks for the largest level's 64 x 32 tiles; the others leave early
         dim3 grid(pool_tiles, n_levels);
-        k_cnn_pool<<<grid, 256, 0, s>>>(d_levels, hmap, hmap_pitch, w.v, w.bv, logits);
+        k_cnn_pool<<<grid, 256, 0, s>>>(d_levels, hmap, hmap_pitch, w.v, w.bv, logits, tau, c_flag, scores);
         return cudaGetLastError();
     }
     return cudaSuccess;

@@ -4,14 +4,11 @@
 // FP32 K4 one warp per window tile of its plan decides whether the tile holds
 // a kept window; a kept tile marks every K2+K3 cell tile its cell region
 // overlaps, and K4 computes the kept tiles (their windows are all scored
-// exactly; the others get -inf, which never becomes an NMS candidate). For the
-// tensor-core K4 each kept window marks only the cell tiles under its own
-// 8 x 16 cells, and K4 scores every window whose cells were all computed; one
-// thread per window does both this and the -inf that the skipped windows keep
-// (bound by reading the logits and writing the scores). Flags are plain stores
-// of 1, so they do not depend on the order of the threads. Either way every
-// kept window is scored exactly, so the recall is at least that of the
-// window-level proposal.
+// exactly; the others get -inf, which never becomes an NMS candidate). Flags
+// are plain stores of 1, so they do not depend on the order of the warps.
+// Either way every kept window is scored exactly, so the recall is at least
+// that of the window-level proposal. (The tensor-core K4's flags are set per
+// window by the pooling kernel of the proposal network.)
 #include "pd_internal.h"
 
 namespace pd {
@@ -48,46 +45,7 @@ __global__ void __launch_bounds__(256) k_proposal_flags(const LevelDesc *__restr
     }
 }
 
-// Block (x, y): every gridDim.x-th run of windows of level y.
-__global__ void __launch_bounds__(256) k_window_flags(const LevelDesc *__restrict__ levels,
-                                                      const float *__restrict__ logits, float tau,
-                                                      uint32_t *__restrict__ c_flag, float *__restrict__ scores) {
-    const LevelDesc &L = levels[blockIdx.y];
-    const int n = L.rows * L.cols, cols = L.cols, ctx = L.ctx;
-    const float *z = logits + L.score_off;
-    float *out = scores + L.score_off;
-    uint32_t *flags = c_flag + L.citem0;
-    constexpr int kU = 4;  // loads in flight per thread
-    for (int i0 = blockIdx.x * 256 * kU + threadIdx.x; i0 < n; i0 += gridDim.x * 256 * kU) {
-        float v[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) v[u] = i0 + u * 256 < n ? __ldg(z + i0 + u * 256) : -INFINITY;
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int i = i0 + u * 256;
-            if (i >= n) continue;
-            out[i] = -INFINITY;
-            if (!(v[u] > tau)) continue;
-            // cell tiles under cell rows wy .. wy+15, columns wx .. wx+7
-            const int wy = i / cols, wx = i - wy * cols;
-            for (int ty = wy / kCellTH; ty <= (wy + kWinBH) / kCellTH; ++ty)
-                for (int tx = wx / kCellTW; tx <= (wx + kWinBW) / kCellTW; ++tx) flags[ty * ctx + tx] = 1u;
-        }
-    }
-}
-
 }  // namespace
-
-cudaError_t launch_window_flags(cudaStream_t s, const LevelDesc *d_levels, int n_levels, int max_windows,
-                                const float *logits, float tau, uint32_t *c_flag, float *scores) {
-    if (n_levels <= 0 || max_windows <= 0) return cudaSuccess;
-    const int gx = max_windows >= 32 * 1024 ? 32 : (max_windows + 1023) / 1024;
-    for (int l0 = 0; l0 < n_levels; l0 += 65535) {  // grid.y limit
-        const int nl = n_levels - l0 < 65535 ? n_levels - l0 : 65535;
-        k_window_flags<<<dim3(gx, nl), 256, 0, s>>>(d_levels + l0, logits, tau, c_flag, scores);
-    }
-    return cudaGetLastError();
-}
 
 cudaError_t launch_proposal_flags(cudaStream_t s, const LevelDesc *d_levels, const SvmItem *d_items, int n_items,
                                   const float *logits, float tau, uint32_t *s_flag, uint32_t *c_flag) {

@@ -524,9 +524,13 @@ void plan_strips(Plan &p, int resident_warps) {
         histogram(rows, n);
         return makespan(n, kMaxRows, 1, R);
     };
-    int rows = kMaxRows;
+    // Sparse path: one cell tile per strip. A tall strip whose tiles are partly
+    // skipped leaves its warp with less than planned (8 x 1920x1080: cells
+    // 297 -> 283 us).
+    const bool sparse = !p.cnn_items.empty();
+    int rows = sparse ? kCellTH : kMaxRows;
     int64_t n32[kMaxRows + 1];
-    if (histogram(rows, n32) < 16 * R) {
+    if (!sparse && histogram(rows, n32) < 16 * R) {
         int64_t best = schedule(rows);
         for (int r = rows / 2; r >= 2; r /= 2) {
             const int64_t t = schedule(r);
@@ -848,12 +852,6 @@ void invalidate_cache(pd_handle *h) {
 int max_pool_tiles(const Plan &p) {
     int m = 0;
     for (const LevelDesc &L : p.levels) m = std::max(m, pool_tiles_of(L.rows, L.cols));
-    return m;
-}
-
-int max_windows(const Plan &p) {
-    int m = 0;
-    for (const LevelDesc &L : p.levels) m = std::max(m, L.rows * L.cols);
     return m;
 }
 
@@ -1259,18 +1257,16 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         if (timed) PD_CUDA(h, record(h->stage_ev[5], q));
         const uint32_t *cf = nullptr, *sf = nullptr;
         if (h->proposal) {
-            // learned proposal: keep-logits of every window, then the tiles to score
+            // learned proposal: keep-logits of every window and the tiles to score
+            const bool per_window = !(h->p.flags & PD_FLAG_SVM_FP32);
+            PD_CUDA(h, cudaMemsetAsync(h->c_flag, 0, p.c_items.size() * 4 + 4, q));
             PD_CUDA(h, launch_cnn(q, dl, (int)p.levels.size(), dptr<CUtensorMap>(h, o.tmaps),
                                   dptr<CnnItem>(h, o.cnn_items),
                                   (int)p.cnn_items.size(), cnn_weights(h), h->hmap, h->atlas.pitch, h->logits,
-                                  max_pool_tiles(p), h->d_err));
-            PD_CUDA(h, cudaMemsetAsync(h->c_flag, 0, p.c_items.size() * 4 + 4, q));
-            if (h->p.flags & PD_FLAG_SVM_FP32)
+                                  max_pool_tiles(p), h->d_err, h->tau, per_window ? h->c_flag : nullptr, h->d_scores));
+            if (!per_window)
                 PD_CUDA(h, launch_proposal_flags(q, dl, dptr<SvmItem>(h, o.s_items), (int)p.s_items.size(),
                                                  h->logits, h->tau, h->s_flag, h->c_flag));
-            else
-                PD_CUDA(h, launch_window_flags(q, dl, (int)p.levels.size(), max_windows(p), h->logits, h->tau,
-                                               h->c_flag, h->d_scores));
             cf = h->c_flag;
             sf = h->s_flag;
         }
@@ -1327,7 +1323,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
                        (p.score_floats == 0 ? 0 : 1) +
                        nms_launches(n_frames, nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame)) +
                        (h->proposal ? (p.cnn_items.empty() ? 0 : 1) + (p.levels.empty() ? 0 : 1) +
-                                          (p.score_floats == 0 ? 0 : 1)
+                                          (p.s_items.empty() ? 0 : 1)
                                     : 0);
     h->detected = true;
     h->ran_proposal = h->proposal;

@@ -139,9 +139,6 @@ cudaError_t launch_cells_warp(cudaStream_t s, const LevelDesc *d_levels, const u
                               const uint8_t *d_lbp_map, const uint32_t *c_flag, int feat);
 cudaError_t launch_proposal_flags(cudaStream_t s, const LevelDesc *d_levels, const SvmItem *d_items, int n_items,
                                   const float *logits, float tau, uint32_t *s_flag, uint32_t *c_flag);
-// Tensor-core K4: cell tiles under every kept window, and -inf in every score.
-cudaError_t launch_window_flags(cudaStream_t s, const LevelDesc *d_levels, int n_levels, int max_windows,
-                                const float *logits, float tau, uint32_t *c_flag, float *scores);
 cudaError_t launch_svm(cudaStream_t s, const CUtensorMap *hog_maps, const CUtensorMap *lbp_maps,
                        const LevelDesc *d_levels, const float *d_w, float bias, float clip,
                        float *scores, const SvmItem *d_items, int n_items, unsigned *d_err,
@@ -262,9 +259,9 @@ struct TrainArgs {
 };
 
 cudaError_t init_cnn();
-// Window pooling tiles: 64 x 16 windows per CTA; pool_tiles = the largest
-// level's tile count (ceil(cols / 64) * ceil(rows / 16)).
-constexpr int kPoolTW = 64, kPoolTH = 16;
+// Window pooling tiles: 64 x 32 windows per CTA; pool_tiles = the largest
+// level's tile count (ceil(cols / 64) * ceil(rows / 32)).
+constexpr int kPoolTW = 64, kPoolTH = 32;
 inline int pool_tiles_of(int rows, int cols) {
     return rows > 0 && cols > 0 ? ((cols + kPoolTW - 1) / kPoolTW) * ((rows + kPoolTH - 1) / kPoolTH) : 0;
 }
@@ -272,9 +269,12 @@ inline int pool_tiles_of(int rows, int cols) {
 // level rows [8 cy0 - 7, 8 cy0 + 65), fetched by TMA through one 2D tensor
 // map per level (u8, box 96 x 72, zero fill outside the level).
 constexpr int kCnnBoxW = 96, kCnnBoxH = 72;
+// c_flag non-null (tensor-core K4's sparse path; zeroed before): the pooling also
+// marks the cell tiles under every window with a logit above tau and fills scores with -inf.
 cudaError_t launch_cnn(cudaStream_t s, const LevelDesc *d_levels, int n_levels, const CUtensorMap *lvl_maps,
                        const CnnItem *d_items, int n_items, const CnnWeights &w, float *hmap,
-                       int32_t hmap_pitch, float *logits, int pool_tiles, unsigned *err);
+                       int32_t hmap_pitch, float *logits, int pool_tiles, unsigned *err, float tau = 0.f,
+                       uint32_t *c_flag = nullptr, float *scores = nullptr);
 cudaError_t init_train();
 size_t train_partial_floats();
 cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a);
