@@ -23,12 +23,13 @@
 //    the subtraction n - c does not borrow out of bit 7, which is the
 //    majority of (n7, not c7, bit 7 of (n | 0x80) - (c & 0x7f)); one
 //    subtraction and one 3-input logic operation compare 4 pixels with one
-//    neighbour, and the 8 comparison words fold into 4 codes. A 256-entry
-//    table gives each code's uniform bin as an 8-bit counter of a word of the
-//    lane's own counters ([word][lane] layout: the shared-memory atomics never
-//    collide; exact and order independent; Algorithm 2). A cell's counts are
-//    the sum of its two lanes' counters (each <= 32), written out after the
-//    band's first 4 rows, which complete cell row cy0 + k - 1.
+//    neighbour. The 8 comparisons of a lane's 32 pixels of a cell (4 columns x
+//    8 rows) are 8 bit planes, shifted in row by row, and a uniform code is
+//    one run of ones: the pixels of a code are three planes ANDed and their
+//    number a population count (Algorithm 2 without a histogram in memory).
+//    Counting in shared memory instead (a code -> counter table and an atomic
+//    per pixel) took a third of the kernel's shared-memory wavefronts and kept
+//    that pipe 79% busy (now 58%): 0.961 -> 0.887 ms per 64 x 1242x375 frames.
 //  * HOG (Algorithm 4). One byte permute and two dp2a (weights +1, -1) give
 //    the central differences of two pixels; the accumulator 0x4B400000 makes
 //    the 32-bit result the float 1.5 * 2^23 + g, so one multiply-add turns it
@@ -50,17 +51,24 @@
 //    bin number plus a constant, so they index the column's vote slots
 //    directly. There are 11 slots per column, slot s holding bin
 //    (s - 1) mod 9 (bin -1 and bin 9 wrap), which the epilogue folds back:
-//    the loop needs no wrap logic.
+//    the loop needs no wrap logic. Two pixels share an instruction wherever
+//    both take the same step (fma.rn.f32x2 rounds each half as the scalar
+//    does): 11 fewer instructions per pixel, 0.887 -> 0.828 ms; shared-memory
+//    addresses of the slots as integers, 0.828 -> 0.810.
 //    The slots of lane t's 4 columns sit at 4t + (j ^ ((t >> 3) & 3)), so
 //    that a warp's data-dependent scatter hits 32 distinct banks and the
-//    epilogue reads them with one 16-byte load. Rows outside the cell grid
-//    vote with weight 0 and count nothing (no branch).
+//    epilogue reads them with one 16-byte load.
+// Rows outside the cell grid are whole halves of the level's first and last
+// bands and are not walked (0.810 -> 0.785 ms). What bounds the kernel now:
+// issue (74% of cycles, about 79 instructions per pixel) with 16 warps per SM
+// at 128 registers; 20 warps at 96 registers measured slower (0.875 against
+// 0.828 ms), all of a row's slot loads before its stores no faster.
 // HOG epilogue of cell row r: each lane forms, per bin, the weighted sums of
 // its 4 columns for its own cell and for the neighbouring cell they reach;
 // three shuffles add the 4 lanes that reach a cell (fixed order:
 // deterministic). The LBP counts of a cell go out as 64 bytes, two 16-byte
-// stores per lane (the counter words are already four bins each), or, for
-// callers that ask for planes, bin-plane by bin-plane. At the top and bottom of a
+// stores from each of its two lanes, or, for callers that ask for planes,
+// bin-plane by bin-plane. At the top and bottom of a
 // level the votes of the clamped cell row (Algorithm 5's interpolation
 // clamped into the grid) are added into the first and last row before they
 // are written. The result does not depend on the strip height: every cell
@@ -73,6 +81,7 @@
 #include <type_traits>
 #include <utility>
 
+#include "f32x2.cuh"
 #include "pd_internal.h"
 
 namespace pd {
@@ -83,7 +92,6 @@ constexpr int kSCols = 8 * kCellTW + 8;          // 128 pixel columns walked per
 static_assert(kSCols == 4 * 32, "four pixel columns per lane");
 constexpr int kSlots = kHogBins + 2;             // vote slots per column (bins -1 .. 9)
 constexpr int kRingStride = kSlots * kSCols;     // floats per open cell row
-constexpr int kCntWords = (kLbpBins + 3) / 4;    // words of four 8-bit counters per cell
 constexpr uint32_t kHi = 0x80808080u;
 constexpr float kMagic = 12582912.0f;            // 1.5 * 2^23: dp2a accumulator
 constexpr uint32_t kMagicBits = 0x4B400000u;
@@ -92,10 +100,8 @@ constexpr uint32_t kMagic2Bits = 0x4BC00000u;
 
 struct WarpSmem {
     float R[2 * kRingStride];       // HOG vote slots of the 2 open cell rows
-    uint32_t cnt[kCntWords * 32];   // LBP counters of the open cell row: [word][lane], lane-private
 };
 struct StripSmem {
-    uint2 map[256];                 // LBP code -> (counter word index, increment)
     WarpSmem w[kWarps];
 };
 
@@ -130,17 +136,32 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
-// 2 atan(z) * 9/pi / z as a polynomial in s = z^2 (|z| <= 1): the fitted
-// coefficients scaled to 20-degree bins and doubled (exact: every step of
-// the evaluation scales by 2).
-__device__ __forceinline__ float atan_bins2_poly(float s) {
-    float p = 2.0f * 0.019514326006174088f;
-    p = fmaf(p, s, 2.0f * -0.09626893699169159f);
-    p = fmaf(p, s, 2.0f * 0.22810496389865875f);
-    p = fmaf(p, s, 2.0f * -0.3791072964668274f);
-    p = fmaf(p, s, 2.0f * 0.5674521327018738f);
-    p = fmaf(p, s, 2.0f * -0.9544723033905029f);
-    return fmaf(p, s, 2.0f * 2.8647778034210205f);
+// -2 atan(z) * 9/pi / z as a polynomial in s = z^2 (|z| <= 1), two values at
+// a time: the fitted coefficients scaled to 20-degree bins, doubled and negated
+// (exact: every step of the evaluation scales by -2).
+__device__ __forceinline__ f32x2 atan_bins2_poly(f32x2 s) {
+    f32x2 p = dup2(-2.0f * 0.019514326006174088f);
+    p = fma2(p, s, dup2(-2.0f * -0.09626893699169159f));
+    p = fma2(p, s, dup2(-2.0f * 0.22810496389865875f));
+    p = fma2(p, s, dup2(-2.0f * -0.3791072964668274f));
+    p = fma2(p, s, dup2(-2.0f * 0.5674521327018738f));
+    p = fma2(p, s, dup2(-2.0f * -0.9544723033905029f));
+    return fma2(p, s, dup2(-2.0f * 2.8647778034210205f));
+}
+
+// A vote slot at a shared-memory address (the compiler's own indexing spends a
+// shift per access). Volatile and clobbering: the epilogue reads the slots
+// through ordinary pointers.
+constexpr int kSlotBytes = 4 * kSCols;
+template <int OFF>
+__device__ __forceinline__ float lds(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1 + %2];" : "=f"(v) : "r"(a), "n"(OFF) : "memory");
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ void sts(uint32_t a, float v) {
+    asm volatile("st.shared.f32 [%0 + %1], %2;" ::"r"(a), "n"(OFF), "f"(v) : "memory");
 }
 
 template <class F, int... I>
@@ -148,28 +169,67 @@ __device__ __forceinline__ void static_for(F &&f, std::integer_sequence<int, I..
     (f(std::integral_constant<int, I>{}), ...);
 }
 
-// 4 pixels' n >= c comparisons, as bit 7 of each byte (other bits 0).
-__device__ __forceinline__ uint32_t ge4(uint32_t n, uint32_t c_lo, uint32_t c_not7) {
+// 4 pixels' n >= c comparisons, as bit 7 of each byte (the other bits are not
+// meaningful); cn = ~c.
+__device__ __forceinline__ uint32_t ge4(uint32_t n, uint32_t c_lo, uint32_t cn) {
     const uint32_t t = (n | kHi) - c_lo;
-    const uint32_t n7 = n & kHi;
-    return (n7 & c_not7) | (t & (n7 | c_not7));
+    return (n & cn) | (t & (n | cn));  // majority of n, not c, t
+}
+
+// Uniform codes below 128 in ascending order are runs of ones [s, s + len) with
+// s + len <= 7; run k (1 .. 28; 0 is the empty code) as constants.
+__host__ __device__ constexpr int run_start(int k) {
+    int i = 0;
+    for (int c = 1; c < 128; ++c) {
+        int s = 0;
+        while (!((c >> s) & 1)) ++s;
+        int e = s;
+        while ((c >> e) & 1) ++e;
+        if (c >> e) continue;
+        if (++i == k) return s;
+    }
+    return -1;
+}
+__host__ __device__ constexpr int run_end(int k) {
+    int i = 0;
+    for (int c = 1; c < 128; ++c) {
+        int s = 0;
+        while (!((c >> s) & 1)) ++s;
+        int e = s;
+        while ((c >> e) & 1) ++e;
+        if (c >> e) continue;
+        if (++i == k) return e;
+    }
+    return -1;
+}
+static_assert(run_end(28) == 7 && run_start(28) == 0 && run_start(29) == -1, "28 runs below bit 7");
+
+// The comparison planes of 32 pixels (bit k of their codes in x[k]) -> pixels
+// whose code is one run starting at s (run[s], s < 7), is 0 (none), or has two
+// or more runs (many: not uniform).
+__device__ __forceinline__ void lbp_runs(const uint32_t (&x)[8], uint32_t (&run)[7], uint32_t &none, uint32_t &many) {
+    uint32_t r[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) r[k] = x[k] & ~x[(k + 7) & 7];  // a run starts at k
+    const uint32_t s1 = r[0] ^ r[1] ^ r[2], c1 = (r[0] & r[1]) | (r[2] & (r[0] | r[1]));
+    const uint32_t s2 = r[3] ^ r[4] ^ r[5], c2 = (r[3] & r[4]) | (r[5] & (r[3] | r[4]));
+    const uint32_t s3 = r[6] ^ r[7], c3 = r[6] & r[7];
+    const uint32_t c4 = (s1 & s2) | (s3 & (s1 | s2));
+    many = (c1 | c2 | c3) | c4;
+    const uint32_t one = (s1 ^ s2 ^ s3) & ~many;
+#pragma unroll
+    for (int k = 0; k < 7; ++k) run[k] = r[k] & one;
+    none = ~((x[0] | x[1] | x[2]) | (x[3] | x[4] | x[5]) | (x[6] | x[7]));
 }
 
 template <int FEAT, bool CELLS>  // CELLS: cell-major LBP counts
 __global__ void __launch_bounds__(kWarps * 32, 4)
     k_cells_warp(const LevelDesc *__restrict__ levels, const uint8_t *__restrict__ pyr, CellAtlas atlas,
                  const StripItem *__restrict__ items, int n_items, int *__restrict__ queue,
-                 const uint8_t *__restrict__ lbp_map, const uint32_t *__restrict__ c_flag) {
+                 const uint32_t *__restrict__ c_flag) {
     constexpr bool kHog = (FEAT & kFeatHog) != 0, kLbp = (FEAT & kFeatLbp) != 0;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StripSmem &S = *reinterpret_cast<StripSmem *>(smem_raw);
-    if (kLbp) {
-        for (int i = threadIdx.x; i < 256; i += kWarps * 32) {
-            const int bn = lbp_map[i];
-            S.map[i] = make_uint2((uint32_t)(bn >> 2) * 32u, 1u << ((bn & 3) * 8));
-        }
-        __syncthreads();
-    }
     const int lane = threadIdx.x & 31;
     WarpSmem &Wm = S.w[threadIdx.x >> 5];
     // persistent warps: each takes the next strip (tallest first) until none is left
@@ -181,7 +241,6 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
         const LevelDesc L = levels[it.level];
         const uint8_t *img = pyr + L.img_off;
         const int pitch = L.img_pitch, Wk = L.Wk, Hk = L.Hk, Wc = L.Wc, Hc = L.Hc;
-        const int gridH = 8 * Hc;
         const int cx0 = it.cx0, cy0 = it.cy0, nb = it.cy1 - it.cy0;
         const int tx = cx0 / kCellTW;
         const int x = 8 * cx0 - 4 + 4 * lane;  // first pixel column of this lane
@@ -191,15 +250,17 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
         if (kHog)
             for (int i = lane; i < 2 * kRingStride / 4; i += 32)
                 reinterpret_cast<float4 *>(Wm.R)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (kLbp)
-            for (int i = lane; i < kCntWords * 32; i += 32) Wm.cnt[i] = 0u;
+        uint32_t plane[8];  // LBP comparisons of the last 8 rows: plane k, byte = column, bit = row
+#pragma unroll
+        for (int k = 0; k < 8; ++k) plane[k] = 0u;
 
         // ---- lane constants
         const int sw = (lane >> 3) & 3;
-        // float index of slot 0 of pixel j's column, less the bias of the rounded angle's bits
+        // shared-memory address of slot 0 of pixel j's column, less the bias of the rounded angle's bits
         uint32_t vb[4];
+        const uint32_t slots = (uint32_t)__cvta_generic_to_shared(Wm.R);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) vb[j] = (uint32_t)(4 * lane + (j ^ sw)) + 128u - kMagic2Bits * 128u;
+        for (int j = 0; j < 4; ++j) vb[j] = slots + 4u * (uint32_t)(4 * lane + (j ^ sw)) + 512u - kMagic2Bits * 512u;
         // epilogue x-weights by slot position p (column j = p ^ sw): own cell, neighbour cell
         float wo[4], wn[4];
         {
@@ -221,7 +282,6 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
                 wn[p] = b;
             }
         }
-        const bool core = (unsigned)(lane - 1) < 30u;  // lanes 1..30 own strip pixels (LBP)
         __syncwarp();
 
         // ---- rows
@@ -257,9 +317,10 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
         // weights wa, wb into the vote slots at float indices va[j] (cell row
         // band - 1) and va[j] + dB (cell row band); LBP counts into the lane's counters
         // (a row outside the cell grid votes with weight 0 and counts nothing)
-        auto pixel_row = [&](const Row &ra, const Row &rb, const Row &rc, float wa, float wb, const uint32_t (&va)[4],
-                             int dB, bool valid) {
+        auto pixel_row = [&](const Row &ra, const Row &rb, const Row &rc, float fa, float fb, const uint32_t (&va)[4],
+                             uint32_t dB) {
             if (kHog) {
+                const f32x2 wa = dup2(fa), wb = dup2(fb);
                 const uint32_t P01 = __byte_perm(rb.r, rb.l, 0x5140), P23 = __byte_perm(rb.r, rb.l, 0x7362);
                 const uint32_t Q01 = __byte_perm(rc.c, ra.c, 0x5140), Q23 = __byte_perm(rc.c, ra.c, 0x7362);
                 const int gxb[4] = {dp2a_diff_lo(P01, (int)kMagicBits), dp2a_diff_hi(P01, (int)kMagicBits),
@@ -267,87 +328,120 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
                 const int gyb[4] = {dp2a_diff_lo(Q01, (int)kMagicBits), dp2a_diff_hi(Q01, (int)kMagicBits),
                                     dp2a_diff_lo(Q23, (int)kMagicBits), dp2a_diff_hi(Q23, (int)kMagicBits)};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < 4; j += 2) {  // pixels j, j + 1: packed where both take the same step
                     // half gradients, exact: (1.5 * 2^23 + g) / 2 - 0.75 * 2^23
-                    const float hx = fmaf(__int_as_float(gxb[j]), 0.5f, -0.5f * kMagic);
-                    const float hy = fmaf(__int_as_float(gyb[j]), 0.5f, -0.5f * kMagic);
-                    const float hm = sqrt_approx(fmaf(hx, hx, hy * hy));  // magnitude / 2
-                    const float ax = fabsf(hx), ay = fabsf(hy);
+                    const f32x2 half = dup2(0.5f), bias = dup2(-0.5f * kMagic), neg = dup2(-1.0f);
+                    const f32x2 hx = fma2(pack2(__int_as_float(gxb[j]), __int_as_float(gxb[j + 1])), half, bias);
+                    const f32x2 hy = fma2(pack2(__int_as_float(gyb[j]), __int_as_float(gyb[j + 1])), half, bias);
+                    float x0, x1, y0, y1, q0, q1;
+                    unpack2(hx, x0, x1);
+                    unpack2(hy, y0, y1);
+                    unpack2(fma2(hx, hx, mul2(hy, hy)), q0, q1);
+                    const f32x2 hm = pack2(sqrt_approx(q0), sqrt_approx(q1));  // magnitude / 2
                     // phi = atan(ay / ax) = 45deg + atan(t), t = (ay - ax) / (ay + ax) in [-1, 1];
                     // ax + ay is 0 or >= 0.5: the 1e-30 only turns 0 / 0 into 0
-                    const float t = (ay - ax) * rcp_approx(ax + ay + 1e-30f);
-                    const float u = fmaf(-t, atan_bins2_poly(t * t), 4.5f);  // 2 (4.5 - phi) in bins, in [0, 9]
+                    float d0, d1;
+                    unpack2(add2(pack2(fabsf(x0) + fabsf(y0), fabsf(x1) + fabsf(y1)), dup2(1e-30f)), d0, d1);
+                    const f32x2 t = mul2(pack2(fabsf(y0) - fabsf(x0), fabsf(y1) - fabsf(x1)),
+                                         pack2(rcp_approx(d0), rcp_approx(d1)));
+                    // u = 2 (4.5 - phi) in bins, in [0, 9]
+                    float u0, u1;
+                    unpack2(fma2(t, atan_bins2_poly(mul2(t, t)), dup2(4.5f)), u0, u1);
                     // theta = phi (same signs) or 9 - phi (opposite signs); the vote position is
                     // theta - 0.5, rounded below through theta - 1: p2 = 2 (theta - 1) = 7 -/+ u
-                    const uint32_t flip = (__float_as_uint(hx) ^ __float_as_uint(hy)) & 0x80000000u;
-                    const float p2 = 7.0f - __uint_as_float(__float_as_uint(u) ^ flip);
-                    const float r2 = p2 + kMagic2;                // 2 round(theta - 1) + 3 * 2^23
-                    const float e2 = p2 - (r2 - kMagic2);         // 2 (theta - 1 - round(...)), in [-1, 1]
-                    const int oa = (int)((uint32_t)__float_as_int(r2) * 128u + va[j]);
-                    float *v = Wm.R + oa;
-                    float *w = Wm.R + (oa + dB);
+                    const uint32_t f0 = ~(__float_as_uint(x0) ^ __float_as_uint(y0)) & 0x80000000u;
+                    const uint32_t f1 = ~(__float_as_uint(x1) ^ __float_as_uint(y1)) & 0x80000000u;
+                    const f32x2 p2 = add2(pack2(__uint_as_float(__float_as_uint(u0) ^ f0),
+                                                __uint_as_float(__float_as_uint(u1) ^ f1)), dup2(7.0f));
+                    const f32x2 r2 = add2(p2, dup2(kMagic2));       // 2 round(theta - 1) + 3 * 2^23
+                    const f32x2 rr = add2(r2, dup2(-kMagic2));
+                    const f32x2 e2 = fma2(rr, neg, p2);             // 2 (theta - 1 - round(...)), in [-1, 1]
+                    const f32x2 n2 = fma2(p2, neg, rr);             // -e2
+                    // slot addresses of the two pixels, in the cell rows above and below
+                    const uint32_t v = (uint32_t)__float_as_int(lo2(r2)) * 512u + va[j], w = v + dB;
+                    const uint32_t z = (uint32_t)__float_as_int(hi2(r2)) * 512u + va[j + 1], o = z + dB;
                     // upper / lower bin: magnitude times (1 +/- e2) / 2
-                    const float mo1 = fmaf(hm, e2, hm), mo0 = fmaf(-hm, e2, hm);
-                    v[0] = fmaf(mo0, wa, v[0]);
-                    v[kSCols] = fmaf(mo1, wa, v[kSCols]);
-                    w[0] = fmaf(mo0, wb, w[0]);
-                    w[kSCols] = fmaf(mo1, wb, w[kSCols]);
+                    const f32x2 mo1 = fma2(hm, e2, hm), mo0 = fma2(hm, n2, hm);
+                    const f32x2 a0 = fma2(mo0, wa, pack2(lds<0>(v), lds<0>(z)));
+                    const f32x2 a1 = fma2(mo1, wa, pack2(lds<kSlotBytes>(v), lds<kSlotBytes>(z)));
+                    const f32x2 b0 = fma2(mo0, wb, pack2(lds<0>(w), lds<0>(o)));
+                    const f32x2 b1 = fma2(mo1, wb, pack2(lds<kSlotBytes>(w), lds<kSlotBytes>(o)));
+                    sts<0>(v, lo2(a0));
+                    sts<0>(z, hi2(a0));
+                    sts<kSlotBytes>(v, lo2(a1));
+                    sts<kSlotBytes>(z, hi2(a1));
+                    sts<0>(w, lo2(b0));
+                    sts<0>(o, hi2(b0));
+                    sts<kSlotBytes>(w, lo2(b1));
+                    sts<kSlotBytes>(o, hi2(b1));
                 }
             }
             if (kLbp) {
-                const uint32_t clo = rb.c & ~kHi, cn7 = ~rb.c & kHi;
-                const uint32_t code = (ge4(ra.l, clo, cn7) >> 7) | (ge4(ra.c, clo, cn7) >> 6) |
-                                      (ge4(ra.r, clo, cn7) >> 5) | (ge4(rb.r, clo, cn7) >> 4) |
-                                      (ge4(rc.r, clo, cn7) >> 3) | (ge4(rc.c, clo, cn7) >> 2) |
-                                      (ge4(rc.l, clo, cn7) >> 1) | ge4(rb.l, clo, cn7);
-                if (core && valid) {
+                const uint32_t clo = rb.c & ~kHi, cn = ~rb.c;
+                const uint32_t nb8[8] = {ra.l, ra.c, ra.r, rb.r, rc.r, rc.c, rc.l, rb.l};
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const uint2 e = S.map[(code >> (8 * j)) & 0xffu];
-                        atomicAdd(&Wm.cnt[(int)e.x + lane], e.y);
-                    }
-                }
+                for (int k = 0; k < 8; ++k)
+                    plane[k] = ((plane[k] >> 1) & ~kHi) | (ge4(nb8[k], clo, cn) & kHi);
             }
         };
 
-        // ---- LBP of cell row r = band - 1 is final after the band's first 4 rows:
-        // a cell's counts are its two lanes' counters; write them, clear
-        auto emit_lbp = [&](int band, bool walked) {
-            __syncwarp();  // every lane's counts of row r are in
+        // ---- LBP of cell row r = band - 1 is final after the band's first 4 rows: the planes
+        // hold its 8 rows (older bits are shifted out). A cell is the two lanes 2c + 1 and
+        // 2c + 2, 32 pixels each. The first counts the 29 uniform codes below 128 over both
+        // lanes' planes, the second those above over the complements: the code ranked 57 - k
+        // is the complement of the code ranked k, so both run the same instructions.
+        auto emit_lbp = [&](int band) {
             const int r = band - 1;
-            const int c = lane & 15, half = lane >> 4;
-            if (CELLS) {
-                // words 8 half .. 8 half + 7 of cell c: 32 bytes (the last word is padding)
-                if (walked && need(r) && c < kCellTW && cx0 + c < Wc) {
-                    const uint32_t *cw = Wm.cnt + half * 8 * 32 + 2 * c + 1;
-                    uint32_t v[8];
+            if (!need(r)) return;
+            const uint32_t half = (lane & 1) ^ 1u, flip = 0u - half;
+            uint32_t x[8], ra_[7], rb_[7], none_a, none_b, many_a, many_b, y[8];
 #pragma unroll
-                    for (int i = 0; i < 7; ++i) v[i] = cw[i * 32] + cw[i * 32 + 1];  // counts <= 32 each: no carry
-                    v[7] = half ? 0u : cw[7 * 32] + cw[7 * 32 + 1];
-                    uint4 *dst = reinterpret_cast<uint4 *>(
-                        atlas.lbp + ((int64_t)(L.cell_row + cy0 + r) * atlas.pitch + cx0 + c) * kLbpCellBytes + 32 * half);
-                    dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
-                    dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
-                }
-            } else if (walked && need(r) && c < kCellTW && cx0 + c < Wc) {
-                const int64_t pl = atlas.lbp_plane;
-                // bin planes 32 half .. 32 half + 31 of cell c
-                uint8_t *dst = atlas.lbp + (int64_t)(L.cell_row + cy0 + r) * atlas.pitch + cx0 + c + 32 * half * pl;
-                const uint32_t *cw = Wm.cnt + half * 8 * 32 + 2 * c + 1;
-                const int nw = half ? kCntWords - 8 : 8;
-#pragma unroll 1
-                for (int i = 0; i < nw; ++i) {
-                    const uint32_t val = cw[i * 32] + cw[i * 32 + 1];  // counts <= 32 each: no carry
-                    dst[0] = (uint8_t)val;
-                    dst[pl] = (uint8_t)(val >> 8);
-                    dst[2 * pl] = (uint8_t)(val >> 16);
-                    if (32 * half + 4 * i + 3 < kLbpBins) dst[3 * pl] = (uint8_t)(val >> 24);
-                    dst += 4 * pl;
-                }
+            for (int k = 0; k < 8; ++k) {
+                x[k] = plane[k] ^ flip;
+                y[k] = __shfl_sync(0xffffffffu, plane[k], ((lane - 1) ^ 1) + 1) ^ flip;
             }
-            __syncwarp();  // read before cleared
+            lbp_runs(x, ra_, none_a, many_a);
+            lbp_runs(y, rb_, none_b, many_b);
+            uint32_t q[8];  // counts of the ranks, 4 per word
+            static_for([&](auto K) {
+                constexpr int k = decltype(K)::value;
+                uint32_t n;
+                if constexpr (k == 0) {
+                    n = __popc(none_a) + __popc(none_b);
+                } else {
+                    constexpr int s = run_start(k), e = run_end(k);
+                    n = __popc(ra_[s] & x[e - 1] & ~x[e]) + __popc(rb_[s] & y[e - 1] & ~y[e]);
+                }
+                if constexpr (k % 4 == 0) q[k / 4] = n;
+                else q[k / 4] += n << (8 * (k % 4));
+            }, std::make_integer_sequence<int, 29>{});
+            const uint32_t other = __popc(many_a) + __popc(many_b);
+            // bins 29, 30, 31 are the upper lane's ranks 28, 27, 26
+            const uint32_t top = __shfl_down_sync(0xffffffffu, __byte_perm(q[7], q[6], 0x0670) & 0xffffffu, 1);
+            uint32_t v[8];
 #pragma unroll
-            for (int wd = 0; wd < kCntWords; ++wd) Wm.cnt[wd * 32 + lane] = 0u;
+            for (int i = 0; i < 8; ++i) {
+                // first lane: bins 4i ..; second: bins 32 + 4i .. = ranks 25 - 4i downwards
+                const uint32_t lo = i < 7 ? q[i] : q[7] | (top << 8);
+                const uint32_t hi = i < 6    ? __byte_perm(q[5 - (i < 6 ? i : 0)], q[6 - (i < 6 ? i : 0)], 0x2345)
+                                    : i == 6 ? __byte_perm(q[0], other, 0x7401)
+                                             : 0u;
+                v[i] = half ? hi : lo;
+            }
+            const int c = (lane - 1) >> 1;
+            if (lane < 1 || lane > 2 * kCellTW || cx0 + c >= Wc) return;
+            if (CELLS) {
+                uint4 *dst = reinterpret_cast<uint4 *>(
+                    atlas.lbp + ((int64_t)(L.cell_row + cy0 + r) * atlas.pitch + cx0 + c) * kLbpCellBytes + 32 * half);
+                dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
+                dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
+            } else {
+                const int64_t pl = atlas.lbp_plane;
+                uint8_t *dst = atlas.lbp + (int64_t)(L.cell_row + cy0 + r) * atlas.pitch + cx0 + c + 32 * half * pl;
+#pragma unroll
+                for (int i = 0; i < 32; ++i, dst += pl)
+                    if (i < 27 || !half) *dst = (uint8_t)(v[i >> 2] >> (8 * (i & 3)));
+            }
         };
 
         // ---- HOG of cell row r = band - 1 is final: write it, recycle its slots
@@ -433,44 +527,44 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
             if (!(need(band - 1) || need(band))) {
                 if (walked_prev) {  // recycle row band - 1's slots and counters
                     emit(band, false);
-                    if (kLbp) emit_lbp(band, false);
                 }
                 have = false;
                 walked_prev = false;
                 continue;
             }
+            // rows outside the cell grid: the first half of the level's first band and the
+            // second half of its last one are not walked
+            const int i0 = cy0 + band == 0 ? 2 : 0, i1 = cy0 + band == Hc ? 2 : 4;
             if (!have) {
                 uint32_t w[3];
-                fetch(yb - 1, w);
+                fetch(yb + 2 * i0 - 1, w);
                 ra = mkrow(w);
-                fetch(yb, w);
+                fetch(yb + 2 * i0, w);
                 rb = mkrow(w);
-                fetch(yb + 1, p0);
-                fetch(yb + 2, p1);
+                fetch(yb + 2 * i0 + 1, p0);
+                fetch(yb + 2 * i0 + 2, p1);
             }
             const bool pf = band + 1 <= nb && (need(band) || need(band + 1));
             const int ringA = (band + 1) & 1;
-            const int dB = (ringA ? -1 : 1) * kRingStride;  // floats from row band - 1's slots to row band's
+            const uint32_t dB = (ringA ? -4 : 4) * kRingStride;  // bytes from row band - 1's slots to row band's
             uint32_t va[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) va[j] = vb[j] + (uint32_t)(ringA * kRingStride);
+            for (int j = 0; j < 4; ++j) va[j] = vb[j] + 4u * (uint32_t)(ringA * kRingStride);
+            float wa = (7.5f - 2 * i0) * 0.125f;  // weight of cell row band - 1 in band row k: (7.5 - k) / 8
 #pragma unroll 1
-            for (int i = 0; i < 4; ++i) {
+            for (int i = i0; i < i1; ++i) {
                 const Row c0 = mkrow(p0), c1 = mkrow(p1);
                 if (i < 3 || pf) {
                     fetch(yb + 3 + 2 * i, p0);
                     fetch(yb + 4 + 2 * i, p1);
                 }
-                // band rows k = 2i, 2i + 1: weights (7.5 - k) / 8 and (k + 0.5) / 8;
-                // LBP cell row band - 1 for k < 4, band for k >= 4
-                const float wa0 = (7.5f - 2 * i) * 0.125f;
-                const int y = yb + 2 * i;
-                const bool v0 = y >= 0 && y < gridH, v1 = y + 1 >= 0 && y + 1 < gridH;
-                pixel_row(ra, rb, c0, v0 ? wa0 : 0.f, v0 ? 1.f - wa0 : 0.f, va, dB, v0);
-                pixel_row(rb, c0, c1, v1 ? wa0 - 0.125f : 0.f, v1 ? 1.125f - wa0 : 0.f, va, dB, v1);
+                // band rows 2i, 2i + 1; LBP cell row band - 1 for rows < 4, band for the others
+                pixel_row(ra, rb, c0, wa, 1.f - wa, va, dB);
+                pixel_row(rb, c0, c1, wa - 0.125f, 1.125f - wa, va, dB);
                 ra = c0;
                 rb = c1;
-                if (kLbp && i == 1) emit_lbp(band, true);
+                wa -= 0.25f;
+                if (kLbp && i == 1) emit_lbp(band);
             }
             emit(band, true);
             have = pf;
@@ -481,7 +575,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
 }
 
 using StripFn = void (*)(const LevelDesc *, const uint8_t *, CellAtlas, const StripItem *, int, int *,
-                         const uint8_t *, const uint32_t *);
+                         const uint32_t *);
 // [feature set][cell-major LBP counts]; without LBP the layout does not matter
 const StripFn kStripFns[3][2] = {{k_cells_warp<kFeatHog | kFeatLbp, false>, k_cells_warp<kFeatHog | kFeatLbp, true>},
                                  {k_cells_warp<kFeatHog, false>, k_cells_warp<kFeatHog, false>},
@@ -506,14 +600,14 @@ cudaError_t init_cells_warp() {
 
 cudaError_t launch_cells_warp(cudaStream_t s, const LevelDesc *d_levels, const uint8_t *pyr, CellAtlas atlas,
                               const StripItem *d_items, int n_items, int *d_queue, int sm_count,
-                              const uint8_t *d_lbp_map, const uint32_t *c_flag, int feat) {
+                              const uint32_t *c_flag, int feat) {
     if (n_items <= 0) return cudaSuccess;
     // resident CTAs: 4 per SM (shared memory); the warps share the strip queue. A
     // small plan gets one CTA per strip, so that its warps spread over the SMs.
     static_assert(kWarps * 4 == kStripWarpsPerSm, "resident warps per SM");
     const int grid = std::min(n_items, 4 * sm_count);
     kStripFns[strip_fn_index(feat)][atlas.lbp_cells != 0]<<<grid, kWarps * 32, sizeof(StripSmem), s>>>(
-        d_levels, pyr, atlas, d_items, n_items, d_queue, d_lbp_map, c_flag);
+        d_levels, pyr, atlas, d_items, n_items, d_queue, c_flag);
     return cudaGetLastError();
 }
 

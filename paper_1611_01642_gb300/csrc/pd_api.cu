@@ -872,7 +872,7 @@ cudaError_t launch_cell_stage(pd_handle *h, cudaStream_t s, const LevelDesc *dl,
     const cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
     return launch_cells_warp(s, dl, pyr, atlas, dptr<StripItem>(h, o.strips), (int)p.strips.size(), queue,
-                             h->sm_count, h->d_lbp_map, c_flag, feat);
+                             h->sm_count, c_flag, feat);
 }
 
 }  // namespace

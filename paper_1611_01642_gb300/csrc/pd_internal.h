@@ -136,7 +136,7 @@ cudaError_t init_cells_warp();
 // Persistent warps over a strip queue (*d_queue must be 0 at launch).
 cudaError_t launch_cells_warp(cudaStream_t s, const LevelDesc *d_levels, const uint8_t *pyr, CellAtlas atlas,
                               const StripItem *d_items, int n_items, int *d_queue, int sm_count,
-                              const uint8_t *d_lbp_map, const uint32_t *c_flag, int feat);
+                              const uint32_t *c_flag, int feat);
 cudaError_t launch_proposal_flags(cudaStream_t s, const LevelDesc *d_levels, const SvmItem *d_items, int n_items,
                                   const float *logits, float tau, uint32_t *s_flag, uint32_t *c_flag);
 cudaError_t launch_svm(cudaStream_t s, const CUtensorMap *hog_maps, const CUtensorMap *lbp_maps,
