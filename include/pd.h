@@ -387,11 +387,11 @@ int pd_logits(const pd_handle *h, const float **d_logits, int64_t *total);
  * fixed memory budget -- and so cannot create a pd_handle (pd_create calls
  * cudaMalloc). It computes exactly what pd_nms_maps computes, with the
  * threshold, IoU and caps passed as arguments, and needs no handle.
- * The scratch memory it needs (level descriptors and the decoded box of
- * every candidate) is one static array inside the library, about 270 KB,
- * that every GPU which loads the library holds until the process exits; it
- * limits a call to max_candidates <= 16384 and n_levels <= PD_MAX_LEVELS
- * (larger values, or max_boxes > 16384, return PD_EINVAL). The caller passes inputs and outputs as
+ * The scratch memory it needs (level descriptors) is one static array
+ * inside the library, about 13 KB, that every GPU which loads the library
+ * holds until the process exits; without a handle's scratch a call is
+ * limited to max_candidates <= 16384 and n_levels <= PD_MAX_LEVELS (larger
+ * values, or max_boxes > 16384, return PD_EINVAL). The caller passes inputs and outputs as
  * for pd_nms_maps: d_scores, d_boxes (cap max_boxes) and d_counts (kept,
  * candidates; a candidate overflow writes 0 and -candidates). Every call
  * looks up the array's device address on the current device and sets the

@@ -2,44 +2,53 @@
 // host in the paper; greedy IoU suppression here, on the device).
 //
 // One CTA (1024 threads) per frame, or a thread-block cluster of 2-8 CTAs
-// that share its collection, large sorts and suppression passes when the
-// batch leaves SMs free. A batch of more frames than clusters that fit on the
-// GPU at once runs on persistent clusters that draw frames from a ticket
-// queue, most candidates first (a counting kernel and a one-CTA sort set the
-// order), so the heaviest frames do not start last. Per frame:
-//  1. collects every window of every level with score > threshold into a
-//     shared-memory key list (64-bit keys: the float score mapped to an
-//     order-reversing integer in the high word, level/wy/wx in the low word,
-//     so ascending keys = score descending, then level, wy, wx ascending);
-//     with a candidate cap above 16,384 the key list lives in the frame's
-//     global scratch instead (same steps, slower sort);
-//  2. sorts the keys: a bitonic sort in shared memory, or, for caps above
-//     16,384, bitonic sorts of 16,384-key chunks in shared memory followed by
-//     merge passes over the global key list (each thread merges its slice
-//     of outputs after locating it by binary search on the two runs);
-//  3. decodes every candidate's box once (exactly rounded float division)
-//     into shared memory (over the no longer needed key array, whose keys
-//     move to a per-frame global scratch array) or, for very many
-//     candidates, into that global scratch;
-//  4. walks the candidates in order in batches of the next 64 not yet
+// that share its collection and suppression passes when the batch leaves SMs
+// free. A batch of more frames than clusters that fit on the GPU at once runs
+// on persistent clusters that draw frames from a ticket queue, most candidates
+// first (a counting kernel and a one-CTA sort set the order), so the heaviest
+// frames do not start last. Per frame:
+//  1. every CTA of the cluster collects a share of the windows with score >
+//     threshold into a list of its own: 64-bit keys (the float score mapped to
+//     an order-reversing integer in the high word, level/wy/wx in the low
+//     word, so ascending keys = score descending, then level, wy, wx
+//     ascending) in its shared memory or, with a candidate cap above 16,384,
+//     in its part of the frame's global scratch. The maps of a frame lie back
+//     to back, so the scan is flat and all its loads are independent;
+//  2. the best keys, at most kSeg of them (all of them, or those below a bound
+//     found by a radix select over the cluster's lists), go to the leader,
+//     which sorts them (bitonic, in registers and shuffles up to 64 keys per
+//     warp) and decodes their boxes (exactly rounded float division);
+//  3. the leader walks this segment in batches of the next 64 not yet
 //     suppressed: all threads compute the batch's pairwise suppression bits,
-//     warp 0 resolves the batch (kept iff no kept earlier member suppresses
-//     it), and all threads then suppress the later candidates against the
-//     batch's kept members (their boxes staged in shared memory). This
-//     takes the same decisions as the one-at-a-time greedy walk (candidates
-//     between batch members are already suppressed).
-// The IoU test first evaluates the IoU in float. For boxes of this detector
-// (width >= 64, height >= 128, coordinates < 8192) the float value is within
-// 7e-5 of the exact one: each coordinate sum or difference is off by at most
-// 3 float roundings of values < 8192 (1.5e-3 px), which moves the
-// intersection by at most (w + h) * 1.5e-3 px^2 and the IoU by at most
-// 1.5e-3 * (1/w + 1/h) <= 3.5e-5 through the intersection and as much again
-// through the union. So a float IoU more than 2e-4 away from the threshold
-// decides; otherwise the IoU is recomputed in double precision with
-// explicitly rounded operations (no FMA contraction), which is the exact IEEE
-// evaluation of the definition. Decisions are therefore the same as those of
-// a plain double-precision implementation, and the slow double path runs
-// only for the rare pairs in the band.
+//     every warp resolves the batch (kept iff no kept earlier member
+//     suppresses it) and suppresses its share of the segment against the
+//     batch's kept members. This takes the same decisions as the
+//     one-at-a-time greedy walk (candidates between batch members are already
+//     suppressed);
+//  4. if candidates remain, every CTA drops from its list the segment's keys
+//     and those that the segment's kept boxes suppress, and the next segment
+//     is taken. A later segment's candidates have met every kept box before
+//     them, so the decisions stay those of the sequential walk.
+// What bounds it: the latency of the one frame with the most candidates: about
+// 6,000 cycles per batch of the walk, 15,000 to collect, 4,000 to 8,000 to sort.
+// A scan level by level, a bitonic sort of all candidates and a cluster-wide
+// pass over all of them after every batch took 80 us where this takes 39 (one
+// 1242x375 frame, 1,884 candidates), 317 against 152 (8 frames of 40 levels, up
+// to 10,363 candidates), 117 against 78 (64 frames of 1242x375).
+// The IoU test first evaluates inter - thr * union in float. A coordinate sum or
+// difference is off by at most 3 float roundings of values up to m = max(W, H)
+// (eps = 3 m 2^-24), which moves the intersection by at most (w + h) eps and the
+// IoU by at most eps (1 / w + 1 / h) through the intersection and as much again
+// through the union (1.7e-5 for 64x128 windows of a 2048-pixel frame). So a float
+// IoU further from the threshold than twice that bound for the frame's smallest
+// window (plus 1e-6 for the products)
+// decides. Otherwise the sign of inter - thr * union is taken from pairs of
+// floats, good to 1e-10 of the union, and only nearer pairs go to double
+// precision with explicitly rounded operations (no FMA contraction), the exact
+// IEEE evaluation of the definition. Decisions are therefore the same as those
+// of a plain double-precision implementation. (Double precision runs at two
+// lanes per SM here: a call holds up the other warps' calls for over a
+// thousand cycles, and one pair in a thousand that overlap is in the band.)
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -50,8 +59,11 @@ namespace pd {
 namespace {
 
 constexpr int kThreads = 1024;
-constexpr int kMaxCandidates = 16384;     // keys + flags + kept list fit in shared memory
-constexpr int kMaxCandidatesBig = 65536;  // keys in global scratch
+constexpr int kMaxCandidates = 16384;     // a CTA's list fits in shared memory
+constexpr int kMaxCandidatesBig = 65536;  // lists in global scratch
+constexpr int kSeg = 2048;                // candidates sorted and walked at a time
+constexpr int kDigit = 11;                // radix select: bits per round
+constexpr int kHist = 1 << kDigit;
 constexpr int kMaxBoxes = 16384;
 constexpr int kBatch = 64;                // greedy walk: candidates resolved per block-wide step
 constexpr int kGrid = 32;                 // culling grid: kGrid x kGrid cells over the frame
@@ -61,6 +73,8 @@ static_assert(nms_sched_ints(1) == 2 + kCountBlocks,
 constexpr int kOrderMax = 16384;          // frames the order kernel sorts (more: drawn in index order)
 static_assert(kThreads == 16 * kBatch, "pairwise matrix: 16 threads per batch member");
 static_assert(kThreads == kGrid * kGrid, "one culling cell per thread");
+static_assert(kSeg == 2 * kThreads && kSeg / 32 == 64, "two segment entries per thread, two flag words per lane");
+static_assert(kHist == 2 * kThreads, "two digits per thread");
 
 __device__ __forceinline__ unsigned long long make_key(float s, int level, int wy, int wx) {
     const uint32_t u = __float_as_uint(s);
@@ -69,8 +83,6 @@ __device__ __forceinline__ unsigned long long make_key(float s, int level, int w
            (uint32_t)((level << 24) | (wy << 12) | wx);
 }
 
-__device__ __forceinline__ bool suppresses(const float4 &a, const float4 &b, float thr);
-
 __device__ __noinline__ void decode_f64(long long nx, long long ny, int W, int H, int2 d, pd_box &b) {
     b.x = (float)__ddiv_rn((double)nx, (double)d.x);
     b.y = (float)__ddiv_rn((double)ny, (double)d.y);
@@ -78,16 +90,20 @@ __device__ __noinline__ void decode_f64(long long nx, long long ny, int W, int H
     b.h = (float)__ddiv_rn(128.0 * H, (double)d.y);
 }
 
+// Score of a key's high word.
+__device__ __forceinline__ float key_score(uint32_t hi) {
+    const uint32_t ord = ~hi;
+    return __uint_as_float((ord & 0x80000000u) ? (ord ^ 0x80000000u) : ~ord);
+}
+
 // Box of a key. x = 8*wx*W/Wk etc. are quotients of integers below 2^24, so
 // the correctly rounded float quotient (__fdiv_rn) equals the double quotient
 // rounded to float (a quotient of two such integers cannot lie within 2^-49
 // of a float rounding midpoint without being on it): no double arithmetic.
 __device__ __forceinline__ pd_box decode(unsigned long long key, int W, int H, const int2 *wkhk) {
-    const uint32_t hi = (uint32_t)(key >> 32), lo = (uint32_t)key;
-    const uint32_t ord = ~hi;
-    const uint32_t u = (ord & 0x80000000u) ? (ord ^ 0x80000000u) : ~ord;
+    const uint32_t lo = (uint32_t)key;
     pd_box b;
-    b.score = __uint_as_float(u);
+    b.score = key_score((uint32_t)(key >> 32));
     b.level = (int)(lo >> 24);
     b.wy = (int)((lo >> 12) & 4095);
     b.wx = (int)(lo & 4095);
@@ -129,20 +145,72 @@ __device__ __noinline__ double iou4(const float4 &a, const float4 &b) {
     return iou(x, y);
 }
 
-__device__ __forceinline__ bool suppresses(const float4 &a, const float4 &b, float thr) {
-    const float iw = fminf(a.x + a.z, b.x + b.z) - fmaxf(a.x, b.x);
-    const float ih = fminf(a.y + a.w, b.y + b.w) - fmaxf(a.y, b.y);
-    float fi = 0.f;
-    if (iw > 0.f && ih > 0.f) {
-        const float inter = iw * ih;
-        fi = __fdividef(inter, a.z * a.w + b.z * b.w - inter);
-    }
-    if (fi < thr - 2e-4f) return false;
-    if (fi > thr + 2e-4f) return true;
-    return iou4(a, b) > (double)thr;
+// IoU > thr by pairs of floats (about 46 bits): 1 yes, 0 no, -1 too near to
+// tell. The edges x + w are exact pairs; the sign of inter - thr * union is
+// taken as certain when it is more than 1e-10 of the union away from 0 (each
+// step errs by at most a few 2^-46 of it).
+struct Pair {
+    float h, l;
+};
+__device__ __forceinline__ Pair two_sum(float a, float b) {
+    const float s = a + b, t = s - a;
+    return {s, (a - (s - t)) + (b - t)};
+}
+__device__ __forceinline__ Pair renorm(float h, float l) {
+    const float s = h + l;
+    return {s, l - (s - h)};
+}
+__device__ __forceinline__ Pair two_prod(float a, float b) {
+    const float p = a * b;
+    return {p, fmaf(a, b, -p)};
+}
+__device__ __forceinline__ Pair add(const Pair &a, const Pair &b) {
+    const Pair s = two_sum(a.h, b.h), t = two_sum(a.l, b.l);
+    const Pair v = renorm(s.h, s.l + t.h);
+    return renorm(v.h, v.l + t.l);
+}
+__device__ __forceinline__ Pair mul(const Pair &a, const Pair &b) {
+    const Pair p = two_prod(a.h, b.h);
+    return renorm(p.h, p.l + (a.h * b.l + a.l * b.h));
+}
+__device__ __forceinline__ Pair extent(float a0, float aw, float b0, float bw) {
+    const Pair a = two_sum(a0, aw), b = two_sum(b0, bw);
+    const bool less = a.h < b.h || (a.h == b.h && a.l < b.l);
+    return add(less ? a : b, {-fmaxf(a0, b0), 0.f});
+}
+__device__ __noinline__ int iou_above(const float4 &a, const float4 &b, float thr) {
+    const Pair iw = extent(a.x, a.z, b.x, b.z), ih = extent(a.y, a.w, b.y, b.w);
+    if (iw.h <= 0.f || ih.h <= 0.f) return 0;
+    const Pair inter = mul(iw, ih);
+    const Pair ua = add(add(two_prod(a.z, a.w), two_prod(b.z, b.w)), {-inter.h, -inter.l});
+    const Pair d = add(inter, mul({-thr, 0.f}, ua));
+    if (fabsf(d.h) <= 1e-10f * ua.h) return -1;
+    return d.h > 0.f ? 1 : 0;
 }
 
-constexpr int kSortChunk = 16384;  // keys per shared-memory chunk of the large-cap sort (128 KB)
+// A box as its edges x0, y0, x1, y1 and area, for the float test.
+struct Edges {
+    float4 e;
+    float area;
+};
+__device__ __forceinline__ Edges edges_of(const float4 &b) {
+    return {make_float4(b.x, b.y, b.x + b.z, b.y + b.w), b.z * b.w};
+}
+__device__ __noinline__ bool suppresses_exact(float4 a, float4 b, float thr) {
+    const int p = iou_above(a, b, thr);
+    return p >= 0 ? p != 0 : iou4(a, b) > (double)thr;
+}
+// IoU > thr of boxes a and b (given also as edges), decided in float unless
+// the IoU is within `band` of thr.
+__device__ __forceinline__ bool suppresses(const Edges &a, const float4 &abox, const Edges &b, const float4 &bbox,
+                                           float thr, float band) {
+    const float iw = fmaxf(fminf(a.e.z, b.e.z) - fmaxf(a.e.x, b.e.x), 0.f);
+    const float inter = iw * fmaxf(fminf(a.e.w, b.e.w) - fmaxf(a.e.y, b.e.y), 0.f);
+    const float ua = (a.area + b.area) - inter;
+    const float d = fmaf(-thr, ua, inter);
+    if (fabsf(d) > band * ua) return d > 0.f;
+    return suppresses_exact(abox, bbox, thr);
+}
 
 // Ascending bitonic sort of m = R * kThreads keys in shared memory k, with
 // each thread holding the R consecutive keys [tid R, tid R + R) in registers:
@@ -294,64 +362,111 @@ __device__ __forceinline__ void bitonic_sort_smem(unsigned long long *k, int m, 
     }
 }
 
-// Large caps: keys[0, np) (np a power of two >= n, padded with ~0) sorted
-// ascending by the nr CTAs of a frame's cluster (rank = this CTA): chunks of
-// up to kSortChunk keys sorted in each CTA's shared memory `sm` (chunk c by
-// rank c mod nr), then merge passes doubling the run length, ping-ponging
-// through `tmp` (np keys), each of the nr * kThreads threads merging its
-// slice of the output; the result ends in keys. csync is the cluster-wide
-// barrier (the keys are in global memory).
-template <class Sync>
-__device__ void sort_large(unsigned long long *keys, unsigned long long *tmp, int np, unsigned long long *sm,
-                           int tid, int rank, int nr, Sync &&csync) {
-    const int C = np < kSortChunk ? np : kSortChunk;
-    for (int c0 = rank * C; c0 < np; c0 += nr * C) {
-        for (int i = tid; i < C; i += kThreads) sm[i] = keys[c0 + i];
+// A CTA's shared memory beside its key list.
+struct NmsSmem {
+    unsigned long long key[kSeg];               // the segment (leader)
+    float4 box[kSeg];
+    unsigned long long cmask[kGrid * kGrid];    // culling grid: kept boxes covering each cell
+    int hist[kHist];
+    int kept[kSeg];                             // the segment's kept entries, in order
+    float4 bbx[kBatch];                         // the batch's boxes; a chunk of kept boxes
+    Edges bed[kBatch];                          // the same as edges
+    unsigned long long bcol[kBatch];            // member b: bit a set iff a < b and a suppresses b
+    unsigned long long lohi[2][32];             // per warp: least and greatest key
+    int4 krect[kBatch];                         // kept boxes' cell ranges x0, x1, y0, y1
+    int2 wkhk[PD_MAX_LEVELS];                   // level sizes of this frame
+    int first[PD_MAX_LEVELS];                   // its levels' first windows
+    int cols[PD_MAX_LEVELS];
+    int batch[kBatch];
+    unsigned short rest[kSeg];                  // alive entries after the batch, in order
+    uint32_t alive[kSeg / 32];
+    int wsum[32];
+    unsigned long long lo, hi;                  // least and greatest key of this CTA's list
+    uint32_t keep[2];                           // the batch's kept members
+    int n_list, n_seg, n_kept_seg, done, frame, digit, below;
+};
+
+__device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
+__device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) { return a < b ? b : a; }
+
+// Sorts the segment's m <= kSeg distinct keys ascending. Up to 256 keys by
+// counting the smaller ones, four threads per key. More by the score's place
+// among kHist equal parts of the segment's range of scores (monotone in the
+// key: each float step rounds monotonically): a histogram gives every part its
+// place, and a key's place among the few of its part is again the number of
+// smaller ones. Where a part holds more than kCrowd keys (scores that hardly
+// differ, infinities), by the bitonic network, whose 66 steps for 2,048 keys
+// take 26,000 cycles.
+constexpr int kCrowd = 64;
+__device__ __forceinline__ void sort_segment(NmsSmem &S, int m, int tid) {
+    unsigned long long *k = S.key;
+    const int lane = tid & 31, warp = tid >> 5;
+    if (m <= 256) {
+        const int i = tid >> 2, q = tid & 3;
+        const unsigned long long key = i < m ? k[i] : ~0ull;
+        int c = 0;
+        for (int j = q; j < m; j += 4) c += k[j] < key;
+        c += __shfl_xor_sync(0xffffffffu, c, 1);
+        c += __shfl_xor_sync(0xffffffffu, c, 2);
         __syncthreads();
-        bitonic_sort_smem(sm, C, tid);
-        for (int i = tid; i < C; i += kThreads) keys[c0 + i] = sm[i];
+        if (i < m && q == 0) k[c] = key;
         __syncthreads();
+        return;
     }
-    csync();
-    unsigned long long *src = keys, *dst = tmp;
-    const int g = rank * kThreads + tid;
-    const int per = np / (nr * kThreads);  // outputs per thread (np >= 2 C here, so per divides every pair)
-    for (int w = C; w < np; w <<= 1) {
-        const int o0 = g * per;
-        const int base = o0 & ~(2 * w - 1), d = o0 - base;
-        const unsigned long long *A = src + base, *B = src + base + w;
-        // i = keys taken from A among the pair's first d outputs (A first on ties)
-        int lo = d > w ? d - w : 0, hi = d < w ? d : w;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (A[mid] <= B[d - 1 - mid])
-                lo = mid + 1;
-            else
-                hi = mid;
-        }
-        int i = lo, j = d - lo;
-        unsigned long long a = i < w ? A[i] : ~0ull, b = j < w ? B[j] : ~0ull;
-        for (int k = 0; k < per; ++k) {
-            const bool take_a = j >= w || (i < w && a <= b);
-            if (take_a) {
-                dst[o0 + k] = a;
-                ++i;
-                a = i < w ? A[i] : ~0ull;
-            } else {
-                dst[o0 + k] = b;
-                ++j;
-                b = j < w ? B[j] : ~0ull;
-            }
-        }
-        csync();
-        unsigned long long *t = src;
-        src = dst;
-        dst = t;
+    const bool has0 = tid < m, has1 = tid + kThreads < m;
+    const unsigned long long k0 = has0 ? k[tid] : 0ull, k1 = has1 ? k[tid + kThreads] : 0ull;
+    // least and greatest high words: the greatest and least score
+    const uint32_t h0 = (uint32_t)(k0 >> 32), h1 = (uint32_t)(k1 >> 32);
+    uint32_t mn = __reduce_min_sync(0xffffffffu, min(has0 ? h0 : ~0u, has1 ? h1 : ~0u));
+    uint32_t mx = __reduce_max_sync(0xffffffffu, max(h0, h1));
+    if (lane == 0) S.lohi[0][warp] = ((unsigned long long)mn << 32) | mx;
+    S.hist[2 * tid] = S.hist[2 * tid + 1] = 0;
+    __syncthreads();
+    mn = __reduce_min_sync(0xffffffffu, (uint32_t)(S.lohi[0][lane] >> 32));
+    mx = __reduce_max_sync(0xffffffffu, (uint32_t)S.lohi[0][lane]);
+    const float best = key_score(mn), range = best - key_score(mx);
+    const float scale = range > 0.f && range <= 3e38f ? (float)(kHist - 1) / range : 0.f;
+    auto digit = [&](uint32_t h) { return min((int)((best - key_score(h)) * scale), kHist - 1); };
+    // (scale 0: every key in part 0, also where the product is not a number, and the network sorts)
+    const int d0 = scale > 0.f && has0 ? digit(h0) : 0, d1 = scale > 0.f && has1 ? digit(h1) : 0;
+    const int r0 = has0 ? atomicAdd(&S.hist[d0], 1) : 0, r1 = has1 ? atomicAdd(&S.hist[d1], 1) : 0;
+    __syncthreads();
+    const int c0 = S.hist[2 * tid], c1 = S.hist[2 * tid + 1];
+    if (__syncthreads_or(c0 > kCrowd || c1 > kCrowd)) {
+        const int np = m <= kThreads ? kThreads : 2 * kThreads;
+        for (int i = m + tid; i < np; i += kThreads) k[i] = ~0ull;
+        __syncthreads();
+        if (np == kThreads) bitonic_hybrid<1>(k, 0, np, tid);
+        else bitonic_hybrid<2>(k, 0, np, tid);
+        return;
     }
-    if (src != keys) {
-        for (int i = g; i < np; i += nr * kThreads) keys[i] = src[i];
-        csync();
+    int incl = c0 + c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += a;
     }
+    if (lane == 31) S.wsum[warp] = incl;
+    __syncthreads();
+    int w = lane < warp ? S.wsum[lane] : 0;
+    w = __reduce_add_sync(0xffffffffu, w);
+    const int start = w + incl - c0 - c1;
+    S.hist[2 * tid] = start;  // a digit's first place; the next one's ends it
+    S.hist[2 * tid + 1] = start + c0;
+    __syncthreads();
+    unsigned long long *t = reinterpret_cast<unsigned long long *>(S.box);  // the boxes come later
+    if (has0) t[S.hist[d0] + r0] = k0;
+    if (has1) t[S.hist[d1] + r1] = k1;
+    __syncthreads();
+    auto place = [&](unsigned long long key, int d) {
+        const int a = S.hist[d], e = d + 1 < kHist ? S.hist[d + 1] : m;
+        int c = a;
+        for (int j = a; j < e; ++j) c += t[j] < key;
+        k[c] = key;
+    };
+    if (has0) place(k0, d0);
+    if (has1) place(k1, d1);
+    __syncthreads();
 }
 
 __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ frames,
@@ -361,374 +476,480 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
                                                   pd_box *__restrict__ boxes, int max_boxes,
                                                   int32_t *__restrict__ counts, int n_frames,
                                                   const int *__restrict__ order, int *__restrict__ queue) {
-    extern __shared__ unsigned long long skeys[];  // [cap_pow2] keys (small caps), cap bytes of flags, kept list
-    __shared__ int n_cand;
-    __shared__ int2 wkhk[PD_MAX_LEVELS];  // level sizes of this frame
-    __shared__ int s_done, s_bx_smem;  // leader's state: walk over; boxes on chip
-    __shared__ int s_frame;            // the frame this cluster works on (-1: none left)
-    // A frame is one cluster of C CTAs (C = 1 without a cluster launch). Every
-    // rank collects a share of the frame's candidates into the leader's list;
-    // with large caps (keys in global memory) every rank also sorts and
-    // decodes a share. Rank 0, the leader, sorts small lists and picks and
-    // resolves the batches exactly as a lone CTA would; every rank takes a
-    // 1/C share of each suppression pass, reading the leader's flags and
-    // boxes through distributed shared memory. All ranks pass the same
-    // cluster barriers: what comes next is read from the leader after one.
+    extern __shared__ __align__(16) unsigned char nms_raw[];
+    NmsSmem &S = *reinterpret_cast<NmsSmem *>(nms_raw);
+    // A frame is one cluster of C CTAs (C = 1 without a cluster launch); rank 0
+    // leads. All ranks pass the same cluster barriers: what comes next follows
+    // from values that all of them read after one.
     // Without a queue, cluster i takes frame i. With one (more frames than
     // clusters that fit on the GPU), the clusters are persistent: the leader
     // draws the next ticket, takes that frame of `order` (heaviest first)
-    // and writes it into every rank's s_frame before the barrier that starts
+    // and writes it into every rank's S.frame before the barrier that starts
     // the frame, so all ranks work on the same frame and stop together.
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const bool leader = rank == 0;
-    const int tid = threadIdx.x;
-    int cap_pow2 = 1;
-    while (cap_pow2 < cap) cap_pow2 <<= 1;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool big = cap > kMaxCandidates;
-    if (queue) cluster.sync();  // every CTA of the cluster runs before the leader writes into it
+    NmsSmem &Lead = *cluster.map_shared_rank(&S, 0);
+    auto csync = [&] {
+        if (C > 1) cluster.sync();
+        else __syncthreads();
+    };
+    const bool cull = iou_thr >= 0.5f;
+    csync();  // every CTA of the cluster runs before the leader writes into it
     for (int pass = 0;; ++pass) {
         if (queue) {
             if (leader && tid == 0) {
                 const int t = atomicAdd(queue, 1);
                 const int fr = t < n_frames ? (order ? order[t] : t) : -1;
-                for (int r = 0; r < C; ++r) *cluster.map_shared_rank(&s_frame, r) = fr;
-                n_cand = 0;
+                for (int r = 0; r < C; ++r) cluster.map_shared_rank(&S, r)->frame = fr;
             }
         } else if (tid == 0) {
-            s_frame = pass == 0 ? (int)(blockIdx.x / C) : -1;
-            if (leader) n_cand = 0;
+            S.frame = pass == 0 ? (int)(blockIdx.x / C) : -1;
         }
-        cluster.sync();  // every rank knows the frame; the leader's counter is zero
-        const int f = s_frame;
+        if (tid == 0) S.n_list = S.n_seg = 0;
+        csync();  // every rank knows the frame
+        const int f = S.frame;
         if (f < 0) return;  // the same value in every rank: all leave together
-        const FrameDesc fd = frames[f];
-        float4 *gbx = scratch + (size_t)f * nms_scratch_float4s(cap);
-        unsigned long long *keys = big ? reinterpret_cast<unsigned long long *>(gbx + cap) : skeys;
-        uint8_t *supp = reinterpret_cast<uint8_t *>(big ? skeys : skeys + cap_pow2);
-        const float4 *bx = gbx;
-        const unsigned long long *ksrc = keys;
-        for (int k = tid; k < fd.n_levels; k += kThreads) {
-            const LevelDesc L = levels[fd.first_level + k];
-            wkhk[k] = make_int2(L.Wk, L.Hk);
+        const FrameDesc &fd = frames[f];
+        const int W = fd.W, H = fd.H, nl = fd.n_levels;
+        const LevelDesc *lv = levels + fd.first_level;
+        int n_win = 0;
+        int64_t base = 0;
+        if (nl > 0) {
+            base = lv[0].score_off;
+            n_win = (int)(lv[nl - 1].score_off + (int64_t)lv[nl - 1].rows * lv[nl - 1].cols - base);
         }
-        {
-            // every rank scans its share of the windows (every C-th run of
-            // kThreads * kUnroll of a level) and appends to the leader's list
-            int *cnt = leader ? &n_cand : cluster.map_shared_rank(&n_cand, 0);
-            unsigned long long *kw = big ? keys : leader ? skeys : cluster.map_shared_rank(skeys, 0);
-            for (int k = 0; k < fd.n_levels; ++k) {
-                const LevelDesc L = levels[fd.first_level + k];
-                const int n = L.rows * L.cols;
-                const float *sc = scores + L.score_off;
-                // warp-aggregated appends; kUnroll independent loads per thread are in
-                // flight before any of them is used (the scan is latency-bound otherwise)
-                constexpr int kUnroll = 8;
-                for (int i0 = rank * kThreads * kUnroll; i0 < n; i0 += C * kThreads * kUnroll) {
-                    float sv[kUnroll];
-    #pragma unroll
-                    for (int u = 0; u < kUnroll; ++u) {
-                        const int i = i0 + u * kThreads + tid;
-                        sv[u] = i < n ? __ldg(sc + i) : 0.f;
-                    }
-    #pragma unroll
-                    for (int u = 0; u < kUnroll; ++u) {
-                        const int i = i0 + u * kThreads + tid;
-                        if (i0 + u * kThreads >= n) break;  // block-uniform
-                        const float s = sv[u];
-                        const bool hit = i < n && s > threshold;
-                        const unsigned m = __ballot_sync(0xffffffffu, hit);
-                        int base = 0;
-                        if ((tid & 31) == 0 && m) base = atomicAdd(cnt, __popc(m));
-                        base = __shfl_sync(0xffffffffu, base, 0);
-                        if (hit) {
-                            const int idx = base + __popc(m & ((1u << (tid & 31)) - 1u));
-                            if (idx < cap) {
-                                const int wy = i / L.cols;
-                                kw[idx] = make_key(s, k, wy, i - wy * L.cols);
-                            }
-                        }
-                    }
-                }
-            }
-        }
-        cluster.sync();  // every rank's candidates are in
-        const int n = leader ? n_cand : *cluster.map_shared_rank(&n_cand, 0);
-        if (n > cap) {
-            if (leader && tid == 0) {
-                counts[2 * f] = 0;
-                counts[2 * f + 1] = -n;
-            }
-            cluster.sync();  // nobody moves on while another rank reads its shared memory
-            continue;
-        }
-        int np = 1;
-        while (np < n) np <<= 1;
-        if (big) {
-            // keys and boxes in global memory: every rank sorts and decodes a share
-            for (int i = n + rank * kThreads + tid; i < np; i += C * kThreads) keys[i] = ~0ull;
-            cluster.sync();
-            // the boxes region (cap float4s) is free until the decode below
-            sort_large(keys, reinterpret_cast<unsigned long long *>(gbx), np, skeys, tid, rank, C,
-                       [&] { cluster.sync(); });
-            for (int i = rank * kThreads + tid; i < n; i += C * kThreads) {
-                const pd_box b = decode(keys[i], fd.W, fd.H, wkhk);
-                gbx[i] = make_float4(b.x, b.y, b.w, b.h);
-            }
-            if (leader) {
-                for (int i = tid; i < n; i += kThreads) supp[i] = 0;
-                if (tid == 0) s_bx_smem = 0;
-            }
-        } else if (leader) {
-            for (int i = n + tid; i < np; i += kThreads) keys[i] = ~0ull;
-            __syncthreads();
-            bitonic_sort_smem(keys, np, tid);
-            for (int i = tid; i < n; i += kThreads) supp[i] = 0;
-            __syncthreads();
-            // Decoded boxes: in shared memory when they fit in the key region (the
-            // keys then move to the global scratch, where only kept ones are read
-            // again), otherwise in the global scratch. Each greedy pass reads every
-            // remaining box, so keeping them on chip shortens every pass.
-            if (2 * n <= cap_pow2) {
-                unsigned long long *gkeys = reinterpret_cast<unsigned long long *>(gbx);
-                for (int i = tid; i < n; i += kThreads) gkeys[i] = keys[i];
-                __syncthreads();
-                float4 *sbx = reinterpret_cast<float4 *>(keys);
-                for (int i = tid; i < n; i += kThreads) {  // each thread re-reads only its own writes
-                    const pd_box b = decode(gkeys[i], fd.W, fd.H, wkhk);
-                    sbx[i] = make_float4(b.x, b.y, b.w, b.h);
-                }
-                bx = sbx;
-                ksrc = gkeys;
-            } else {
-                for (int i = tid; i < n; i += kThreads) {
-                    const pd_box b = decode(keys[i], fd.W, fd.H, wkhk);
-                    gbx[i] = make_float4(b.x, b.y, b.w, b.h);
-                }
-            }
-            if (tid == 0) s_bx_smem = bx != gbx;
-        }
-        cluster.sync();  // the leader's candidates, flags and boxes are in place
-        // the flags and the boxes of the walk: the leader's own, or read remotely
-        uint8_t *fl = leader ? supp : cluster.map_shared_rank(supp, 0);
-        if (!leader && *cluster.map_shared_rank(&s_bx_smem, 0))
-            bx = cluster.map_shared_rank(reinterpret_cast<float4 *>(keys), 0);
-        // Greedy walk in batches. All threads find the next (up to) 64 candidates
-        // not yet suppressed, in order (1024 positions per round), and copy their
-        // boxes to shared memory; all threads compute the batch's pairwise
-        // suppression bits (4 pairs each); warp 0 resolves the members (a member
-        // is kept iff no kept member before it suppresses it: the candidates
-        // between members are already suppressed) and copies the kept boxes to
-        // shared memory; then every thread suppresses the later candidates against
-        // them. Same decisions as the sequential definition, with ~64x fewer
-        // block-wide barriers.
-        //
-        // Culling (IoU threshold >= 0.5): if IoU(A, B) > 0.5 then A's centre lies
-        // in B (were it outside B on one axis, A and B would overlap on at most
-        // half of A's extent there, so inter <= |A| / 2, and inter > (|A| + |B|)
-        // / 3 would need |B| < |A| / 2 while inter <= |B| needs |B| > |A| / 2).
-        // Each batch records, for every cell of a 32 x 32 grid over the frame,
-        // which of its kept boxes cover the cell (one cell of margin for
-        // rounding); a candidate is tested only against the kept boxes that cover
-        // its centre's cell (no test at all when none does).
-        __shared__ int batch[kBatch];
-        __shared__ float4 bbx[kBatch], kbx[kBatch];
-        __shared__ unsigned long long bcol[kBatch];  // member b: bit a set iff a < b and a suppresses b
-        __shared__ int n_batch, n_keep, kept_total, scan_pos;
-        __shared__ int wcnt[kThreads / 32];
-        __shared__ unsigned long long cmask[kGrid * kGrid];  // culling grid: kept boxes covering each cell
-        __shared__ int4 krect[kBatch];                       // kept boxes' cell ranges x0, x1, y0, y1
-        int *kept_idx = reinterpret_cast<int *>(supp + ((cap + 15) & ~15));
-        const int warp = tid >> 5, lane = tid & 31;
-        const bool cull = iou_thr >= 0.5f;
-        const float gsx = (float)kGrid / (float)fd.W, gsy = (float)kGrid / (float)fd.H;
-        if (tid == 0 && leader) {
-            kept_total = 0;
-            scan_pos = 0;
+        for (int k = tid; k < nl; k += kThreads) {
+            const LevelDesc &L = lv[k];
+            S.wkhk[k] = make_int2(L.Wk, L.Hk);
+            S.first[k] = (int)(L.score_off - base);
+            S.cols[k] = L.cols;
         }
         __syncthreads();
-        while (true) {
-            if (leader) {
-                // ---- the next batch: the first kBatch alive candidates at or after scan_pos
-                {
-                    int cnt = 0, pos = scan_pos;
-                    while (cnt < kBatch && pos < n) {
-                        const int j = pos + tid;
-                        const bool alive = j < n && !fl[j];
-                        const unsigned m = __ballot_sync(0xffffffffu, alive);
-                        if (lane == 0) wcnt[warp] = __popc(m);
-                        __syncthreads();
-                        int before = 0, total = 0;
-    #pragma unroll 8
-                        for (int w = 0; w < kThreads / 32; ++w) {
-                            const int c = wcnt[w];
-                            before += w < warp ? c : 0;
-                            total += c;
+        // the float test's band (see above): from the frame's size and its smallest window
+        int wk = 1, hk = 1;
+        for (int k = lane; k < nl; k += 32) {
+            wk = max(wk, S.wkhk[k].x);
+            hk = max(hk, S.wkhk[k].y);
+        }
+        wk = __reduce_max_sync(0xffffffffu, wk);
+        hk = __reduce_max_sync(0xffffffffu, hk);
+        const float band = 4.f * (3.f * 5.9604645e-8f * (float)max(W, H)) *
+                               ((float)wk / (64.f * (float)W) + (float)hk / (128.f * (float)H)) + 1e-6f;
+        unsigned long long *list = big ? reinterpret_cast<unsigned long long *>(scratch + (size_t)f * nms_scratch_float4s(cap))
+                                       : reinterpret_cast<unsigned long long *>(nms_raw + sizeof(NmsSmem));
+        // ---- 1. candidates: this rank's share of the windows (every C-th run of
+        // kThreads * kU), kU independent loads in flight; warp-aggregated appends.
+        // With lists in global memory a first scan counts, which gives every rank its part.
+        const float *sc = scores + base;
+        auto scan = [&](bool count_only) {
+            constexpr int kU = 4;
+            for (int i0 = rank * kThreads * kU; i0 < n_win; i0 += C * kThreads * kU) {
+                float v[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int i = i0 + u * kThreads + tid;
+                    v[u] = i < n_win ? __ldg(sc + i) : -INFINITY;
+                }
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int i = i0 + u * kThreads + tid;
+                    const bool hit = i < n_win && v[u] > threshold;
+                    const unsigned m = __ballot_sync(0xffffffffu, hit);
+                    if (!m) continue;
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(&S.n_list, __popc(m));
+                    if (count_only) continue;
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                    if (hit && (big || at < cap)) {
+                        int lo = 0, hi = nl - 1;  // the window's level: the last one that starts at or before it
+                        while (lo < hi) {
+                            const int mid = (lo + hi + 1) >> 1;
+                            if (S.first[mid] <= i) lo = mid;
+                            else hi = mid - 1;
                         }
-                        const int slot = cnt + before + __popc(m & ((1u << lane) - 1u));
-                        if (alive && slot < kBatch) {
-                            batch[slot] = j;
-                            bbx[slot] = bx[j];
-                            if (slot == kBatch - 1) scan_pos = j + 1;  // stop right after the last member
-                        }
-                        if (cnt + total < kBatch && tid == 0) scan_pos = min(pos + kThreads, n);
-                        cnt = min(cnt + total, kBatch);
-                        pos += kThreads;
-                        __syncthreads();  // wcnt reused by the next round; scan_pos, batch visible
+                        const int w = i - S.first[lo], wy = w / S.cols[lo];
+                        list[at] = make_key(v[u], lo, wy, w - wy * S.cols[lo]);
                     }
-                    if (tid == 0) n_batch = cnt;
+                }
+            }
+        };
+        scan(big);
+        csync();  // every rank's count is in
+        int n = 0, before = 0;
+        for (int r = 0; r < C; ++r) {
+            const int c = cluster.map_shared_rank(&S, r)->n_list;
+            n += c;
+            before += r < rank ? c : 0;
+        }
+        if (n == 0 || n > cap) {
+            if (leader && tid == 0) {
+                counts[2 * f] = 0;
+                counts[2 * f + 1] = n > cap ? -n : 0;
+            }
+            csync();  // nobody clears its count while another rank reads it
+            continue;
+        }
+        int n_list = S.n_list;  // this rank's list
+        if (big) {
+            csync();  // the counts have been read
+            list += before;
+            if (tid == 0) S.n_list = 0;
+            __syncthreads();
+            scan(false);
+            __syncthreads();
+        }
+        int alive = n, kept_total = 0;  // candidates left in the cluster; kept boxes (leader)
+        pd_box *out = boxes + (size_t)f * max_boxes;
+        for (;;) {
+            // ---- 2. the segment: all keys, or those below the bound of a radix select
+            unsigned long long bound = ~0ull;
+            if (alive > kSeg) {
+                unsigned long long mn = ~0ull, mx = 0ull;
+                for (int i = tid; i < n_list; i += kThreads) {
+                    const unsigned long long k = list[i];
+                    mn = umin64(mn, k);
+                    mx = umax64(mx, k);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    mn = umin64(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+                    mx = umax64(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                }
+                if (lane == 0) {
+                    S.lohi[0][warp] = mn;
+                    S.lohi[1][warp] = mx;
                 }
                 __syncthreads();
-                const int nb = n_batch;
-                if (nb > 0) {
+                if (warp == 0) {
+                    mn = S.lohi[0][lane];
+                    mx = S.lohi[1][lane];
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        mn = umin64(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+                        mx = umax64(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                    }
+                    if (lane == 0) {
+                        S.lo = mn;
+                        S.hi = mx;
+                    }
+                }
+                csync();
+                mn = ~0ull;
+                mx = 0ull;
+                for (int r = 0; r < C; ++r) {
+                    mn = umin64(mn, cluster.map_shared_rank(&S, r)->lo);
+                    mx = umax64(mx, cluster.map_shared_rank(&S, r)->hi);
+                }
+                // digits of kDigit bits from the highest bit in which the keys differ; the keys
+                // of the digits below the one that overfills the segment are taken, and that
+                // one is split further while they are less than half a segment
+                int top = 64 - __clzll((long long)(mn ^ mx));  // bits [0, top) differ (at least 12: the keys are distinct)
+                unsigned long long prefix = top < 64 ? mn >> top << top : 0ull;
+                int taken = 0;
+                for (;;) {
+                    const int shift = top > kDigit ? top - kDigit : 0;
+                    for (int i = tid; i < kHist; i += kThreads) S.hist[i] = 0;
+                    __syncthreads();
+                    for (int i = tid; i < n_list; i += kThreads) {
+                        const unsigned long long k = list[i];
+                        if (top == 64 || (k >> top) == (prefix >> top)) atomicAdd(&S.hist[(int)(k >> shift) & (kHist - 1)], 1);
+                    }
+                    csync();
+                    // every rank adds up all histograms (two digits per thread) and finds the digit
+                    int c0 = 0, c1 = 0;
+                    for (int r = 0; r < C; ++r) {
+                        const int2 c = *reinterpret_cast<const int2 *>(&cluster.map_shared_rank(&S, r)->hist[2 * tid]);
+                        c0 += c.x;
+                        c1 += c.y;
+                    }
+                    int incl = c0 + c1;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int a = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += a;
+                    }
+                    if (lane == 31) S.wsum[warp] = incl;
+                    __syncthreads();
+                    int excl = taken + incl - c0 - c1;
+                    for (int w = 0; w < warp; ++w) excl += S.wsum[w];
+                    // one thread holds the first digit whose keys no longer fit
+                    if (excl <= kSeg && excl + c0 > kSeg) {
+                        S.digit = 2 * tid;
+                        S.below = excl;
+                    } else if (excl + c0 <= kSeg && excl + c0 + c1 > kSeg) {
+                        S.digit = 2 * tid + 1;
+                        S.below = excl + c0;
+                    }
+                    csync();  // found; nobody clears its histogram while another rank reads it
+                    taken = S.below;
+                    prefix |= (unsigned long long)S.digit << shift;
+                    top = shift;
+                    if (taken >= kSeg / 2 || shift == 0) break;
+                }
+                bound = prefix - 1ull;  // the keys below the digit
+            }
+            for (int i0 = 0; i0 < n_list; i0 += kThreads) {
+                const int i = i0 + tid;
+                const unsigned long long k = i < n_list ? list[i] : 0ull;
+                const bool take = i < n_list && k <= bound;
+                const unsigned m = __ballot_sync(0xffffffffu, take);
+                if (!m) continue;
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&Lead.n_seg, __popc(m));
+                at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                if (take && at < kSeg) Lead.key[at] = k;  // (the select keeps it below)
+            }
+            csync();  // the segment is with the leader
+            // ---- 3. the leader sorts and walks it
+            if (leader) {
+                const int m = min(S.n_seg, kSeg);
+                sort_segment(S, m, tid);
+                for (int i = tid; i < m; i += kThreads) {
+                    const pd_box b = decode(S.key[i], W, H, S.wkhk);
+                    S.box[i] = make_float4(b.x, b.y, b.w, b.h);
+                }
+                if (tid < kSeg / 32) {
+                    const int left = m - 32 * tid;
+                    S.alive[tid] = left >= 32 ? 0xffffffffu : left > 0 ? (1u << left) - 1u : 0u;
+                }
+                __syncthreads();
+                const float4 own0 = S.box[tid], own1 = S.box[tid + kThreads];  // (unused past m)
+                int kept_seg = 0;
+                for (;;) {
+                    // the next (up to) 64 alive entries, in order: every warp ranks the entries of its
+                    // two flag words by the words' prefix counts
+                    const uint32_t wa = S.alive[2 * lane], wb = S.alive[2 * lane + 1];
+                    int incl = __popc(wa) + __popc(wb);
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int a = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += a;
+                    }
+                    const int total = __shfl_sync(0xffffffffu, incl, 31);
+                    if (total == 0 || kept_total >= max_boxes) break;
+                    const int nb = min(total, kBatch);
+                    uint32_t mine[2];
+                    bool member[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int word = warp + 32 * h, src = word >> 1;
+                        const uint32_t a = __shfl_sync(0xffffffffu, wa, src), b = __shfl_sync(0xffffffffu, wb, src);
+                        const int pre = __shfl_sync(0xffffffffu, incl, src) - __popc(b) - (word & 1 ? 0 : __popc(a));
+                        mine[h] = word & 1 ? b : a;
+                        const int slot = pre + __popc(mine[h] & ((1u << lane) - 1u));
+                        const bool on = (mine[h] >> lane) & 1u;
+                        member[h] = on && slot < kBatch;
+                        if (on && !member[h]) S.rest[slot - kBatch] = (unsigned short)(tid + h * kThreads);
+                        if (member[h]) {
+                            const float4 b = h ? own1 : own0;
+                            S.batch[slot] = tid + h * kThreads;
+                            S.bbx[slot] = b;
+                            S.bed[slot] = edges_of(b);
+                        }
+                    }
+                    __syncthreads();
                     {
                         // member b = tid / 16 is tested against members a = 4 (tid % 16) .. + 3
                         // (a < b); the 16 threads of a member OR their bits together
                         const int b = tid >> 4, a0 = (tid & 15) * 4;
                         unsigned long long bits = 0;
-                        if (b < nb) {
-                            const float4 bb = bbx[b];
-    #pragma unroll
+                        if (b < nb && a0 < b) {
+                            const Edges bb = S.bed[b];
+#pragma unroll
                             for (int q = 0; q < 4; ++q) {
                                 const int a = a0 + q;
-                                if (a < b && suppresses(bbx[a], bb, iou_thr)) bits |= 1ull << a;
+                                if (a < b && suppresses(S.bed[a], S.bbx[a], bb, S.bbx[b], iou_thr, band)) bits |= 1ull << a;
                             }
                         }
-    #pragma unroll
+#pragma unroll
                         for (int o = 8; o > 0; o >>= 1) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
-                        if ((tid & 15) == 0 && b < kBatch) bcol[b] = bits;
+                        if ((tid & 15) == 0) S.bcol[b] = bits;
                     }
                     __syncthreads();
+                    // Resolve in rounds (warp 0): a member is dropped once a kept member suppresses
+                    // it, and kept once every member that could suppress it is decided and none of
+                    // them is kept. This reaches the in-order result (induction on the member
+                    // index) in as many rounds as the longest chain of suppressions. Lane l decides
+                    // members l and l + 32; only members before it can suppress a member.
                     if (warp == 0) {
-                        // Resolve in rounds: a member is dropped once a kept member
-                        // suppresses it, and kept once every member that could suppress it
-                        // is decided and none of them is kept. This reaches the in-order
-                        // result (induction on the member index) in as many rounds as the
-                        // longest chain of suppressions.
-                        const unsigned long long all = nb == 64 ? ~0ull : ((1ull << nb) - 1ull);
-                        const unsigned long long c0 = bcol[lane], c1 = bcol[lane + 32];
-                        unsigned long long keep = 0, decided = ~all;
-                        while (decided != ~0ull) {
-                            const bool k0 = !((decided >> lane) & 1ull) && !(c0 & keep) && !(c0 & ~decided);
-                            const bool d0 = k0 || (!((decided >> lane) & 1ull) && (c0 & keep));
-                            const bool k1 = !((decided >> (lane + 32)) & 1ull) && !(c1 & keep) && !(c1 & ~decided);
-                            const bool d1 = k1 || (!((decided >> (lane + 32)) & 1ull) && (c1 & keep));
-                            keep |= (unsigned long long)__ballot_sync(0xffffffffu, k0) |
-                                    ((unsigned long long)__ballot_sync(0xffffffffu, k1) << 32);
-                            decided |= (unsigned long long)__ballot_sync(0xffffffffu, d0) |
-                                       ((unsigned long long)__ballot_sync(0xffffffffu, d1) << 32);
+                        const uint32_t c0 = (uint32_t)S.bcol[lane];
+                        const uint32_t c1 = (uint32_t)S.bcol[lane + 32], c2 = (uint32_t)(S.bcol[lane + 32] >> 32);
+                        uint32_t kl = 0, kh = 0;                       // kept, low and high members
+                        uint32_t ul = nb >= 32 ? ~0u : (1u << nb) - 1u;  // undecided
+                        uint32_t uh = nb <= 32 ? 0u : nb == 64 ? ~0u : (1u << (nb - 32)) - 1u;
+                        while (ul | uh) {
+                            const bool u0 = (ul >> lane) & 1u, u1 = (uh >> lane) & 1u;
+                            const bool s0 = c0 & kl, s1 = (c1 & kl) | (c2 & kh);   // suppressed
+                            const bool k0 = u0 && !s0 && !(c0 & ul), k1 = u1 && !s1 && !((c1 & ul) | (c2 & uh));
+                            kl |= __ballot_sync(0xffffffffu, k0);
+                            kh |= __ballot_sync(0xffffffffu, k1);
+                            ul &= ~__ballot_sync(0xffffffffu, u0 && (k0 || s0));
+                            uh &= ~__ballot_sync(0xffffffffu, u1 && (k1 || s1));
                         }
                         // the cap on kept boxes: only the first (max_boxes - kept so far) in order
-                        const int kt = kept_total;
-                        const int room = max_boxes - kt;
-                        while (__popcll(keep) > room) keep &= ~(1ull << (63 - __clzll(keep)));
-    #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int m = lane + 32 * h;
-                            if (m < nb && ((keep >> m) & 1ull)) {
-                                const int r = __popcll(keep & ((1ull << m) - 1ull));
-                                kept_idx[kt + r] = batch[m];
-                                kbx[r] = bbx[m];
-                            }
+                        while (__popc(kl) + __popc(kh) > max_boxes - kept_total) {
+                            if (kh) kh &= ~(0x80000000u >> __clz((int)kh));
+                            else kl &= ~(0x80000000u >> __clz((int)kl));
                         }
-                        if (lane == 0) {
-                            n_keep = __popcll(keep);
-                            kept_total = kt + __popcll(keep);
+                        if (lane < 2) S.keep[lane] = lane ? kh : kl;
+                    }
+                    // the members leave the flags meanwhile
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t off = __ballot_sync(0xffffffffu, member[h]);
+                        if (lane == 0) S.alive[warp + 32 * h] = mine[h] & ~off;
+                    }
+                    __syncthreads();
+                    const uint32_t keep[2] = {S.keep[0], S.keep[1]};
+                    const int n_keep = __popc(keep[0]) + __popc(keep[1]);
+                    const uint32_t kw = warp ? keep[1] : keep[0];
+                    if (tid < kBatch && ((kw >> lane) & 1u)) {  // warps 0 and 1
+                        const int r = (warp ? __popc(keep[0]) : 0) + __popc(kw & ((1u << lane) - 1u));
+                        const int e = S.batch[tid];
+                        const unsigned long long key = S.key[e];
+                        const uint32_t lo = (uint32_t)key;
+                        const float4 bc = S.bbx[tid];
+                        pd_box b;
+                        b.x = bc.x;
+                        b.y = bc.y;
+                        b.w = bc.z;
+                        b.h = bc.w;
+                        b.score = key_score((uint32_t)(key >> 32));
+                        b.level = (int)(lo >> 24);
+                        b.wy = (int)((lo >> 12) & 4095);
+                        b.wx = (int)(lo & 4095);
+                        out[kept_total + r] = b;
+                        S.kept[kept_seg + r] = e;
+                    }
+                    // the segment's later entries against the batch's kept members: 1 to 32 threads
+                    // per entry, as many as the block has for the entries that are left
+                    const int n_rest = total - nb;
+                    int per = 1;
+                    while (per < 32 && 2 * per * n_rest <= kThreads) per *= 2;
+                    const int sub = tid & (per - 1);
+                    // the members this thread tests: every per-th, from sub
+                    const uint32_t part = (per == 1    ? ~0u
+                                           : per == 2  ? 0x55555555u
+                                           : per == 4  ? 0x11111111u
+                                           : per == 8  ? 0x01010101u
+                                           : per == 16 ? 0x00010001u
+                                                       : 1u) << sub;
+                    for (int i0 = 0; i0 < n_rest; i0 += kThreads / per) {
+                        const int i = i0 + tid / per;
+                        bool gone = false;
+                        int e = 0;
+                        if (i < n_rest) {
+                            e = S.rest[i];
+                            const float4 bj = S.box[e];
+                            const Edges ej = edges_of(bj);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+                                for (uint32_t k = keep[h] & part; k && !gone; k &= k - 1u) {
+                                    const int j = 32 * h + __ffs((int)k) - 1;
+                                    gone = suppresses(S.bed[j], S.bbx[j], ej, bj, iou_thr, band);
+                                }
+                        }
+                        for (int o = per / 2; o > 0; o >>= 1) gone |= __shfl_xor_sync(0xffffffffu, (int)gone, o) != 0;
+                        if (gone && sub == 0) atomicAnd(&S.alive[e >> 5], ~(1u << (e & 31)));
+                    }
+                    kept_total += n_keep;
+                    kept_seg += n_keep;
+                    __syncthreads();
+                }
+                if (tid == 0) {
+                    S.n_kept_seg = kept_seg;
+                    S.done = kept_total >= max_boxes;
+                    S.n_seg = 0;
+                }
+            }
+            if (bound == ~0ull) break;  // nothing is left behind the segment
+            csync();  // the segment is walked
+            if (Lead.done) break;
+            // ---- 4. drop the segment's keys and what its kept boxes suppress, 64 of them at a time
+            const int nk = Lead.n_kept_seg;
+            const float gsx = (float)kGrid / (float)W, gsy = (float)kGrid / (float)H;
+            // one run of keys per thread: test each against all kept boxes of the chunk; more:
+            // only against those that cover its centre's cell
+            const bool grid = cull && n_list > kThreads;
+            for (int k0 = 0; k0 < nk || k0 == 0; k0 += kBatch) {
+                const int kc = min(kBatch, nk - k0);
+                if (tid < kc) {
+                    const float4 b = Lead.box[Lead.kept[k0 + tid]];
+                    S.bbx[tid] = b;
+                    S.bed[tid] = edges_of(b);
+                    S.krect[tid] = make_int4(max((int)floorf(b.x * gsx) - 1, 0),
+                                             min((int)floorf((b.x + b.z) * gsx) + 1, kGrid - 1),
+                                             max((int)floorf(b.y * gsy) - 1, 0),
+                                             min((int)floorf((b.y + b.w) * gsy) + 1, kGrid - 1));
+                }
+                __syncthreads();
+                if (grid) {
+                    // Culling (IoU threshold >= 0.5): if IoU(A, B) > 0.5 then A's centre lies
+                    // in B (were it outside B on one axis, A and B would overlap on at most
+                    // half of A's extent there, so inter <= |A| / 2, and inter > (|A| + |B|)
+                    // / 3 would need |B| < |A| / 2 while inter <= |B| needs |B| > |A| / 2).
+                    // For every cell of a 32 x 32 grid over the frame: which of the kept boxes
+                    // cover it (one cell of margin for rounding).
+                    const int cx = tid & (kGrid - 1), cy = tid / kGrid;
+                    unsigned long long m = 0ull;
+                    for (int k = 0; k < kc; ++k) {
+                        const int4 r = S.krect[k];
+                        if (cx >= r.x && cx <= r.y && cy >= r.z && cy <= r.w) m |= 1ull << k;
+                    }
+                    S.cmask[tid] = m;
+                    __syncthreads();
+                }
+                int left = 0;  // keys kept so far (the list is compacted in place, a run at a time)
+                for (int i0 = 0; i0 < n_list; i0 += kThreads) {
+                    const int i = i0 + tid;
+                    const unsigned long long key = i < n_list ? list[i] : 0ull;
+                    bool stay = i < n_list && key > bound;
+                    if (stay && kc > 0) {
+                        const pd_box b = decode(key, W, H, S.wkhk);
+                        const float4 bj = make_float4(b.x, b.y, b.w, b.h);
+                        const Edges ej = edges_of(bj);
+                        if (grid) {
+                            const int cx = min(max((int)floorf((b.x + 0.5f * b.w) * gsx), 0), kGrid - 1);
+                            const int cy = min(max((int)floorf((b.y + 0.5f * b.h) * gsy), 0), kGrid - 1);
+                            const unsigned long long m = S.cmask[cy * kGrid + cx];
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+                                for (uint32_t k = (uint32_t)(m >> (32 * h)); k && stay; k &= k - 1u) {
+                                    const int j = 32 * h + __ffs((int)k) - 1;
+                                    stay = !suppresses(S.bed[j], S.bbx[j], ej, bj, iou_thr, band);
+                                }
+                        } else {
+                            for (int j = 0; j < kc && stay; ++j)
+                                stay = !suppresses(S.bed[j], S.bbx[j], ej, bj, iou_thr, band);
                         }
                     }
+                    const unsigned m = __ballot_sync(0xffffffffu, stay);
+                    if (lane == 0) S.wsum[warp] = __popc(m);
+                    __syncthreads();  // also: the run has been read
+                    const int c = S.wsum[lane];
+                    const int total = __reduce_add_sync(0xffffffffu, c);
+                    const int at = left + __reduce_add_sync(0xffffffffu, lane < warp ? c : 0);
+                    if (stay) list[at + __popc(m & ((1u << lane) - 1u))] = key;
+                    left += total;
+                    __syncthreads();
                 }
-                __syncthreads();
-                if (tid == 0) s_done = nb == 0 || kept_total >= max_boxes;
+                n_list = left;
             }
-            cluster.sync();  // the batch is resolved (or the walk is over)
-            if (leader ? s_done : *cluster.map_shared_rank(&s_done, 0)) break;
-            int nk, sp;
-            if (leader) {
-                nk = n_keep;
-                sp = scan_pos;
-            } else {  // the kept boxes of the batch and the scan start, from the leader
-                nk = *cluster.map_shared_rank(&n_keep, 0);
-                sp = *cluster.map_shared_rank(&scan_pos, 0);
-                const float4 *lk = cluster.map_shared_rank(kbx, 0);
-                for (int k = tid; k < nk; k += kThreads) kbx[k] = lk[k];
-                __syncthreads();
+            if (tid == 0) S.n_list = n_list;
+            csync();  // the lists are compacted, the leader's segment is free
+            alive = 0;
+            for (int r = 0; r < C; ++r) alive += cluster.map_shared_rank(&S, r)->n_list;
+            if (alive == 0) {
+                csync();  // nobody clears its count while another rank reads it
+                break;
             }
-            if (cull) {
-                // grid cells under each kept box, with one cell of margin; then per
-                // cell (one per thread) the set of kept boxes that cover it
-                if (tid < nk) {
-                    const float4 b = kbx[tid];
-                    krect[tid] = make_int4(max((int)floorf(b.x * gsx) - 1, 0),
-                                           min((int)floorf((b.x + b.z) * gsx) + 1, kGrid - 1),
-                                           max((int)floorf(b.y * gsy) - 1, 0),
-                                           min((int)floorf((b.y + b.w) * gsy) + 1, kGrid - 1));
-                }
-                __syncthreads();
-                const int cx = tid & (kGrid - 1), cy = tid / kGrid;
-                unsigned long long m = 0ull;
-                for (int k = 0; k < nk; ++k) {
-                    const int4 r = krect[k];
-                    if (cx >= r.x && cx <= r.y && cy >= r.z && cy <= r.w) m |= 1ull << k;
-                }
-                cmask[tid] = m;
-                __syncthreads();
-            }
-            int j = sp + rank * kThreads + tid;  // this rank's share: every C-th run of kThreads
-            float4 bnext = j < n ? bx[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-            for (; j < n; j += C * kThreads) {
-                // the next box is loaded while this one is tested (global for large caps)
-                const float4 bj = bnext;
-                if (j + C * kThreads < n) bnext = bx[j + C * kThreads];
-                if (fl[j]) continue;
-                bool hit = false;
-                if (cull) {
-                    // only the kept boxes that cover the centre's cell can suppress it
-                    const int cx = min(max((int)floorf((bj.x + 0.5f * bj.z) * gsx), 0), kGrid - 1);
-                    const int cy = min(max((int)floorf((bj.y + 0.5f * bj.w) * gsy), 0), kGrid - 1);
-                    unsigned long long m = cmask[cy * kGrid + cx];
-                    while (m && !hit) {
-                        const int k = __ffsll((long long)m) - 1;
-                        m &= m - 1ull;
-                        hit = suppresses(kbx[k], bj, iou_thr);
-                    }
-                } else {
-                    for (int k = 0; k < nk && !hit; k += 4) {
-                        // four tests in flight (kept boxes past nk repeat the first one)
-                        const bool h0 = suppresses(kbx[k], bj, iou_thr);
-                        const bool h1 = suppresses(kbx[k + 1 < nk ? k + 1 : 0], bj, iou_thr);
-                        const bool h2 = suppresses(kbx[k + 2 < nk ? k + 2 : 0], bj, iou_thr);
-                        const bool h3 = suppresses(kbx[k + 3 < nk ? k + 3 : 0], bj, iou_thr);
-                        hit = h0 || h1 || h2 || h3;
-                    }
-                }
-                if (hit) fl[j] = 1;
-            }
-            cluster.sync();  // every rank's share of the pass is done
         }
-        cluster.sync();  // nobody moves on while another rank reads its shared memory
-        if (!leader) continue;
-        const int kept = kept_total;
-        pd_box *out = boxes + (size_t)f * max_boxes;
-        for (int k = tid; k < kept; k += kThreads) {
-            const int c = kept_idx[k];
-            const unsigned long long key = ksrc[c];
-            const float4 bc = bx[c];
-            const uint32_t hi = (uint32_t)(key >> 32), lo = (uint32_t)key;
-            const uint32_t ord = ~hi;
-            pd_box b;
-            b.x = bc.x;
-            b.y = bc.y;
-            b.w = bc.z;
-            b.h = bc.w;
-            b.score = __uint_as_float((ord & 0x80000000u) ? (ord ^ 0x80000000u) : ~ord);
-            b.level = (int)(lo >> 24);
-            b.wy = (int)((lo >> 12) & 4095);
-            b.wx = (int)(lo & 4095);
-            out[k] = b;
-        }
-        if (tid == 0) {
-            counts[2 * f] = kept;
+        if (leader && tid == 0) {
+            counts[2 * f] = kept_total;
             counts[2 * f + 1] = n;
         }
     }
@@ -793,14 +1014,10 @@ __global__ void __launch_bounds__(kThreads) k_nms_order(const int *__restrict__ 
     if (tid == 0) *queue = 0;
 }
 
-size_t nms_smem(int cap, int max_boxes) {
+size_t nms_smem(int cap) {
     int p = 1;
     while (p < cap) p <<= 1;
-    const size_t keys = cap > kMaxCandidates ? 0 : (size_t)p * sizeof(unsigned long long);
-    const size_t walk = keys + (size_t)((cap + 15) & ~15) + 4 * (size_t)max_boxes;
-    // large caps: the sort's key chunks use the same shared memory first
-    const size_t chunk = cap > kMaxCandidates ? (size_t)kSortChunk * sizeof(unsigned long long) : 0;
-    return walk > chunk ? walk : chunk;
+    return sizeof(NmsSmem) + (cap > kMaxCandidates ? 0 : (size_t)p * sizeof(unsigned long long));
 }
 
 }  // namespace
@@ -813,7 +1030,7 @@ int log2_cluster(int c) { return c == 8 ? 3 : c == 4 ? 2 : c == 2 ? 1 : 0; }
 }  // namespace
 
 cudaError_t init_nms(bool occupancy) {
-    const int smem = (int)nms_smem(kMaxCandidates, kMaxBoxes);
+    const int smem = (int)nms_smem(kMaxCandidates);
     cudaError_t e = cudaFuncSetAttribute(k_nms, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_nms_order, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -851,7 +1068,7 @@ cudaError_t init_nms(bool occupancy) {
 }
 
 int nms_cluster_for(int n_frames, int sm_count, int max_cand) {
-    // the CTAs of a frame share its suppression passes; only while every CTA
+    // the CTAs of a frame share its collection and passes; only while every CTA
     // still gets an SM of its own (one 1024-thread CTA per SM), or, for large
     // candidate lists, while two rounds of clusters cover the frames (the
     // clusters then draw the frames heaviest first)
@@ -877,7 +1094,7 @@ cudaError_t launch_nms(cudaStream_t s, const FrameDesc *d_frames, const LevelDes
     if (max_cand < 1 || max_cand > kMaxCandidatesBig || max_boxes < 1 || max_boxes > kMaxBoxes ||
         cluster < 1 || cluster > 8 || (cluster & (cluster - 1)))
         return cudaErrorInvalidValue;
-    const size_t smem = nms_smem(max_cand, max_boxes);
+    const size_t smem = nms_smem(max_cand);
     // more frames than clusters that fit at once: persistent clusters over a
     // ticket queue, frames ordered by their candidate counts (most first)
     int *queue = nullptr, *order = nullptr;
@@ -922,9 +1139,8 @@ cudaError_t launch_nms(cudaStream_t s, const FrameDesc *d_frames, const LevelDes
 
 // ---------------------------------------------------------------------------
 // Allocation-free NMS (pd_nms_noalloc). The kernel above needs device memory
-// beyond its inputs and outputs: the frame / level descriptors it reads and
-// the per-candidate decoded boxes. For callers that cannot allocate device
-// memory, that scratch lives in one file-scope array that every GPU loading
+// beyond its inputs and outputs: the frame / level descriptors it reads. For
+// callers that cannot allocate device memory, that scratch lives in one file-scope array that every GPU loading
 // this library holds until the process exits. A small set-up kernel copies
 // the level geometry (passed by value) into it before the unchanged NMS
 // kernel runs.
@@ -936,7 +1152,6 @@ constexpr int kNoAllocMaxLevels = PD_MAX_LEVELS;
 struct NoAllocScratch {
     FrameDesc frame;
     LevelDesc levels[kNoAllocMaxLevels];
-    float4 boxes[kNoAllocMaxCandidates];  // decoded candidate boxes
 };
 
 struct NoAllocGeometry {
@@ -1013,7 +1228,7 @@ extern "C" int pd_nms_noalloc(void *stream, const float *d_scores, int n_levels,
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     k_nms_noalloc_setup<<<1, 128, 0, s>>>(g, scratch);
     if (cudaGetLastError() != cudaSuccess) return PD_ECUDA;
-    if (launch_nms(s, &scratch->frame, scratch->levels, 1, d_scores, threshold, nms_iou, scratch->boxes,
+    if (launch_nms(s, &scratch->frame, scratch->levels, 1, d_scores, threshold, nms_iou, nullptr,
                    max_candidates, d_boxes, max_boxes, d_counts) != cudaSuccess)
         return PD_ECUDA;
     return PD_OK;

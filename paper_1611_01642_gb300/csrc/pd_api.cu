@@ -264,7 +264,7 @@ struct pd_handle {
     int64_t score_cap = 0;
     pd_box *d_boxes = nullptr;
     int32_t *d_counts = nullptr;  // [2 * max_frames]
-    float4 *d_nms_scratch = nullptr;  // [max_frames][max_candidates] decoded candidate boxes
+    float4 *d_nms_scratch = nullptr;  // candidate keys per frame (caps above 16,384)
     unsigned *d_err = nullptr;
     uint8_t *d_frames = nullptr;  // host-input staging for pd_detect_host
     int64_t frames_cap = 0;

@@ -165,13 +165,10 @@ cudaError_t launch_svm_tc(cudaStream_t s, const CUtensorMap &hog_map, const CUte
                           const unsigned char *d_consts, float bias, float clip, float *scores,
                           const uint32_t *c_flag, unsigned *d_err, int hog_planes = kHogBins,
                           const CUtensorMap *level_maps = nullptr);
-// Per-frame NMS scratch (float4 units) for a candidate cap: the decoded
-// boxes, plus the sort keys when the cap is above 16,384 (shared memory
-// holds them below).
+// Per-frame NMS scratch (float4 units) for a candidate cap: the candidates'
+// 64-bit keys when the cap is above 16,384 (shared memory holds them below).
 __host__ __device__ inline size_t nms_scratch_float4s(int cap) {
-    size_t p = 1;
-    while (p < (size_t)cap) p <<= 1;
-    return cap > 16384 ? (size_t)cap + p / 2 : (size_t)cap;
+    return cap > 16384 ? ((size_t)cap + 1) / 2 : 0;
 }
 // cluster: CTAs per frame (1, 2, 4 or 8; a thread-block cluster that shares
 // the frame's suppression passes); nms_cluster_for picks it for a batch.
