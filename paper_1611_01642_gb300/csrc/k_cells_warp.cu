@@ -74,6 +74,27 @@
 // are written. The result does not depend on the strip height: every cell
 // row sums its votes in the same order.
 //
+// Per-block HOG (kFeatHogBlock, Algorithm 5 read per 16x16 block): a block's
+// 4 cell histograms take only the block's own pixels, with the votes of the
+// shared grid left unclamped (a vote towards a cell outside the block is
+// dropped). Cell (cy, cx) sits at one of 4 places q = 2a + b of the blocks
+// that contain it (a = 0: it is the block's top cell, so the block spans
+// pixel rows [8cy, 8cy + 16); a = 1: rows [8cy - 8, 8cy + 8); b likewise on
+// x), and the kernel writes its 4 restricted histograms Q_q to planes
+// 9q + bin. Block (by, bx) is then [Q_0(by, bx), Q_1(by, bx+1),
+// Q_2(by+1, bx), Q_3(by+1, bx+1)]. The walk and its votes are the shared
+// grid's: of the rows that vote into cell row t, A = [8t - 4, 8t),
+// B = [8t, 8t + 8) and C = [8t + 8, 8t + 12), a = 1 takes A and B, a = 0 takes
+// B and C, and the ends of A, B and C are ends of half bands. So the slots are
+// summed over the columns three times per cell row: after A (set aside, slots
+// cleared), after B (with A: a = 1) and after C (a = 0); of a cell's 16 columns
+// b drops the first or the last 4, one b per lane of the cell. Against a CTA
+// of 128 threads per 15 x 8-cell tile, one column per thread, which voted
+// three times per pixel and counted LBP by shared-memory atomics: 583 -> 309 us
+// per 16 x 1242x375 frames (the shared grid: about 200). What bounds it: the
+// shared-memory pipe, where the column sums and the second clear add about
+// 170 wavefronts per cell row to the walk's 370.
+//
 // Sparse path: c_flag marks the 15 x 8-cell tiles to compute; a band is
 // walked when one of its two cell rows lies in a marked tile, and a cell
 // row is written when its tile is marked.
@@ -98,11 +119,18 @@ constexpr uint32_t kMagicBits = 0x4B400000u;
 constexpr float kMagic2 = 25165824.0f;           // 3 * 2^23 (spacing 2): rounds to even integers
 constexpr uint32_t kMagic2Bits = 0x4BC00000u;
 
+template <bool PB>
 struct WarpSmem {
     float R[2 * kRingStride];       // HOG vote slots of the 2 open cell rows
 };
+template <>
+struct WarpSmem<true> {
+    float R[2 * kRingStride];
+    float top[kHogBins][32];        // per-block HOG: per lane, the votes of the 4 pixel rows above the open cell row
+};
+template <bool PB>
 struct StripSmem {
-    WarpSmem w[kWarps];
+    WarpSmem<PB> w[kWarps];
 };
 
 struct Row {
@@ -138,8 +166,21 @@ __device__ __forceinline__ float rcp_approx(float x) {
 
 // -2 atan(z) * 9/pi / z as a polynomial in s = z^2 (|z| <= 1), two values at
 // a time: the fitted coefficients scaled to 20-degree bins, doubled and negated
-// (exact: every step of the evaluation scales by -2).
+// (exact: every step of the evaluation scales by -2). PREC: one degree more (15,
+// fitted to the least largest error), 3.3e-7 bin instead of 8.9e-7 in float32;
+// the histograms' error is 1.1e-7 of their norm with it and 2.9e-7 without.
+template <bool PREC>
 __device__ __forceinline__ f32x2 atan_bins2_poly(f32x2 s) {
+    if constexpr (PREC) {
+        f32x2 p = dup2(-2.0f * -0.01161547377705574f);
+        p = fma2(p, s, dup2(-2.0f * 0.06263275444507599f));
+        p = fma2(p, s, dup2(-2.0f * -0.16017703711986542f));
+        p = fma2(p, s, dup2(-2.0f * 0.2762286365032196f));
+        p = fma2(p, s, dup2(-2.0f * -0.39845290780067444f));
+        p = fma2(p, s, dup2(-2.0f * 0.571427047252655f));
+        p = fma2(p, s, dup2(-2.0f * -0.9548301696777344f));
+        return fma2(p, s, dup2(-2.0f * 2.8647871017456055f));
+    }
     f32x2 p = dup2(-2.0f * 0.019514326006174088f);
     p = fma2(p, s, dup2(-2.0f * -0.09626893699169159f));
     p = fma2(p, s, dup2(-2.0f * 0.22810496389865875f));
@@ -228,10 +269,11 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
                  const StripItem *__restrict__ items, int n_items, int *__restrict__ queue,
                  const uint32_t *__restrict__ c_flag) {
     constexpr bool kHog = (FEAT & kFeatHog) != 0, kLbp = (FEAT & kFeatLbp) != 0;
+    constexpr bool kPb = (FEAT & kFeatHogBlock) != 0;  // per-block HOG
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    StripSmem &S = *reinterpret_cast<StripSmem *>(smem_raw);
+    StripSmem<kPb> &S = *reinterpret_cast<StripSmem<kPb> *>(smem_raw);
     const int lane = threadIdx.x & 31;
-    WarpSmem &Wm = S.w[threadIdx.x >> 5];
+    WarpSmem<kPb> &Wm = S.w[threadIdx.x >> 5];
     // persistent warps: each takes the next strip (tallest first) until none is left
     for (;;) {
         int item = lane == 0 ? atomicAdd(queue, 1) : 0;
@@ -250,6 +292,10 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
         if (kHog)
             for (int i = lane; i < 2 * kRingStride / 4; i += 32)
                 reinterpret_cast<float4 *>(Wm.R)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (kPb) {
+#pragma unroll
+            for (int h = 0; h < kHogBins; ++h) Wm.top[h][lane] = 0.f;  // a level's first cell row has no rows above it
+        }
         uint32_t plane[8];  // LBP comparisons of the last 8 rows: plane k, byte = column, bit = row
 #pragma unroll
         for (int k = 0; k < 8; ++k) plane[k] = 0u;
@@ -274,7 +320,8 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
                     const float ux = ((float)xc - 3.5f) * 0.125f;
                     const float fx = floorf(ux);
                     const float w1 = ux - fx, w0 = 1.f - w1;
-                    const int c0 = clampi((int)fx, 0, Wc - 1), c1 = clampi((int)fx + 1, 0, Wc - 1);
+                    const int c0 = kPb ? (int)fx : clampi((int)fx, 0, Wc - 1);
+                    const int c1 = kPb ? (int)fx + 1 : clampi((int)fx + 1, 0, Wc - 1);
                     a = (c0 == own ? w0 : 0.f) + (c1 == own ? w1 : 0.f);
                     b = (c0 == nbr ? w0 : 0.f) + (c1 == nbr ? w1 : 0.f);
                 }
@@ -346,7 +393,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
                                          pack2(rcp_approx(d0), rcp_approx(d1)));
                     // u = 2 (4.5 - phi) in bins, in [0, 9]
                     float u0, u1;
-                    unpack2(fma2(t, atan_bins2_poly(mul2(t, t)), dup2(4.5f)), u0, u1);
+                    unpack2(fma2(t, atan_bins2_poly<kPb>(mul2(t, t)), dup2(4.5f)), u0, u1);
                     // theta = phi (same signs) or 9 - phi (opposite signs); the vote position is
                     // theta - 0.5, rounded below through theta - 1: p2 = 2 (theta - 1) = 7 -/+ u
                     const uint32_t f0 = ~(__float_as_uint(x0) ^ __float_as_uint(y0)) & 0x80000000u;
@@ -444,6 +491,72 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
             }
         };
 
+        // ---- HOG bin h of a cell row: the lane's columns of the slots at Rl (bin h is slot
+        // h + 1; bin 0 also slot 10, bin 8 also slot 0), weighted for its own cell and for
+        // the neighbouring cell they reach
+        auto columns = [&](const float *Rl, int h, float &own, float &nbv) {
+            float4 v = *reinterpret_cast<const float4 *>(Rl + (h + 1) * kSCols);
+            if (h == 0 || h == kHogBins - 1) {
+                const float4 u = *reinterpret_cast<const float4 *>(Rl + (h == 0 ? kSlots - 1 : 0) * kSCols);
+                v.x += u.x;
+                v.y += u.y;
+                v.z += u.z;
+                v.w += u.w;
+            }
+            own = wo[0] * v.x;
+            own = fmaf(wo[1], v.y, own);
+            own = fmaf(wo[2], v.z, own);
+            own = fmaf(wo[3], v.w, own);
+            nbv = wn[0] * v.x;
+            nbv = fmaf(wn[1], v.y, nbv);
+            nbv = fmaf(wn[2], v.z, nbv);
+            nbv = fmaf(wn[3], v.w, nbv);
+        };
+        auto clear = [&](float *Rl) {  // only this lane wrote its columns
+#pragma unroll
+            for (int s = 0; s < kSlots; ++s)
+                *reinterpret_cast<float4 *>(Rl + s * kSCols) = make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+
+        // ---- per-block HOG: bin h of the cell's blocks on one side of it. Lane 2c + 1 sums the
+        // columns of the block that starts at cell c (b = 0), lane 2c + 2 those of the block
+        // that ends with it (b = 1).
+        auto block_sum = [&](const float *Rl, int h) {
+            float own, nbv;
+            columns(Rl, h, own, nbv);
+            const float o = __shfl_sync(0xffffffffu, own, ((lane - 1) ^ 1) + 1);
+            const float n = __shfl_sync(0xffffffffu, nbv, (lane & 1) ? lane + 2 : lane - 2);
+            return (own + o) + n;
+        };
+        auto block_dst = [&](int r, int a) {  // plane 9 (2a + b) of the cell
+            return atlas.hog + (int64_t)((2 * a + ((lane & 1) ^ 1)) * kHogBins) * atlas.hog_plane +
+                   (int64_t)(L.cell_row + cy0 + r) * atlas.pitch + cx0 + ((lane - 1) >> 1);
+        };
+        const bool block_st = lane >= 1 && lane <= 2 * kCellTW && cx0 + ((lane - 1) >> 1) < Wc;
+        // After a band's first 4 rows, cell row band - 1 has the votes of its own 8 rows: with
+        // those of the 4 rows above it they are the blocks that end with the row (a = 1). Cell
+        // row band has the votes of the 4 rows above it: set aside, its slots start again.
+        auto emit_half = [&](int band) {
+            if constexpr (kPb) {
+                const int ringA = (band + 1) & 1, ringB = band & 1;
+                if (need(band - 1)) {
+                    const float *Ra = Wm.R + ringA * kRingStride + 4 * lane;
+                    float *dst = block_dst(band - 1, 1);
+#pragma unroll
+                    for (int h = 0; h < kHogBins; ++h) {
+                        const float v = Wm.top[h][lane] + block_sum(Ra, h);
+                        if (block_st) dst[(int64_t)h * atlas.hog_plane] = v;
+                    }
+                }
+                if (need(band)) {
+                    float *Rb = Wm.R + ringB * kRingStride + 4 * lane;
+#pragma unroll
+                    for (int h = 0; h < kHogBins; ++h) Wm.top[h][lane] = block_sum(Rb, h);
+                    clear(Rb);
+                }
+            }
+        };
+
         // ---- HOG of cell row r = band - 1 is final: write it, recycle its slots
         auto emit = [&](int band, bool walked) {
             const int ringA = (band + 1) & 1, ringB = band & 1;
@@ -452,6 +565,19 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
             const int64_t rowoff = (int64_t)(L.cell_row + cy0 + r) * atlas.pitch;
             if (kHog) {
                 float *Ra = Wm.R + ringA * kRingStride + 4 * lane;
+                if (kPb) {
+                    // the 4 rows below the cell row added: the blocks that start with it (a = 0)
+                    if (out) {
+                        float *dst = block_dst(r, 0);
+#pragma unroll
+                        for (int h = 0; h < kHogBins; ++h) {
+                            const float v = block_sum(Ra, h);
+                            if (block_st) dst[(int64_t)h * atlas.hog_plane] = v;
+                        }
+                    }
+                    clear(Ra);
+                    return;
+                }
                 if (walked && band == 0 && cy0 == 0) {
                     // top of the level: the rows above cell row 0 vote into row 0
                     float *Rb = Wm.R + ringB * kRingStride + 4 * lane;
@@ -483,23 +609,8 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
                     float *dst = atlas.hog + rowoff + cx0 + ((lane - 1) >> 1);
 #pragma unroll
                     for (int h = 0; h < kHogBins; ++h) {
-                        // bin h is slot h + 1; bin 0 also slot 10, bin 8 also slot 0
-                        float4 v = *reinterpret_cast<const float4 *>(Ra + (h + 1) * kSCols);
-                        if (h == 0 || h == kHogBins - 1) {
-                            const float4 u = *reinterpret_cast<const float4 *>(Ra + (h == 0 ? kSlots - 1 : 0) * kSCols);
-                            v.x += u.x;
-                            v.y += u.y;
-                            v.z += u.z;
-                            v.w += u.w;
-                        }
-                        float own = wo[0] * v.x;
-                        own = fmaf(wo[1], v.y, own);
-                        own = fmaf(wo[2], v.z, own);
-                        own = fmaf(wo[3], v.w, own);
-                        float nbv = wn[0] * v.x;
-                        nbv = fmaf(wn[1], v.y, nbv);
-                        nbv = fmaf(wn[2], v.z, nbv);
-                        nbv = fmaf(wn[3], v.w, nbv);
+                        float own, nbv;
+                        columns(Ra, h, own, nbv);
                         // cell (t - 1) / 2 at odd lane t: own(t) + own(t + 1) + nb(t - 1) + nb(t + 2)
                         const float o_next = __shfl_down_sync(0xffffffffu, own, 1);
                         const float n_prev = __shfl_up_sync(0xffffffffu, nbv, 1);
@@ -508,10 +619,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
                         if (st) dst[(int64_t)h * atlas.hog_plane] = tot;
                     }
                 }
-                // clear the slots of row r for row r + 2 (only this lane wrote them)
-#pragma unroll
-                for (int s = 0; s < kSlots; ++s)
-                    *reinterpret_cast<float4 *>(Ra + s * kSCols) = make_float4(0.f, 0.f, 0.f, 0.f);
+                clear(Ra);  // for row r + 2
             }
         };
 
@@ -564,6 +672,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
                 ra = c0;
                 rb = c1;
                 wa -= 0.25f;
+                if (kPb && i == 1) emit_half(band);
                 if (kLbp && i == 1) emit_lbp(band);
             }
             emit(band, true);
@@ -576,23 +685,30 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
 
 using StripFn = void (*)(const LevelDesc *, const uint8_t *, CellAtlas, const StripItem *, int, int *,
                          const uint32_t *);
+constexpr int kBlk = kFeatHogBlock;
 // [feature set][cell-major LBP counts]; without LBP the layout does not matter
-const StripFn kStripFns[3][2] = {{k_cells_warp<kFeatHog | kFeatLbp, false>, k_cells_warp<kFeatHog | kFeatLbp, true>},
+const StripFn kStripFns[5][2] = {{k_cells_warp<kFeatHog | kFeatLbp, false>, k_cells_warp<kFeatHog | kFeatLbp, true>},
                                  {k_cells_warp<kFeatHog, false>, k_cells_warp<kFeatHog, false>},
-                                 {k_cells_warp<kFeatLbp, false>, k_cells_warp<kFeatLbp, true>}};
+                                 {k_cells_warp<kFeatLbp, false>, k_cells_warp<kFeatLbp, true>},
+                                 {k_cells_warp<kFeatHog | kFeatLbp | kBlk, false>,
+                                  k_cells_warp<kFeatHog | kFeatLbp | kBlk, true>},
+                                 {k_cells_warp<kFeatHog | kBlk, false>, k_cells_warp<kFeatHog | kBlk, false>}};
 
 int strip_fn_index(int feat) {
-    if (feat == kFeatHog) return 1;
+    const int blk = (feat & kBlk) ? 3 : 0;
+    if ((feat & ~kBlk) == kFeatHog) return blk + 1;
     if (feat == kFeatLbp) return 2;
-    return 0;
+    return blk;
 }
+
+int strip_smem(int index) { return (int)(index >= 3 ? sizeof(StripSmem<true>) : sizeof(StripSmem<false>)); }
 
 }  // namespace
 
 cudaError_t init_cells_warp() {
-    for (int i = 0; i < 6; ++i) {
+    for (int i = 0; i < 10; ++i) {
         const cudaError_t e = cudaFuncSetAttribute(kStripFns[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)sizeof(StripSmem));
+                                                   strip_smem(i / 2));
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -606,7 +722,8 @@ cudaError_t launch_cells_warp(cudaStream_t s, const LevelDesc *d_levels, const u
     // small plan gets one CTA per strip, so that its warps spread over the SMs.
     static_assert(kWarps * 4 == kStripWarpsPerSm, "resident warps per SM");
     const int grid = std::min(n_items, 4 * sm_count);
-    kStripFns[strip_fn_index(feat)][atlas.lbp_cells != 0]<<<grid, kWarps * 32, sizeof(StripSmem), s>>>(
+    const int k = strip_fn_index(feat);
+    kStripFns[k][atlas.lbp_cells != 0]<<<grid, kWarps * 32, strip_smem(k), s>>>(
         d_levels, pyr, atlas, d_items, n_items, d_queue, c_flag);
     return cudaGetLastError();
 }

@@ -61,7 +61,6 @@ struct Plan {
     std::vector<FrameDesc> frames;
     std::vector<LevelDesc> levels;
     std::vector<ResizeItem> r_items;
-    std::vector<CellItem> c_items;
     std::vector<StripItem> strips;
     std::vector<SvmItem> s_items;
     std::vector<TcItem> t_items;
@@ -72,6 +71,7 @@ struct Plan {
     int64_t score_floats = 0;
     int32_t atlas_rows = 0;
     int32_t max_wc = 0;
+    int32_t c_tiles = 0;  // cell tiles of all levels (sparse path: one flag each)
     // frames of equal size share their Q11 tables: (W, H) -> first level index
     std::map<std::pair<int, int>, int> tab_owner;
 
@@ -80,7 +80,6 @@ struct Plan {
         frames.clear();
         levels.clear();
         r_items.clear();
-        c_items.clear();
         strips.clear();
         s_items.clear();
         t_items.clear();
@@ -88,13 +87,13 @@ struct Plan {
         tabs.clear();
         tc_widths.clear();
         pyr_bytes = score_floats = 0;
-        atlas_rows = max_wc = 0;
+        atlas_rows = max_wc = c_tiles = 0;
     }
 };
 
 // Byte offsets of the plan's sections inside the packed descriptor block.
 struct Packed {
-    int64_t frames, levels, r_items, c_items, strips, s_items, t_items, cnn_items, tabs, tmaps, tc_maps, total;
+    int64_t frames, levels, r_items, strips, s_items, t_items, cnn_items, tabs, tmaps, tc_maps, total;
 };
 
 Packed pack_layout(const Plan &p) {
@@ -108,7 +107,6 @@ Packed pack_layout(const Plan &p) {
     o.frames = take((int64_t)p.frames.size() * sizeof(FrameDesc));
     o.levels = take((int64_t)p.levels.size() * sizeof(LevelDesc));
     o.r_items = take((int64_t)p.r_items.size() * sizeof(ResizeItem));
-    o.c_items = take((int64_t)p.c_items.size() * sizeof(CellItem));
     o.strips = take((int64_t)p.strips.size() * sizeof(StripItem));
     o.s_items = take((int64_t)p.s_items.size() * sizeof(SvmItem));
     o.t_items = take((int64_t)p.t_items.size() * sizeof(TcItem));
@@ -632,8 +630,7 @@ void k1_tables(Plan &p, LevelDesc &L, int W, int H, int Wk, int Hk) {
 // planning time: a pd_cell_features call on a 1920x1080 level planned for 50 us
 // what it never launched.)
 constexpr unsigned kPlanResize = 1;   // K1 tables
-constexpr unsigned kPlanTiles = 2;    // cell tiles (per-block HOG, sparse flags)
-constexpr unsigned kPlanWindows = 4;  // FP32 K4 window tiles
+constexpr unsigned kPlanWindows = 2;  // FP32 K4 window tiles
 
 // Adds one level to the plan (descriptor, and the tables and items of `what`).
 void plan_level(Plan &p, unsigned what, int frame, int level, int W, int H, int Wk, int Hk, int64_t img_off,
@@ -669,11 +666,9 @@ void plan_level(Plan &p, unsigned what, int frame, int level, int W, int H, int 
     }
     const int li = (int)p.levels.size();
     L.hsrc = li;
-    L.citem0 = (int32_t)p.c_items.size();
+    L.citem0 = p.c_tiles;
     L.ctx = (L.Wc + kCellTW - 1) / kCellTW;
-    if (what & kPlanTiles)
-        for (int cy = 0; cy < L.Hc; cy += kCellTH)
-            for (int cx = 0; cx < L.Wc; cx += kCellTW) p.c_items.push_back({li, cx, cy, 0});
+    p.c_tiles += L.ctx * ((L.Hc + kCellTH - 1) / kCellTH);
     if (what & kPlanWindows) plan_windows(p.s_items, li, L.rows, L.cols, tile_cost);
     p.atlas_rows += L.Hc;
     p.score_floats += (int64_t)L.rows * L.cols;
@@ -771,7 +766,6 @@ int upload_plan(pd_handle *h, cudaStream_t s, const Plan &p, Packed &o, const ui
     put(o.frames, p.frames.data(), p.frames.size() * sizeof(FrameDesc));
     put(o.levels, p.levels.data(), p.levels.size() * sizeof(LevelDesc));
     put(o.r_items, p.r_items.data(), p.r_items.size() * sizeof(ResizeItem));
-    put(o.c_items, p.c_items.data(), p.c_items.size() * sizeof(CellItem));
     put(o.strips, p.strips.data(), p.strips.size() * sizeof(StripItem));
     put(o.s_items, p.s_items.data(), p.s_items.size() * sizeof(SvmItem));
     put(o.t_items, p.t_items.data(), p.t_items.size() * sizeof(TcItem));
@@ -860,14 +854,10 @@ const T *dptr(pd_handle *h, int64_t off) {
     return reinterpret_cast<const T *>(h->d_desc + off);
 }
 
-// K2+K3 of a plan: the warp-per-strip kernel, or for per-block HOG the
-// CTA-per-tile kernel.
+// K2+K3 of a plan.
 cudaError_t launch_cell_stage(pd_handle *h, cudaStream_t s, const LevelDesc *dl, const uint8_t *pyr,
                               const CellAtlas &atlas, const Plan &p, const Packed &o, const uint32_t *c_flag,
                               int feat) {
-    if (feat & kFeatHogBlock)
-        return launch_cells(s, dl, pyr, atlas, dptr<CellItem>(h, o.c_items), (int)p.c_items.size(), h->d_lbp_map,
-                            c_flag, feat);
     int *queue = h->d_queue + 1;  // the strip counter (K4's is d_queue[0])
     const cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
@@ -995,7 +985,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
         return code;
     };
     if (cudaGetDevice(&h->device) != cudaSuccess) return bail(PD_ECUDA);
-    if (init_resize() != cudaSuccess || init_cells() != cudaSuccess || init_cells_warp() != cudaSuccess ||
+    if (init_resize() != cudaSuccess || init_cells_warp() != cudaSuccess ||
         init_svm() != cudaSuccess || init_svm_tc() != cudaSuccess ||
         init_nms() != cudaSuccess || init_train() != cudaSuccess ||
         init_cnn() != cudaSuccess)
@@ -1016,7 +1006,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     // tables (frames of different sizes do not share them).
     {
         Plan one;
-        plan_frame(one, kPlanResize | kPlanTiles, *params, nullptr, params->max_width, params->max_height, params->max_width);
+        plan_frame(one, kPlanResize, *params, nullptr, params->max_width, params->max_height, params->max_width);
         int64_t s_bound = 0;
         for (const LevelDesc &L : one.levels) {
             int64_t most = 0;
@@ -1037,15 +1027,14 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
         int64_t cnn_bound = 0;
         for (const LevelDesc &L : one.levels)
             cnn_bound += (int64_t)((L.Hc + kCnnTile - 1) / kCnnTile) * ((L.Wc + kCnnTile - 1) / kCnnTile);
-        h->flag_cap = F * std::max<int64_t>(s_bound, (int64_t)one.c_items.size()) + 64;
+        h->flag_cap = F * std::max<int64_t>(s_bound, (int64_t)one.c_tiles) + 64;
         h->desc_cap = round_up(F * (int64_t)one.levels.size() * (int64_t)sizeof(CUtensorMap), 64) + 128 +
                       round_up(2 * (int64_t)std::max(worst.max_wc, 1) * (int64_t)sizeof(CUtensorMap), 64) + 64 +
                       round_up(F * cnn_bound * (int64_t)sizeof(CnnItem), 16) +
                       round_up(F * (int64_t)sizeof(FrameDesc), 16) +
                       round_up(F * (int64_t)one.levels.size() * (int64_t)sizeof(LevelDesc), 16) +
                       round_up(F * (int64_t)one.r_items.size() * (int64_t)sizeof(ResizeItem), 16) +
-                      round_up(F * (int64_t)one.c_items.size() * (int64_t)sizeof(CellItem), 16) +
-                      round_up(4 * F * (int64_t)one.c_items.size() * (int64_t)sizeof(StripItem), 16) +  // 2-row strips
+                      round_up(5 * F * (int64_t)one.c_tiles * (int64_t)sizeof(StripItem), 16) +  // 2-row strips: 4 per tile
                       round_up(F * s_bound * (int64_t)sizeof(SvmItem), 16) +
                       round_up((F * t_bound + 4 * kTcFineItems) * (int64_t)sizeof(TcItem), 16) +
                       round_up(F * (int64_t)one.tabs.size() * 4, 16) + 4096;
@@ -1208,9 +1197,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         invalidate_cache(h);
         p.clear();
         const bool fp32 = (h->p.flags & PD_FLAG_SVM_FP32) != 0;
-        const unsigned what = kPlanResize |
-                              (h->proposal || (h->p.flags & PD_FLAG_HOG_PER_BLOCK) ? kPlanTiles : 0u) |
-                              (fp32 ? kPlanWindows : 0u);
+        const unsigned what = kPlanResize | (fp32 ? kPlanWindows : 0u);
         for (int f = 0; f < n_frames; ++f) {
             int r = plan_frame(p, what, h->p, d_frames[f], widths[f], heights[f], pitches[f],
                                h->proposal ? kSparseTileCost : h->tile_cost, h->proposal);
@@ -1223,7 +1210,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         }
         plan_strips(p, h->sm_count * kStripWarpsPerSm);
         if (p.atlas_rows > h->atlas.rows || p.pyr_bytes > h->pyr_cap || p.score_floats > h->score_cap ||
-            (int64_t)p.s_items.size() > h->flag_cap || (int64_t)p.c_items.size() > h->flag_cap)
+            (int64_t)p.s_items.size() > h->flag_cap || p.c_tiles > h->flag_cap)
             return fail(h, PD_EINVAL, "batch exceeds the arena");
         // full descriptor upload, once per batch shape
         int r = upload_plan(h, s, p, h->packed, h->d_pyr);
@@ -1259,7 +1246,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         if (h->proposal) {
             // learned proposal: keep-logits of every window and the tiles to score
             const bool per_window = !(h->p.flags & PD_FLAG_SVM_FP32);
-            PD_CUDA(h, cudaMemsetAsync(h->c_flag, 0, p.c_items.size() * 4 + 4, q));
+            PD_CUDA(h, cudaMemsetAsync(h->c_flag, 0, (size_t)p.c_tiles * 4 + 4, q));
             PD_CUDA(h, launch_cnn(q, dl, (int)p.levels.size(), dptr<CUtensorMap>(h, o.tmaps),
                                   dptr<CnnItem>(h, o.cnn_items),
                                   (int)p.cnn_items.size(), cnn_weights(h), h->hmap, h->atlas.pitch, h->logits,
@@ -1714,9 +1701,8 @@ int pd_cell_features(pd_handle *h, void *stream, const uint8_t *d_level, int Wk,
         cell_pitch % 16 != 0 || hog_plane < (int64_t)Hc * cell_pitch || lbp_plane < (int64_t)Hc * cell_pitch)
         return fail(h, PD_EINVAL, "pd_cell_features: bad argument");
     Plan p;
-    const bool per_block = (features_of(h->p.flags) & kFeatHogBlock) != 0;
-    plan_level(p, per_block ? kPlanTiles : 0u, 0, 0, Wk, Hk, Wk, Hk, 0, pitch);
-    if (!per_block) plan_strips(p, h->sm_count * kStripWarpsPerSm);
+    plan_level(p, 0u, 0, 0, Wk, Hk, Wk, Hk, 0, pitch);
+    plan_strips(p, h->sm_count * kStripWarpsPerSm);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     Packed o;
     int r = upload_plan(h, s, p, o);

@@ -47,8 +47,8 @@ struct LevelDesc {
                         // weights (2048 - a) | a << 16 (16-byte aligned; unused lanes 0)
     int32_t ytab_off;   // K1 row table: per output row an int2 {byte offset of its top source row's
                         // quad row (source row * 4 * kResizeQP), (8192 - 4 a) | 4 a << 16}
-    int32_t citem0;     // index of this level's first K2+K3 item
-    int32_t ctx;        // K2+K3 tiles per row of cells
+    int32_t citem0;     // index of this level's first cell tile (15 x 8 cells)
+    int32_t ctx;        // cell tiles per row of cells
     int32_t xbnd_off;   // per K1 source-tile column t: first column group whose first source is >= 128 t
     int32_t ybnd_off;   // per K1 source-tile row t: first output row whose source is >= 32 t
     int32_t rgroup;     // K1 output columns per group: 4, or 1 when a group of 4 reaches past the halo
@@ -61,7 +61,6 @@ struct LevelDesc {
 
 // Work items (one CTA each).
 struct ResizeItem { int32_t frame, x0, y0, pad; };   // source tile of a frame
-struct CellItem { int32_t level, cx0, cy0, pad; };   // cell tile of a level
 struct SvmItem { int32_t level, wx0, wy0, shape; };  // window tile of a level, tile shape index
 struct TcItem { int32_t level, wx0, wy0, wy1; };     // tensor-core K4: window columns [wx0, wx0 + 26), rows [wy0, wy1)
 struct StripItem { int32_t level, cx0, cy0, cy1; };  // K2+K3 warp: cells [cx0, cx0 + 15) x rows [cy0, cy1)
@@ -75,7 +74,7 @@ __host__ __device__ inline int resize_quad_index(int d) { return d + (d >> 5); }
 // K1 quad row pitch in words: > resize_quad_index(kResizeBW - 2) and 1 mod 32, so that
 // quad rows sy and sy + 1 start one bank apart
 constexpr int kResizeQP = 193;
-constexpr int kCellTW = 15;     // cells per cell tile along x (8*15+8 = 128 columns: 128 threads, or 32 lanes x 4)
+constexpr int kCellTW = 15;     // cells per cell tile along x (8*15+8 = 128 columns: 32 lanes x 4)
 constexpr int kCellTH = 8;      // cells per cell tile along y
 constexpr int kStripTiles = 4;  // cell tiles per K2+K3 strip (one warp each), top to bottom, at most
 constexpr int kStripWarpsPerSm = 16;  // K2+K3 warps resident per SM (4 CTAs of 4)
@@ -113,7 +112,6 @@ struct CellAtlas {
 };
 
 // One-time per-device kernel attribute set-up (dynamic shared memory opt-in).
-cudaError_t init_cells();
 cudaError_t init_svm();
 cudaError_t init_nms(bool occupancy = true);  // occupancy: also the clusters that fit (for the launch policy)
 cudaError_t init_resize();
@@ -123,15 +121,10 @@ cudaError_t init_resize();
 cudaError_t launch_resize(cudaStream_t s, const FrameDesc *d_frames, const LevelDesc *d_levels,
                           const int32_t *d_tabs, uint8_t *pyr, const ResizeItem *d_items,
                           int n_items, int k1_groups = 8);
-// CTA-per-tile K2+K3 for per-block HOG: feat = kFeatHogBlock | kFeatHog
-// (| kFeatLbp); 36 HOG planes, the 4 block-restricted histograms of every
-// cell, plane 9 q + bin. Other feature sets: cudaErrorInvalidValue (they
-// run on launch_cells_warp).
 constexpr int kFeatHog = 1, kFeatLbp = 2, kFeatHogBlock = 4;
-cudaError_t launch_cells(cudaStream_t s, const LevelDesc *d_levels, const uint8_t *pyr,
-                         CellAtlas atlas, const CellItem *d_items, int n_items, const uint8_t *d_lbp_map,
-                         const uint32_t *c_flag = nullptr, int feat = kFeatHog | kFeatLbp);
-// Default K2+K3 (HOG and / or LBP without per-block HOG): one warp per strip.
+// K2+K3: one warp per strip. feat: HOG and / or LBP; kFeatHogBlock | kFeatHog
+// (| kFeatLbp) for 36 HOG planes, the 4 block-restricted histograms of every
+// cell, plane 9 q + bin.
 cudaError_t init_cells_warp();
 // Persistent warps over a strip queue (*d_queue must be 0 at launch).
 cudaError_t launch_cells_warp(cudaStream_t s, const LevelDesc *d_levels, const uint8_t *pyr, CellAtlas atlas,
