@@ -2,11 +2,21 @@
 //
 // Every pyramid level is a fixed-point bilinear resample (11-bit weights) of
 // the frame itself, not of the previous level (downsampled levels, and the
-// optional upsampled ones placed before them). One CTA owns a 128x32 source
-// tile of one frame: it stages the tile (plus a right halo of up to 32
-// columns and one bottom row) in shared memory once and then writes, for
-// every level of that frame, the output pixels it owns. The frame is read
-// from HBM once for all levels, and each level pixel is written once.
+// optional upsampled ones placed before them). One CTA owns a 128x64 source
+// tile of one frame (128x32 in a small plan): it stages the tile (plus a right
+// halo of up to 32 columns and one bottom row) in shared memory once and then
+// writes, for every level of that frame, the output pixels it owns. The frame
+// is read from HBM once for all levels, and each level pixel is written once.
+//
+// What bounds it: instructions (issue 66% of cycles, the integer-multiply pipe
+// 68%), about 20 per output pixel. A warp's task (8 column groups of a level by
+// all its rows in the tile) costs some 60 instructions before its first row,
+// and rows go 4 at a time, so a taller tile pays less per pixel: 64 x 1242x375
+// frames 234 us in 32-row tiles of 256 threads, 197 us in 64-row tiles of 512
+// (the divisions by the staged width as multiplications are 10 of these).
+// While the 32-row tiles of a plan fit the chip in one round the frame is as
+// slow as its slowest tile, and 512 threads on 32 rows are the faster ones:
+// one 1242x375 frame 19.5 us (256 threads), 18.7 (64 rows), 13.9 (32 rows).
 //
 // Ownership: output row y belongs to the tile row holding its top source row;
 // output columns go in groups of 4 (one 32-bit store), and a group belongs to
@@ -34,26 +44,34 @@
 namespace pd {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;
 constexpr int kTW = kResizeTW;                 // 128 source columns per tile
-constexpr int kTH = kResizeTH;                 // 32 source rows per tile
 constexpr int kTP = 176;                       // staged byte row pitch (>= kResizeBW + 8, 16-byte multiple)
 constexpr int kQP = kResizeQP;                 // quad row pitch in words
 constexpr int kML = PD_MAX_LEVELS;
-constexpr int kStageIters = ((kTH + 1) * ((kResizeBW + 3) / 4) + kThreads - 1) / kThreads;  // staged words per thread
 static_assert(kTP >= kResizeBW + 8 && kTP % 16 == 0, "staged row pitch");
 static_assert(kQP > (kResizeBW - 2) + ((kResizeBW - 2) >> 5) && kQP % 32 == 1 && kQP <= 256, "quad row pitch");
 
-// Dynamic shared memory layout (bytes).
-constexpr int kOffTile = 0;
-constexpr int kOffQuad = kOffTile + (kTH + 1) * kTP;
-constexpr int kOffRng = kOffQuad + ((kTH * kQP * 4 + 15) & ~15);  // int4 per level: first group, groups, first row, rows
-constexpr int kOffCnt = kOffRng + kML * 16;             // int per level: warp tasks (-1: the copied level)
-constexpr int kOffPre = kOffCnt + kML * 4;              // int per level + 1: first task
-constexpr int kOffMisc = kOffPre + (kML + 1) * 4;       // copied level, task counter
-constexpr int kOffLvl = (kOffMisc + 16 + 15) & ~15;     // per level: the fields the task loop reads
-constexpr int kSmemBytes = kOffLvl + kML * 32;
-static_assert(kOffQuad % 16 == 0 && kOffRng % 16 == 0, "alignment");
+// Dynamic shared memory layout (bytes) of a tile of TH source rows.
+template <int TH>
+struct Layout {
+    static constexpr int kTile = 0;
+    static constexpr int kQuad = kTile + (TH + 1) * kTP;
+    static constexpr int kRng = kQuad + ((TH * kQP * 4 + 15) & ~15);  // int4 per level: first group, groups, first row, rows
+    static constexpr int kCnt = kRng + kML * 16;            // int per level: warp tasks (-1: the copied level)
+    static constexpr int kPre = kCnt + kML * 4;             // int per level + 1: first task
+    static constexpr int kMisc = kPre + (kML + 1) * 4;      // copied level, task counter
+    static constexpr int kLvl = (kMisc + 16 + 15) & ~15;    // per level: the fields the task loop reads
+    static constexpr int kBytes = kLvl + kML * 32;
+    static_assert(kQuad % 16 == 0 && kRng % 16 == 0, "alignment");
+};
+static_assert(kResizeCtas * (Layout<2 * kResizeTH>::kBytes + 1024) <= 227 * 1024, "resident CTAs");
+static_assert(kThreads / 8 >= 2 * kResizeTH, "the copied level: 16 bytes per thread, 8 threads per row");
+
+// i / n as i * div20(n) >> 20: exact for i < (kTH + 1) n, n <= 40 (the remainder's
+// excess i (div20(n) n - 2^20) / 2^20 stays below 65 * 40 / 2^20 < 1 / n).
+static_assert((2 * kResizeTH + 1) * ((kResizeBW + 3) / 4) * ((kResizeBW + 3) / 4) < (1 << 20), "div20");
+__device__ __forceinline__ uint32_t div20(int n) { return ((1u << 20) + (uint32_t)n - 1u) / (uint32_t)n; }
 
 // One output pixel: its quad (taps) at shared-memory byte address qa, packed
 // column weights and scaled row weights; the output byte is byte 3.
@@ -71,31 +89,34 @@ __device__ __forceinline__ uint32_t pack4(uint32_t o0, uint32_t o1, uint32_t o2,
 }
 
 // kCG column groups per warp task; the warp's lanes are kCG groups x kRS row slices.
-template <int kCG>
-__global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restrict__ frames,
-                                                        const LevelDesc *__restrict__ levels,
-                                                        const int32_t *__restrict__ tabs,
-                                                        uint8_t *__restrict__ pyr,
-                                                        const ResizeItem *__restrict__ items) {
+template <int kCG, int kTH>
+__global__ void __launch_bounds__(kThreads, kResizeCtas) k_resize(const FrameDesc *__restrict__ frames,
+                                                                  const LevelDesc *__restrict__ levels,
+                                                                  const int32_t *__restrict__ tabs,
+                                                                  uint8_t *__restrict__ pyr,
+                                                                  const ResizeItem *__restrict__ items) {
+    using Lay = Layout<kTH>;
+    constexpr int kStageIters = ((kTH + 1) * ((kResizeBW + 3) / 4) + kThreads - 1) / kThreads;  // staged words per thread
     constexpr int kRS = 32 / kCG;
     extern __shared__ __align__(16) uint8_t smem[];
-    uint8_t *tile = smem + kOffTile;
-    uint32_t *quad = reinterpret_cast<uint32_t *>(smem + kOffQuad);
-    int4 *s_rng = reinterpret_cast<int4 *>(smem + kOffRng);
-    int *s_cnt = reinterpret_cast<int *>(smem + kOffCnt);
-    int *s_pre = reinterpret_cast<int *>(smem + kOffPre);
-    int *s_misc = reinterpret_cast<int *>(smem + kOffMisc);
+    uint8_t *tile = smem + Lay::kTile;
+    uint32_t *quad = reinterpret_cast<uint32_t *>(smem + Lay::kQuad);
+    int4 *s_rng = reinterpret_cast<int4 *>(smem + Lay::kRng);
+    int *s_cnt = reinterpret_cast<int *>(smem + Lay::kCnt);
+    int *s_pre = reinterpret_cast<int *>(smem + Lay::kPre);
+    int *s_misc = reinterpret_cast<int *>(smem + Lay::kMisc);
     // per level: {img_off lo, img_off hi, pitch, Wk}, {rgroup, xtab_off, xq_off, ytab_off}
-    int4 *s_lvl = reinterpret_cast<int4 *>(smem + kOffLvl);
+    int4 *s_lvl = reinterpret_cast<int4 *>(smem + Lay::kLvl);
 
     const ResizeItem it = items[blockIdx.x];
     const FrameDesc fd = frames[it.frame];
     const int tid = threadIdx.x, lane = tid & 31;
     const int n = fd.n_levels;
-    const int tcx = it.x0 / kTW, tcy = it.y0 / kTH;
+    const int tcx = it.x0 / kTW;
+    const int tcy0 = it.y0 / kResizeTH;  // the row bounds are per kResizeTH source rows
+    const int tcy1 = min(tcy0 + kTH / kResizeTH, (fd.H + kResizeTH - 1) / kResizeTH);
 
-
-    // Stage source rows y0 .. y0+32 (clamped to the frame), bytes [x0, x0 + bw)
+    // Stage source rows y0 .. y0+kTH (clamped to the frame), bytes [x0, x0 + bw)
     // with columns at or past the right edge replaced by the last one. Aligned
     // 32-bit loads, each holding at least one byte of the row, realigned by a
     // funnel shift (the frame may be read straight from pinned host memory).
@@ -103,6 +124,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restr
     {
         const int bw = fd.rbw;
         const int nw = (bw + 3) >> 2;
+        const uint32_t inv_nw = div20(nw);
         const int nvalid = min(bw, fd.W - it.x0);
         uint32_t w0[kStageIters], w1[kStageIters];
 #pragma unroll
@@ -110,7 +132,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restr
             const int i = tid + u * kThreads;
             w0[u] = w1[u] = 0u;
             if (i < (kTH + 1) * nw) {
-                const int r = i / nw, j = i - r * nw;
+                const int r = (int)((uint32_t)i * inv_nw >> 20), j = i - r * nw;
                 const int y = min(it.y0 + r, fd.H - 1);
                 const uintptr_t a = reinterpret_cast<uintptr_t>(fd.ptr + (size_t)y * fd.pitch + it.x0);
                 const int m = (int)(a & 3);
@@ -125,7 +147,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restr
         for (int k = tid; k < n; k += kThreads) {
             const LevelDesc &L = levels[fd.first_level + k];
             const int gs = __ldg(tabs + L.xbnd_off + tcx), ge = __ldg(tabs + L.xbnd_off + tcx + 1);
-            const int rs = __ldg(tabs + L.ybnd_off + tcy), re = __ldg(tabs + L.ybnd_off + tcy + 1);
+            const int rs = __ldg(tabs + L.ybnd_off + tcy0), re = __ldg(tabs + L.ybnd_off + tcy1);
             const bool copy = L.Wk == fd.W && L.Hk == fd.H && L.img_pitch % 16 == 0 &&
                               ((reinterpret_cast<uintptr_t>(pyr + L.img_off)) & 15) == 0;
             const int ng = ge - gs, nr = re - rs;
@@ -142,7 +164,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restr
         for (int u = 0; u < kStageIters; ++u) {
             const int i = tid + u * kThreads;
             if (i < (kTH + 1) * nw) {
-                const int r = i / nw, j = i - r * nw;
+                const int r = (int)((uint32_t)i * inv_nw >> 20), j = i - r * nw;
                 const int y = min(it.y0 + r, fd.H - 1);
                 const uint8_t *p = fd.ptr + (size_t)y * fd.pitch + it.x0;
                 const int m = (int)(reinterpret_cast<uintptr_t>(p) & 3);
@@ -193,8 +215,9 @@ __global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restr
     // at word resize_quad_index(c) of quad row r (the skew spreads strided reads over banks).
     {
         const int nq4 = (fd.rbw - 1 + 3) >> 2;
+        const uint32_t inv_nq4 = div20(nq4);
         for (int i = tid; i < kTH * nq4; i += kThreads) {
-            const int r = i / nq4, j = i - r * nq4;
+            const int r = (int)((uint32_t)i * inv_nq4 >> 20), j = i - r * nq4;
             const uint8_t *t0 = tile + r * kTP + 4 * j;
             const uint32_t a0 = *reinterpret_cast<const uint32_t *>(t0);
             const uint32_t a1 = *reinterpret_cast<const uint32_t *>(t0 + 4);
@@ -215,7 +238,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restr
         const LevelDesc &L = levels[fd.first_level + kc];
         const int r = tid >> 3, c = (tid & 7) * 16;
         const int y = it.y0 + r, x = it.x0 + c;
-        if (y < L.Hk && x < L.Wk) {
+        if (r < kTH && y < L.Hk && x < L.Wk) {
             const uint4 v = *reinterpret_cast<const uint4 *>(tile + r * kTP + c);
             uint8_t *o = pyr + L.img_off + (size_t)y * L.img_pitch + x;
             if (x + 16 <= L.Wk) {
@@ -231,7 +254,8 @@ __global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restr
     __syncthreads();
 
     // Every other level: warp tasks of kCG column groups x all the tile's rows
-    // of the level, taken from a shared counter. Lane = (row slice j, group c):
+    // of the level; a warp's first is its own, the others come off a shared
+    // counter. Lane = (row slice j, group c):
     // it keeps its group's weights and quad addresses in registers and walks
     // rows j, j + 4, ... (consecutive groups of a row store 32 contiguous bytes).
     const int total = s_pre[n];
@@ -239,11 +263,11 @@ __global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restr
         (uint32_t)__cvta_generic_to_shared(quad) - (uint32_t)(it.y0 * kQP * 4);
     const int c = lane & (kCG - 1), j = lane / kCG;
     int k = -1;
-    for (;;) {
-        int t = 0;
-        if (lane == 0) t = atomicAdd(&s_misc[1], 1);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= total) break;
+    auto next = [&] {
+        const int n = lane == 0 ? kThreads / 32 + atomicAdd(&s_misc[1], 1) : 0;
+        return __shfl_sync(0xffffffffu, n, 0);
+    };
+    for (int t = tid >> 5; t < total; t = next()) {
         while (t >= s_pre[k + 1]) ++k;
         const int4 rg = s_rng[k];
         const int g = (t - s_pre[k]) * kCG + c;
@@ -302,23 +326,30 @@ __global__ void __launch_bounds__(kThreads, 6) k_resize(const FrameDesc *__restr
 
 }  // namespace
 
+namespace {
+using ResizeFn = void (*)(const FrameDesc *, const LevelDesc *, const int32_t *, uint8_t *, const ResizeItem *);
+// [column groups per task 4, 8, 16][tile rows kResizeTH, 2 kResizeTH]
+const ResizeFn kResizeFns[3][2] = {{k_resize<4, kResizeTH>, k_resize<4, 2 * kResizeTH>},
+                                   {k_resize<8, kResizeTH>, k_resize<8, 2 * kResizeTH>},
+                                   {k_resize<16, kResizeTH>, k_resize<16, 2 * kResizeTH>}};
+const int kResizeSmem[2] = {Layout<kResizeTH>::kBytes, Layout<2 * kResizeTH>::kBytes};
+}  // namespace
+
 cudaError_t init_resize() {
-    cudaError_t e = cudaFuncSetAttribute(k_resize<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_resize<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_resize<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    return e;
+    for (int i = 0; i < 6; ++i) {
+        const cudaError_t e = cudaFuncSetAttribute(kResizeFns[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   kResizeSmem[i % 2]);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_resize(cudaStream_t s, const FrameDesc *d_frames, const LevelDesc *d_levels,
                           const int32_t *d_tabs, uint8_t *pyr, const ResizeItem *d_items,
-                          int n_items, int k1_groups) {
+                          int n_items, bool tall, int k1_groups) {
     if (n_items <= 0) return cudaSuccess;
-    if (k1_groups == 4)
-        k_resize<4><<<n_items, kThreads, kSmemBytes, s>>>(d_frames, d_levels, d_tabs, pyr, d_items);
-    else if (k1_groups == 16)
-        k_resize<16><<<n_items, kThreads, kSmemBytes, s>>>(d_frames, d_levels, d_tabs, pyr, d_items);
-    else
-        k_resize<8><<<n_items, kThreads, kSmemBytes, s>>>(d_frames, d_levels, d_tabs, pyr, d_items);
+    const int g = k1_groups == 4 ? 0 : k1_groups == 16 ? 2 : 1;
+    kResizeFns[g][tall]<<<n_items, kThreads, kResizeSmem[tall], s>>>(d_frames, d_levels, d_tabs, pyr, d_items);
     return cudaGetLastError();
 }
 

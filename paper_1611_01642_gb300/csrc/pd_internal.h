@@ -67,7 +67,8 @@ struct StripItem { int32_t level, cx0, cy0, cy1; };  // K2+K3 warp: cells [cx0, 
 
 // Tiles.
 constexpr int kResizeTW = 128;  // source tile width  (pixels)
-constexpr int kResizeTH = 32;   // source tile height (pixels)
+constexpr int kResizeTH = 32;   // source tile height (pixels); plans of many tiles take 2 kResizeTH
+constexpr int kResizeCtas = 3;  // K1 CTAs resident per SM
 constexpr int kResizeBW = 160;  // source bytes staged per tile row at most (tile + right halo)
 // K1 shared-memory quad word of source column d of a tile row (skewed by d / 32)
 __host__ __device__ inline int resize_quad_index(int d) { return d + (d >> 5); }
@@ -117,10 +118,10 @@ cudaError_t init_nms(bool occupancy = true);  // occupancy: also the clusters th
 cudaError_t init_resize();
 
 // Kernel launchers (host functions defined next to their kernels).
-// k1_groups: column groups per warp task (4, 8 or 16)
+// tall: tiles of 2 kResizeTH rows; k1_groups: column groups per warp task (4, 8 or 16)
 cudaError_t launch_resize(cudaStream_t s, const FrameDesc *d_frames, const LevelDesc *d_levels,
                           const int32_t *d_tabs, uint8_t *pyr, const ResizeItem *d_items,
-                          int n_items, int k1_groups = 8);
+                          int n_items, bool tall, int k1_groups = 8);
 constexpr int kFeatHog = 1, kFeatLbp = 2, kFeatHogBlock = 4;
 // K2+K3: one warp per strip. feat: HOG and / or LBP; kFeatHogBlock | kFeatHog
 // (| kFeatLbp) for 36 HOG planes, the 4 block-restricted histograms of every
