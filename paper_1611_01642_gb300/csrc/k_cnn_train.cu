@@ -15,18 +15,23 @@
 //
 // What bounds them: the convolutions are 3 x 468 multiply-adds per pyramid
 // pixel, and dz is fp32, so they run on the FP32 pipe, two multiply-adds per
-// instruction (fma.rn.f32x2 over pairs of channels). Every kernel walks a
-// contiguous share of the batch's tiles with persistent blocks; the operands
-// of a tile sit in shared memory, columns split by parity so that a stride-2
-// window is unit stride, and a thread holds 4 to 8 positions times 8 to 16
-// channels, so that one broadcast weight load feeds 4 to 8 instructions.
-// Weight gradients stay in registers over a block's whole share and leave as
-// one partial per block, summed in block order by the last kernel.
+// instruction (fma.rn.f32x2 over pairs of channels or positions). Every kernel
+// walks a contiguous share of the batch's tiles with persistent blocks; the
+// operands of a tile sit in shared memory, the next tile's arrive there
+// (cp.async) while this one is worked on, and a thread holds 4 to 8 positions
+// times 4 to 16 channels (or 4 channels times 9 taps), so that one broadcast
+// load feeds 4 to 8 instructions. Weight gradients stay in registers over a
+// block's whole share and leave as one partial per block, summed in block
+// order by the last kernel.
 // 4 x 1280x720 frames (38 M pyramid pixels, 36 levels each), one step:
 // 74.4 -> 6.67 ms against one thread per position with all levels of a weight's
-// gradient in one block (weight gradient of layer 1 and data gradient of layer 2
-// 49.8 -> 2.05, weight gradients of layers 2 and 3 9.2 -> 1.31 and 6.6 -> 0.75,
-// data gradient of layer 3 6.1 -> 0.55, forward convolutions 2.5 -> 1.65 ms).
+// gradient in one block, and 6.67 -> 3.55 ms by fetching ahead (half of every
+// warp's waiting was for the tile's loads, with 8 to 16 warps per SM to hide
+// them): weight gradient of layer 1 with the data gradient of layer 2 2.05 ->
+// 0.72, weight gradients of layers 2 and 3 1.31 -> 0.76 and 0.75 -> 0.39, data
+// gradient of layer 3 0.55 -> 0.33, forward convolutions 0.84 -> 0.49 and 0.61
+// -> 0.34 ms. The FP32 pipe is now 54 to 76% busy in them; in the two data
+// gradients shared memory's 75% comes first.
 #include "pd_internal.h"
 
 #include <cuda_bf16.h>
@@ -67,6 +72,25 @@ struct Walk {
         }
     }
 };
+
+// ---- staging: before a block works on a tile it starts the copies of the next
+// one into its other buffer (cp.async, 16 bytes per copy, zeros outside the
+// plane); a thread waits for its own copies and the block's barrier hands them over.
+__device__ __forceinline__ uint32_t smem_at(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// 16 bytes to shared memory, of which the first n come from src and the rest are 0 (n <= 0: all)
+__device__ __forceinline__ void copy16(void *dst, const void *src, int n) {
+    n = min(max(n, 0), 16);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_at(dst)), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// One chunk of row y, elements [x, x + 16 / sizeof(T)), of a plane of H rows and
+// W valid columns (row pitch P); zeros outside.
+template <class T>
+__device__ __forceinline__ void copy_row16(void *dst, const T *plane, int y, int x, int H, int W, int P) {
+    const bool in = y >= 0 && y < H && x >= 0 && x < W;
+    copy16(dst, in ? plane + (int64_t)y * P + x : plane, in ? (int)sizeof(T) * (W - x) : 0);
+}
 
 constexpr int kXE = 64, kXO = 68;  // input tile row pitches: even columns, odd columns (from -1)
 
@@ -160,76 +184,84 @@ __global__ void __launch_bounds__(256) t_conv1(const TrainLevel *__restrict__ tl
     }
 }
 
-constexpr int kAP = 36;  // bf16 row pitch of a staged activation tile (32 even columns, 33 odd ones)
-
 // ---- layers 2 and 3: 32 x 8 positions per tile, 4 positions x 16 output
-// channels per thread, 16 input channels staged at a time. Per input channel
-// and window row: 3 activation loads and 12 broadcast weight loads for 96
-// packed multiply-adds.
+// channels per thread; kCS input channels are worked on while the next kCS
+// (or the next tile's first) arrive. Activations stay two bf16 columns to a
+// word: per input channel and window row 2 activation loads and 12 broadcast
+// weight loads for 96 packed multiply-adds.
+constexpr int kAP = 36;  // words per staged activation row: columns 2 j0 - 8 ..
+template <int CIN>
+struct ConvSmem {
+    static constexpr int kCS = 128 / CIN;  // 8 or 4: three blocks per SM
+    float ws[CIN * 9 * 32];                // [c][tap][o]
+    uint32_t as[2][kCS * 17 * kAP];
+};
 template <int CIN, bool LAST>
 __global__ void __launch_bounds__(128) t_conv23(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
                                                 const __nv_bfloat16 *__restrict__ act, const float *__restrict__ w,
                                                 const float *__restrict__ b, __nv_bfloat16 *__restrict__ out16,
                                                 float *__restrict__ out32) {
-    extern __shared__ __align__(16) float smem_f[];
-    float *ws = smem_f;                                                      // [CIN][9][32]
-    __nv_bfloat16 *E = reinterpret_cast<__nv_bfloat16 *>(ws + CIN * 9 * 32);  // [16][17][kAP]
-    __nv_bfloat16 *O = E + 16 * 17 * kAP;
-    __shared__ float bs[32];
+    constexpr int kCS = ConvSmem<CIN>::kCS;
+    extern __shared__ __align__(16) unsigned char smem_b[];
+    ConvSmem<CIN> &S = *reinterpret_cast<ConvSmem<CIN> *>(smem_b);
     const int tid = threadIdx.x;
     for (int i = tid; i < CIN * 9 * 32; i += 128) {
         const int o = i & 31, ct = i >> 5;
-        ws[i] = w[o * CIN * 9 + ct];
+        S.ws[i] = w[o * CIN * 9 + ct];
     }
-    if (tid < 32) bs[tid] = b[tid];
     const int o0 = 16 * (tid >> 6), g = tid & 7, ir = (tid >> 3) & 7;
     constexpr int GRID = LAST ? 2 : 0;
-    for (Walk<GRID> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+    Walk<GRID> wk(tl, n_tl, n_tiles);
+    auto fetch = [&](uint32_t *as, int cb) {  // this thread's share of channels cb .. of the tile of wk
         const TrainLevel &T = tl[wk.k];
         const int Hi = LAST ? T.H2 : T.H1, Wi = LAST ? T.W2 : T.W1, Pi = LAST ? T.P2 : T.P1;
-        const int Ho = LAST ? T.H3 : T.H2, Wo = LAST ? T.W3 : T.W2, Po = LAST ? T.P3 : T.P2;
-        const int64_t in_off = LAST ? T.a2 : T.a1;
-        const int ntx = (Wo + 31) / 32, lt = wk.local();
+        const int ntx = ((LAST ? T.W3 : T.W2) + 31) / 32, lt = wk.local();
         const int i0 = 8 * (lt / ntx), j0 = 32 * (lt % ntx);
+        const __nv_bfloat16 *a = act + (LAST ? T.a2 : T.a1) + (int64_t)cb * Hi * Pi;
+        for (int e = tid; e < kCS * 17 * 9; e += 128) {
+            const int cr = e / 9, q = e - 9 * cr, cc = cr / 17, r = cr - 17 * cc;
+            copy_row16(as + 4 * e, a + (int64_t)cc * Hi * Pi, 2 * i0 + r - 1, 2 * j0 - 8 + 8 * q, Hi, Wi, Pi);
+        }
+    };
+    f32x2 bias[8];
+#pragma unroll
+    for (int o = 0; o < 8; ++o) bias[o] = pack2(b[o0 + 2 * o], b[o0 + 2 * o + 1]);
+    int buf = 0;
+    if (wk.valid()) fetch(S.as[0], 0);
+    while (wk.valid()) {
+        const TrainLevel &T = tl[wk.k];
+        const int Ho = LAST ? T.H3 : T.H2, Wo = LAST ? T.W3 : T.W2, Po = LAST ? T.P3 : T.P2;
+        const int64_t out_off = LAST ? T.a3 : T.a2;
+        const int ntx = (Wo + 31) / 32, lt = wk.local();
+        const int i = 8 * (lt / ntx) + ir, j = 32 * (lt % ntx) + 4 * g;
         f32x2 acc[4][8];
-        for (int c0 = 0; c0 < CIN; c0 += 16) {
-            __syncthreads();
-            for (int i = tid; i < 16 * 17 * 33; i += 128) {
-                const int cr = i / 33, m = i - 33 * cr - 1;
-                const int cc = cr / 17, r = cr - 17 * cc;
-                const int y = 2 * i0 + r - 1, x = 2 * (j0 + m);
-                uint32_t v = 0u;
-                if (y >= 0 && y < Hi && x >= 0 && x < Wi) {
-                    v = *reinterpret_cast<const uint32_t *>(act + in_off + ((int64_t)(c0 + cc) * Hi + y) * Pi + x);
-                    if (x + 1 >= Wi) v &= 0xffffu;
-                }
-                if (m >= 0) reinterpret_cast<uint16_t *>(E)[cr * kAP + m] = (uint16_t)v;
-                reinterpret_cast<uint16_t *>(O)[cr * kAP + m + 1] = (uint16_t)(v >> 16);
-            }
-            __syncthreads();
-            if (c0 == 0) {
 #pragma unroll
-                for (int o = 0; o < 8; ++o) {
-                    const f32x2 bb = pack2(bs[o0 + 2 * o], bs[o0 + 2 * o + 1]);
+        for (int o = 0; o < 8; ++o)
 #pragma unroll
-                    for (int p = 0; p < 4; ++p) acc[p][o] = bb;
-                }
+            for (int p = 0; p < 4; ++p) acc[p][o] = bias[o];
+#pragma unroll 1
+        for (int cb = 0; cb < CIN; cb += kCS, buf ^= 1) {
+            copies_done();
+            __syncthreads();  // these channels are here, and the other buffer is free
+            if (cb + kCS < CIN) {
+                fetch(S.as[buf ^ 1], cb + kCS);
+            } else {
+                wk.step(n_tiles);
+                if (wk.valid()) fetch(S.as[buf ^ 1], 0);
             }
 #pragma unroll 1
-            for (int c = 0; c < 16; ++c) {
+            for (int c = 0; c < kCS; ++c) {
 #pragma unroll
                 for (int dy = 0; dy < 3; ++dy) {
-                    const int row = (c * 17 + 2 * ir + dy) * kAP + 4 * g;
-                    const uint2 e = *reinterpret_cast<const uint2 *>(E + row);
-                    const uint2 od = *reinterpret_cast<const uint2 *>(O + row);
-                    const uint32_t ol = reinterpret_cast<const uint16_t *>(O)[row + 4];
-                    const f32x2 v0[4] = {dup2(bf_lo(od.x)), dup2(bf_hi(od.x)), dup2(bf_lo(od.y)), dup2(bf_hi(od.y))};
-                    const f32x2 v1[4] = {dup2(bf_lo(e.x)), dup2(bf_hi(e.x)), dup2(bf_lo(e.y)), dup2(bf_hi(e.y))};
-                    const f32x2 v2[4] = {v0[1], v0[2], v0[3], dup2(bf_lo(ol))};
+                    const uint32_t *row = S.as[buf] + (c * 17 + 2 * ir + dy) * kAP + 4 + 4 * g;
+                    const uint4 u = *reinterpret_cast<const uint4 *>(row);
+                    const f32x2 v0[4] = {dup2(bf_hi(row[-1])), dup2(bf_hi(u.x)), dup2(bf_hi(u.y)), dup2(bf_hi(u.z))};
+                    const f32x2 v1[4] = {dup2(bf_lo(u.x)), dup2(bf_lo(u.y)), dup2(bf_lo(u.z)), dup2(bf_lo(u.w))};
+                    const f32x2 v2[4] = {v0[1], v0[2], v0[3], dup2(bf_hi(u.w))};
 #pragma unroll
                     for (int dx = 0; dx < 3; ++dx) {
                         const f32x2 *v = dx == 0 ? v0 : dx == 1 ? v1 : v2;
-                        const float *wp = ws + ((c0 + c) * 9 + dy * 3 + dx) * 32 + o0;
+                        const float *wp = S.ws + ((cb + c) * 9 + dy * 3 + dx) * 32 + o0;
 #pragma unroll
                         for (int o = 0; o < 8; o += 2) {
                             const ulonglong2 ww = *reinterpret_cast<const ulonglong2 *>(wp + 2 * o);
@@ -243,14 +275,13 @@ __global__ void __launch_bounds__(128) t_conv23(const TrainLevel *__restrict__ t
                 }
             }
         }
-        const int i = i0 + ir, j = j0 + 4 * g;
         if (i < Ho && j < Po) {
 #pragma unroll
             for (int o = 0; o < 16; ++o) {
                 float v[4];
 #pragma unroll
                 for (int p = 0; p < 4; ++p) v[p] = fmaxf(o & 1 ? hi2(acc[p][o >> 1]) : lo2(acc[p][o >> 1]), 0.f);
-                const int64_t at = (LAST ? T.a3 : T.a2) + ((int64_t)(o0 + o) * Ho + i) * Po + j;
+                const int64_t at = out_off + ((int64_t)(o0 + o) * Ho + i) * Po + j;
                 if (LAST) {
                     *reinterpret_cast<float4 *>(out32 + at) = make_float4(v[0], v[1], v[2], v[3]);
                 } else {
@@ -344,14 +375,16 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // ---- gradients of V, bv (32 x 16 windows per tile in shared memory, one
 // thread per template position and half of the rows) and of wh, bh (32 x 8
-// cells per tile, a warp per 4 channels). Partial p of a block: 0..127 V,
+// cells per tile, a warp per 4 channels; it also turns a3 into dz3 = wh dh (a3 > 0),
+// in place, 0 outside the cells). Partial p of a block: 0..127 V,
 // 128 bv, 129..160 wh, 161 bh.
 constexpr int kSmallParts = 162;
 __global__ void __launch_bounds__(256) t_small_grads(const TrainLevel *__restrict__ tl, int n_tl, int n_win_tiles,
                                                      int n_cell_tiles, const LevelDesc *__restrict__ levels,
                                                      const float *__restrict__ dz, const float *__restrict__ hmap,
                                                      const float *__restrict__ dh, int32_t hp,
-                                                     const float *__restrict__ a3, float *__restrict__ part) {
+                                                     const float *__restrict__ wh, float *__restrict__ a3,
+                                                     float *__restrict__ part) {
     __shared__ float sd[16 * 32], sh[31 * 40], red[256 + 8];
     const int tid = threadIdx.x, q = tid & 127, half = tid >> 7, lane = tid & 31, warp = tid >> 5;
     const int r = q >> 3, s = q & 7;
@@ -381,22 +414,32 @@ __global__ void __launch_bounds__(256) t_small_grads(const TrainLevel *__restric
         }
     }
     float aw[4] = {0.f, 0.f, 0.f, 0.f}, ab = 0.f;
+    const float4 wh4 = reinterpret_cast<const float4 *>(wh)[warp];
+    const float who[4] = {wh4.x, wh4.y, wh4.z, wh4.w};
     for (Walk<2> wk(tl, n_tl, n_cell_tiles); wk.valid(); wk.step(n_cell_tiles)) {
         const TrainLevel &T = tl[wk.k];
         const LevelDesc &L = levels[T.level];
         const int ntx = (T.W3 + 31) / 32, lt = wk.local();
         const int y0 = 8 * (lt / ntx), x = 32 * (lt % ntx) + lane;
         const int64_t plane = (int64_t)T.H3 * T.P3;
+        if (x >= T.W3) continue;
+        float *src = a3 + T.a3 + 4 * warp * plane + (int64_t)y0 * T.P3 + x;
+        const float *dp = dh + (int64_t)(L.cell_row + y0) * hp + x;
+        float d[8], v[8][4];
 #pragma unroll
         for (int yy = 0; yy < 8; ++yy) {
-            const int y = y0 + yy;
-            if (y < L.Hc && x < L.Wc) {
-                const float d = dh[(int64_t)(L.cell_row + y) * hp + x];
-                const float *src = a3 + T.a3 + 4 * warp * plane + (int64_t)y * T.P3 + x;
+            d[yy] = y0 + yy < L.Hc && x < L.Wc ? dp[(int64_t)yy * hp] : 0.f;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) aw[c] = fmaf(d, src[c * plane], aw[c]);
-                ab += d;
+            for (int c = 0; c < 4; ++c) v[yy][c] = y0 + yy < T.H3 ? src[c * plane + yy * T.P3] : 0.f;
+        }
+#pragma unroll
+        for (int yy = 0; yy < 8; ++yy) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                aw[c] = fmaf(d[yy], v[yy][c], aw[c]);
+                if (y0 + yy < T.H3) src[c * plane + yy * T.P3] = v[yy][c] > 0.f ? who[c] * d[yy] : 0.f;
             }
+            ab += d[yy];
         }
     }
     float *out = part + (int64_t)blockIdx.x * kSmallParts;
@@ -414,28 +457,20 @@ __global__ void __launch_bounds__(256) t_small_grads(const TrainLevel *__restric
     if (tid == 0) out[161] = ab;
 }
 
-// dz3[o] of layer-3 position (i, j): wh[o] dh (a3 > 0) on the cells, else 0.
-__device__ __forceinline__ float dz3_at(const TrainLevel &T, const LevelDesc &L, const float *a3, const float *dh,
-                                        int32_t hp, float who, int o, int i, int j) {
-    if (i >= L.Hc || j >= L.Wc) return 0.f;
-    const float a = a3[T.a3 + ((int64_t)o * T.H3 + i) * T.P3 + j];
-    return a > 0.f ? who * dh[(int64_t)(L.cell_row + i) * hp + j] : 0.f;
-}
-
 // Data gradient of a stride-2 layer for two horizontally adjacent quads of
 // input positions (2i, 2i+1) x (4 columns) and 8 input channels: a quad takes
 // 9 products per (output channel, input channel) from the 2 x 2 output
 // positions it reaches. d: the tile's output gradients [32][dplane], row pitch
-// DP, at (i, j); ws: [32 o][9 taps][CIN] weights at the thread's channels.
+// DP, at (i, j); ws: [32 o][9 taps][CIN] weights at the thread's 2 NP channels.
 // acc[quad][2 * row + column][channel pair].
-template <int CIN, int DP>
-__device__ __forceinline__ void quad_pair(const float *d, int dplane, const float *ws, f32x2 (&acc)[2][4][4]) {
+template <int CIN, int DP, int NP>
+__device__ __forceinline__ void quad_pair(const float *d, int dplane, const float *ws, f32x2 (&acc)[2][4][NP]) {
 #pragma unroll
     for (int q = 0; q < 2; ++q)
 #pragma unroll
         for (int p = 0; p < 4; ++p)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[q][p][c] = 0ull;
+            for (int c = 0; c < NP; ++c) acc[q][p][c] = 0ull;
 #pragma unroll 1
     for (int o = 0; o < 32; ++o) {
         const float *dp = d + o * dplane;
@@ -450,16 +485,18 @@ __device__ __forceinline__ void quad_pair(const float *d, int dplane, const floa
         constexpr int kCol[9] = {0, 1, 0, 0, 0, 1, 0, 1, 0};
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(wo + kTap[k] * CIN);
-            const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(wo + kTap[k] * CIN + 4);
+            ulonglong2 w[NP / 2];
+#pragma unroll
+            for (int c = 0; c < NP / 2; ++c) w[c] = *reinterpret_cast<const ulonglong2 *>(wo + kTap[k] * CIN + 4 * c);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const f32x2 v = kRow[k] ? bot[q + kCol[k]] : top[q + kCol[k]];
-                f32x2(&a)[4] = acc[q][kPos[k]];
-                a[0] = fma2(w0.x, v, a[0]);
-                a[1] = fma2(w0.y, v, a[1]);
-                a[2] = fma2(w1.x, v, a[2]);
-                a[3] = fma2(w1.y, v, a[3]);
+                f32x2(&a)[NP] = acc[q][kPos[k]];
+#pragma unroll
+                for (int c = 0; c < NP / 2; ++c) {
+                    a[2 * c] = fma2(w[c].x, v, a[2 * c]);
+                    a[2 * c + 1] = fma2(w[c].y, v, a[2 * c + 1]);
+                }
             }
         }
     }
@@ -467,52 +504,71 @@ __device__ __forceinline__ void quad_pair(const float *d, int dplane, const floa
 
 // ---- dz2 = (a2 > 0) * data gradient of layer 3: a tile is 16 x 8 quads
 // (32 x 16 layer-2 positions), 64 quad pairs x 4 groups of 8 channels.
-constexpr int kD3P = 18;  // staged dz3 row pitch (17 columns)
+constexpr int kD3P = 20;  // staged dz3 row pitch (17 columns)
+struct Dz2Smem {
+    float ws[32 * 9 * 32];           // [o][tap][c]
+    float ds[2][32 * 9 * kD3P];      // dz3 [o][i][j]
+    __nv_bfloat16 a2[32 * 16 * 32];  // [c][row][column] of the tile worked on
+};
 __global__ void __launch_bounds__(256) t_dz2(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
-                                             const LevelDesc *__restrict__ levels, const float *__restrict__ a3,
-                                             const float *__restrict__ dh, int32_t hp, const float *__restrict__ wh,
-                                             const float *__restrict__ w, const __nv_bfloat16 *__restrict__ act,
-                                             float *__restrict__ dz2) {
-    extern __shared__ __align__(16) float smem_f[];
-    float *ws = smem_f;               // [32 o][9][32 c]
-    float *ds = smem_f + 32 * 9 * 32;  // [32 o][9][kD3P]
-    __shared__ float whs[32];
+                                             const float *__restrict__ dz3, const float *__restrict__ w,
+                                             const __nv_bfloat16 *__restrict__ act, float *__restrict__ dz2) {
+    extern __shared__ __align__(16) unsigned char smem_b[];
+    Dz2Smem &S = *reinterpret_cast<Dz2Smem *>(smem_b);
     const int tid = threadIdx.x;
     for (int i = tid; i < 32 * 9 * 32; i += 256) {
         const int c = i & 31, ot = i >> 5, o = ot / 9;
-        ws[i] = w[(o * 32 + c) * 9 + ot - 9 * o];
+        S.ws[i] = w[(o * 32 + c) * 9 + ot - 9 * o];
     }
-    if (tid < 32) whs[tid] = wh[tid];
-    const int c0 = 8 * (tid >> 6), qx = tid & 7, qr = (tid >> 3) & 7;
-    for (Walk<3> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+    Walk<3> wk(tl, n_tl, n_tiles);
+    auto fetch = [&](float *ds) {  // this thread's share of the tile of wk
         const TrainLevel &T = tl[wk.k];
-        const LevelDesc &L = levels[T.level];
         const int ntx = (T.W3 + 15) / 16, lt = wk.local();
-        const int i0 = 8 * (lt / ntx), j0 = 16 * (lt % ntx);
-        __syncthreads();
-        for (int e = tid; e < 32 * 9 * 17; e += 256) {
-            const int oi = e / 17, j = e - 17 * oi, o = oi / 9, i = oi - 9 * o;
-            ds[oi * kD3P + j] = dz3_at(T, L, a3, dh, hp, whs[o], o, i0 + i, j0 + j);
+        const int i0 = 8 * (lt / ntx), j0 = 16 * (lt % ntx), H3 = T.H3, W3 = T.W3, P3 = T.P3;
+        const float *d = dz3 + T.a3;
+        for (int e = tid; e < 32 * 9 * 5; e += 256) {
+            const int oi = e / 5, q = e - 5 * oi, o = oi / 9, i = oi - 9 * o;
+            copy_row16(ds + 4 * e, d + (int64_t)o * H3 * P3, i0 + i, j0 + 4 * q, H3, W3, P3);
         }
-        __syncthreads();
+    };
+    const int c0 = 8 * (tid >> 6), qx = tid & 7, qr = (tid >> 3) & 7;
+    if (wk.valid()) fetch(S.ds[0]);
+#pragma unroll 1
+    for (int b = 0; wk.valid(); b ^= 1) {
+        copies_done();
+        __syncthreads();  // this tile is here, the other buffer and the mask are free
+        const TrainLevel &T = tl[wk.k];
+        const int H2 = T.H2, W2 = T.W2, P2 = T.P2;
+        const int ntx = (T.W3 + 15) / 16, lt = wk.local();
+        const int y0 = 16 * (lt / ntx), x0 = 32 * (lt % ntx);
+        const __nv_bfloat16 *a2 = act + T.a2;
+        float *out = dz2 + T.d2;
+#pragma unroll
+        for (int e = tid; e < 32 * 16 * 4; e += 256) {
+            const int c = e >> 6, r = (e >> 2) & 15, q = e & 3;
+            copy_row16(S.a2 + 8 * e, a2 + (int64_t)c * H2 * P2, y0 + r, x0 + 8 * q, H2, W2, P2);
+        }
+        wk.step(n_tiles);
+        if (wk.valid()) fetch(S.ds[b ^ 1]);
         f32x2 acc[2][4][4];
-        quad_pair<32, kD3P>(ds + qr * kD3P + 2 * qx, 9 * kD3P, ws + c0, acc);
-        const int x = 2 * j0 + 4 * qx;
+        quad_pair<32, kD3P, 4>(S.ds[b] + qr * kD3P + 2 * qx, 9 * kD3P, S.ws + c0, acc);
+        copies_done();
+        __syncthreads();  // the mask is there
+        const int x = x0 + 4 * qx;
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
-            const int y = 2 * (i0 + qr) + a;
-            if (y >= T.H2 || x >= T.P2) continue;
+            const int y = y0 + 2 * qr + a;
+            if (y >= H2 || x >= P2) continue;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                const int64_t at = ((int64_t)(c0 + c) * T.H2 + y) * T.P2 + x;
-                const uint2 m = *reinterpret_cast<const uint2 *>(act + T.a2 + at);
+                const uint2 m = *reinterpret_cast<const uint2 *>(S.a2 + ((c0 + c) * 16 + 2 * qr + a) * 32 + 4 * qx);
                 float v[4];
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
                     const f32x2 s = acc[p >> 1][2 * a + (p & 1)][c >> 1];
                     v[p] = c & 1 ? hi2(s) : lo2(s);
                 }
-                *reinterpret_cast<float4 *>(dz2 + T.d2 + at) =
+                *reinterpret_cast<float4 *>(out + ((int64_t)(c0 + c) * H2 + y) * P2 + x) =
                     make_float4(bf_lo(m.x) > 0.f ? v[0] : 0.f, bf_hi(m.x) > 0.f ? v[1] : 0.f,
                                 bf_lo(m.y) > 0.f ? v[2] : 0.f, bf_hi(m.y) > 0.f ? v[3] : 0.f);
             }
@@ -521,89 +577,125 @@ __global__ void __launch_bounds__(256) t_dz2(const TrainLevel *__restrict__ tl, 
 }
 
 // ---- layer 1's weight gradient. dz1 = (a1 > 0) * data gradient of layer 2 is
-// only needed for it, so a thread keeps its 8 positions x 8 channels of dz1 in
+// only needed for it, so a thread keeps its 8 positions x 4 channels of dz1 in
 // registers and adds their products with the input pixels to its own sums;
 // dz1 is never written (it would be 2 x 64 bytes per position of traffic). A
-// tile is 32 x 8 quads (64 x 16 layer-1 positions): 128 quad pairs x 2 channel groups.
-constexpr int kD2P = 34;  // staged dz2 row pitch (33 columns)
+// tile is 32 x 8 quads (64 x 16 layer-1 positions): 128 quad pairs x 4 channel
+// groups. (8 channels per thread, 8 warps and a ninth to copy: 168 registers, so
+// that the loads of the weights were waited for, 1.01 ms against 0.72.)
+constexpr int kD2P = 36;  // staged dz2 row pitch (33 columns)
 constexpr int kW1Parts = 160;
-__global__ void __launch_bounds__(256, 1) t_dw1(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
+struct Dw1Stage {
+    float ds[32 * 9 * kD2P];         // dz2 [o][i][j]
+    __nv_bfloat16 a1[16 * 16 * 64];  // [c][row][column]
+    uint8_t raw[33 * 144];           // input rows, bytes from column 4 j0 - 16
+};
+struct Dw1Smem {
+    float ws[32 * 9 * 16];           // [o][tap][c]
+    Dw1Stage st[2];
+    float E[33 * kXE], O[33 * kXO];  // input pixels
+    float lut[256];
+    float red[16 * 40];
+};
+__global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
                                                 const LevelDesc *__restrict__ levels,
                                                 const uint8_t *__restrict__ pyr, const float *__restrict__ in_tab,
                                                 const float *__restrict__ w, const __nv_bfloat16 *__restrict__ act,
                                                 const float *__restrict__ dz2, float *__restrict__ part) {
-    extern __shared__ __align__(16) float smem_f[];
-    float *ws = smem_f;                  // [32 o][9][16 c]
-    float *ds = ws + 32 * 9 * 16;        // [32 o][9][kD2P]
-    float *E = ds + 32 * 9 * kD2P;       // [33][kXE]
-    float *O = E + 33 * kXE;             // [33][kXO]
-    __shared__ float lut[256], red[8 * 80];
+    extern __shared__ __align__(16) unsigned char smem_b[];
+    Dw1Smem &S = *reinterpret_cast<Dw1Smem *>(smem_b);
     const int tid = threadIdx.x;
-    lut[tid] = in_tab[tid];
-    for (int i = tid; i < 32 * 9 * 16; i += 256) {
+    if (tid < 256) S.lut[tid] = in_tab[tid];
+    for (int i = tid; i < 32 * 9 * 16; i += 512) {
         const int c = i & 15, ot = i >> 4, o = ot / 9;
-        ws[i] = w[(o * 16 + c) * 9 + ot - 9 * o];
+        S.ws[i] = w[(o * 16 + c) * 9 + ot - 9 * o];
     }
-    const int c0 = 8 * (tid >> 7), qx = tid & 15, qr = (tid >> 4) & 7;
-    f32x2 sum[10][4];
-#pragma unroll
-    for (int k = 0; k < 10; ++k)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) sum[k][c] = 0ull;
-    for (Walk<0> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+    Walk<0> wk(tl, n_tl, n_tiles);
+    auto fetch = [&](Dw1Stage &st) {  // this thread's share of the tile of wk
         const TrainLevel &T = tl[wk.k];
         const LevelDesc &L = levels[T.level];
         const int ntx = (T.W2 + 31) / 32, lt = wk.local();
         const int i0 = 8 * (lt / ntx), j0 = 32 * (lt % ntx);
-        __syncthreads();
-        stage_pixels(pyr + L.img_off, L.img_pitch, L.Wk, L.Hk, lut, 2 * i0, 2 * j0, E, O);
-        for (int e = tid; e < 32 * 9 * 33; e += 256) {
-            const int oi = e / 33, j = e - 33 * oi, o = oi / 9, i = oi - 9 * o;
-            ds[oi * kD2P + j] = i0 + i < T.H2 && j0 + j < T.W2
-                                    ? dz2[T.d2 + ((int64_t)o * T.H2 + i0 + i) * T.P2 + j0 + j]
-                                    : 0.f;
+        if (tid < 33 * 9) {
+            const int r = tid / 9, q = tid - 9 * r;
+            copy_row16(st.raw + 16 * tid, pyr + L.img_off, 4 * i0 + r - 1, 4 * j0 - 16 + 16 * q, L.Hk, L.Wk, L.img_pitch);
         }
-        __syncthreads();
-        f32x2 acc[2][4][4];
-        quad_pair<16, kD2P>(ds + qr * kD2P + 2 * qx, 9 * kD2P, ws + c0, acc);
-        // relu mask of a1 (and the layer's edge)
-        const int x = 2 * j0 + 4 * qx;
+        const int H2 = T.H2, W2 = T.W2, P2 = T.P2, H1 = T.H1, W1 = T.W1, P1 = T.P1;
+        const float *d = dz2 + T.d2;
+        for (int e = tid; e < 32 * 9 * 9; e += 512) {
+            const int row = e / 9, q = e - 9 * row, o = row / 9, i = row - 9 * o;
+            copy_row16(st.ds + 4 * e, d + (int64_t)o * H2 * P2, i0 + i, j0 + 4 * q, H2, W2, P2);
+        }
+        const __nv_bfloat16 *a1 = act + T.a1;
+#pragma unroll
+        for (int e = tid; e < 16 * 16 * 8; e += 512) {
+            const int c = e >> 7, r = (e >> 3) & 15, q = e & 7;
+            copy_row16(st.a1 + 8 * e, a1 + (int64_t)c * H1 * P1, 2 * i0 + r, 2 * j0 + 8 * q, H1, W1, P1);
+        }
+    };
+    const int c0 = 4 * (tid >> 7), qx = tid & 15, qr = (tid >> 4) & 7;
+    f32x2 sum[10][2];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) sum[k][0] = sum[k][1] = 0ull;
+    if (wk.valid()) fetch(S.st[0]);
+#pragma unroll 1
+    for (int b = 0; wk.valid(); b ^= 1) {
+        copies_done();
+        __syncthreads();  // this tile is here, and the other buffer is free
+        const Dw1Stage &st = S.st[b];
+        {
+            const TrainLevel &T = tl[wk.k];
+            const LevelDesc &L = levels[T.level];
+            const int ntx = (T.W2 + 31) / 32, lt = wk.local();
+            const int y0 = 32 * (lt / ntx) - 1, x0 = 128 * (lt % ntx) - 4;
+            for (int e = tid; e < 33 * 33; e += 512) {
+                const int r = e / 33, w4 = e - 33 * r, y = y0 + r, x = x0 + 4 * w4, m = 2 * w4 - 2;
+                const uint32_t v = *reinterpret_cast<const uint32_t *>(st.raw + r * 144 + 12 + 4 * w4);
+                const bool in = y >= 0 && y < L.Hk && x >= 0;
+                if (m >= 0) {
+                    S.E[r * kXE + m] = in && x < L.Wk ? S.lut[v & 255u] : 0.f;
+                    S.O[r * kXO + m + 1] = in && x + 1 < L.Wk ? S.lut[(v >> 8) & 255u] : 0.f;
+                    S.E[r * kXE + m + 1] = in && x + 2 < L.Wk ? S.lut[(v >> 16) & 255u] : 0.f;
+                }
+                S.O[r * kXO + m + 2] = in && x + 3 < L.Wk ? S.lut[v >> 24] : 0.f;
+            }
+        }
+        wk.step(n_tiles);
+        if (wk.valid()) fetch(S.st[b ^ 1]);
+        f32x2 acc[2][4][2];
+        quad_pair<16, kD2P, 2>(st.ds + qr * kD2P + 2 * qx, 9 * kD2P, S.ws + c0, acc);
+        // relu mask of a1 (0 outside the level)
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
-            const int y = 2 * (i0 + qr) + a;
-            const bool in = y < T.H1 && x < T.P1;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                uint2 m0 = make_uint2(0u, 0u), m1 = m0;
-                if (in) {
-                    const __nv_bfloat16 *src = act + T.a1 + ((int64_t)(c0 + 2 * c) * T.H1 + y) * T.P1 + x;
-                    m0 = *reinterpret_cast<const uint2 *>(src);
-                    m1 = *reinterpret_cast<const uint2 *>(src + (int64_t)T.H1 * T.P1);
-                }
+            for (int c = 0; c < 2; ++c) {
+                const __nv_bfloat16 *src = st.a1 + ((c0 + 2 * c) * 16 + 2 * qr + a) * 64 + 4 * qx;
+                const uint2 m0 = *reinterpret_cast<const uint2 *>(src);
+                const uint2 m1 = *reinterpret_cast<const uint2 *>(src + 16 * 64);
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
                     const uint32_t u0 = p < 2 ? m0.x : m0.y, u1 = p < 2 ? m1.x : m1.y;
-                    const bool ok = x + p < T.W1;
-                    const bool k0 = ok && (p & 1 ? bf_hi(u0) : bf_lo(u0)) > 0.f;
-                    const bool k1 = ok && (p & 1 ? bf_hi(u1) : bf_lo(u1)) > 0.f;
+                    const bool k0 = (p & 1 ? bf_hi(u0) : bf_lo(u0)) > 0.f;
+                    const bool k1 = (p & 1 ? bf_hi(u1) : bf_lo(u1)) > 0.f;
                     f32x2 &s = acc[p >> 1][2 * a + (p & 1)][c];
                     s = pack2(k0 ? lo2(s) : 0.f, k1 ? hi2(s) : 0.f);
                 }
             }
         }
+        __syncthreads();  // the pixels are there
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
 #pragma unroll
             for (int dy = 0; dy < 3; ++dy) {
                 const int r = 2 * (2 * qr + a) + dy;
-                const float4 e = *reinterpret_cast<const float4 *>(E + r * kXE + 4 * qx);
-                const float4 o4 = *reinterpret_cast<const float4 *>(O + r * kXO + 4 * qx);
+                const float4 e = *reinterpret_cast<const float4 *>(S.E + r * kXE + 4 * qx);
+                const float4 o4 = *reinterpret_cast<const float4 *>(S.O + r * kXO + 4 * qx);
                 const f32x2 ev[4] = {dup2(e.x), dup2(e.y), dup2(e.z), dup2(e.w)};
-                const f32x2 ov[5] = {dup2(o4.x), dup2(o4.y), dup2(o4.z), dup2(o4.w), dup2(O[r * kXO + 4 * qx + 4])};
+                const f32x2 ov[5] = {dup2(o4.x), dup2(o4.y), dup2(o4.z), dup2(o4.w), dup2(S.O[r * kXO + 4 * qx + 4])};
 #pragma unroll
                 for (int p = 0; p < 4; ++p)
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
+                    for (int c = 0; c < 2; ++c) {
                         const f32x2 d = acc[p >> 1][2 * a + (p & 1)][c];
                         sum[3 * dy][c] = fma2(d, ov[p], sum[3 * dy][c]);
                         sum[3 * dy + 1][c] = fma2(d, ev[p], sum[3 * dy + 1][c]);
@@ -613,133 +705,145 @@ __global__ void __launch_bounds__(256, 1) t_dw1(const TrainLevel *__restrict__ t
             }
         }
     }
-    const int warp = tid >> 5, lane = tid & 31;
 #pragma unroll
     for (int k = 0; k < 10; ++k)
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
+        for (int c = 0; c < 4; ++c) {
             const float v = warp_sum(c & 1 ? hi2(sum[k][c >> 1]) : lo2(sum[k][c >> 1]));
-            if (lane == 0) red[warp * 80 + k * 8 + c] = v;
+            if ((tid & 31) == 0) S.red[(tid >> 5) * 40 + k * 4 + c] = v;
         }
     __syncthreads();
     if (tid < kW1Parts) {  // order: 144 weights [c][tap], 16 biases
         const int c = tid < 144 ? tid / 9 : tid - 144, k = tid < 144 ? tid % 9 : 9;
-        const int at = (c >> 3) * 4 * 80 + k * 8 + (c & 7);
-        part[(int64_t)blockIdx.x * kW1Parts + tid] = ((red[at] + red[at + 80]) + red[at + 160]) + red[at + 240];
+        const float *r = S.red + (c >> 2) * 4 * 40 + k * 4 + (c & 3);
+        part[(int64_t)blockIdx.x * kW1Parts + tid] = ((r[0] + r[40]) + r[80]) + r[120];
     }
 }
 
 // ---- weight gradients of layers 2 and 3: dW[o][c][tap] = sum over positions
 // of dz[o] a[c at the tap]. A tile is 16 x 8 positions; a thread holds one
-// input channel x 4 output channels x 9 taps (CIN = 16: the two halves of the
-// block take half of the rows each). Lanes are channels: the activation planes
-// are an odd number of words apart (no bank conflict), dz is a broadcast.
-constexpr int kWAP = 33, kWAC = 17 * kWAP;  // staged activation row pitch (16 even, 17 odd columns), plane
-constexpr int kWDP = 36;                    // staged dz: words per position
-static_assert(kWAC % 2 == 1, "planes an odd number of words apart");
+// input channel x 4 output channels x 9 taps, in pairs of positions (so that
+// the gradients pair up as they lie), and a half or a quarter of the tile's
+// rows. Lanes are channels: dz is a broadcast. Activations stay two bf16
+// columns to a word until they are used. All threads fetch the next tile while
+// they work on this one.
+constexpr int kWAP = 20, kWAC = 17 * kWAP;  // staged activations: words per row (columns 2 j0 - 8 ..), per channel
+constexpr int kWDP = 132;                   // staged dz: floats per output channel (128 positions)
+static_assert(kWAC % 32 == 20, "8 channels of a row in 8 different quads of banks");
 template <int CIN>
-__global__ void __launch_bounds__(256) t_dw23(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
-                                              const LevelDesc *__restrict__ levels, const float *__restrict__ a3,
-                                              const float *__restrict__ dh, int32_t hp, const float *__restrict__ wh,
-                                              const __nv_bfloat16 *__restrict__ act, const float *__restrict__ dz2,
+struct Dw23Stage {
+    float ds[32 * kWDP];
+    uint32_t as[CIN * kWAC];
+};
+template <int CIN>
+__global__ void __launch_bounds__(512) t_dw23(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
+                                              const __nv_bfloat16 *__restrict__ act, const float *__restrict__ dz,
                                               float *__restrict__ part) {
     constexpr bool LAST = CIN == 32;
-    constexpr int kRows = LAST ? 8 : 4;
-    extern __shared__ __align__(16) float smem_f[];
-    float *ds = smem_f;                // [128 positions][kWDP]
-    float *as = smem_f + 128 * kWDP;   // [CIN][17][16 even | 17 odd columns]
-    __shared__ float whs[32];
+    constexpr int kTeam = 8 * CIN, kParts = 512 / kTeam, kRows = 8 / kParts;  // threads of one part of the rows
+    extern __shared__ __align__(16) unsigned char smem_b[];
+    Dw23Stage<CIN> *st = reinterpret_cast<Dw23Stage<CIN> *>(smem_b);
     const int tid = threadIdx.x;
-    if (LAST && tid < 32) whs[tid] = wh[tid];
-    const int c = tid % CIN, og = (tid / CIN) & 7, r0 = LAST ? 0 : 4 * (tid >> 7);
-    f32x2 acc[9][2], accb[2] = {0ull, 0ull};
+    const int c = tid % CIN, og = (tid / CIN) & 7, part_i = tid / kTeam;
+    f32x2 acc[4][9];
+    float bias = 0.f;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) acc[k][0] = acc[k][1] = 0ull;
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[u][k] = 0ull;
     constexpr int GRID = LAST ? 3 : 1;
-    for (Walk<GRID> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+    Walk<GRID> wk(tl, n_tl, n_tiles);
+    auto fetch = [&](Dw23Stage<CIN> &S) {  // this thread's share of the tile of wk
         const TrainLevel &T = tl[wk.k];
-        const LevelDesc &L = levels[T.level];
         const int Hi = LAST ? T.H2 : T.H1, Wi = LAST ? T.W2 : T.W1, Pi = LAST ? T.P2 : T.P1;
-        const int Wo = LAST ? T.W3 : T.W2;
-        const int64_t in_off = LAST ? T.a2 : T.a1;
+        const int Ho = LAST ? T.H3 : T.H2, Wo = LAST ? T.W3 : T.W2, Po = LAST ? T.P3 : T.P2;
         const int ntx = (Wo + 15) / 16, lt = wk.local();
         const int i0 = 8 * (lt / ntx), j0 = 16 * (lt % ntx);
-        __syncthreads();
-        for (int e = tid; e < 32 * 128; e += 256) {
-            const int o = e >> 7, p = e & 127, i = i0 + (p >> 4), j = j0 + (p & 15);
-            float v;
-            if (LAST) v = dz3_at(T, L, a3, dh, hp, whs[o], o, i, j);
-            else v = i < T.H2 && j < T.W2 ? dz2[T.d2 + ((int64_t)o * T.H2 + i) * T.P2 + j] : 0.f;
-            ds[p * kWDP + o] = v;
+        const float *d = dz + (LAST ? T.a3 : T.d2);
+#pragma unroll
+        for (int e = tid; e < 32 * 8 * 4; e += 512) {
+            const int o = e >> 5, i = (e >> 2) & 7, q = e & 3;
+            copy_row16(S.ds + o * kWDP + i * 16 + 4 * q, d + (int64_t)o * Ho * Po, i0 + i, j0 + 4 * q, Ho, Wo, Po);
         }
-        for (int e = tid; e < CIN * 17 * 17; e += 256) {
-            const int cr = e / 17, m = e - 17 * cr - 1, cc = cr / 17, r = cr - 17 * cc;
-            const int y = 2 * i0 + r - 1, x = 2 * (j0 + m);
-            uint32_t v = 0u;
-            if (y >= 0 && y < Hi && x >= 0 && x < Wi) {
-                v = *reinterpret_cast<const uint32_t *>(act + in_off + ((int64_t)cc * Hi + y) * Pi + x);
-                if (x + 1 >= Wi) v &= 0xffffu;
-            }
-            float *row = as + cc * kWAC + r * kWAP;
-            if (m >= 0) row[m] = bf_lo(v);
-            row[16 + m + 1] = bf_hi(v);
+        const __nv_bfloat16 *a = act + (LAST ? T.a2 : T.a1);
+        for (int e = tid; e < CIN * 17 * 5; e += 512) {
+            const int cr = e / 5, q = e - 5 * cr, cc = cr / 17, r = cr - 17 * cc;
+            copy_row16(S.as + 4 * e, a + (int64_t)cc * Hi * Pi, 2 * i0 + r - 1, 2 * j0 - 8 + 8 * q, Hi, Wi, Pi);
         }
-        __syncthreads();
+    };
+    if (wk.valid()) fetch(st[0]);
 #pragma unroll 1
-        for (int i = r0; i < r0 + kRows; ++i) {
-            const float *ap = as + c * kWAC + 2 * i * kWAP;
-            const float *dp = ds + i * 16 * kWDP + 4 * og;
-            f32x2 od[3];
+    for (int b = 0; wk.valid(); b ^= 1) {
+        copies_done();
+        __syncthreads();  // this tile is here, and the other buffer is free
+        wk.step(n_tiles);
+        if (wk.valid()) fetch(st[b ^ 1]);
+        const Dw23Stage<CIN> &S = st[b];
+        {
+            const float4 *d = reinterpret_cast<const float4 *>(S.ds + (tid >> 4) * kWDP + 8 * (tid & 15));
+            const float4 u = d[0], v = d[1];
+            bias += ((u.x + u.y) + (u.z + u.w)) + ((v.x + v.y) + (v.z + v.w));
+        }
+#pragma unroll 1
+        for (int i = part_i * kRows; i < (part_i + 1) * kRows; ++i) {
+            const uint32_t *ap = S.as + c * kWAC + 2 * i * kWAP + 4;
+            const float *dp = S.ds + 4 * og * kWDP + 16 * i;
+            uint32_t prev[3];
 #pragma unroll
-            for (int dy = 0; dy < 3; ++dy) od[dy] = dup2(ap[dy * kWAP + 16]);
+            for (int dy = 0; dy < 3; ++dy) prev[dy] = ap[dy * kWAP - 1];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const ulonglong2 d = *reinterpret_cast<const ulonglong2 *>(dp + j * kWDP);
-                accb[0] = add2(accb[0], d.x);
-                accb[1] = add2(accb[1], d.y);
+            for (int j = 0; j < 16; j += 4) {
+                ulonglong2 d[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) d[u] = *reinterpret_cast<const ulonglong2 *>(dp + u * kWDP + j);
 #pragma unroll
                 for (int dy = 0; dy < 3; ++dy) {
-                    const f32x2 e = dup2(ap[dy * kWAP + j]), on = dup2(ap[dy * kWAP + 17 + j]);
-                    acc[3 * dy][0] = fma2(d.x, od[dy], acc[3 * dy][0]);
-                    acc[3 * dy][1] = fma2(d.y, od[dy], acc[3 * dy][1]);
-                    acc[3 * dy + 1][0] = fma2(d.x, e, acc[3 * dy + 1][0]);
-                    acc[3 * dy + 1][1] = fma2(d.y, e, acc[3 * dy + 1][1]);
-                    acc[3 * dy + 2][0] = fma2(d.x, on, acc[3 * dy + 2][0]);
-                    acc[3 * dy + 2][1] = fma2(d.y, on, acc[3 * dy + 2][1]);
-                    od[dy] = on;
+                    const uint4 w = *reinterpret_cast<const uint4 *>(ap + dy * kWAP + j);
+                    const f32x2 l0 = pack2(bf_hi(prev[dy]), bf_hi(w.x)), l1 = pack2(bf_hi(w.y), bf_hi(w.z));
+                    const f32x2 e0 = pack2(bf_lo(w.x), bf_lo(w.y)), e1 = pack2(bf_lo(w.z), bf_lo(w.w));
+                    const f32x2 r0 = pack2(bf_hi(w.x), bf_hi(w.y)), r1 = pack2(bf_hi(w.z), bf_hi(w.w));
+                    prev[dy] = w.w;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        acc[u][3 * dy] = fma2(d[u].x, l0, acc[u][3 * dy]);
+                        acc[u][3 * dy + 1] = fma2(d[u].x, e0, acc[u][3 * dy + 1]);
+                        acc[u][3 * dy + 2] = fma2(d[u].x, r0, acc[u][3 * dy + 2]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        acc[u][3 * dy] = fma2(d[u].y, l1, acc[u][3 * dy]);
+                        acc[u][3 * dy + 1] = fma2(d[u].y, e1, acc[u][3 * dy + 1]);
+                        acc[u][3 * dy + 2] = fma2(d[u].y, r1, acc[u][3 * dy + 2]);
+                    }
                 }
             }
         }
     }
-    float v[10][4];
+    // the parts' sums, in order
+    float *x = reinterpret_cast<float *>(smem_b);
+    __syncthreads();
+    if (part_i) {
 #pragma unroll
-    for (int k = 0; k < 10; ++k) {
-        unpack2(k < 9 ? acc[k][0] : accb[0], v[k][0], v[k][1]);
-        unpack2(k < 9 ? acc[k][1] : accb[1], v[k][2], v[k][3]);
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) x[(u * 9 + k) * (512 - kTeam) + tid - kTeam] = lo2(acc[u][k]) + hi2(acc[u][k]);
     }
-    if (!LAST) {  // add the second half's sums to the first's
-        __syncthreads();
-        if (tid >= 128) {
-#pragma unroll
-            for (int k = 0; k < 10; ++k)
-#pragma unroll
-                for (int u = 0; u < 4; ++u) smem_f[(k * 4 + u) * 128 + tid - 128] = v[k][u];
-        }
-        __syncthreads();
-        if (tid >= 128) return;
-#pragma unroll
-        for (int k = 0; k < 10; ++k)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[k][u] += smem_f[(k * 4 + u) * 128 + tid];
-    }
+    __syncthreads();
     float *out = part + (int64_t)blockIdx.x * (32 * CIN * 9 + 32);
+    if (!part_i) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int o = 4 * og + u;
+        for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int k = 0; k < 9; ++k) out[(o * CIN + c) * 9 + k] = v[k][u];
-        if (c == 0) out[32 * CIN * 9 + o] = v[9][u];
+            for (int k = 0; k < 9; ++k) {
+                float v = lo2(acc[u][k]) + hi2(acc[u][k]);
+#pragma unroll
+                for (int q = 0; q + 1 < kParts; ++q) v += x[(u * 9 + k) * (512 - kTeam) + q * kTeam + tid];
+                out[((4 * og + u) * CIN + c) * 9 + k] = v;
+            }
     }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) bias += __shfl_xor_sync(0xffffffffu, bias, o);
+    if ((tid & 15) == 0) out[32 * CIN * 9 + (tid >> 4)] = bias;
 }
 
 // Conv weights are rounded to bf16 in the working copy the forward pass uses.
@@ -796,11 +900,13 @@ __global__ void __launch_bounds__(256) t_finish(const float *__restrict__ p1, in
     }
 }
 
-constexpr size_t conv23_smem(int cin) { return (size_t)cin * 9 * 32 * 4 + 2 * 16 * 17 * kAP * 2; }
-constexpr size_t kDz2Smem = (size_t)(32 * 9 * 32 + 32 * 9 * kD3P) * 4;
-constexpr size_t kDw1Smem = (size_t)(32 * 9 * 16 + 32 * 9 * kD2P + 33 * (kXE + kXO)) * 4;
-constexpr size_t dw23_smem(int cin) { return (size_t)(128 * kWDP + cin * kWAC) * 4; }
-static_assert(dw23_smem(16) >= 40 * 128 * 4, "the halves' exchange fits");
+constexpr size_t conv23_smem(int cin) { return cin == 16 ? sizeof(ConvSmem<16>) : sizeof(ConvSmem<32>); }
+constexpr size_t kDz2Smem = sizeof(Dz2Smem);
+static_assert(2 * (kDz2Smem + 1024) <= 228 * 1024, "two blocks per SM");
+constexpr size_t kDw1Smem = sizeof(Dw1Smem);
+static_assert(kDw1Smem <= 227 * 1024, "one block per SM");
+constexpr size_t dw23_smem(int cin) { return cin == 16 ? 2 * sizeof(Dw23Stage<16>) : 2 * sizeof(Dw23Stage<32>); }
+static_assert(dw23_smem(16) >= 36 * 384 * 4 && dw23_smem(32) >= 36 * 256 * 4, "the parts' exchange fits");
 
 }  // namespace
 
@@ -837,7 +943,7 @@ cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a) {
                                   a.act16);
     t_conv23<16, false><<<3 * G, 128, conv23_smem(16), s>>>(a.tl, nl, a.tiles[0], a.act16, a.wr + kOffW2,
                                                             a.wr + kOffB2, a.act16, nullptr);
-    t_conv23<32, true><<<2 * G, 128, conv23_smem(32), s>>>(a.tl, nl, a.tiles[2], a.act16, a.wr + kOffW3,
+    t_conv23<32, true><<<3 * G, 128, conv23_smem(32), s>>>(a.tl, nl, a.tiles[2], a.act16, a.wr + kOffW3,
                                                            a.wr + kOffB3, nullptr, a.act32);
     t_head_fwd<<<g2, blk, 0, s>>>(a.tl, a.levels, a.act32, a.wr + kOffWh, a.wr + kOffBh, a.hmap, a.hp);
     cudaError_t e = cudaGetLastError();
@@ -853,14 +959,12 @@ cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a) {
     t_loss<<<dim3(kLossParts, nl), 256, 0, s>>>(a.tl, a.levels, a.logits, a.scores, a.label_thr, a.pos_weight, a.inv_n,
                                                 a.dz, a.level_loss);
     t_pool_bwd_h<<<dim3(48, nl), blk, 0, s>>>(a.tl, a.levels, a.dz, a.wr + kOffV, a.dh, a.hp);
-    t_small_grads<<<G, blk, 0, s>>>(a.tl, nl, a.tiles[4], a.tiles[2], a.levels, a.dz, a.hmap, a.dh, a.hp, a.act32, ps);
-    t_dw23<32><<<G, blk, dw23_smem(32), s>>>(a.tl, nl, a.tiles[3], a.levels, a.act32, a.dh, a.hp, a.wr + kOffWh,
-                                             a.act16, nullptr, p3);
-    t_dz2<<<G, blk, kDz2Smem, s>>>(a.tl, nl, a.tiles[3], a.levels, a.act32, a.dh, a.hp, a.wr + kOffWh, a.wr + kOffW3,
-                                   a.act16, a.dz2);
-    t_dw23<16><<<G, blk, dw23_smem(16), s>>>(a.tl, nl, a.tiles[1], a.levels, nullptr, nullptr, 0, nullptr, a.act16,
-                                             a.dz2, p2);
-    t_dw1<<<G, blk, kDw1Smem, s>>>(a.tl, nl, a.tiles[0], a.levels, a.pyr, a.w.in_tab, a.wr + kOffW2, a.act16, a.dz2,
+    t_small_grads<<<G, blk, 0, s>>>(a.tl, nl, a.tiles[4], a.tiles[2], a.levels, a.dz, a.hmap, a.dh, a.hp,
+                                     a.wr + kOffWh, a.act32, ps);  // and a3 becomes dz3
+    t_dw23<32><<<G, 512, dw23_smem(32), s>>>(a.tl, nl, a.tiles[3], a.act16, a.act32, p3);
+    t_dz2<<<G, blk, kDz2Smem, s>>>(a.tl, nl, a.tiles[3], a.act32, a.wr + kOffW3, a.act16, a.dz2);
+    t_dw23<16><<<G, 512, dw23_smem(16), s>>>(a.tl, nl, a.tiles[1], a.act16, a.dz2, p2);
+    t_dw1<<<G, 512, kDw1Smem, s>>>(a.tl, nl, a.tiles[0], a.levels, a.pyr, a.w.in_tab, a.wr + kOffW2, a.act16, a.dz2,
                                    p1);
     t_finish<<<(kCnnParams + 31) / 32, blk, 0, s>>>(p1, G, p2, G, p3, G, ps, G, a.grad, a.master, a.m, a.v, a.wr, a.lr,
                                                     a.beta1, a.beta2, a.eps, a.c1, a.c2);
