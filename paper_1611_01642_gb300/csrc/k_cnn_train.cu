@@ -25,12 +25,12 @@
 // order by the last kernel.
 // 4 x 1280x720 frames (38 M pyramid pixels, 36 levels each), one step:
 // 74.4 -> 6.67 ms against one thread per position with all levels of a weight's
-// gradient in one block, and 6.67 -> 3.55 ms by fetching ahead (half of every
+// gradient in one block, and 6.67 -> 3.44 ms by fetching ahead (half of every
 // warp's waiting was for the tile's loads, with 8 to 16 warps per SM to hide
 // them): weight gradient of layer 1 with the data gradient of layer 2 2.05 ->
-// 0.72, weight gradients of layers 2 and 3 1.31 -> 0.76 and 0.75 -> 0.39, data
+// 0.72, weight gradients of layers 2 and 3 1.31 -> 0.67 and 0.75 -> 0.38, data
 // gradient of layer 3 0.55 -> 0.33, forward convolutions 0.84 -> 0.49 and 0.61
-// -> 0.34 ms. The FP32 pipe is now 54 to 76% busy in them; in the two data
+// -> 0.34 ms. The FP32 pipe is now 50 to 76% busy in them; in the two data
 // gradients shared memory's 75% comes first.
 #include "pd_internal.h"
 
@@ -722,11 +722,14 @@ __global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ t
 
 // ---- weight gradients of layers 2 and 3: dW[o][c][tap] = sum over positions
 // of dz[o] a[c at the tap]. A tile is 16 x 8 positions; a thread holds one
-// input channel x 4 output channels x 9 taps, in pairs of positions (so that
+// input channel x 8 output channels x 9 taps, in pairs of positions (so that
 // the gradients pair up as they lie), and a half or a quarter of the tile's
 // rows. Lanes are channels: dz is a broadcast. Activations stay two bf16
-// columns to a word until they are used. All threads fetch the next tile while
-// they work on this one.
+// columns to a word until they are used: taking them apart costs 12 operations
+// per 4 columns and row against 6 packed multiply-adds per output channel, so a thread
+// takes 8 output channels and 255 registers (4 and twice the warps: 0.76 and
+// 0.39 ms, now 0.67 and 0.38). All threads fetch the next tile while they work
+// on this one.
 constexpr int kWAP = 20, kWAC = 17 * kWAP;  // staged activations: words per row (columns 2 j0 - 8 ..), per channel
 constexpr int kWDP = 132;                   // staged dz: floats per output channel (128 positions)
 static_assert(kWAC % 32 == 20, "8 channels of a row in 8 different quads of banks");
@@ -736,19 +739,19 @@ struct Dw23Stage {
     uint32_t as[CIN * kWAC];
 };
 template <int CIN>
-__global__ void __launch_bounds__(512) t_dw23(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
+__global__ void __launch_bounds__(256, 1) t_dw23(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
                                               const __nv_bfloat16 *__restrict__ act, const float *__restrict__ dz,
                                               float *__restrict__ part) {
     constexpr bool LAST = CIN == 32;
-    constexpr int kTeam = 8 * CIN, kParts = 512 / kTeam, kRows = 8 / kParts;  // threads of one part of the rows
+    constexpr int kTeam = 4 * CIN, kParts = 256 / kTeam, kRows = 8 / kParts;  // threads of one part of the rows
     extern __shared__ __align__(16) unsigned char smem_b[];
     Dw23Stage<CIN> *st = reinterpret_cast<Dw23Stage<CIN> *>(smem_b);
     const int tid = threadIdx.x;
-    const int c = tid % CIN, og = (tid / CIN) & 7, part_i = tid / kTeam;
-    f32x2 acc[4][9];
+    const int c = tid % CIN, og = (tid / CIN) & 3, part_i = tid / kTeam;
+    f32x2 acc[8][9];
     float bias = 0.f;
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < 8; ++u)
 #pragma unroll
         for (int k = 0; k < 9; ++k) acc[u][k] = 0ull;
     constexpr int GRID = LAST ? 3 : 1;
@@ -761,12 +764,12 @@ __global__ void __launch_bounds__(512) t_dw23(const TrainLevel *__restrict__ tl,
         const int i0 = 8 * (lt / ntx), j0 = 16 * (lt % ntx);
         const float *d = dz + (LAST ? T.a3 : T.d2);
 #pragma unroll
-        for (int e = tid; e < 32 * 8 * 4; e += 512) {
+        for (int e = tid; e < 32 * 8 * 4; e += 256) {
             const int o = e >> 5, i = (e >> 2) & 7, q = e & 3;
             copy_row16(S.ds + o * kWDP + i * 16 + 4 * q, d + (int64_t)o * Ho * Po, i0 + i, j0 + 4 * q, Ho, Wo, Po);
         }
         const __nv_bfloat16 *a = act + (LAST ? T.a2 : T.a1);
-        for (int e = tid; e < CIN * 17 * 5; e += 512) {
+        for (int e = tid; e < CIN * 17 * 5; e += 256) {
             const int cr = e / 5, q = e - 5 * cr, cc = cr / 17, r = cr - 17 * cc;
             copy_row16(S.as + 4 * e, a + (int64_t)cc * Hi * Pi, 2 * i0 + r - 1, 2 * j0 - 8 + 8 * q, Hi, Wi, Pi);
         }
@@ -780,22 +783,22 @@ __global__ void __launch_bounds__(512) t_dw23(const TrainLevel *__restrict__ tl,
         if (wk.valid()) fetch(st[b ^ 1]);
         const Dw23Stage<CIN> &S = st[b];
         {
-            const float4 *d = reinterpret_cast<const float4 *>(S.ds + (tid >> 4) * kWDP + 8 * (tid & 15));
-            const float4 u = d[0], v = d[1];
-            bias += ((u.x + u.y) + (u.z + u.w)) + ((v.x + v.y) + (v.z + v.w));
+            const float4 *d = reinterpret_cast<const float4 *>(S.ds + (tid >> 3) * kWDP + 4 * (tid & 7));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) bias += (d[8 * q].x + d[8 * q].y) + (d[8 * q].z + d[8 * q].w);
         }
 #pragma unroll 1
         for (int i = part_i * kRows; i < (part_i + 1) * kRows; ++i) {
             const uint32_t *ap = S.as + c * kWAC + 2 * i * kWAP + 4;
-            const float *dp = S.ds + 4 * og * kWDP + 16 * i;
+            const float *dp = S.ds + 8 * og * kWDP + 16 * i;
             uint32_t prev[3];
 #pragma unroll
             for (int dy = 0; dy < 3; ++dy) prev[dy] = ap[dy * kWAP - 1];
 #pragma unroll
             for (int j = 0; j < 16; j += 4) {
-                ulonglong2 d[4];
+                ulonglong2 d[8];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) d[u] = *reinterpret_cast<const ulonglong2 *>(dp + u * kWDP + j);
+                for (int u = 0; u < 8; ++u) d[u] = *reinterpret_cast<const ulonglong2 *>(dp + u * kWDP + j);
 #pragma unroll
                 for (int dy = 0; dy < 3; ++dy) {
                     const uint4 w = *reinterpret_cast<const uint4 *>(ap + dy * kWAP + j);
@@ -804,17 +807,17 @@ __global__ void __launch_bounds__(512) t_dw23(const TrainLevel *__restrict__ tl,
                     const f32x2 r0 = pack2(bf_hi(w.x), bf_hi(w.y)), r1 = pack2(bf_hi(w.z), bf_hi(w.w));
                     prev[dy] = w.w;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        acc[u][3 * dy] = fma2(d[u].x, l0, acc[u][3 * dy]);
-                        acc[u][3 * dy + 1] = fma2(d[u].x, e0, acc[u][3 * dy + 1]);
-                        acc[u][3 * dy + 2] = fma2(d[u].x, r0, acc[u][3 * dy + 2]);
-                    }
+                    for (int u = 0; u < 8; ++u) acc[u][3 * dy] = fma2(l0, d[u].x, acc[u][3 * dy]);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        acc[u][3 * dy] = fma2(d[u].y, l1, acc[u][3 * dy]);
-                        acc[u][3 * dy + 1] = fma2(d[u].y, e1, acc[u][3 * dy + 1]);
-                        acc[u][3 * dy + 2] = fma2(d[u].y, r1, acc[u][3 * dy + 2]);
-                    }
+                    for (int u = 0; u < 8; ++u) acc[u][3 * dy + 1] = fma2(e0, d[u].x, acc[u][3 * dy + 1]);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) acc[u][3 * dy + 2] = fma2(r0, d[u].x, acc[u][3 * dy + 2]);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) acc[u][3 * dy] = fma2(l1, d[u].y, acc[u][3 * dy]);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) acc[u][3 * dy + 1] = fma2(e1, d[u].y, acc[u][3 * dy + 1]);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) acc[u][3 * dy + 2] = fma2(r1, d[u].y, acc[u][3 * dy + 2]);
                 }
             }
         }
@@ -824,26 +827,26 @@ __global__ void __launch_bounds__(512) t_dw23(const TrainLevel *__restrict__ tl,
     __syncthreads();
     if (part_i) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 8; ++u)
 #pragma unroll
-            for (int k = 0; k < 9; ++k) x[(u * 9 + k) * (512 - kTeam) + tid - kTeam] = lo2(acc[u][k]) + hi2(acc[u][k]);
+            for (int k = 0; k < 9; ++k) x[(u * 9 + k) * (256 - kTeam) + tid - kTeam] = lo2(acc[u][k]) + hi2(acc[u][k]);
     }
     __syncthreads();
     float *out = part + (int64_t)blockIdx.x * (32 * CIN * 9 + 32);
     if (!part_i) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 8; ++u)
 #pragma unroll
             for (int k = 0; k < 9; ++k) {
                 float v = lo2(acc[u][k]) + hi2(acc[u][k]);
 #pragma unroll
-                for (int q = 0; q + 1 < kParts; ++q) v += x[(u * 9 + k) * (512 - kTeam) + q * kTeam + tid];
-                out[((4 * og + u) * CIN + c) * 9 + k] = v;
+                for (int q = 0; q + 1 < kParts; ++q) v += x[(u * 9 + k) * (256 - kTeam) + q * kTeam + tid];
+                out[((8 * og + u) * CIN + c) * 9 + k] = v;
             }
     }
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) bias += __shfl_xor_sync(0xffffffffu, bias, o);
-    if ((tid & 15) == 0) out[32 * CIN * 9 + (tid >> 4)] = bias;
+    for (int o = 4; o > 0; o >>= 1) bias += __shfl_xor_sync(0xffffffffu, bias, o);
+    if ((tid & 7) == 0) out[32 * CIN * 9 + (tid >> 3)] = bias;
 }
 
 // Conv weights are rounded to bf16 in the working copy the forward pass uses.
@@ -906,7 +909,7 @@ static_assert(2 * (kDz2Smem + 1024) <= 228 * 1024, "two blocks per SM");
 constexpr size_t kDw1Smem = sizeof(Dw1Smem);
 static_assert(kDw1Smem <= 227 * 1024, "one block per SM");
 constexpr size_t dw23_smem(int cin) { return cin == 16 ? 2 * sizeof(Dw23Stage<16>) : 2 * sizeof(Dw23Stage<32>); }
-static_assert(dw23_smem(16) >= 36 * 384 * 4 && dw23_smem(32) >= 36 * 256 * 4, "the parts' exchange fits");
+static_assert(dw23_smem(16) >= 72 * 192 * 4 && dw23_smem(32) >= 72 * 128 * 4, "the parts' exchange fits");
 
 }  // namespace
 
@@ -961,9 +964,9 @@ cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a) {
     t_pool_bwd_h<<<dim3(48, nl), blk, 0, s>>>(a.tl, a.levels, a.dz, a.wr + kOffV, a.dh, a.hp);
     t_small_grads<<<G, blk, 0, s>>>(a.tl, nl, a.tiles[4], a.tiles[2], a.levels, a.dz, a.hmap, a.dh, a.hp,
                                      a.wr + kOffWh, a.act32, ps);  // and a3 becomes dz3
-    t_dw23<32><<<G, 512, dw23_smem(32), s>>>(a.tl, nl, a.tiles[3], a.act16, a.act32, p3);
+    t_dw23<32><<<G, 256, dw23_smem(32), s>>>(a.tl, nl, a.tiles[3], a.act16, a.act32, p3);
     t_dz2<<<G, blk, kDz2Smem, s>>>(a.tl, nl, a.tiles[3], a.act32, a.wr + kOffW3, a.act16, a.dz2);
-    t_dw23<16><<<G, 512, dw23_smem(16), s>>>(a.tl, nl, a.tiles[1], a.act16, a.dz2, p2);
+    t_dw23<16><<<G, 256, dw23_smem(16), s>>>(a.tl, nl, a.tiles[1], a.act16, a.dz2, p2);
     t_dw1<<<G, 512, kDw1Smem, s>>>(a.tl, nl, a.tiles[0], a.levels, a.pyr, a.w.in_tab, a.wr + kOffW2, a.act16, a.dz2,
                                    p1);
     t_finish<<<(kCnnParams + 31) / 32, blk, 0, s>>>(p1, G, p2, G, p3, G, ps, G, a.grad, a.master, a.m, a.v, a.wr, a.lr,
