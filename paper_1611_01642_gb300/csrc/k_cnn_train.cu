@@ -25,12 +25,12 @@
 // order by the last kernel.
 // 4 x 1280x720 frames (38 M pyramid pixels, 36 levels each), one step:
 // 74.4 -> 6.67 ms against one thread per position with all levels of a weight's
-// gradient in one block, and 6.67 -> 3.44 ms by fetching ahead (half of every
+// gradient in one block, and 6.67 -> 3.30 ms by fetching ahead (half of every
 // warp's waiting was for the tile's loads, with 8 to 16 warps per SM to hide
 // them): weight gradient of layer 1 with the data gradient of layer 2 2.05 ->
-// 0.72, weight gradients of layers 2 and 3 1.31 -> 0.67 and 0.75 -> 0.38, data
-// gradient of layer 3 0.55 -> 0.33, forward convolutions 0.84 -> 0.49 and 0.61
-// -> 0.34 ms. The FP32 pipe is now 50 to 76% busy in them; in the two data
+// 0.69, weight gradients of layers 2 and 3 1.31 -> 0.67 and 0.75 -> 0.38, data
+// gradient of layer 3 0.55 -> 0.33, forward convolutions 0.20 -> 0.15, 0.84 ->
+// 0.49 and 0.61 -> 0.35 ms. The FP32 pipe is now 50 to 76% busy in them; in the two data
 // gradients shared memory's 75% comes first.
 #include "pd_internal.h"
 
@@ -94,47 +94,66 @@ __device__ __forceinline__ void copy_row16(void *dst, const T *plane, int y, int
 
 constexpr int kXE = 64, kXO = 68;  // input tile row pitches: even columns, odd columns (from -1)
 
-// Input pixels of the 64 x 16 layer-1 positions from (i0, j0): E[r][j] = x at
-// column 2 (j0 + j), O[r][j] = x at column 2 (j0 + j) - 1, row 2 i0 + r - 1;
-// zero outside the level. Level rows are 4-byte aligned (pitch a multiple of 16).
-__device__ __forceinline__ void stage_pixels(const uint8_t *img, int pitch, int Wk, int Hk, const float *lut, int i0,
-                                             int j0, float *E, float *O) {
-    for (int i = threadIdx.x; i < 33 * 33; i += 256) {
-        const int r = i / 33, w = i - 33 * r;
-        const int y = 2 * i0 + r - 1, c = 2 * j0 - 4 + 4 * w;
-        uint32_t v = 0u;
-        const bool in = y >= 0 && y < Hk && c >= 0 && c < pitch;
-        if (in) v = *reinterpret_cast<const uint32_t *>(img + (int64_t)y * pitch + c);
-        const int m = 2 * w - 2;
+// Input of the 64 x 16 layer-1 positions from (i0, j0): rows 2 i0 - 1 .., 144
+// bytes from column 2 j0 - 16. copy_pixels: thread e's copy (e < 33 * 9).
+constexpr int kRawP = 144;
+__device__ __forceinline__ void copy_pixels(uint8_t *raw, const uint8_t *img, const LevelDesc &L, int i0, int j0, int e) {
+    const int r = e / 9, q = e - 9 * r;
+    copy_row16(raw + 16 * e, img, 2 * i0 + r - 1, 2 * j0 - 16 + 16 * q, L.Hk, L.Wk, L.img_pitch);
+}
+// E[r][j] = x at column 2 (j0 + j), O[r][j] = x at column 2 (j0 + j) - 1, row
+// 2 i0 + r - 1; zero outside the level.
+template <int THREADS>
+__device__ __forceinline__ void spread_pixels(const uint8_t *raw, const LevelDesc &L, const float *lut, int i0, int j0,
+                                              float *E, float *O) {
+    const int Wk = L.Wk, Hk = L.Hk;
+    for (int e = threadIdx.x; e < 33 * 33; e += THREADS) {
+        const int r = e / 33, w4 = e - 33 * r, y = 2 * i0 + r - 1, x = 2 * j0 - 4 + 4 * w4, m = 2 * w4 - 2;
+        const uint32_t v = *reinterpret_cast<const uint32_t *>(raw + r * kRawP + 12 + 4 * w4);
+        const bool in = y >= 0 && y < Hk && x >= 0;
         if (m >= 0) {
-            E[r * kXE + m] = in && c < Wk ? lut[v & 255u] : 0.f;
-            O[r * kXO + m + 1] = in && c + 1 < Wk ? lut[(v >> 8) & 255u] : 0.f;
-            E[r * kXE + m + 1] = in && c + 2 < Wk ? lut[(v >> 16) & 255u] : 0.f;
+            E[r * kXE + m] = in && x < Wk ? lut[v & 255u] : 0.f;
+            O[r * kXO + m + 1] = in && x + 1 < Wk ? lut[(v >> 8) & 255u] : 0.f;
+            E[r * kXE + m + 1] = in && x + 2 < Wk ? lut[(v >> 16) & 255u] : 0.f;
         }
-        O[r * kXO + m + 2] = in && c + 3 < Wk ? lut[v >> 24] : 0.f;
+        O[r * kXO + m + 2] = in && x + 3 < Wk ? lut[v >> 24] : 0.f;
     }
 }
 
 // ---- layer 1: 64 x 16 positions per tile, 4 positions x 16 channels per
 // thread. The sum of a channel runs over (dy, dx) in order, as everywhere.
-// Bound by its stores (a1 is 32 bytes per position) and the staging.
+// Bound by issue and its stores (a1 is 32 bytes per position): 154 us, 197
+// before the pixels of the next tile were fetched ahead.
 __global__ void __launch_bounds__(256) t_conv1(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
                                                const LevelDesc *__restrict__ levels, const uint8_t *__restrict__ pyr,
                                                const float *__restrict__ in_tab, const float *__restrict__ w,
                                                const float *__restrict__ b, __nv_bfloat16 *__restrict__ act) {
     __shared__ __align__(16) float E[33 * kXE], O[33 * kXO], ws[9 * 16], bs[16], lut[256];
+    __shared__ __align__(16) uint8_t raw[2][33 * kRawP];
     const int tid = threadIdx.x;
     lut[tid] = in_tab[tid];
     if (tid < 144) ws[(tid % 9) * 16 + tid / 9] = w[tid];
     if (tid < 16) bs[tid] = b[tid];
     const int g = tid & 15, ir = tid >> 4;
-    for (Walk<0> wk(tl, n_tl, n_tiles); wk.valid(); wk.step(n_tiles)) {
+    Walk<0> wk(tl, n_tl, n_tiles);
+    auto fetch = [&](uint8_t *dst) {
+        const TrainLevel &T = tl[wk.k];
+        const LevelDesc &L = levels[T.level];
+        const int ntx = (T.W2 + 31) / 32, lt = wk.local();
+        for (int e = tid; e < 33 * 9; e += 256)
+            copy_pixels(dst, pyr + L.img_off, L, 16 * (lt / ntx), 64 * (lt % ntx), e);
+    };
+    if (wk.valid()) fetch(raw[0]);
+    for (int buf = 0; wk.valid(); buf ^= 1) {
         const TrainLevel &T = tl[wk.k];
         const LevelDesc &L = levels[T.level];
         const int ntx = (T.W2 + 31) / 32, lt = wk.local();
         const int i0 = 16 * (lt / ntx), j0 = 64 * (lt % ntx);
+        copies_done();
         __syncthreads();
-        stage_pixels(pyr + L.img_off, L.img_pitch, L.Wk, L.Hk, lut, i0, j0, E, O);
+        spread_pixels<256>(raw[buf], L, lut, i0, j0, E, O);
+        wk.step(n_tiles);
+        if (wk.valid()) fetch(raw[buf ^ 1]);
         __syncthreads();
         f32x2 acc[4][8];
 #pragma unroll
@@ -188,19 +207,25 @@ __global__ void __launch_bounds__(256) t_conv1(const TrainLevel *__restrict__ tl
 // channels per thread; kCS input channels are worked on while the next kCS
 // (or the next tile's first) arrive. Activations stay two bf16 columns to a
 // word: per input channel and window row 2 activation loads and 12 broadcast
-// weight loads for 96 packed multiply-adds.
+// weight loads for 96 packed multiply-adds. Layer 3 forms the head on its way
+// out: h = bh + wh . a3 on the cells, channel by channel (a kernel of its own
+// read a3 back for it, 68 us; layer 3 takes 5 us longer).
 constexpr int kAP = 36;  // words per staged activation row: columns 2 j0 - 8 ..
 template <int CIN>
 struct ConvSmem {
     static constexpr int kCS = 128 / CIN;  // 8 or 4: three blocks per SM
     float ws[CIN * 9 * 32];                // [c][tap][o]
     uint32_t as[2][kCS * 17 * kAP];
+    float4 head[64];                       // layer 3: bh + wh . a3 over the first 16 channels
+    float wh[32];
 };
 template <int CIN, bool LAST>
 __global__ void __launch_bounds__(128) t_conv23(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
                                                 const __nv_bfloat16 *__restrict__ act, const float *__restrict__ w,
                                                 const float *__restrict__ b, __nv_bfloat16 *__restrict__ out16,
-                                                float *__restrict__ out32) {
+                                                float *__restrict__ out32, const LevelDesc *__restrict__ levels,
+                                                const float *__restrict__ wh, const float *__restrict__ bh,
+                                                float *__restrict__ hmap, int32_t hp) {
     constexpr int kCS = ConvSmem<CIN>::kCS;
     extern __shared__ __align__(16) unsigned char smem_b[];
     ConvSmem<CIN> &S = *reinterpret_cast<ConvSmem<CIN> *>(smem_b);
@@ -209,6 +234,7 @@ __global__ void __launch_bounds__(128) t_conv23(const TrainLevel *__restrict__ t
         const int o = i & 31, ct = i >> 5;
         S.ws[i] = w[o * CIN * 9 + ct];
     }
+    if (LAST && tid < 32) S.wh[tid] = wh[tid];
     const int o0 = 16 * (tid >> 6), g = tid & 7, ir = (tid >> 3) & 7;
     constexpr int GRID = LAST ? 2 : 0;
     Walk<GRID> wk(tl, n_tl, n_tiles);
@@ -232,6 +258,7 @@ __global__ void __launch_bounds__(128) t_conv23(const TrainLevel *__restrict__ t
         const TrainLevel &T = tl[wk.k];
         const int Ho = LAST ? T.H3 : T.H2, Wo = LAST ? T.W3 : T.W2, Po = LAST ? T.P3 : T.P2;
         const int64_t out_off = LAST ? T.a3 : T.a2;
+        const int tl_level = T.level;
         const int ntx = (Wo + 31) / 32, lt = wk.local();
         const int i = 8 * (lt / ntx) + ir, j = 32 * (lt % ntx) + 4 * g;
         f32x2 acc[4][8];
@@ -275,6 +302,29 @@ __global__ void __launch_bounds__(128) t_conv23(const TrainLevel *__restrict__ t
                 }
             }
         }
+        if (LAST) {  // h on the cells, channel by channel: the first two warps, then the others
+            const LevelDesc &L = levels[tl_level];
+            float h[4];
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                if ((o0 != 0) == (half != 0)) {
+                    const float4 h0 = half ? S.head[tid & 63] : make_float4(bh[0], bh[0], bh[0], bh[0]);
+                    h[0] = h0.x, h[1] = h0.y, h[2] = h0.z, h[3] = h0.w;
+#pragma unroll
+                    for (int o = 0; o < 16; ++o)
+#pragma unroll
+                        for (int p = 0; p < 4; ++p)
+                            h[p] = fmaf(S.wh[o0 + o], fmaxf(o & 1 ? hi2(acc[p][o >> 1]) : lo2(acc[p][o >> 1]), 0.f), h[p]);
+                    if (!half) S.head[tid & 63] = make_float4(h[0], h[1], h[2], h[3]);
+                }
+                if (!half) __syncthreads();
+            }
+            if (o0 && i < L.Hc) {
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+                    if (j + p < L.Wc) hmap[(int64_t)(L.cell_row + i) * hp + j + p] = h[p];
+            }
+        }
         if (i < Ho && j < Po) {
 #pragma unroll
             for (int o = 0; o < 16; ++o) {
@@ -293,24 +343,6 @@ __global__ void __launch_bounds__(128) t_conv23(const TrainLevel *__restrict__ t
                 }
             }
         }
-    }
-}
-
-// ---- head: h = bh + wh . a3 on the cells of the level
-__global__ void t_head_fwd(const TrainLevel *__restrict__ tl, const LevelDesc *__restrict__ levels,
-                           const float *__restrict__ a3, const float *__restrict__ wh,
-                           const float *__restrict__ bh, float *__restrict__ hmap, int32_t hp) {
-    const TrainLevel &T = tl[blockIdx.y];
-    const LevelDesc &L = levels[T.level];
-    const int n = L.Hc * L.Wc;
-    const int64_t plane = (int64_t)T.H3 * T.P3;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const int cy = p / L.Wc, cx = p - cy * L.Wc;
-        const float *src = a3 + T.a3 + (int64_t)cy * T.P3 + cx;
-        float h = bh[0];
-#pragma unroll
-        for (int c = 0; c < 32; ++c) h = fmaf(__ldg(wh + c), src[c * plane], h);
-        hmap[(int64_t)(L.cell_row + cy) * hp + cx] = h;
     }
 }
 
@@ -582,13 +614,13 @@ __global__ void __launch_bounds__(256) t_dz2(const TrainLevel *__restrict__ tl, 
 // dz1 is never written (it would be 2 x 64 bytes per position of traffic). A
 // tile is 32 x 8 quads (64 x 16 layer-1 positions): 128 quad pairs x 4 channel
 // groups. (8 channels per thread, 8 warps and a ninth to copy: 168 registers, so
-// that the loads of the weights were waited for, 1.01 ms against 0.72.)
+// that the loads of the weights were waited for, 1.01 ms against 0.69.)
 constexpr int kD2P = 36;  // staged dz2 row pitch (33 columns)
 constexpr int kW1Parts = 160;
 struct Dw1Stage {
     float ds[32 * 9 * kD2P];         // dz2 [o][i][j]
     __nv_bfloat16 a1[16 * 16 * 64];  // [c][row][column]
-    uint8_t raw[33 * 144];           // input rows, bytes from column 4 j0 - 16
+    uint8_t raw[33 * kRawP];         // input pixels
 };
 struct Dw1Smem {
     float ws[32 * 9 * 16];           // [o][tap][c]
@@ -616,10 +648,7 @@ __global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ t
         const LevelDesc &L = levels[T.level];
         const int ntx = (T.W2 + 31) / 32, lt = wk.local();
         const int i0 = 8 * (lt / ntx), j0 = 32 * (lt % ntx);
-        if (tid < 33 * 9) {
-            const int r = tid / 9, q = tid - 9 * r;
-            copy_row16(st.raw + 16 * tid, pyr + L.img_off, 4 * i0 + r - 1, 4 * j0 - 16 + 16 * q, L.Hk, L.Wk, L.img_pitch);
-        }
+        if (tid < 33 * 9) copy_pixels(st.raw, pyr + L.img_off, L, 2 * i0, 2 * j0, tid);
         const int H2 = T.H2, W2 = T.W2, P2 = T.P2, H1 = T.H1, W1 = T.W1, P1 = T.P1;
         const float *d = dz2 + T.d2;
         for (int e = tid; e < 32 * 9 * 9; e += 512) {
@@ -647,18 +676,7 @@ __global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ t
             const TrainLevel &T = tl[wk.k];
             const LevelDesc &L = levels[T.level];
             const int ntx = (T.W2 + 31) / 32, lt = wk.local();
-            const int y0 = 32 * (lt / ntx) - 1, x0 = 128 * (lt % ntx) - 4;
-            for (int e = tid; e < 33 * 33; e += 512) {
-                const int r = e / 33, w4 = e - 33 * r, y = y0 + r, x = x0 + 4 * w4, m = 2 * w4 - 2;
-                const uint32_t v = *reinterpret_cast<const uint32_t *>(st.raw + r * 144 + 12 + 4 * w4);
-                const bool in = y >= 0 && y < L.Hk && x >= 0;
-                if (m >= 0) {
-                    S.E[r * kXE + m] = in && x < L.Wk ? S.lut[v & 255u] : 0.f;
-                    S.O[r * kXO + m + 1] = in && x + 1 < L.Wk ? S.lut[(v >> 8) & 255u] : 0.f;
-                    S.E[r * kXE + m + 1] = in && x + 2 < L.Wk ? S.lut[(v >> 16) & 255u] : 0.f;
-                }
-                S.O[r * kXO + m + 2] = in && x + 3 < L.Wk ? S.lut[v >> 24] : 0.f;
-            }
+            spread_pixels<512>(st.raw, L, S.lut, 16 * (lt / ntx), 64 * (lt % ntx), S.E, S.O);
         }
         wk.step(n_tiles);
         if (wk.valid()) fetch(S.st[b ^ 1]);
@@ -936,7 +954,6 @@ cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a) {
     const dim3 blk(256);
     const int nl = a.n_levels;
     if (nl <= 0) return cudaSuccess;
-    const dim3 g2(8, nl);
     // persistent blocks: a fixed number, so that the sums' order does not depend on the device
     constexpr int G = kTrainBlocks;
     float *p1 = a.part, *p2 = p1 + (size_t)G * kW1Parts, *p3 = p2 + (size_t)G * (kOffW3 - kOffW2),
@@ -945,10 +962,11 @@ cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a) {
     t_conv1<<<4 * G, blk, 0, s>>>(a.tl, nl, a.tiles[0], a.levels, a.pyr, a.w.in_tab, a.wr + kOffW1, a.wr + kOffB1,
                                   a.act16);
     t_conv23<16, false><<<3 * G, 128, conv23_smem(16), s>>>(a.tl, nl, a.tiles[0], a.act16, a.wr + kOffW2,
-                                                            a.wr + kOffB2, a.act16, nullptr);
+                                                            a.wr + kOffB2, a.act16, nullptr, nullptr, nullptr, nullptr,
+                                                            nullptr, 0);
     t_conv23<32, true><<<3 * G, 128, conv23_smem(32), s>>>(a.tl, nl, a.tiles[2], a.act16, a.wr + kOffW3,
-                                                           a.wr + kOffB3, nullptr, a.act32);
-    t_head_fwd<<<g2, blk, 0, s>>>(a.tl, a.levels, a.act32, a.wr + kOffWh, a.wr + kOffBh, a.hmap, a.hp);
+                                                           a.wr + kOffB3, nullptr, a.act32, a.levels, a.wr + kOffWh,
+                                                           a.wr + kOffBh, a.hmap, a.hp);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // pooling forward: the inference pooling kernel (identical sums) over the
