@@ -475,7 +475,8 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
                                                   float iou_thr, int cap, float4 *__restrict__ scratch,
                                                   pd_box *__restrict__ boxes, int max_boxes,
                                                   int32_t *__restrict__ counts, int n_frames,
-                                                  const int *__restrict__ order, int *__restrict__ queue) {
+                                                  const int *__restrict__ order, int *__restrict__ queue,
+                                                  const unsigned *__restrict__ err, unsigned *__restrict__ err_out) {
     extern __shared__ __align__(16) unsigned char nms_raw[];
     NmsSmem &S = *reinterpret_cast<NmsSmem *>(nms_raw);
     // A frame is one cluster of C CTAs (C = 1 without a cluster launch); rank 0
@@ -498,6 +499,7 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
         else __syncthreads();
     };
     const bool cull = iou_thr >= 0.5f;
+    if (err_out && blockIdx.x == 0 && tid == 0) *err_out = *err;
     csync();  // every CTA of the cluster runs before the leader writes into it
     for (int pass = 0;; ++pass) {
         if (queue) {
@@ -1089,7 +1091,7 @@ int nms_launches(int n_frames, int cluster) {
 cudaError_t launch_nms(cudaStream_t s, const FrameDesc *d_frames, const LevelDesc *d_levels,
                        int n_frames, const float *scores, float threshold, float iou,
                        float4 *scratch, int max_cand, pd_box *boxes, int max_boxes,
-                       int32_t *counts, int cluster, int *sched) {
+                       int32_t *counts, int cluster, int *sched, const unsigned *err, unsigned *err_out) {
     if (n_frames <= 0) return cudaSuccess;
     if (max_cand < 1 || max_cand > kMaxCandidatesBig || max_boxes < 1 || max_boxes > kMaxBoxes ||
         cluster < 1 || cluster > 8 || (cluster & (cluster - 1)))
@@ -1118,7 +1120,7 @@ cudaError_t launch_nms(cudaStream_t s, const FrameDesc *d_frames, const LevelDes
     }
     if (cluster == 1) {
         k_nms<<<n_clusters, kThreads, smem, s>>>(d_frames, d_levels, scores, threshold, iou, max_cand, scratch,
-                                                 boxes, max_boxes, counts, n_frames, order, queue);
+                                                 boxes, max_boxes, counts, n_frames, order, queue, err, err_out);
         return cudaGetLastError();
     }
     cudaLaunchConfig_t cfg = {};
@@ -1134,7 +1136,7 @@ cudaError_t launch_nms(cudaStream_t s, const FrameDesc *d_frames, const LevelDes
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_nms, d_frames, d_levels, scores, threshold, iou, max_cand, scratch, boxes,
-                              max_boxes, counts, n_frames, (const int *)order, queue);
+                              max_boxes, counts, n_frames, (const int *)order, queue, err, err_out);
 }
 
 // ---------------------------------------------------------------------------

@@ -94,7 +94,8 @@ __global__ void __launch_bounds__(kThreads, kResizeCtas) k_resize(const FrameDes
                                                                   const LevelDesc *__restrict__ levels,
                                                                   const int32_t *__restrict__ tabs,
                                                                   uint8_t *__restrict__ pyr,
-                                                                  const ResizeItem *__restrict__ items) {
+                                                                  const ResizeItem *__restrict__ items,
+                                                                  int *__restrict__ zero) {
     using Lay = Layout<kTH>;
     constexpr int kStageIters = ((kTH + 1) * ((kResizeBW + 3) / 4) + kThreads - 1) / kThreads;  // staged words per thread
     constexpr int kRS = 32 / kCG;
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(kThreads, kResizeCtas) k_resize(const FrameDes
     // per level: {img_off lo, img_off hi, pitch, Wk}, {rgroup, xtab_off, xq_off, ytab_off}
     int4 *s_lvl = reinterpret_cast<int4 *>(smem + Lay::kLvl);
 
+    if (zero && blockIdx.x == 0 && threadIdx.x < kStepWords) zero[threadIdx.x] = 0;
     const ResizeItem it = items[blockIdx.x];
     const FrameDesc fd = frames[it.frame];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -327,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, kResizeCtas) k_resize(const FrameDes
 }  // namespace
 
 namespace {
-using ResizeFn = void (*)(const FrameDesc *, const LevelDesc *, const int32_t *, uint8_t *, const ResizeItem *);
+using ResizeFn = void (*)(const FrameDesc *, const LevelDesc *, const int32_t *, uint8_t *, const ResizeItem *, int *);
 // [column groups per task 4, 8, 16][tile rows kResizeTH, 2 kResizeTH]
 const ResizeFn kResizeFns[3][2] = {{k_resize<4, kResizeTH>, k_resize<4, 2 * kResizeTH>},
                                    {k_resize<8, kResizeTH>, k_resize<8, 2 * kResizeTH>},
@@ -346,10 +348,10 @@ cudaError_t init_resize() {
 
 cudaError_t launch_resize(cudaStream_t s, const FrameDesc *d_frames, const LevelDesc *d_levels,
                           const int32_t *d_tabs, uint8_t *pyr, const ResizeItem *d_items,
-                          int n_items, bool tall, int k1_groups) {
+                          int n_items, bool tall, int k1_groups, int *zero) {
     if (n_items <= 0) return cudaSuccess;
     const int g = k1_groups == 4 ? 0 : k1_groups == 16 ? 2 : 1;
-    kResizeFns[g][tall]<<<n_items, kThreads, kResizeSmem[tall], s>>>(d_frames, d_levels, d_tabs, pyr, d_items);
+    kResizeFns[g][tall]<<<n_items, kThreads, kResizeSmem[tall], s>>>(d_frames, d_levels, d_tabs, pyr, d_items, zero);
     return cudaGetLastError();
 }
 

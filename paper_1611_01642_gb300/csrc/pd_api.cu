@@ -275,7 +275,9 @@ struct pd_handle {
     int32_t *h_counts = nullptr;   // mapped: [2 * max_frames] kept / candidates
     pd_box *m_boxes = nullptr;     // device views of the two mapped buffers
     int32_t *m_counts = nullptr;
-    unsigned *h_err = nullptr;
+    unsigned *h_err = nullptr;     // mapped: the error word of the last step (NMS writes it)
+    unsigned *m_err = nullptr;     // its device view
+    bool err_stage = false;        // a stage call has used d_err since
     cudaEvent_t desc_done = nullptr;
     cudaEvent_t stage_ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     bool timed = false;
@@ -304,7 +306,7 @@ struct pd_handle {
     // tensor maps over the atlases, one pair per tile shape of the FP32 K4
     CUtensorMap hog_map[kSvmShapes]{}, lbp_map[kSvmShapes]{};
     unsigned char *d_tc_consts = nullptr;    // tensor-core K4: B operand and LBP table
-    int *d_queue = nullptr;                  // [2]: K4's and K2+K3's item counters (zeroed before each launch)
+    int *d_queue = nullptr;                  // [2]: K4's and K2+K3's item counters (zero at each launch; after d_err)
     int *d_nms_sched = nullptr;              // NMS ticket counter, frame order and candidate counts
     int sm_count = 1;
     float tile_cost[kSvmShapes] = {kDefaultTileCost[0], kDefaultTileCost[1], kDefaultTileCost[2],
@@ -867,14 +869,11 @@ const T *dptr(pd_handle *h, int64_t off) {
     return reinterpret_cast<const T *>(h->d_desc + off);
 }
 
-// K2+K3 of a plan.
+// K2+K3 of a plan (its strip counter is 0 at launch).
 cudaError_t launch_cell_stage(pd_handle *h, cudaStream_t s, const LevelDesc *dl, const uint8_t *pyr,
                               const CellAtlas &atlas, const Plan &p, const Packed &o, const uint32_t *c_flag,
                               int feat) {
-    int *queue = h->d_queue + 1;  // the strip counter (K4's is d_queue[0])
-    const cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
-    return launch_cells_warp(s, dl, pyr, atlas, dptr<StripItem>(h, o.strips), (int)p.strips.size(), queue,
+    return launch_cells_warp(s, dl, pyr, atlas, dptr<StripItem>(h, o.strips), (int)p.strips.size(), h->d_queue + 1,
                              h->sm_count, c_flag, feat);
 }
 
@@ -1133,6 +1132,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     if (cudaHostGetDevicePointer(reinterpret_cast<void **>(&h->m_boxes), h->h_boxes, 0) != cudaSuccess ||
         cudaHostGetDevicePointer(reinterpret_cast<void **>(&h->m_counts), h->h_counts, 0) != cudaSuccess)
         return bail(PD_ECUDA);
+    h->m_err = reinterpret_cast<unsigned *>(h->m_counts + 2 * params->max_frames);
     if (cudaEventCreateWithFlags(&h->desc_done, cudaEventDisableTiming) != cudaSuccess)
         return bail(PD_ECUDA);
     if (cudaEventRecord(h->desc_done, 0) != cudaSuccess) return bail(PD_ECUDA);
@@ -1251,10 +1251,13 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         if (n_frames)
             PD_CUDA(h, cudaMemcpyAsync(h->d_desc + o.frames, h->h_desc + o.frames,
                                        p.frames.size() * sizeof(FrameDesc), cudaMemcpyHostToDevice, q));
-        PD_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(unsigned), q));
+        // the error word and the item counters start a step as 0: K1 clears them
+        // (as memsets they were 3 of a step's 8 graph nodes)
+        int *zero = reinterpret_cast<int *>(h->d_err);
+        if (p.r_items.empty()) PD_CUDA(h, cudaMemsetAsync(zero, 0, kStepWords * sizeof(int), q));
         if (timed) PD_CUDA(h, record(h->stage_ev[0], q));
         PD_CUDA(h, launch_resize(q, df, dl, dptr<int32_t>(h, o.tabs), h->d_pyr, dptr<ResizeItem>(h, o.r_items),
-                                 (int)p.r_items.size(), p.tall, h->tuning.k1_groups));
+                                 (int)p.r_items.size(), p.tall, h->tuning.k1_groups, zero));
         if (timed) PD_CUDA(h, record(h->stage_ev[5], q));
         const uint32_t *cf = nullptr, *sf = nullptr;
         if (h->proposal) {
@@ -1278,7 +1281,6 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
             PD_CUDA(h, launch_svm(q, h->hog_map, h->lbp_map, dl, h->d_w, h->bias, h->p.l2hys_clip, h->d_scores,
                                   dptr<SvmItem>(h, o.s_items), (int)p.s_items.size(), h->d_err, sf));
         } else {
-            PD_CUDA(h, cudaMemsetAsync(h->d_queue, 0, sizeof(int), q));
             PD_CUDA(h, launch_svm_tc(q, CUtensorMap{}, CUtensorMap{}, dl, dptr<TcItem>(h, o.t_items),
                                      (int)p.t_items.size(), h->d_queue, h->sm_count, h->d_tc_consts, h->bias,
                                      h->p.l2hys_clip, h->d_scores, cf, h->d_err, hog_planes_of(h->p.flags),
@@ -1289,7 +1291,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
                               h->d_nms_scratch, h->p.max_candidates_per_frame, h->m_boxes,
                               h->p.max_boxes_per_frame, h->m_counts,
                               nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame),
-                              h->d_nms_sched));
+                              h->d_nms_sched, h->d_err, h->m_err));
         if (timed) PD_CUDA(h, record(h->stage_ev[4], q));
         return PD_OK;
     };
@@ -1320,6 +1322,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         if (r != PD_OK) return r;
     }
     PD_CUDA(h, cudaEventRecord(h->graph_done, s));
+    h->err_stage = false;
     h->last_launches = (p.r_items.empty() ? 0 : 1) + (p.strips.empty() ? 0 : 1) +
                        (p.score_floats == 0 ? 0 : 1) +
                        nms_launches(n_frames, nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame)) +
@@ -1369,8 +1372,12 @@ int pd_sync(pd_handle *h) {
     if (!h) return PD_EINVAL;
     if (!h->detected) return fail(h, PD_ESTATE, "pd_sync without pd_detect");
     const int nf = (int)h->plan.frames.size();
-    PD_CUDA(h, cudaMemcpyAsync(h->h_err, h->d_err, 4, cudaMemcpyDeviceToHost, h->stream));
-    PD_CUDA(h, cudaStreamSynchronize(h->stream));  // boxes and counts are already in host memory
+    // Boxes, counts and the step's error word are already in host memory, written
+    // by NMS (the word is copied where no NMS ran or a stage call came after:
+    // as a copy it cost every step about 8 us).
+    if (h->err_stage || nf == 0)
+        PD_CUDA(h, cudaMemcpyAsync(h->h_err, h->d_err, 4, cudaMemcpyDeviceToHost, h->stream));
+    PD_CUDA(h, cudaStreamSynchronize(h->stream));
     int status = PD_OK;
     if (*h->h_err & kErrTimeout) status = fail(h, PD_ETIMEOUT, "device wait timed out");
     else if (*h->h_err & kErrBounds) status = fail(h, PD_EBOUNDS, "device bounds check fired");
@@ -1458,6 +1465,7 @@ int pd_cnn_forward(pd_handle *h, void *stream, const uint8_t *d_level, int Wk, i
     Packed o;
     int r = upload_plan(h, s, p, o, d_level);
     if (r != PD_OK) return r;
+    h->err_stage = true;
     PD_CUDA(h, launch_cnn(s, dptr<LevelDesc>(h, o.levels), p.levels[0].rows > 0 ? 1 : 0,
                           dptr<CUtensorMap>(h, o.tmaps), dptr<CnnItem>(h, o.cnn_items), (int)p.cnn_items.size(),
                           cnn_weights(h), d_h, h_pitch, d_logits, max_pool_tiles(p), h->d_err));
@@ -1729,6 +1737,7 @@ int pd_cell_features(pd_handle *h, void *stream, const uint8_t *d_level, int Wk,
     a.lbp_plane = lbp_plane;
     a.pitch = cell_pitch;
     a.rows = Hc;
+    PD_CUDA(h, cudaMemsetAsync(h->d_queue + 1, 0, sizeof(int), s));
     PD_CUDA(h, launch_cell_stage(h, s, dptr<LevelDesc>(h, o.levels), d_level, a, p, o, nullptr,
                                  kFeatHog | kFeatLbp | (features_of(h->p.flags) & kFeatHogBlock)));
     return PD_OK;
@@ -1769,12 +1778,12 @@ int pd_window_scores(pd_handle *h, void *stream, const float *d_hog, int64_t hog
     Packed o;
     int r = upload_plan(h, s, p, o);
     if (r != PD_OK) return r;
-    PD_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(unsigned), s));
+    PD_CUDA(h, cudaMemsetAsync(h->d_err, 0, 2 * sizeof(int), s));  // and K4's item counter
+    h->err_stage = true;
     if (fp32) {
         PD_CUDA(h, launch_svm(s, hm, lm, dptr<LevelDesc>(h, o.levels), h->d_w, h->bias, h->p.l2hys_clip,
                               d_scores, dptr<SvmItem>(h, o.s_items), (int)p.s_items.size(), h->d_err));
     } else {
-        PD_CUDA(h, cudaMemsetAsync(h->d_queue, 0, sizeof(int), s));
         PD_CUDA(h, launch_lbp_cells(s, d_lbp, lbp_plane, cell_pitch, cells_x, cells_y, cells));
         PD_CUDA(h, launch_svm_tc(s, th, tl, dptr<LevelDesc>(h, o.levels), dptr<TcItem>(h, o.t_items),
                                  (int)p.t_items.size(), h->d_queue, h->sm_count, h->d_tc_consts, h->bias,

@@ -118,10 +118,12 @@ cudaError_t init_nms(bool occupancy = true);  // occupancy: also the clusters th
 cudaError_t init_resize();
 
 // Kernel launchers (host functions defined next to their kernels).
-// tall: tiles of 2 kResizeTH rows; k1_groups: column groups per warp task (4, 8 or 16)
+// tall: tiles of 2 kResizeTH rows; k1_groups: column groups per warp task (4, 8 or 16); zero: the
+// kStepWords words that a step starts with cleared (the error word and the item counters)
+constexpr int kStepWords = 3;
 cudaError_t launch_resize(cudaStream_t s, const FrameDesc *d_frames, const LevelDesc *d_levels,
                           const int32_t *d_tabs, uint8_t *pyr, const ResizeItem *d_items,
-                          int n_items, bool tall, int k1_groups = 8);
+                          int n_items, bool tall, int k1_groups = 8, int *zero = nullptr);
 constexpr int kFeatHog = 1, kFeatLbp = 2, kFeatHogBlock = 4;
 // K2+K3: one warp per strip. feat: HOG and / or LBP; kFeatHogBlock | kFeatHog
 // (| kFeatLbp) for 36 HOG planes, the 4 block-restricted histograms of every
@@ -174,7 +176,8 @@ __host__ __device__ inline size_t nms_scratch_float4s(int cap) {
 cudaError_t launch_nms(cudaStream_t s, const FrameDesc *d_frames, const LevelDesc *d_levels,
                        int n_frames, const float *scores, float threshold, float iou,
                        float4 *scratch, int max_cand, pd_box *boxes, int max_boxes,
-                       int32_t *counts, int cluster = 1, int *sched = nullptr);
+                       int32_t *counts, int cluster = 1, int *sched = nullptr, const unsigned *err = nullptr,
+                       unsigned *err_out = nullptr);  // err_out: where the step's error word *err goes
 int nms_cluster_for(int n_frames, int sm_count, int max_cand);
 // launch_nms with sched runs the persistent form (count, order, NMS kernels)
 bool nms_persistent(int n_frames, int cluster);
