@@ -29,12 +29,14 @@
 //     and those that the segment's kept boxes suppress, and the next segment
 //     is taken. A later segment's candidates have met every kept box before
 //     them, so the decisions stay those of the sequential walk.
-// What bounds it: the latency of the one frame with the most candidates: about
-// 6,000 cycles per batch of the walk, 15,000 to collect, 4,000 to 8,000 to sort.
+// What bounds it: the latency of the one frame with the most candidates: 3,000
+// to 10,000 cycles per batch of the walk, 15,000 to collect, 4,000 to 8,000 to sort.
 // A scan level by level, a bitonic sort of all candidates and a cluster-wide
-// pass over all of them after every batch took 80 us where this takes 39 (one
-// 1242x375 frame, 1,884 candidates), 317 against 152 (8 frames of 40 levels, up
-// to 10,363 candidates), 117 against 78 (64 frames of 1242x375).
+// pass over all of them after every batch took 80 us where this takes 31 (one
+// 1242x375 frame, 1,884 candidates), 317 against 137 (8 frames of 40 levels, up
+// to 10,363 candidates), 117 against 68 (64 frames of 1242x375). Of these 37, 152
+// and 76 had a batch's edges 32 bytes apart: 16 lanes on one bank group, and the
+// pairwise bits took 3,700 cycles per batch where they take about 1,200.
 // The IoU test first evaluates inter - thr * union in float. A coordinate sum or
 // difference is off by at most 3 float roundings of values up to m = max(W, H)
 // (eps = 3 m 2^-24), which moves the intersection by at most (w + h) eps and the
@@ -70,6 +72,7 @@ constexpr int kGrid = 32;                 // culling grid: kGrid x kGrid cells o
 constexpr int kCountBlocks = 32;          // blocks per frame counting its candidates
 static_assert(nms_sched_ints(1) == 2 + kCountBlocks,
               "scheduling scratch: the ticket, then per frame its order slot and counts");
+constexpr int kSoloWindows = 8192;        // frames of at most this many windows: one CTA (two rounds of loads)
 constexpr int kOrderMax = 16384;          // frames the order kernel sorts (more: drawn in index order)
 static_assert(kThreads == 16 * kBatch, "pairwise matrix: 16 threads per batch member");
 static_assert(kThreads == kGrid * kGrid, "one culling cell per thread");
@@ -370,7 +373,8 @@ struct NmsSmem {
     int hist[kHist];
     int kept[kSeg];                             // the segment's kept entries, in order
     float4 bbx[kBatch];                         // the batch's boxes; a chunk of kept boxes
-    Edges bed[kBatch];                          // the same as edges
+    float4 be[kBatch];                          // the same as edges, and areas (apart: 16 threads read
+    float ba[kBatch];                           // 16 members in a row without bank conflicts)
     unsigned long long bcol[kBatch];            // member b: bit a set iff a < b and a suppresses b
     unsigned long long lohi[2][32];             // per warp: least and greatest key
     int4 krect[kBatch];                         // kept boxes' cell ranges x0, x1, y0, y1
@@ -384,6 +388,13 @@ struct NmsSmem {
     unsigned long long lo, hi;                  // least and greatest key of this CTA's list
     uint32_t keep[2];                           // the batch's kept members
     int n_list, n_seg, n_kept_seg, done, frame, digit, below;
+    __device__ __forceinline__ Edges edges(int i) const { return {be[i], ba[i]}; }
+    __device__ __forceinline__ void set_box(int i, const float4 &b) {
+        const Edges e = edges_of(b);
+        bbx[i] = b;
+        be[i] = e.e;
+        ba[i] = e.area;
+    }
 };
 
 __device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
@@ -500,8 +511,8 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
     };
     const bool cull = iou_thr >= 0.5f;
     if (err_out && blockIdx.x == 0 && tid == 0) *err_out = *err;
-    csync();  // every CTA of the cluster runs before the leader writes into it
-    for (int pass = 0;; ++pass) {
+    if (queue) csync();  // every CTA of the cluster runs before the leader writes into it
+    for (;;) {
         if (queue) {
             if (leader && tid == 0) {
                 const int t = atomicAdd(queue, 1);
@@ -509,10 +520,11 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
                 for (int r = 0; r < C; ++r) cluster.map_shared_rank(&S, r)->frame = fr;
             }
         } else if (tid == 0) {
-            S.frame = pass == 0 ? (int)(blockIdx.x / C) : -1;
+            S.frame = (int)(blockIdx.x / C);
         }
         if (tid == 0) S.n_list = S.n_seg = 0;
-        csync();  // every rank knows the frame
+        if (queue) csync();  // every rank knows the frame
+        else __syncthreads();
         const int f = S.frame;
         if (f < 0) return;  // the same value in every rank: all leave together
         const FrameDesc &fd = frames[f];
@@ -592,7 +604,8 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
                 counts[2 * f] = 0;
                 counts[2 * f + 1] = n > cap ? -n : 0;
             }
-            csync();  // nobody clears its count while another rank reads it
+            csync();  // nobody clears its count or leaves while another rank reads it
+            if (!queue) return;
             continue;
         }
         int n_list = S.n_list;  // this rank's list
@@ -749,22 +762,21 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
                         if (member[h]) {
                             const float4 b = h ? own1 : own0;
                             S.batch[slot] = tid + h * kThreads;
-                            S.bbx[slot] = b;
-                            S.bed[slot] = edges_of(b);
+                            S.set_box(slot, b);
                         }
                     }
                     __syncthreads();
                     {
-                        // member b = tid / 16 is tested against members a = 4 (tid % 16) .. + 3
+                        // member b = tid / 16 is tested against members a = tid % 16, + 16, ..
                         // (a < b); the 16 threads of a member OR their bits together
-                        const int b = tid >> 4, a0 = (tid & 15) * 4;
+                        const int b = tid >> 4, a0 = tid & 15;
                         unsigned long long bits = 0;
                         if (b < nb && a0 < b) {
-                            const Edges bb = S.bed[b];
+                            const Edges bb = S.edges(b);
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
-                                const int a = a0 + q;
-                                if (a < b && suppresses(S.bed[a], S.bbx[a], bb, S.bbx[b], iou_thr, band)) bits |= 1ull << a;
+                                const int a = a0 + 16 * q;
+                                if (a < b && suppresses(S.edges(a), S.bbx[a], bb, S.bbx[b], iou_thr, band)) bits |= 1ull << a;
                             }
                         }
 #pragma unroll
@@ -852,7 +864,7 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
                             for (int h = 0; h < 2; ++h)
                                 for (uint32_t k = keep[h] & part; k && !gone; k &= k - 1u) {
                                     const int j = 32 * h + __ffs((int)k) - 1;
-                                    gone = suppresses(S.bed[j], S.bbx[j], ej, bj, iou_thr, band);
+                                    gone = suppresses(S.edges(j), S.bbx[j], ej, bj, iou_thr, band);
                                 }
                         }
                         for (int o = per / 2; o > 0; o >>= 1) gone |= __shfl_xor_sync(0xffffffffu, (int)gone, o) != 0;
@@ -881,8 +893,7 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
                 const int kc = min(kBatch, nk - k0);
                 if (tid < kc) {
                     const float4 b = Lead.box[Lead.kept[k0 + tid]];
-                    S.bbx[tid] = b;
-                    S.bed[tid] = edges_of(b);
+                    S.set_box(tid, b);
                     S.krect[tid] = make_int4(max((int)floorf(b.x * gsx) - 1, 0),
                                              min((int)floorf((b.x + b.z) * gsx) + 1, kGrid - 1),
                                              max((int)floorf(b.y * gsy) - 1, 0),
@@ -922,11 +933,11 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
                             for (int h = 0; h < 2; ++h)
                                 for (uint32_t k = (uint32_t)(m >> (32 * h)); k && stay; k &= k - 1u) {
                                     const int j = 32 * h + __ffs((int)k) - 1;
-                                    stay = !suppresses(S.bed[j], S.bbx[j], ej, bj, iou_thr, band);
+                                    stay = !suppresses(S.edges(j), S.bbx[j], ej, bj, iou_thr, band);
                                 }
                         } else {
                             for (int j = 0; j < kc && stay; ++j)
-                                stay = !suppresses(S.bed[j], S.bbx[j], ej, bj, iou_thr, band);
+                                stay = !suppresses(S.edges(j), S.bbx[j], ej, bj, iou_thr, band);
                         }
                     }
                     const unsigned m = __ballot_sync(0xffffffffu, stay);
@@ -953,6 +964,12 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
         if (leader && tid == 0) {
             counts[2 * f] = kept_total;
             counts[2 * f + 1] = n;
+        }
+        if (!queue) {
+            // one frame per cluster: after the last segment nobody reads another rank's
+            // memory unless there were several (their bookkeeping is the leader's)
+            if (n > kSeg) csync();
+            return;
         }
     }
 }
@@ -1069,7 +1086,10 @@ cudaError_t init_nms(bool occupancy) {
     return cudaSuccess;
 }
 
-int nms_cluster_for(int n_frames, int sm_count, int max_cand) {
+int nms_cluster_for(int n_frames, int sm_count, int max_cand, int64_t windows) {
+    // few windows: a second round of a CTA's loads costs less than the cluster's
+    // barriers (320x240 frame, 139 candidates: 18.4 us with 8 CTAs, 16.4 with one)
+    if (windows <= kSoloWindows) return 1;
     // the CTAs of a frame share its collection and passes; only while every CTA
     // still gets an SM of its own (one 1024-thread CTA per SM), or, for large
     // candidate lists, while two rounds of clusters cover the frames (the

@@ -864,6 +864,16 @@ int max_pool_tiles(const Plan &p) {
     return m;
 }
 
+int64_t max_windows(const Plan &p) {
+    int64_t m = 0;
+    for (const FrameDesc &f : p.frames) {
+        int64_t n = 0;
+        for (int k = 0; k < f.n_levels; ++k) n += (int64_t)p.levels[f.first_level + k].rows * p.levels[f.first_level + k].cols;
+        m = std::max(m, n);
+    }
+    return m;
+}
+
 template <class T>
 const T *dptr(pd_handle *h, int64_t off) {
     return reinterpret_cast<const T *>(h->d_desc + off);
@@ -1247,6 +1257,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
     auto record = [&](cudaEvent_t e, cudaStream_t q) {
         return capturing ? cudaEventRecordWithFlags(e, q, cudaEventRecordExternal) : cudaEventRecord(e, q);
     };
+    const int cluster = nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame, max_windows(p));
     auto enqueue = [&](cudaStream_t q) -> int {
         if (n_frames)
             PD_CUDA(h, cudaMemcpyAsync(h->d_desc + o.frames, h->h_desc + o.frames,
@@ -1290,7 +1301,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         PD_CUDA(h, launch_nms(q, df, dl, n_frames, h->d_scores, h->p.threshold, h->p.nms_iou,
                               h->d_nms_scratch, h->p.max_candidates_per_frame, h->m_boxes,
                               h->p.max_boxes_per_frame, h->m_counts,
-                              nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame),
+                              cluster,
                               h->d_nms_sched, h->d_err, h->m_err));
         if (timed) PD_CUDA(h, record(h->stage_ev[4], q));
         return PD_OK;
@@ -1325,7 +1336,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
     h->err_stage = false;
     h->last_launches = (p.r_items.empty() ? 0 : 1) + (p.strips.empty() ? 0 : 1) +
                        (p.score_floats == 0 ? 0 : 1) +
-                       nms_launches(n_frames, nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame)) +
+                       nms_launches(n_frames, cluster) +
                        (h->proposal ? (p.cnn_items.empty() ? 0 : 1) + (p.levels.empty() ? 0 : 1) +
                                           (p.s_items.empty() ? 0 : 1)
                                     : 0);
@@ -1829,7 +1840,7 @@ int pd_nms_maps(pd_handle *h, void *stream, const float *d_scores, int n_levels,
     PD_CUDA(h, launch_nms(s, dptr<FrameDesc>(h, o.frames), dptr<LevelDesc>(h, o.levels), 1, d_scores,
                           h->p.threshold, h->p.nms_iou, h->d_nms_scratch, h->p.max_candidates_per_frame,
                           d_boxes, max_boxes, d_counts,
-                          nms_cluster_for(1, h->sm_count, h->p.max_candidates_per_frame)));
+                          nms_cluster_for(1, h->sm_count, h->p.max_candidates_per_frame, max_windows(p))));
     return PD_OK;
 }
 

@@ -178,7 +178,7 @@ cudaError_t launch_nms(cudaStream_t s, const FrameDesc *d_frames, const LevelDes
                        float4 *scratch, int max_cand, pd_box *boxes, int max_boxes,
                        int32_t *counts, int cluster = 1, int *sched = nullptr, const unsigned *err = nullptr,
                        unsigned *err_out = nullptr);  // err_out: where the step's error word *err goes
-int nms_cluster_for(int n_frames, int sm_count, int max_cand);
+int nms_cluster_for(int n_frames, int sm_count, int max_cand, int64_t windows);  // windows: of the largest frame
 // launch_nms with sched runs the persistent form (count, order, NMS kernels)
 bool nms_persistent(int n_frames, int cluster);
 int nms_launches(int n_frames, int cluster);  // kernels launch_nms with sched starts
