@@ -90,7 +90,7 @@
 // cleared), after B (with A: a = 1) and after C (a = 0); of a cell's 16 columns
 // b drops the first or the last 4, one b per lane of the cell. Against a CTA
 // of 128 threads per 15 x 8-cell tile, one column per thread, which voted
-// three times per pixel and counted LBP by shared-memory atomics: 583 -> 309 us
+// three times per pixel and counted LBP by shared-memory atomics: 583 -> 271 us
 // per 16 x 1242x375 frames (the shared grid: about 200). What bounds it: the
 // shared-memory pipe, where the column sums and the second clear add about
 // 170 wavefronts per cell row to the walk's 370.

@@ -501,10 +501,14 @@ void plan_tc(Plan &p, int max_rows, int sm_count) {
 void plan_strips(Plan &p, int resident_warps) {
     // A strip of r cell rows costs r + 1 bands of 8 pixel rows (one band of
     // halo), and the persistent warps take strips, tallest first, until none
-    // is left. Of the heights 32, 16, ..., 2 the planner takes the one whose
-    // schedule ends first, a shorter one only if it ends at least 3% sooner:
-    // with many rounds of strips per warp that is 32 (least halo); with few,
-    // a shorter height evens out the last round. The schedule (each strip to
+    // is left. Of the heights 32, 16, ..., 2 the planner takes the one of least
+    // cost, a shorter one only if it costs at least 5% less: with many rounds
+    // of strips per warp that is 32 (least halo); with few, a shorter height
+    // evens out the last round. Cost: the bands of the schedule plus a quarter
+    // of the height. The schedule lets all warps go equally fast, but an SM with
+    // idle warps is slower as a whole, and the taller the strips, the longer
+    // SMs end apart (16 x 1242x375: 32 rows 35 bands but 260 us, 16 rows 36
+    // bands and 228 us; 8 frames, 16 rows 140 us, 8 rows 135). The schedule (each strip to
     // the warp that is free first) is simulated when 32-row strips make fewer
     // than 16 rounds, from the histogram of strip heights with warps counted
     // per integer time (strips of one height go to the free warps in bulk).
@@ -526,6 +530,7 @@ void plan_strips(Plan &p, int resident_warps) {
         histogram(rows, n);
         return makespan(n, kMaxRows, 1, R);
     };
+    auto cost = [&](int rows) { return 4 * schedule(rows) + rows; };
     // Sparse path: one cell tile per strip. A tall strip whose tiles are partly
     // skipped leaves its warp with less than planned (8 x 1920x1080: cells
     // 297 -> 283 us).
@@ -533,10 +538,10 @@ void plan_strips(Plan &p, int resident_warps) {
     int rows = sparse ? kCellTH : kMaxRows;
     int64_t n32[kMaxRows + 1];
     if (!sparse && histogram(rows, n32) < 16 * R) {
-        int64_t best = schedule(rows);
+        int64_t best = cost(rows);
         for (int r = rows / 2; r >= 2; r /= 2) {
-            const int64_t t = schedule(r);
-            if (100 * t <= 97 * best) {
+            const int64_t t = cost(r);
+            if (100 * t <= 95 * best) {
                 best = t;
                 rows = r;
             }
