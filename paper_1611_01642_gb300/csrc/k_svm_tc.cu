@@ -46,17 +46,23 @@
 //    and stored.
 // A has three stages and D two buffers: the producers build steps s + 1 and
 // s + 2 and the epilogue reads step s - 1 while step s's MMAs run.
-// What bounds it: a step takes about 2,250 cycles: a HOG or LBP warp needs
-// about 1,750 for its 300 instructions (3.5 warps per scheduler, fixed latencies
-// and the shared-memory pipe, 51% busy), the 18 MMAs 1,010 to 1,500; handing on
-// the finished stores later, or a packed bf16 split, changed nothing.
-// 64 x 1242x375 frames: 0.334 ms; 0.661 ms with one strip of 104 columns per
+// What bounds it: a step takes about 1,850 cycles, and the LBP warps, the HOG
+// warps and the MMA warp are all busy for most of it: an LBP warp needs about
+// 1,500 for its 320 instructions (3.5 warps per scheduler, fixed latencies and the
+// shared-memory pipe, half busy), a HOG warp 1,400, the 18 MMAs 1,000 to issue
+// and 1,280 to finish, and each wait on a barrier that is already complete costs
+// about 100. The LBP warps were alone the slowest (1,780) while they held the
+// spread sums of both cell rows and all of a step's results in registers, so
+// that only a few table reads were in flight, and added the table's address
+// to each. Handing on the finished stores later, or a packed bf16 split, changed
+// nothing.
+// 64 x 1242x375 frames: 0.293 ms (0.332 with those LBP warps and the MMAs
+// issued by lane 0 alone); 0.661 ms with one strip of 104 columns per
 // CTA, LBP planes read a byte per bin and summed in place, and a single warp
 // issuing the MMAs between its epilogue rows (3,400 cycles per row, 901 rows
-// per frame; now 693 steps); two A stages instead of three: 0.344 ms. One
-// 1242x375 frame: 84 -> 31 us, with items cut until every SM has work (see the
-// planner). 14 warps leave 128 registers per thread (4 warps on a scheduler),
-// which the epilogue's loads are staged for.
+// per frame; now 693 steps). One 1242x375 frame: 84 -> 27 us, with items cut
+// until every SM has work (see the planner). 14 warps leave 128 registers per
+// thread (4 warps on a scheduler), which the epilogue's loads are staged for.
 // Per-block HOG (Algorithm 5 read per block): each staged cell row holds 36
 // HOG planes, the cell's 4 block-restricted histograms (plane 9 q + bin, q =
 // its place in the block); a block takes q = 0, 1 from its upper row and
@@ -235,6 +241,12 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
                    "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), \
                    "+f"(v[14]), "+f"(v[15])::"memory")
 
+// true in one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
 // bf16 high and low parts of a pair of floats, packed (first float in the low half)
 __device__ __forceinline__ void split2(f32x2 x, uint32_t &hi, uint32_t &lo) {
     float a, b;
@@ -303,34 +315,36 @@ __device__ __forceinline__ void build_hog(const float (&x)[36], float clip, uint
     tst2(lanes + a_lo(stage, 1), lo + 16);
 }
 
-// Horizontal sums of the LBP counts of a cell and its right neighbour, times 4
-// (table byte offsets), two 16-bit counts per word: even[w] bins 4w, 4w+2,
-// odd[w] bins 4w+1, 4w+3. Cells are 64 bytes, 16-byte chunks swizzled by the
-// cell's bits 1, 2. Counts are at most 64, so byte sums do not carry (larger
-// ones would only give another entry of the 512-entry table).
-__device__ __forceinline__ void lbp_row(const uint8_t *base, int cell, uint32_t (&even)[15], uint32_t (&odd)[15]) {
+// Horizontal sums of the LBP counts of a cell and its right neighbour, four
+// bins per word. Cells are 64 bytes, 16-byte chunks swizzled by the cell's bits
+// 1, 2. Counts are at most 64, so byte sums do not carry (larger ones would only
+// give another entry of the 512-entry table).
+__device__ __forceinline__ void lbp_row(const uint8_t *base, int cell, uint32_t (&h)[15]) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const uint4 x = *reinterpret_cast<const uint4 *>(base + cell * 64 + ((k ^ ((cell >> 1) & 3)) << 4));
         const uint4 y =
             *reinterpret_cast<const uint4 *>(base + (cell + 1) * 64 + ((k ^ (((cell + 1) >> 1) & 3)) << 4));
-        const uint32_t h[4] = {x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w};
+        const uint32_t v[4] = {x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w};
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (4 * k + u < 15) {
-                even[4 * k + u] = (h[u] << 2) & 0x03fc03fcu;
-                odd[4 * k + u] = (h[u] >> 6) & 0x03fc03fcu;
-            }
+            if (4 * k + u < 15) h[4 * k + u] = v[u];
     }
 }
 
-// bf16 split pairs of four bins from the table: columns 2 w, 2 w + 1 of the LBP part
-__device__ __forceinline__ void lbp_word(const uint32_t *tab, uint32_t e, uint32_t o, uint32_t *hi, uint32_t *lo) {
-    const uint8_t *t = reinterpret_cast<const uint8_t *>(tab);
-    const uint32_t v0 = *reinterpret_cast<const uint32_t *>(t + (e & 0xffffu));
-    const uint32_t v1 = *reinterpret_cast<const uint32_t *>(t + (o & 0xffffu));
-    const uint32_t v2 = *reinterpret_cast<const uint32_t *>(t + (e >> 16));
-    const uint32_t v3 = *reinterpret_cast<const uint32_t *>(t + (o >> 16));
+__device__ __forceinline__ uint32_t table_word(uint32_t at) {  // read-only once the constants are there
+    uint32_t v;
+    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at));
+    return v;
+}
+// bf16 split pairs of four bins from the table (columns 2 w, 2 w + 1 of the LBP
+// part): u, l the bins' sums of the upper and the lower cell row; base: the table's
+// shared-memory address, in both halves (it is below 2^16, so two addresses fit a word).
+__device__ __forceinline__ void lbp_word(uint32_t base, uint32_t u, uint32_t l, uint32_t *hi, uint32_t *lo) {
+    const uint32_t e = 4u * (__byte_perm(u, 0u, 0x4240) + __byte_perm(l, 0u, 0x4240)) + base;  // bins 4 w, 4 w + 2
+    const uint32_t o = 4u * (__byte_perm(u, 0u, 0x4341) + __byte_perm(l, 0u, 0x4341)) + base;  // bins 4 w + 1, 4 w + 3
+    const uint32_t v0 = table_word(e & 0xffffu), v1 = table_word(o & 0xffffu);
+    const uint32_t v2 = table_word(e >> 16), v3 = table_word(o >> 16);
     hi[0] = __byte_perm(v0, v1, 0x5410);
     lo[0] = __byte_perm(v0, v1, 0x7632);
     hi[1] = __byte_perm(v2, v3, 0x5410);
@@ -350,7 +364,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     TcSmem &S = *reinterpret_cast<TcSmem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (smem_u32(smem_raw) & 1023u) {  // operand and TMA alignment: never expected
+    // operand and TMA alignment, table addresses of 16 bits: never expected to fail
+    if ((smem_u32(smem_raw) & 1023u) || smem_u32(S.tab) + kTabBytes > 65536u) {
         if (tid == 0) atomicOr(err, kErrTimeout);
         return;
     }
@@ -445,40 +460,47 @@ __global__ void __launch_bounds__(kThreads, 1)
                 publish(s);
             }
         } else {
-            uint32_t ue[15], uo[15];  // the upper cell row's sums
+            const uint32_t base = smem_u32(S.tab) * 0x10001u;
+            uint32_t up[15];  // the upper cell row's sums
 #pragma unroll
-            for (int t = 0; t < 15; ++t) ue[t] = uo[t] = 0u;
+            for (int t = 0; t < 15; ++t) up[t] = 0u;
             for (uint32_t s = 0; ok; ++s) {
                 if (!(ok = warp_wait(&S.cfull[s % kSlots], (s / kSlots) & 1u))) break;
                 const uint32_t kind = S.meta[s % kMeta][g].flags & 3u;
                 if (kind == 3u) break;
-                uint32_t e[15], o[15];
-                lbp_row(S.slot[s % kSlots].lbp[g], lane, e, o);
+                uint32_t h[15];
+                lbp_row(S.slot[s % kSlots].lbp[g], lane, h);
                 __syncwarp();
                 if (lane == 0) arrive(&S.cempty[s % kSlots]);
-                uint32_t hi[30], lo[30];
-                if (kind == 2u) {
-#pragma unroll
-                    for (int w = 0; w < 15; ++w) lbp_word(S.tab, ue[w] + e[w], uo[w] + o[w], hi + 2 * w, lo + 2 * w);
-                }
-#pragma unroll
-                for (int w = 0; w < 15; ++w) {
-                    ue[w] = e[w];
-                    uo[w] = o[w];
-                }
                 if (!(ok = stage_free(s))) break;
                 if (kind == 2u) {
+                    // words 0, 1-2, 3-6, 7-10, 11-14: stored as they are ready, so that few
+                    // registers are live and many table reads in flight
                     tc_fence_after();
-                    const uint32_t a = lanes + a_hi(s % kStages), b = lanes + a_lo(s % kStages, 1);
+                    const uint32_t a = lanes + a_hi(s % kStages), b = lanes + a_lo(s % kStages, 1),
+                                   c = lanes + a_lo(s % kStages, 2);
+                    uint32_t hi[8], lo[8];
+#pragma unroll
+                    for (int w = 0; w < 3; ++w) lbp_word(base, up[w], h[w], hi + 2 * w, lo + 2 * w);
                     tst2(a + 18, hi);
                     tst4(a + 20, hi + 2);
-                    tst8(a + 24, hi + 6);
-                    tst16(a + 32, hi + 14);
                     tst2(b + 2, lo);
                     tst4(b + 4, lo + 2);
-                    tst8(b + 8, lo + 6);
-                    tst16(lanes + a_lo(s % kStages, 2), lo + 14);
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) lbp_word(base, up[3 + w], h[3 + w], hi + 2 * w, lo + 2 * w);
+                    tst8(a + 24, hi);
+                    tst8(b + 8, lo);
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+#pragma unroll
+                        for (int w = 0; w < 4; ++w)
+                            lbp_word(base, up[7 + 4 * q + w], h[7 + 4 * q + w], hi + 2 * w, lo + 2 * w);
+                        tst8(a + 32 + 8 * q, hi);
+                        tst8(c + 8 * q, lo);
+                    }
                 }
+#pragma unroll
+                for (int w = 0; w < 15; ++w) up[w] = h[w];
                 publish(s);
             }
         }
@@ -547,31 +569,35 @@ __global__ void __launch_bounds__(kThreads, 1)
                 scores[m.out + lane] = (m.keep >> lane) & 1u ? acc[kWinBH - 1] : -INFINITY;
         }
     } else if (warp == 12) {
-        // ---- MMA issue
-        if (lane == 0 && bar_wait(S, &S.bfull, 0, err)) {
-            const uint32_t b_base = smem_u32(S.b);
-            for (uint32_t s = 0;; ++s) {
-                if (!bar_wait(S, &S.mready[s % kMeta], (s / kMeta) & 1u, err)) break;
-                if ((S.meta[s % kMeta][0].flags & 3u) == 3u) break;
-                const uint32_t st = s % kStages;
-                if (!bar_wait(S, &S.afull[st], (s / kStages) & 1u, err)) break;
-                if (s >= 2 && !bar_wait(S, &S.dempty[s & 1], ((s >> 1) - 1) & 1u, err)) break;
-                tc_fence_after();
-                const uint32_t d = tmem + (s & 1) * 128;
-                const uint32_t ah = tmem + a_hi(st);  // 8 columns per K step
+        // ---- MMA issue. The whole warp walks the loop and one elected lane issues: the
+        // loop's values are uniform, so each MMA finds its operands where it reads them
+        // (a loop of lane 0 alone took 8 us longer for 64 x 1242x375 frames).
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint32_t b_base = smem_u32(S.b);
+        bool ok = warp_wait(&S.bfull, 0);
+        for (uint32_t s = 0; ok; ++s) {
+            const uint32_t st = s % kStages;
+            if (!warp_wait(&S.mready[s % kMeta], (s / kMeta) & 1u)) break;
+            if (__any_sync(0xffffffffu, (S.meta[s % kMeta][0].flags & 3u) == 3u)) break;
+            if (!warp_wait(&S.afull[st], (s / kStages) & 1u)) break;
+            if (s >= 2 && !warp_wait(&S.dempty[s & 1], ((s >> 1) - 1) & 1u)) break;
+            tc_fence_after();
+            const uint32_t d = tm + (s & 1) * 128;
+            const uint32_t ah = tm + a_hi(st);  // 8 columns per K step
+            if (elect_one()) {
 #pragma unroll
                 for (int k = 0; k < 6; ++k) umma_ts(d, ah + 8 * k, umma_desc(b_base + 256 * k), k > 0);
 #pragma unroll
                 for (int k = 0; k < 6; ++k)
-                    umma_ts(d, tmem + a_lo(st, k / 2) + 8 * (k & 1), umma_desc(b_base + 256 * k), 1);
+                    umma_ts(d, tm + a_lo(st, k / 2) + 8 * (k & 1), umma_desc(b_base + 256 * k), 1);
 #pragma unroll
                 for (int k = 0; k < 6; ++k) umma_ts(d, ah + 8 * k, umma_desc(b_base + 12 * 128 + 256 * k), 1);
                 umma_commit(&S.aempty[st]);
                 umma_commit(&S.dfull[s & 1]);
-                committed = s + 1;
             }
+            __syncwarp();
+            committed = s + 1;
         }
-        __syncwarp();
     } else {
         // ---- items and cell rows; lane g < 4 serves group g. A group draws its next item when
         // it needs it: the ring of slots covers the chain of loads, and a ticket drawn ahead
