@@ -18,20 +18,20 @@
 // instruction (fma.rn.f32x2 over pairs of channels or positions). Every kernel
 // walks a contiguous share of the batch's tiles with persistent blocks; the
 // operands of a tile sit in shared memory, the next tile's arrive there
-// (cp.async) while this one is worked on, and a thread holds 4 to 8 positions
-// times 4 to 16 channels (or 4 channels times 9 taps), so that one broadcast
+// (cp.async) while this one is worked on, and a thread holds 4 to 16 positions
+// times 4 to 16 channels (or 8 channels times 9 taps), so that one broadcast
 // load feeds 4 to 8 instructions. Weight gradients stay in registers over a
 // block's whole share and leave as one partial per block, summed in block
 // order by the last kernel.
 // 4 x 1280x720 frames (38 M pyramid pixels, 36 levels each), one step:
 // 74.4 -> 6.67 ms against one thread per position with all levels of a weight's
-// gradient in one block, and 6.67 -> 3.30 ms by fetching ahead (half of every
+// gradient in one block, and 6.67 -> 3.25 ms by fetching ahead (half of every
 // warp's waiting was for the tile's loads, with 8 to 16 warps per SM to hide
 // them): weight gradient of layer 1 with the data gradient of layer 2 2.05 ->
-// 0.69, weight gradients of layers 2 and 3 1.31 -> 0.67 and 0.75 -> 0.38, data
-// gradient of layer 3 0.55 -> 0.33, forward convolutions 0.20 -> 0.15, 0.84 ->
-// 0.49 and 0.61 -> 0.35 ms. The FP32 pipe is now 50 to 76% busy in them; in the two data
-// gradients shared memory's 75% comes first.
+// 0.675, weight gradients of layers 2 and 3 1.31 -> 0.67 and 0.75 -> 0.38, data
+// gradient of layer 3 0.55 -> 0.31, forward convolutions 0.20 -> 0.15, 0.84 ->
+// 0.49 and 0.61 -> 0.35 ms. The FP32 pipe is now 50 to 76% busy in them;
+// what is left is its throttle and dispatch stalls more than waiting.
 #include "pd_internal.h"
 
 #include <cuda_bf16.h>
@@ -489,26 +489,29 @@ __global__ void __launch_bounds__(256) t_small_grads(const TrainLevel *__restric
     if (tid == 0) out[161] = ab;
 }
 
-// Data gradient of a stride-2 layer for two horizontally adjacent quads of
-// input positions (2i, 2i+1) x (4 columns) and 8 input channels: a quad takes
-// 9 products per (output channel, input channel) from the 2 x 2 output
-// positions it reaches. d: the tile's output gradients [32][dplane], row pitch
-// DP, at (i, j); ws: [32 o][9 taps][CIN] weights at the thread's 2 NP channels.
-// acc[quad][2 * row + column][channel pair].
-template <int CIN, int DP, int NP>
-__device__ __forceinline__ void quad_pair(const float *d, int dplane, const float *ws, f32x2 (&acc)[2][4][NP]) {
+// Data gradient of a stride-2 layer for 2 x 2 quads of input positions (a quad
+// is (2i, 2i+1) x (2j, 2j+1)) and 4 input channels: a quad takes 9 products per
+// (output channel, input channel) from the 2 x 2 output positions it reaches. d: the
+// tile's output gradients [32][dplane], row pitch DP, at (i, j); ws: [32 o][9
+// taps][CIN] weights at the thread's channels.
+// acc[quad row][quad column][2 * row + column][channel pair].
+template <int CIN, int DP>
+__device__ __forceinline__ void quad_block(const float *d, int dplane, const float *ws, f32x2 (&acc)[2][2][4][2]) {
 #pragma unroll
-    for (int q = 0; q < 2; ++q)
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int p = 0; p < 4; ++p)
-#pragma unroll
-            for (int c = 0; c < NP; ++c) acc[q][p][c] = 0ull;
+        for (int p = 0; p < 4; ++p) acc[q >> 1][q & 1][p][0] = acc[q >> 1][q & 1][p][1] = 0ull;
 #pragma unroll 1
     for (int o = 0; o < 32; ++o) {
         const float *dp = d + o * dplane;
-        const float2 t = *reinterpret_cast<const float2 *>(dp), u = *reinterpret_cast<const float2 *>(dp + DP);
-        const f32x2 top[3] = {dup2(t.x), dup2(t.y), dup2(dp[2])};
-        const f32x2 bot[3] = {dup2(u.x), dup2(u.y), dup2(dp[DP + 2])};
+        f32x2 v[3][3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const float2 t = *reinterpret_cast<const float2 *>(dp + r * DP);
+            v[r][0] = dup2(t.x);
+            v[r][1] = dup2(t.y);
+            v[r][2] = dup2(dp[r * DP + 2]);
+        }
         const float *wo = ws + o * 9 * CIN;
         // tap, input position (2 * row + column), output position (row, column)
         constexpr int kTap[9] = {4, 3, 5, 1, 7, 0, 2, 6, 8};
@@ -517,25 +520,20 @@ __device__ __forceinline__ void quad_pair(const float *d, int dplane, const floa
         constexpr int kCol[9] = {0, 1, 0, 0, 0, 1, 0, 1, 0};
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            ulonglong2 w[NP / 2];
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(wo + kTap[k] * CIN);
 #pragma unroll
-            for (int c = 0; c < NP / 2; ++c) w[c] = *reinterpret_cast<const ulonglong2 *>(wo + kTap[k] * CIN + 4 * c);
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const f32x2 v = kRow[k] ? bot[q + kCol[k]] : top[q + kCol[k]];
-                f32x2(&a)[NP] = acc[q][kPos[k]];
-#pragma unroll
-                for (int c = 0; c < NP / 2; ++c) {
-                    a[2 * c] = fma2(w[c].x, v, a[2 * c]);
-                    a[2 * c + 1] = fma2(w[c].y, v, a[2 * c + 1]);
-                }
+            for (int q = 0; q < 4; ++q) {
+                const f32x2 x = v[(q >> 1) + kRow[k]][(q & 1) + kCol[k]];
+                f32x2(&a)[2] = acc[q >> 1][q & 1][kPos[k]];
+                a[0] = fma2(w.x, x, a[0]);
+                a[1] = fma2(w.y, x, a[1]);
             }
         }
     }
 }
 
 // ---- dz2 = (a2 > 0) * data gradient of layer 3: a tile is 16 x 8 quads
-// (32 x 16 layer-2 positions), 64 quad pairs x 4 groups of 8 channels.
+// (32 x 16 layer-2 positions), 32 blocks of 2 x 2 quads x 8 groups of 4 channels.
 constexpr int kD3P = 20;  // staged dz3 row pitch (17 columns)
 struct Dz2Smem {
     float ws[32 * 9 * 32];           // [o][tap][c]
@@ -563,7 +561,7 @@ __global__ void __launch_bounds__(256) t_dz2(const TrainLevel *__restrict__ tl, 
             copy_row16(ds + 4 * e, d + (int64_t)o * H3 * P3, i0 + i, j0 + 4 * q, H3, W3, P3);
         }
     };
-    const int c0 = 8 * (tid >> 6), qx = tid & 7, qr = (tid >> 3) & 7;
+    const int c0 = 4 * (tid >> 5), qx = tid & 7, qy = (tid >> 3) & 3;
     if (wk.valid()) fetch(S.ds[0]);
 #pragma unroll 1
     for (int b = 0; wk.valid(); b ^= 1) {
@@ -582,22 +580,22 @@ __global__ void __launch_bounds__(256) t_dz2(const TrainLevel *__restrict__ tl, 
         }
         wk.step(n_tiles);
         if (wk.valid()) fetch(S.ds[b ^ 1]);
-        f32x2 acc[2][4][4];
-        quad_pair<32, kD3P, 4>(S.ds[b] + qr * kD3P + 2 * qx, 9 * kD3P, S.ws + c0, acc);
+        f32x2 acc[2][2][4][2];
+        quad_block<32, kD3P>(S.ds[b] + 2 * qy * kD3P + 2 * qx, 9 * kD3P, S.ws + c0, acc);
         copies_done();
         __syncthreads();  // the mask is there
         const int x = x0 + 4 * qx;
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            const int y = y0 + 2 * qr + a;
+        for (int a = 0; a < 4; ++a) {
+            const int y = y0 + 4 * qy + a;
             if (y >= H2 || x >= P2) continue;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const uint2 m = *reinterpret_cast<const uint2 *>(S.a2 + ((c0 + c) * 16 + 2 * qr + a) * 32 + 4 * qx);
+            for (int c = 0; c < 4; ++c) {
+                const uint2 m = *reinterpret_cast<const uint2 *>(S.a2 + ((c0 + c) * 16 + 4 * qy + a) * 32 + 4 * qx);
                 float v[4];
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
-                    const f32x2 s = acc[p >> 1][2 * a + (p & 1)][c >> 1];
+                    const f32x2 s = acc[a >> 1][p >> 1][2 * (a & 1) + (p & 1)][c >> 1];
                     v[p] = c & 1 ? hi2(s) : lo2(s);
                 }
                 *reinterpret_cast<float4 *>(out + ((int64_t)(c0 + c) * H2 + y) * P2 + x) =
@@ -609,12 +607,13 @@ __global__ void __launch_bounds__(256) t_dz2(const TrainLevel *__restrict__ tl, 
 }
 
 // ---- layer 1's weight gradient. dz1 = (a1 > 0) * data gradient of layer 2 is
-// only needed for it, so a thread keeps its 8 positions x 4 channels of dz1 in
-// registers and adds their products with the input pixels to its own sums;
+// only needed for it, so a thread keeps its 4 x 4 positions x 4 channels of dz1
+// in registers and adds their products with the input pixels to its own sums;
 // dz1 is never written (it would be 2 x 64 bytes per position of traffic). A
-// tile is 32 x 8 quads (64 x 16 layer-1 positions): 128 quad pairs x 4 channel
-// groups. (8 channels per thread, 8 warps and a ninth to copy: 168 registers, so
-// that the loads of the weights were waited for, 1.01 ms against 0.69.)
+// tile is 32 x 8 quads (64 x 16 layer-1 positions): 64 blocks of 2 x 2 quads x 4
+// channel groups. (Two quads and 4 channels per thread on twice the warps: shared
+// memory 76% busy, 0.69 ms against 0.675; two quads and 8 channels, with a ninth
+// warp to copy: 168 registers, the loads of the weights waited for, 1.01 ms.)
 constexpr int kD2P = 36;  // staged dz2 row pitch (33 columns)
 constexpr int kW1Parts = 160;
 struct Dw1Stage {
@@ -627,9 +626,9 @@ struct Dw1Smem {
     Dw1Stage st[2];
     float E[33 * kXE], O[33 * kXO];  // input pixels
     float lut[256];
-    float red[16 * 40];
+    float red[8 * 40];
 };
-__global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
+__global__ void __launch_bounds__(256, 1) t_dw1(const TrainLevel *__restrict__ tl, int n_tl, int n_tiles,
                                                 const LevelDesc *__restrict__ levels,
                                                 const uint8_t *__restrict__ pyr, const float *__restrict__ in_tab,
                                                 const float *__restrict__ w, const __nv_bfloat16 *__restrict__ act,
@@ -637,8 +636,8 @@ __global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ t
     extern __shared__ __align__(16) unsigned char smem_b[];
     Dw1Smem &S = *reinterpret_cast<Dw1Smem *>(smem_b);
     const int tid = threadIdx.x;
-    if (tid < 256) S.lut[tid] = in_tab[tid];
-    for (int i = tid; i < 32 * 9 * 16; i += 512) {
+    S.lut[tid] = in_tab[tid];
+    for (int i = tid; i < 32 * 9 * 16; i += 256) {
         const int c = i & 15, ot = i >> 4, o = ot / 9;
         S.ws[i] = w[(o * 16 + c) * 9 + ot - 9 * o];
     }
@@ -648,21 +647,21 @@ __global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ t
         const LevelDesc &L = levels[T.level];
         const int ntx = (T.W2 + 31) / 32, lt = wk.local();
         const int i0 = 8 * (lt / ntx), j0 = 32 * (lt % ntx);
-        if (tid < 33 * 9) copy_pixels(st.raw, pyr + L.img_off, L, 2 * i0, 2 * j0, tid);
+        for (int e = tid; e < 33 * 9; e += 256) copy_pixels(st.raw, pyr + L.img_off, L, 2 * i0, 2 * j0, e);
         const int H2 = T.H2, W2 = T.W2, P2 = T.P2, H1 = T.H1, W1 = T.W1, P1 = T.P1;
         const float *d = dz2 + T.d2;
-        for (int e = tid; e < 32 * 9 * 9; e += 512) {
+        for (int e = tid; e < 32 * 9 * 9; e += 256) {
             const int row = e / 9, q = e - 9 * row, o = row / 9, i = row - 9 * o;
             copy_row16(st.ds + 4 * e, d + (int64_t)o * H2 * P2, i0 + i, j0 + 4 * q, H2, W2, P2);
         }
         const __nv_bfloat16 *a1 = act + T.a1;
 #pragma unroll
-        for (int e = tid; e < 16 * 16 * 8; e += 512) {
+        for (int e = tid; e < 16 * 16 * 8; e += 256) {
             const int c = e >> 7, r = (e >> 3) & 15, q = e & 7;
             copy_row16(st.a1 + 8 * e, a1 + (int64_t)c * H1 * P1, 2 * i0 + r, 2 * j0 + 8 * q, H1, W1, P1);
         }
     };
-    const int c0 = 4 * (tid >> 7), qx = tid & 15, qr = (tid >> 4) & 7;
+    const int c0 = 4 * (tid >> 6), qx = tid & 15, qy = (tid >> 4) & 3;
     f32x2 sum[10][2];
 #pragma unroll
     for (int k = 0; k < 10; ++k) sum[k][0] = sum[k][1] = 0ull;
@@ -676,18 +675,18 @@ __global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ t
             const TrainLevel &T = tl[wk.k];
             const LevelDesc &L = levels[T.level];
             const int ntx = (T.W2 + 31) / 32, lt = wk.local();
-            spread_pixels<512>(st.raw, L, S.lut, 16 * (lt / ntx), 64 * (lt % ntx), S.E, S.O);
+            spread_pixels<256>(st.raw, L, S.lut, 16 * (lt / ntx), 64 * (lt % ntx), S.E, S.O);
         }
         wk.step(n_tiles);
         if (wk.valid()) fetch(S.st[b ^ 1]);
-        f32x2 acc[2][4][2];
-        quad_pair<16, kD2P, 2>(st.ds + qr * kD2P + 2 * qx, 9 * kD2P, S.ws + c0, acc);
+        f32x2 acc[2][2][4][2];
+        quad_block<16, kD2P>(st.ds + 2 * qy * kD2P + 2 * qx, 9 * kD2P, S.ws + c0, acc);
         // relu mask of a1 (0 outside the level)
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < 4; ++a) {
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                const __nv_bfloat16 *src = st.a1 + ((c0 + 2 * c) * 16 + 2 * qr + a) * 64 + 4 * qx;
+                const __nv_bfloat16 *src = st.a1 + ((c0 + 2 * c) * 16 + 4 * qy + a) * 64 + 4 * qx;
                 const uint2 m0 = *reinterpret_cast<const uint2 *>(src);
                 const uint2 m1 = *reinterpret_cast<const uint2 *>(src + 16 * 64);
 #pragma unroll
@@ -695,17 +694,17 @@ __global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ t
                     const uint32_t u0 = p < 2 ? m0.x : m0.y, u1 = p < 2 ? m1.x : m1.y;
                     const bool k0 = (p & 1 ? bf_hi(u0) : bf_lo(u0)) > 0.f;
                     const bool k1 = (p & 1 ? bf_hi(u1) : bf_lo(u1)) > 0.f;
-                    f32x2 &s = acc[p >> 1][2 * a + (p & 1)][c];
+                    f32x2 &s = acc[a >> 1][p >> 1][2 * (a & 1) + (p & 1)][c];
                     s = pack2(k0 ? lo2(s) : 0.f, k1 ? hi2(s) : 0.f);
                 }
             }
         }
         __syncthreads();  // the pixels are there
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < 4; ++a) {
 #pragma unroll
             for (int dy = 0; dy < 3; ++dy) {
-                const int r = 2 * (2 * qr + a) + dy;
+                const int r = 2 * (4 * qy + a) + dy;
                 const float4 e = *reinterpret_cast<const float4 *>(S.E + r * kXE + 4 * qx);
                 const float4 o4 = *reinterpret_cast<const float4 *>(S.O + r * kXO + 4 * qx);
                 const f32x2 ev[4] = {dup2(e.x), dup2(e.y), dup2(e.z), dup2(e.w)};
@@ -714,7 +713,7 @@ __global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ t
                 for (int p = 0; p < 4; ++p)
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
-                        const f32x2 d = acc[p >> 1][2 * a + (p & 1)][c];
+                        const f32x2 d = acc[a >> 1][p >> 1][2 * (a & 1) + (p & 1)][c];
                         sum[3 * dy][c] = fma2(d, ov[p], sum[3 * dy][c]);
                         sum[3 * dy + 1][c] = fma2(d, ev[p], sum[3 * dy + 1][c]);
                         sum[3 * dy + 2][c] = fma2(d, ov[p + 1], sum[3 * dy + 2][c]);
@@ -733,8 +732,8 @@ __global__ void __launch_bounds__(512, 1) t_dw1(const TrainLevel *__restrict__ t
     __syncthreads();
     if (tid < kW1Parts) {  // order: 144 weights [c][tap], 16 biases
         const int c = tid < 144 ? tid / 9 : tid - 144, k = tid < 144 ? tid % 9 : 9;
-        const float *r = S.red + (c >> 2) * 4 * 40 + k * 4 + (c & 3);
-        part[(int64_t)blockIdx.x * kW1Parts + tid] = ((r[0] + r[40]) + r[80]) + r[120];
+        const float *r = S.red + (c >> 2) * 2 * 40 + k * 4 + (c & 3);
+        part[(int64_t)blockIdx.x * kW1Parts + tid] = r[0] + r[40];
     }
 }
 
@@ -985,7 +984,7 @@ cudaError_t launch_train_step(cudaStream_t s, const TrainArgs &a) {
     t_dw23<32><<<G, 256, dw23_smem(32), s>>>(a.tl, nl, a.tiles[3], a.act16, a.act32, p3);
     t_dz2<<<G, blk, kDz2Smem, s>>>(a.tl, nl, a.tiles[3], a.act32, a.wr + kOffW3, a.act16, a.dz2);
     t_dw23<16><<<G, 256, dw23_smem(16), s>>>(a.tl, nl, a.tiles[1], a.act16, a.dz2, p2);
-    t_dw1<<<G, 512, kDw1Smem, s>>>(a.tl, nl, a.tiles[0], a.levels, a.pyr, a.w.in_tab, a.wr + kOffW2, a.act16, a.dz2,
+    t_dw1<<<G, 256, kDw1Smem, s>>>(a.tl, nl, a.tiles[0], a.levels, a.pyr, a.w.in_tab, a.wr + kOffW2, a.act16, a.dz2,
                                    p1);
     t_finish<<<(kCnnParams + 31) / 32, blk, 0, s>>>(p1, G, p2, G, p3, G, ps, G, a.grad, a.master, a.m, a.v, a.wr, a.lr,
                                                     a.beta1, a.beta2, a.eps, a.c1, a.c2);
