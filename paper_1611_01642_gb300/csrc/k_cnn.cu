@@ -11,16 +11,18 @@
 //
 // k_cnn_fwd: persistent CTAs (8 warps, two per SM), each walking 8x8-cell
 // tiles. The 72x96 input bytes of the next tile are fetched by TMA
-// while the current tile is computed. Per tile: the pixels become bf16 x
+// while the current tile is computed, and its pixels and layer 1 are done while
+// the current tile's layer 3 is on the tensor cores; the head of the last tile
+// goes with the current one's layer 2. Per tile: the pixels become bf16 x
 // (zero outside the level: the padding of layer 1); layer 1 runs on the
 // tensor cores as a GEMM over 4x4 pixel patches (a stride-2 3x3 window at
 // (2r-1, 2c-1) is the top-left 3x3 of the 4x4 patch there; the 7 extra taps
 // carry zero weights; mma.sync m16n8k16), giving 35x35x16 activations.
-// What bounds it: the phases of a tile follow one another behind block
-// barriers (issue 47%, barrier and tensor-memory waits), so the conversion and
-// layer 1's index arithmetic are in the way: 8 pixels per conversion step with
+// What bounds it: issue (about half of the cycles), and the phases of a tile
+// follow one another behind block barriers: 8 pixels per conversion step with
 // packed float operations and positions stepped instead of divided took it
-// from 279 to 243 us per 8 x 1920x1080 frames (network on every 4th level).
+// from 279 to 243 us per 8 x 1920x1080 frames (network on every 4th level), the
+// next tile's work under layer 3's MMAs (4 barriers per tile instead of 7) to 230.
 // Layer 2 (17x17x32, K = 9 taps x 16) and layer 3 (8x8x32, K = 9 x 32) are
 // implicit GEMMs on the 5th-generation tensor cores: one thread issues
 // tcgen05.mma with both operands in shared memory (no-swizzle K-major
@@ -50,7 +52,7 @@ constexpr int R1 = 2 * R2 + 1;   // 35 layer-1 positions per side
 constexpr int XR = 2 * R1 + 2;   // 72 pixel rows/columns under the 4x4 patches
 constexpr int kRawW = kCnnBoxW;  // staged bytes per row: pixels x0-9 .. x0+86 (TMA box)
 static_assert(XR == kCnnBoxH, "input box height");
-static_assert((XR * kRawW) % 128 == 0, "second raw buffer stays 128-byte aligned");
+static_assert((XR * kRawW) % 16 == 0, "the planes after the raw buffer are 16-byte aligned");
 static_assert(XR % 8 == 0, "8 pixels per conversion step");
 constexpr int XBW = 44;          // bf16 pixel row stride in words (72 used, padded for banks)
 // Activations are stored as 16-byte rows of 8 bf16 channels, split by
@@ -78,13 +80,17 @@ constexpr int kEdge = 2 * R2 - 1; // 33 edge positions
 constexpr uint32_t kTmemCols = 128;  // L2 core accumulators in columns [0,64), L3 in [64,96)
 constexpr uint64_t kWaitNs = 1000000000ull;
 
+// A tile of the walk: its first cell, and what its phases read of its level.
+struct TileInfo {
+    int level, cy0, cx0, Hk, Wk, Hc, Wc, cell_row;
+};
+
 struct CnnSmem {
-    uint8_t raw[2][XR][kRawW];   // input bytes, double buffered (TMA destinations: 128-byte aligned)
+    uint8_t raw[XR][kRawW];      // input bytes (TMA destination: 128-byte aligned)
     uint4 a1[2 * 2 * PS1];       // [channel group 0..1][parity] planes of layer 1
-    union {
-        uint32_t xb[XR * XBW];   // bf16 pixel pairs (dead once layer 1 is done)
-        uint4 a2[4 * 2 * PS2];   // [channel group 0..3][parity] planes of layer 2
-    } u;
+    uint4 a2[4 * 2 * PS2];       // [channel group 0..3][parity] planes of layer 2
+    uint32_t xb[XR * XBW];       // bf16 pixel pairs
+    TileInfo info[4];            // tiles i - 1 .. i + 2 of the walk
     uint8_t w2c[9 * kBTapBytes];      // layer-2 B operands, one per tap
     uint8_t w3c[9 * 2 * kBTapBytes];  // layer-3 B operands, per tap and input-channel half
     float b2[32];
@@ -92,9 +98,8 @@ struct CnnSmem {
     float wh[32];
     float hpart[2][64];
     unsigned long long bar;      // MMA completion (one phase per commit)
-    unsigned long long inbar[2]; // input tile arrival, one per raw buffer
+    unsigned long long inbar;    // input tile arrival
     uint32_t tmem;               // tensor-memory base of this CTA
-    int failed;
 };
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -185,7 +190,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 }
 
 // Every thread waits (bounded) for phase `parity` of the MMA barrier; a wait
-// that gives up sets the error word and the CTA's failed flag.
+// that gives up sets the error word.
 __device__ __forceinline__ bool mma_wait(CnnSmem &S, uint32_t parity, unsigned *err) {
     const uint32_t a = smem_u32(&S.bar);
     uint32_t ok = 0;
@@ -198,10 +203,7 @@ __device__ __forceinline__ bool mma_wait(CnnSmem &S, uint32_t parity, unsigned *
             : "memory");
         if (ok || global_ns() - t0 > kWaitNs) break;
     }
-    if (!ok) {
-        S.failed = 1;
-        if (err) atomicOr(err, kErrTimeout);
-    }
+    if (!ok && err) atomicOr(err, kErrTimeout);
     return ok != 0;
 }
 
@@ -210,7 +212,7 @@ __device__ __forceinline__ bool mma_wait(CnnSmem &S, uint32_t parity, unsigned *
 // x coordinate is a multiple of 16 bytes; outside the level the box reads
 // zeros, and the conversion zeroes those pixels anyway).
 __device__ __forceinline__ void load_input(uint8_t (*raw)[kRawW], unsigned long long *bar,
-                                           const CUtensorMap *__restrict__ maps, const CnnItem &it) {
+                                           const CUtensorMap *__restrict__ maps, const TileInfo &it) {
     const uint32_t b = smem_u32(bar);
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"((uint32_t)(kRawW * XR))
                  : "memory");
@@ -252,20 +254,25 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
     CnnSmem &S = *reinterpret_cast<CnnSmem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t = lane & 3;
-    int item = blockIdx.x;
-    if (item >= n_items) return;
+    const int n_mine = (n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    if (n_mine <= 0) return;
     if (smem_u32(S.raw) & 127u) {  // TMA destinations need 128-byte alignment: never expected
         if (tid == 0 && err) atomicOr(err, kErrTimeout);
         return;
     }
+    auto fill_info = [&](int i) {
+        const CnnItem it = items[blockIdx.x + (int64_t)i * gridDim.x];
+        const LevelDesc &L = levels[it.level];
+        S.info[i & 3] = {it.level, it.cy0, it.cx0, L.Hk, L.Wk, L.Hc, L.Wc, L.cell_row};
+    };
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&S.inbar[0])));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&S.inbar[1])));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&S.inbar)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        load_input(S.raw[0], &S.inbar[0], lvl_maps, items[item]);
+        fill_info(0);
+        load_input(S.raw, &S.inbar, lvl_maps, S.info[0]);
+        if (n_mine > 1) fill_info(1);
     }
-    // thread 0: loads issued and not yet consumed (bit b: raw buffer b) and their phase parities
-    uint32_t pend = tid == 0 ? 1u : 0u, ppar = 0u;
+    int loads = 1;  // input tiles sent for (thread 0's count is the one used)
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem)),
@@ -275,7 +282,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&S.bar)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        S.failed = 0;
     }
     // canonical B operands of layers 2 and 3 from the bf16-rounded weights
     for (int i = tid; i < 9 * 32 * 16; i += kThreads) {
@@ -314,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
     const float b1r[4] = {wts.b1[2 * t], wts.b1[2 * t + 1], wts.b1[8 + 2 * t], wts.b1[8 + 2 * t + 1]};
     const float bh = wts.bh[0];
     const uint32_t a1_base = smem_u32(&S.a1[0]);
-    const uint32_t a2_base = smem_u32(&S.u.a2[0]);
+    const uint32_t a2_base = smem_u32(&S.a2[0]);
     const uint32_t w2c_base = smem_u32(S.w2c), w3c_base = smem_u32(S.w3c);
     async_proxy_fence();  // the B operands are read by the tensor cores
     tc_fence_before();
@@ -323,38 +329,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
     const uint32_t tmem = S.tmem;
     uint32_t phase = 0;  // parity of the next MMA barrier phase
 
-    for (int iter = 0; item < n_items && !S.failed; ++iter, item += gridDim.x) {
-        const int cur = iter & 1;
-        const int next = item + gridDim.x;
-        if (tid == 0 && next < n_items) {
-            async_proxy_fence();  // the buffer's previous bytes were read by the generic proxy
-            load_input(S.raw[cur ^ 1], &S.inbar[cur ^ 1], lvl_maps, items[next]);
-            pend |= 1u << (cur ^ 1);
-            ppar = (ppar & ~(1u << (cur ^ 1))) | ((((uint32_t)(iter + 1) >> 1) & 1u) << (cur ^ 1));
-        }
-        // this tile's input: phase iter / 2 of its buffer's barrier (CTA-uniform decision)
-        const bool in_ok = bar_wait(&S.inbar[cur], (uint32_t)(iter >> 1) & 1u);
-        if (tid == 0 && in_ok) pend &= ~(1u << cur);
-        if (__syncthreads_or(!in_ok)) {
-            if (tid == 0) {
-                S.failed = 1;
-                if (err) atomicOr(err, kErrTimeout);
-            }
-            break;
-        }
-
-        const CnnItem it = items[item];
-        const LevelDesc L = levels[it.level];
-        const int Hk = L.Hk, Wk = L.Wk;
-        const int H1 = (Hk + 1) / 2, W1 = (Wk + 1) / 2;
-        const int H2 = (H1 + 1) / 2, W2 = (W1 + 1) / 2;
-        const int y3 = it.cy0, x3 = it.cx0;                  // tile origin (cells)
-        const int y2 = 2 * y3 - 1, x2 = 2 * x3 - 1;          // layer-2 region origin
-        const int y1 = 2 * y2 - 1, x1 = 2 * x2 - 1;          // layer-1 region origin
-        const int y0 = 2 * y1 - 1, x0 = 2 * x1 - 1;          // pixel region origin
-        const bool interior1 = y1 >= 0 && x1 >= 0 && y1 + R1 <= H1 && x1 + R1 <= W1;
-        const bool interior2 = y2 >= 0 && x2 >= 0 && y2 + R2 <= H2 && x2 + R2 <= W2;
-
+    // ---- the phases of a tile; what each needs of it comes from S.info
+    auto convert = [&](const TileInfo &T) {
+        const int Hk = T.Hk, Wk = T.Wk, y0 = 8 * T.cy0 - 7, x0 = 8 * T.cx0 - 7;  // pixel region origin
         // ---- pixels -> bf16 x; xb[r][c] = x(y0 + r, x0 + c) = raw[r][c + 9].
         // x = bf16(L/255 - 0.5): one fma in float32 rounded once to bf16 equals
         // the correctly rounded value for all 256 inputs (checked exhaustively
@@ -363,7 +340,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
         const bool interior0 = y0 >= 0 && x0 >= 0 && y0 + XR <= Hk && x0 + XR <= Wk;
         for (int k = tid; k < XR * (XR / 8); k += kThreads) {
             const int r = k / (XR / 8), j = k - r * (XR / 8);
-            const uint32_t *rw = reinterpret_cast<const uint32_t *>(S.raw[cur][r]) + 2 * j + 2;
+            const uint32_t *rw = reinterpret_cast<const uint32_t *>(S.raw[r]) + 2 * j + 2;
             const uint32_t m = rw[1];
             const uint32_t v[2] = {__byte_perm(rw[0], m, 0x4321), __byte_perm(m, rw[2], 0x4321)};  // bytes 8j + 9 ..
             uint32_t o[4];
@@ -385,15 +362,18 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
                     o[h] &= (rin && x >= 0 && x < Wk ? 0xffffu : 0u) | (rin && x + 1 >= 0 && x + 1 < Wk ? 0xffff0000u : 0u);
                 }
             }
-            *reinterpret_cast<uint4 *>(&S.u.xb[r * XBW + 4 * j]) = make_uint4(o[0], o[1], o[2], o[3]);
+            *reinterpret_cast<uint4 *>(&S.xb[r * XBW + 4 * j]) = make_uint4(o[0], o[1], o[2], o[3]);
         }
-        __syncthreads();
+    };
+    auto layer1 = [&](const TileInfo &T) {
+        const int H1 = (T.Hk + 1) / 2, W1 = (T.Wk + 1) / 2, y1 = 4 * T.cy0 - 3, x1 = 4 * T.cx0 - 3;  // region origin
+        const bool interior1 = y1 >= 0 && x1 >= 0 && y1 + R1 <= H1 && x1 + R1 <= W1;
         // ---- layer 1 on tensor cores (mma.sync): 1225 positions x 16 channels, K = 16 (4x4 patch)
         // A warp's tiles are 128 positions (3 rows and 23 columns) apart.
         int r0 = rs0, c0 = cs0, r1 = rs1, c1 = cs1, pr = prs, pc = pcs;
         for (int mt = warp; mt < M1T; mt += kThreads / 32) {
-            const uint32_t *x0w = &S.u.xb[(2 * r0 + (t >> 1)) * XBW + c0 + (t & 1)];
-            const uint32_t *x1w = &S.u.xb[(2 * r1 + (t >> 1)) * XBW + c1 + (t & 1)];
+            const uint32_t *x0w = &S.xb[(2 * r0 + (t >> 1)) * XBW + c0 + (t & 1)];
+            const uint32_t *x1w = &S.xb[(2 * r1 + (t >> 1)) * XBW + c1 + (t & 1)];
             const uint32_t a0 = x0w[0], a1 = x1w[0], a2 = x0w[2 * XBW], a3 = x1w[2 * XBW];
             float acc[2][4];
 #pragma unroll
@@ -422,10 +402,64 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
             next_tile(r1, c1);
             next_tile(pr, pc);
         }
-        async_proxy_fence();  // layer-1 planes are read by the tensor cores next
+    };
+    auto head = [&]() {
+        // ---- layer-3 epilogue and head: M = 64 rows sit in lanes 32 q + (0..15) of
+        // quadrant q (rows 16 q .. 16 q + 15); warps 0-3 take channels 0-15, warps 4-7 16-31
+        {
+            const int q = warp & 3, half = warp >> 2;
+            float v[16];
+            tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + 64 + 16 * half, v);
+            float hp = 0.f;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int ch = 16 * half + i;
+                hp = fmaf(fmaxf(v[i] + S.b3[ch], 0.f), S.wh[ch], hp);
+            }
+            if (lane < 16) S.hpart[half][16 * q + lane] = hp;
+        }
+    };
+    auto store_head = [&](const TileInfo &T) {
+        if (tid < 64) {
+            const int cy = T.cy0 + (tid >> 3), cx = T.cx0 + (tid & 7);
+            if (cy < T.Hc && cx < T.Wc)
+                hmap[(int64_t)(T.cell_row + cy) * hmap_pitch + cx] = bh + S.hpart[0][tid] + S.hpart[1][tid];
+        }
+    };
+    // the tile whose input has arrived becomes bf16 pixels, the next tile is sent for (CTA-uniform result)
+    auto take_input = [&](int i) {
+        const bool in_ok = bar_wait(&S.inbar, (uint32_t)i & 1u);
+        convert(S.info[i & 3]);
+        if (__syncthreads_or(!in_ok)) {
+            if (tid == 0 && err) atomicOr(err, kErrTimeout);
+            return false;
+        }
+        if (tid == 0 && i + 1 < n_mine) {
+            async_proxy_fence();  // the buffer's bytes were read by the generic proxy
+            load_input(S.raw, &S.inbar, lvl_maps, S.info[(i + 1) & 3]);
+            loads = i + 2;
+        }
+        return true;
+    };
+    // ends a phase whose planes the tensor cores read next
+    auto hand_over = [&] {
+        async_proxy_fence();
         tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
+    };
+
+    bool ok = take_input(0);
+    if (ok) {
+        layer1(S.info[0]);
+        hand_over();
+    }
+    __syncthreads();
+    tc_fence_after();
+    for (int i = 0; ok && i < n_mine; ++i) {
+        const TileInfo &T = S.info[i & 3];
+        const int Hk = T.Hk, Wk = T.Wk;
+        const int H2 = ((Hk + 1) / 2 + 1) / 2, W2 = ((Wk + 1) / 2 + 1) / 2;
+        const int y2 = 2 * T.cy0 - 1, x2 = 2 * T.cx0 - 1;  // layer-2 region origin
+        const bool interior2 = y2 >= 0 && x2 >= 0 && y2 + R2 <= H2 && x2 + R2 <= W2;
         // ---- layer 2, outputs [0,16)^2 on tcgen05: two 16-row x 8-column blocks (M = 128),
         // N = 32, K = 16 per tap. A for tap (dy, dx), block c0: rows 2r + dy of the
         // parity-(dx & 1) plane, columns c0 + dx / 2 + 0..7; 8-row groups 2 plane rows apart.
@@ -442,6 +476,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
                 }
             umma_commit(&S.bar);
         }
+        // meanwhile: the last tile's head, the edges, and the tile after the next
+        if (i > 0) head();
+        if (tid == kThreads - 32 && i + 2 < n_mine) fill_info(i + 2);
         // ---- layer 2 edges (row 16, column 16: 33 positions) on mma.sync, meanwhile
         if (warp < 3) {
             const int mt = warp;
@@ -479,9 +516,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
                         in0 ? relu_pack_bf16(acc[2 * h + 1][0], acc[2 * h + 1][1]) : 0u,
                         in1 ? relu_pack_bf16(acc[2 * h + 1][2], acc[2 * h + 1][3]) : 0u);
         }
-        if (__syncthreads_or(!mma_wait(S, phase, err))) break;  // CTA-uniform
+        ok = !__syncthreads_or(!mma_wait(S, phase, err));  // CTA-uniform
+        if (!ok) break;
         phase ^= 1u;
         tc_fence_after();
+        if (i > 0) store_head(S.info[(i - 1) & 3]);
         // ---- layer-2 core epilogue: warp w reads lanes 32 (w % 4) .. + 31 of block w / 4:
         // lane m = 32 (w % 4) + l holds output (r, c) = (m / 8, 8 (w / 4) + m % 8), 32 channels
         {
@@ -501,12 +540,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
                     q.y = in ? relu_pack_bf16(v[8 * gg + 2] + bb[2], v[8 * gg + 3] + bb[3]) : 0u;
                     q.z = in ? relu_pack_bf16(v[8 * gg + 4] + bb[4], v[8 * gg + 5] + bb[5]) : 0u;
                     q.w = in ? relu_pack_bf16(v[8 * gg + 6] + bb[6], v[8 * gg + 7] + bb[7]) : 0u;
-                    S.u.a2[(grp * 2 + (c & 1)) * PS2 + r * C2P + (c >> 1)] = q;
+                    S.a2[(grp * 2 + (c & 1)) * PS2 + r * C2P + (c >> 1)] = q;
                 }
             }
         }
-        async_proxy_fence();  // layer-2 planes are read by the tensor cores next
-        tc_fence_before();
+        hand_over();
         __syncthreads();
         tc_fence_after();
         // ---- layer 3 on tcgen05: 8 x 8 outputs (M = 64), N = 32, K = 9 taps x 2 halves x 16
@@ -524,34 +562,23 @@ __global__ void __launch_bounds__(kThreads, 2) k_cnn_fwd(const LevelDesc *__rest
                 }
             umma_commit(&S.bar);
         }
-        if (__syncthreads_or(!mma_wait(S, phase, err))) break;  // CTA-uniform
+        // meanwhile: the next tile's pixels and layer 1
+        if (i + 1 < n_mine) {
+            ok = take_input(i + 1);
+            if (ok) layer1(S.info[(i + 1) & 3]);
+        }
+        hand_over();
+        ok = !__syncthreads_or(!mma_wait(S, phase, err)) && ok;
         phase ^= 1u;
         tc_fence_after();
-        // ---- layer-3 epilogue and head: M = 64 rows sit in lanes 32 q + (0..15) of
-        // quadrant q (rows 16 q .. 16 q + 15); warps 0-3 take channels 0-15, warps 4-7 16-31
-        {
-            const int q = warp & 3, half = warp >> 2;
-            float v[16];
-            tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + 64 + 16 * half, v);
-            float hp = 0.f;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int ch = 16 * half + i;
-                hp = fmaf(fmaxf(v[i] + S.b3[ch], 0.f), S.wh[ch], hp);
-            }
-            if (lane < 16) S.hpart[half][16 * q + lane] = hp;
-        }
-        __syncthreads();
-        if (tid < 64) {
-            const int cy = y3 + (tid >> 3), cx = x3 + (tid & 7);
-            if (cy < L.Hc && cx < L.Wc)
-                hmap[(int64_t)(L.cell_row + cy) * hmap_pitch + cx] = bh + S.hpart[0][tid] + S.hpart[1][tid];
-        }
     }
-    // drain loads still in flight (bounded) before the CTA leaves
-    if (tid == 0)
-        for (int b = 0; b < 2; ++b)
-            if ((pend >> b) & 1u) bar_wait(&S.inbar[b], (ppar >> b) & 1u);
+    if (ok) {
+        head();
+        __syncthreads();
+        store_head(S.info[(n_mine - 1) & 3]);
+    }
+    // drain the load still in flight (bounded) before the CTA leaves
+    if (tid == 0) bar_wait(&S.inbar, (uint32_t)(loads - 1) & 1u);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
