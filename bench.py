@@ -861,7 +861,7 @@ def run_gpu(args):
                   "peak_basis": f"{sm_count} SMs x 128 lanes x {sm_mhz} MHz, one op per lane slot "
                                 f"({OPS_PER_CELL_PIXEL} algorithmic ops per cell-grid pixel; max SM clock, "
                                 f"{peak_kind})",
-                  # ncu, same source: fraction of cycles the schedulers issued (the kernel runs ~1.9
+                  # ncu, same source: fraction of cycles the schedulers issued (the kernel runs ~1.4
                   # instructions per algorithmic op: addressing, shared-memory traffic, control)
                   "issue_active_frac": None if args.hog_per_block else recorded_traffic(
                       "k_cells_warp_1242x375_b32.txt", "k_cells_warp.cu", "issue_active_frac")}
