@@ -25,11 +25,12 @@
 //    subtraction and one 3-input logic operation compare 4 pixels with one
 //    neighbour. The 8 comparisons of a lane's 32 pixels of a cell (4 columns x
 //    8 rows) are 8 bit planes, shifted in row by row, and a uniform code is
-//    one run of ones: the pixels of a code are three planes ANDed and their
-//    number a population count (Algorithm 2 without a histogram in memory).
+//    one run of ones around the circle: the pixels of a code are three planes
+//    ANDed and their number a population count (Algorithm 2 without a histogram
+//    in memory).
 //    Counting in shared memory instead (a code -> counter table and an atomic
 //    per pixel) took a third of the kernel's shared-memory wavefronts and kept
-//    that pipe 79% busy (now 58%): 0.961 -> 0.887 ms per 64 x 1242x375 frames.
+//    that pipe 79% busy (now 57%): 0.961 -> 0.887 ms per 64 x 1242x375 frames.
 //  * HOG (Algorithm 4). One byte permute and two dp2a (weights +1, -1) give
 //    the central differences of two pixels; the accumulator 0x4B400000 makes
 //    the 32-bit result the float 1.5 * 2^23 + g, so one multiply-add turns it
@@ -59,8 +60,11 @@
 //    that a warp's data-dependent scatter hits 32 distinct banks and the
 //    epilogue reads them with one 16-byte load.
 // Rows outside the cell grid are whole halves of the level's first and last
-// bands and are not walked (0.810 -> 0.785 ms). What bounds the kernel now:
-// issue (74% of cycles, about 79 instructions per pixel) with 16 warps per SM
+// bands and are not walked (0.810 -> 0.785 ms). Each lane of a cell counts its
+// own 32 pixels of all bins and swaps half of them with the other (both lanes'
+// pixels for half of the bins took 80 instructions more per cell row: 0.785 ->
+// 0.766 ms). What bounds the kernel now:
+// issue (73% of cycles, about 77 instructions per pixel) with 16 warps per SM
 // at 128 registers; 20 warps at 96 registers measured slower (0.875 against
 // 0.828 ms), all of a row's slot loads before its stores no faster.
 // HOG epilogue of cell row r: each lane forms, per bin, the weighted sums of
@@ -90,7 +94,7 @@
 // cleared), after B (with A: a = 1) and after C (a = 0); of a cell's 16 columns
 // b drops the first or the last 4, one b per lane of the cell. Against a CTA
 // of 128 threads per 15 x 8-cell tile, one column per thread, which voted
-// three times per pixel and counted LBP by shared-memory atomics: 583 -> 271 us
+// three times per pixel and counted LBP by shared-memory atomics: 583 -> 266 us
 // per 16 x 1242x375 frames (the shared grid: about 200). What bounds it: the
 // shared-memory pipe, where the column sums and the second clear add about
 // 170 wavefronts per cell row to the walk's 370.
@@ -217,38 +221,34 @@ __device__ __forceinline__ uint32_t ge4(uint32_t n, uint32_t c_lo, uint32_t cn) 
     return (n & cn) | (t & (n | cn));  // majority of n, not c, t
 }
 
-// Uniform codes below 128 in ascending order are runs of ones [s, s + len) with
-// s + len <= 7; run k (1 .. 28; 0 is the empty code) as constants.
-__host__ __device__ constexpr int run_start(int k) {
-    int i = 0;
-    for (int c = 1; c < 128; ++c) {
-        int s = 0;
-        while (!((c >> s) & 1)) ++s;
-        int e = s;
-        while ((c >> e) & 1) ++e;
-        if (c >> e) continue;
-        if (++i == k) return s;
+// Uniform codes in ascending order (at most two changes around the circle): code of
+// bin b, 0 .. 57. All but 0 and 255 are one run of ones, from run_start over
+// run_length positions around the circle.
+__host__ __device__ constexpr int uniform_code(int b) {
+    int i = -1;
+    for (int c = 0; c < 256; ++c) {
+        int changes = 0;
+        for (int k = 0; k < 8; ++k) changes += ((c >> k) & 1) != ((c >> ((k + 1) & 7)) & 1);
+        if (changes <= 2 && ++i == b) return c;
     }
     return -1;
 }
-__host__ __device__ constexpr int run_end(int k) {
-    int i = 0;
-    for (int c = 1; c < 128; ++c) {
-        int s = 0;
-        while (!((c >> s) & 1)) ++s;
-        int e = s;
-        while ((c >> e) & 1) ++e;
-        if (c >> e) continue;
-        if (++i == k) return e;
-    }
+__host__ __device__ constexpr int run_start(int c) {
+    for (int k = 0; k < 8; ++k)
+        if (((c >> k) & 1) && !((c >> ((k + 7) & 7)) & 1)) return k;
     return -1;
 }
-static_assert(run_end(28) == 7 && run_start(28) == 0 && run_start(29) == -1, "28 runs below bit 7");
+__host__ __device__ constexpr int run_length(int c) {
+    int n = 0;
+    for (int k = 0; k < 8; ++k) n += (c >> k) & 1;
+    return n;
+}
+static_assert(uniform_code(0) == 0 && uniform_code(57) == 255 && uniform_code(58) == -1, "58 uniform codes");
 
 // The comparison planes of 32 pixels (bit k of their codes in x[k]) -> pixels
-// whose code is one run starting at s (run[s], s < 7), is 0 (none), or has two
-// or more runs (many: not uniform).
-__device__ __forceinline__ void lbp_runs(const uint32_t (&x)[8], uint32_t (&run)[7], uint32_t &none, uint32_t &many) {
+// whose code is one run starting at s (run[s]) or has two or more runs (many: not
+// uniform). Codes 0 and 255 have none.
+__device__ __forceinline__ void lbp_runs(const uint32_t (&x)[8], uint32_t (&run)[8], uint32_t &many) {
     uint32_t r[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) r[k] = x[k] & ~x[(k + 7) & 7];  // a run starts at k
@@ -257,10 +257,8 @@ __device__ __forceinline__ void lbp_runs(const uint32_t (&x)[8], uint32_t (&run)
     const uint32_t s3 = r[6] ^ r[7], c3 = r[6] & r[7];
     const uint32_t c4 = (s1 & s2) | (s3 & (s1 | s2));
     many = (c1 | c2 | c3) | c4;
-    const uint32_t one = (s1 ^ s2 ^ s3) & ~many;
 #pragma unroll
-    for (int k = 0; k < 7; ++k) run[k] = r[k] & one;
-    none = ~((x[0] | x[1] | x[2]) | (x[3] | x[4] | x[5]) | (x[6] | x[7]));
+    for (int k = 0; k < 8; ++k) run[k] = r[k] & ~many;
 }
 
 template <int FEAT, bool CELLS>  // CELLS: cell-major LBP counts
@@ -434,46 +432,36 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
 
         // ---- LBP of cell row r = band - 1 is final after the band's first 4 rows: the planes
         // hold its 8 rows (older bits are shifted out). A cell is the two lanes 2c + 1 and
-        // 2c + 2, 32 pixels each. The first counts the 29 uniform codes below 128 over both
-        // lanes' planes, the second those above over the complements: the code ranked 57 - k
-        // is the complement of the code ranked k, so both run the same instructions.
+        // 2c + 2, 32 pixels each: each counts its own (59 bins, a byte each), they swap
+        // halves of the bins and the first writes bins 0 .. 31, the second the others.
         auto emit_lbp = [&](int band) {
             const int r = band - 1;
             if (!need(r)) return;
-            const uint32_t half = (lane & 1) ^ 1u, flip = 0u - half;
-            uint32_t x[8], ra_[7], rb_[7], none_a, none_b, many_a, many_b, y[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                x[k] = plane[k] ^ flip;
-                y[k] = __shfl_sync(0xffffffffu, plane[k], ((lane - 1) ^ 1) + 1) ^ flip;
-            }
-            lbp_runs(x, ra_, none_a, many_a);
-            lbp_runs(y, rb_, none_b, many_b);
-            uint32_t q[8];  // counts of the ranks, 4 per word
-            static_for([&](auto K) {
-                constexpr int k = decltype(K)::value;
-                uint32_t n;
-                if constexpr (k == 0) {
-                    n = __popc(none_a) + __popc(none_b);
-                } else {
-                    constexpr int s = run_start(k), e = run_end(k);
-                    n = __popc(ra_[s] & x[e - 1] & ~x[e]) + __popc(rb_[s] & y[e - 1] & ~y[e]);
+            const uint32_t half = (lane & 1) ^ 1u;
+            uint32_t run[8], many;
+            lbp_runs(plane, run, many);
+            uint32_t q[16];  // counts, 4 bins per word
+            static_for([&](auto B) {
+                constexpr int bin = decltype(B)::value;
+                uint32_t n = 0u;
+                if constexpr (bin == 0) {
+                    n = __popc(~((plane[0] | plane[1] | plane[2]) | (plane[3] | plane[4] | plane[5]) | (plane[6] | plane[7])));
+                } else if constexpr (bin == 57) {
+                    n = __popc((plane[0] & plane[1] & plane[2]) & (plane[3] & plane[4] & plane[5]) & (plane[6] & plane[7]));
+                } else if constexpr (bin == 58) {
+                    n = __popc(many);
+                } else if constexpr (bin < 58) {
+                    constexpr int s = run_start(uniform_code(bin)), e = s + run_length(uniform_code(bin));
+                    n = __popc(run[s] & plane[(e - 1) & 7] & ~plane[e & 7]);
                 }
-                if constexpr (k % 4 == 0) q[k / 4] = n;
-                else q[k / 4] += n << (8 * (k % 4));
-            }, std::make_integer_sequence<int, 29>{});
-            const uint32_t other = __popc(many_a) + __popc(many_b);
-            // bins 29, 30, 31 are the upper lane's ranks 28, 27, 26
-            const uint32_t top = __shfl_down_sync(0xffffffffu, __byte_perm(q[7], q[6], 0x0670) & 0xffffffu, 1);
+                if constexpr (bin % 4 == 0) q[bin / 4] = n;
+                else if constexpr (bin <= 58) q[bin / 4] += n << (8 * (bin % 4));
+            }, std::make_integer_sequence<int, 64>{});
             uint32_t v[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                // first lane: bins 4i ..; second: bins 32 + 4i .. = ranks 25 - 4i downwards
-                const uint32_t lo = i < 7 ? q[i] : q[7] | (top << 8);
-                const uint32_t hi = i < 6    ? __byte_perm(q[5 - (i < 6 ? i : 0)], q[6 - (i < 6 ? i : 0)], 0x2345)
-                                    : i == 6 ? __byte_perm(q[0], other, 0x7401)
-                                             : 0u;
-                v[i] = half ? hi : lo;
+                const uint32_t give = half ? q[i] : q[8 + i], keep = half ? q[8 + i] : q[i];
+                v[i] = keep + __shfl_sync(0xffffffffu, give, ((lane - 1) ^ 1) + 1);
             }
             const int c = (lane - 1) >> 1;
             if (lane < 1 || lane > 2 * kCellTW || cx0 + c >= Wc) return;
