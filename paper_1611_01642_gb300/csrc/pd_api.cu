@@ -533,9 +533,11 @@ void plan_strips(Plan &p, int resident_warps) {
     auto cost = [&](int rows) { return 4 * schedule(rows) + rows; };
     // Sparse path: one cell tile per strip. A tall strip whose tiles are partly
     // skipped leaves its warp with less than planned (8 x 1920x1080: cells
-    // 297 -> 283 us).
+    // 297 -> 283 us; two tiles 288 against 271 later). Two tiles, for less halo,
+    // from 12 tiles per warp on (16 frames, 17 tiles per warp: 499 -> 489; 8
+    // frames have 8).
     const bool sparse = !p.cnn_items.empty();
-    int rows = sparse ? kCellTH : kMaxRows;
+    int rows = !sparse ? kMaxRows : p.c_tiles >= 12 * R ? 2 * kCellTH : kCellTH;
     int64_t n32[kMaxRows + 1];
     if (!sparse && histogram(rows, n32) < 16 * R) {
         int64_t best = cost(rows);
