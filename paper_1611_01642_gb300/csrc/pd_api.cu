@@ -11,7 +11,9 @@
 // Every level owns a band of atlas rows, so one pair of tensor maps (encoded
 // once) covers all levels of all frames. The plan also carries the work
 // lists of the four kernels and the Q11 resample tables; it is packed into a
-// pinned host buffer and sent with one asynchronous copy per pd_detect.
+// pinned host buffer and sent with one asynchronous copy per batch shape (and
+// per stage call). The frame pointers go with every pd_detect, from a pinned
+// buffer of their own.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -270,7 +272,8 @@ struct pd_handle {
     int64_t frames_cap = 0;
     int64_t level_cap = 0, r_cap = 0, c_cap = 0, s_cap = 0, tab_cap = 0;
     // pinned host
-    unsigned char *h_desc = nullptr;
+    unsigned char *h_desc = nullptr;   // a plan on its way to d_desc (free once desc_done has passed)
+    FrameDesc *h_step_frames = nullptr;  // after it: the frame section that a step sends (free once graph_done has passed)
     pd_box *h_boxes = nullptr;     // mapped: written by the NMS kernel
     int32_t *h_counts = nullptr;   // mapped: [2 * max_frames] kept / candidates
     pd_box *m_boxes = nullptr;     // device views of the two mapped buffers
@@ -1137,7 +1140,9 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     h->proposal = params->use_proposal != 0;
     h->tau = params->keep_logit_threshold;
 
-    if (cudaMallocHost(&h->h_desc, h->desc_cap) != cudaSuccess) return bail(PD_ENOMEM);
+    if (cudaMallocHost(&h->h_desc, h->desc_cap + (size_t)params->max_frames * sizeof(FrameDesc)) != cudaSuccess)
+        return bail(PD_ENOMEM);
+    h->h_step_frames = reinterpret_cast<FrameDesc *>(h->h_desc + h->desc_cap);
     // Results land in mapped pinned host memory: NMS writes the kept boxes and
     // counts there directly, so pd_sync needs no device-to-host copies.
     if (cudaHostAlloc(&h->h_boxes, (size_t)params->max_frames * params->max_boxes_per_frame * sizeof(pd_box),
@@ -1249,12 +1254,13 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         h->sig = sig;
         h->cache_valid = true;
     }
-    // frame pointers change from call to call: rewrite only that section
+    // Frame pointers change from call to call: every step sends that section again, from
+    // a buffer of its own, which the last step's copy must have left (a plan for another
+    // batch shape or a stage call's is written while that copy may still be queued).
     PD_CUDA(h, cudaEventSynchronize(h->graph_done));
-    PD_CUDA(h, cudaEventSynchronize(h->desc_done));
     for (int f = 0; f < n_frames; ++f) p.frames[f].ptr = d_frames[f];
     const Packed &o = h->packed;
-    if (n_frames) std::memcpy(h->h_desc + o.frames, p.frames.data(), p.frames.size() * sizeof(FrameDesc));
+    if (n_frames) std::memcpy(h->h_step_frames, p.frames.data(), p.frames.size() * sizeof(FrameDesc));
     const FrameDesc *df = dptr<FrameDesc>(h, o.frames);
     const LevelDesc *dl = dptr<LevelDesc>(h, o.levels);
     const bool timed = (h->p.flags & PD_FLAG_STAGE_TIMING) != 0;
@@ -1267,7 +1273,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
     const int cluster = nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame, max_windows(p));
     auto enqueue = [&](cudaStream_t q) -> int {
         if (n_frames)
-            PD_CUDA(h, cudaMemcpyAsync(h->d_desc + o.frames, h->h_desc + o.frames,
+            PD_CUDA(h, cudaMemcpyAsync(h->d_desc + o.frames, h->h_step_frames,
                                        p.frames.size() * sizeof(FrameDesc), cudaMemcpyHostToDevice, q));
         // the error word and the item counters start a step as 0: K1 clears them
         // (as memsets they were 3 of a step's 8 graph nodes)
@@ -1337,7 +1343,10 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
         PD_CUDA(h, cudaGraphLaunch(h->graph, s));
     } else {
         int r = enqueue(s);
-        if (r != PD_OK) return r;
+        if (r != PD_OK) {
+            cudaEventRecord(h->graph_done, s);  // what was enqueued still reads h_step_frames
+            return r;
+        }
     }
     PD_CUDA(h, cudaEventRecord(h->graph_done, s));
     h->err_stage = false;
