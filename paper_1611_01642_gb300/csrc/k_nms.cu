@@ -38,7 +38,8 @@
 // and 76 had a batch's edges 32 bytes apart: 16 lanes on one bank group, and the
 // pairwise bits took 3,700 cycles per batch where they take about 1,200.
 // The IoU test first evaluates inter - thr * union in float. A coordinate sum or
-// difference is off by at most 3 float roundings of values up to m = max(W, H)
+// difference is off by at most 3 float roundings of values up to m, the frame's
+// size or, for maps that reach beyond it, their farthest edge
 // (eps = 3 m 2^-24), which moves the intersection by at most (w + h) eps and the
 // IoU by at most eps (1 / w + 1 / h) through the intersection and as much again
 // through the union (1.7e-5 for 64x128 windows of a 2048-pixel frame). So a float
@@ -68,7 +69,7 @@ constexpr int kDigit = 11;                // radix select: bits per round
 constexpr int kHist = 1 << kDigit;
 constexpr int kMaxBoxes = 16384;
 constexpr int kBatch = 64;                // greedy walk: candidates resolved per block-wide step
-constexpr int kGrid = 32;                 // culling grid: kGrid x kGrid cells over the frame
+constexpr int kGrid = 32;                 // culling grid: kGrid x kGrid cells over the boxes' extent
 constexpr int kCountBlocks = 32;          // blocks per frame counting its candidates
 static_assert(nms_sched_ints(1) == 2 + kCountBlocks,
               "scheduling scratch: the ticket, then per frame its order slot and counts");
@@ -543,7 +544,7 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
             S.cols[k] = L.cols;
         }
         __syncthreads();
-        // the float test's band (see above): from the frame's size and its smallest window
+        // the float test's band (see above): from the boxes' extent and the smallest window
         int wk = 1, hk = 1;
         for (int k = lane; k < nl; k += 32) {
             wk = max(wk, S.wkhk[k].x);
@@ -551,7 +552,7 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
         }
         wk = __reduce_max_sync(0xffffffffu, wk);
         hk = __reduce_max_sync(0xffffffffu, hk);
-        const float band = 4.f * (3.f * 5.9604645e-8f * (float)max(W, H)) *
+        const float band = 4.f * (3.f * 5.9604645e-8f * fmaxf(fd.ex, fd.ey)) *
                                ((float)wk / (64.f * (float)W) + (float)hk / (128.f * (float)H)) + 1e-6f;
         unsigned long long *list = big ? reinterpret_cast<unsigned long long *>(scratch + (size_t)f * nms_scratch_float4s(cap))
                                        : reinterpret_cast<unsigned long long *>(nms_raw + sizeof(NmsSmem));
@@ -885,7 +886,7 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
             if (Lead.done) break;
             // ---- 4. drop the segment's keys and what its kept boxes suppress, 64 of them at a time
             const int nk = Lead.n_kept_seg;
-            const float gsx = (float)kGrid / (float)W, gsy = (float)kGrid / (float)H;
+            const float gsx = (float)kGrid / fd.ex, gsy = (float)kGrid / fd.ey;
             // one run of keys per thread: test each against all kept boxes of the chunk; more:
             // only against those that cover its centre's cell
             const bool grid = cull && n_list > kThreads;
@@ -905,7 +906,7 @@ __global__ void __launch_bounds__(kThreads) k_nms(const FrameDesc *__restrict__ 
                     // in B (were it outside B on one axis, A and B would overlap on at most
                     // half of A's extent there, so inter <= |A| / 2, and inter > (|A| + |B|)
                     // / 3 would need |B| < |A| / 2 while inter <= |B| needs |B| > |A| / 2).
-                    // For every cell of a 32 x 32 grid over the frame: which of the kept boxes
+                    // For every cell of a 32 x 32 grid over the boxes' extent: which of the kept boxes
                     // cover it (one cell of margin for rounding).
                     const int cx = tid & (kGrid - 1), cy = tid / kGrid;
                     unsigned long long m = 0ull;
@@ -1178,6 +1179,7 @@ struct NoAllocScratch {
 
 struct NoAllocGeometry {
     int32_t W, H, n_levels, pad;
+    float ex, ey;
     int32_t Wk[kNoAllocMaxLevels], Hk[kNoAllocMaxLevels];
     int32_t rows[kNoAllocMaxLevels], cols[kNoAllocMaxLevels];
     int64_t score_off[kNoAllocMaxLevels];
@@ -1196,6 +1198,8 @@ __global__ void k_nms_noalloc_setup(const __grid_constant__ NoAllocGeometry g, N
         f.H = g.H;
         f.first_level = 0;
         f.n_levels = g.n_levels;
+        f.ex = g.ex;
+        f.ey = g.ey;
         s->frame = f;
     }
     for (int k = threadIdx.x; k < g.n_levels; k += blockDim.x) {
@@ -1228,6 +1232,8 @@ extern "C" int pd_nms_noalloc(void *stream, const float *d_scores, int n_levels,
     g.W = W;
     g.H = H;
     g.n_levels = n_levels;
+    g.ex = (float)W;
+    g.ey = (float)H;
     int64_t off = 0;
     for (int k = 0; k < n_levels; ++k) {
         if (rows[k] < 0 || cols[k] < 0 || rows[k] > 4096 || cols[k] > 4096 || Wk[k] < 1 || Hk[k] < 1)
@@ -1238,6 +1244,7 @@ extern "C" int pd_nms_noalloc(void *stream, const float *d_scores, int n_levels,
         g.cols[k] = cols[k];
         g.score_off[k] = off;
         off += (int64_t)rows[k] * cols[k];
+        add_extent(g.ex, g.ey, W, H, Wk[k], Hk[k], rows[k], cols[k]);
     }
     // Every call: the current device's address of the scratch array (the
     // host-side symbol is only a stand-in) and the kernel's shared-memory

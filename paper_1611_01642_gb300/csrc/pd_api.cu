@@ -708,6 +708,8 @@ int plan_frame(Plan &p, unsigned what, const pd_params &prm, const uint8_t *ptr,
     fd.W = W;
     fd.H = H;
     fd.pitch = pitch;
+    fd.ex = (float)W;
+    fd.ey = (float)H;
     fd.first_level = (int32_t)p.levels.size();
     fd.n_levels = n;
     const int f = (int)p.frames.size();
@@ -1831,6 +1833,8 @@ int pd_nms_maps(pd_handle *h, void *stream, const float *d_scores, int n_levels,
     FrameDesc fd{};
     fd.W = W;
     fd.H = H;
+    fd.ex = (float)W;
+    fd.ey = (float)H;
     fd.first_level = 0;
     fd.n_levels = n_levels;
     int64_t off = 0;
@@ -1846,6 +1850,7 @@ int pd_nms_maps(pd_handle *h, void *stream, const float *d_scores, int n_levels,
         L.cols = cols[k];
         L.score_off = off;
         off += (int64_t)rows[k] * cols[k];
+        add_extent(fd.ex, fd.ey, W, H, Wk[k], Hk[k], rows[k], cols[k]);
         p.levels.push_back(L);
     }
     p.frames.push_back(fd);

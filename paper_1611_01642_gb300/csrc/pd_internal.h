@@ -5,6 +5,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "../../include/pd.h"
@@ -29,7 +30,14 @@ struct FrameDesc {
     int32_t W, H, pitch;
     int32_t first_level, n_levels;  // range in the LevelDesc table
     int32_t rbw;                    // K1: source bytes staged per tile row (max of the levels' rspan)
+    float ex, ey;                   // NMS: right and lower end of all boxes, at least W and H
 };
+// Extends ex, ey by the last window of a rows x cols map (a caller's map may reach beyond the frame).
+inline void add_extent(float &ex, float &ey, int W, int H, int Wk, int Hk, int rows, int cols) {
+    if (rows <= 0 || cols <= 0) return;
+    ex = fmaxf(ex, (float)((8.0 * cols + 56) * W / Wk));
+    ey = fmaxf(ey, (float)((8.0 * rows + 120) * H / Hk));
+}
 
 // One (frame, level).
 struct LevelDesc {
