@@ -763,24 +763,28 @@ __global__ void __launch_bounds__(kThreads, 1)
 #undef PD_WAIT_X16
 
 // LBP count planes [59][rows][pitch] -> 64 bytes per cell, [rows][width][64]
-// (bins 59..63 zero): one thread per 16 bins of a cell. For callers' planes;
+// (bins 59..63 zero): one thread per 16 bins of a cell, a block per row (or
+// every kRowBlocks-th: a grid has no more). For callers' planes;
 // the detector's own cells are written that way.
+constexpr int kRowBlocks = 65535;
 __global__ void __launch_bounds__(128) k_lbp_cells(const uint8_t *__restrict__ planes, int64_t plane, int pitch,
-                                                   int width, uint8_t *__restrict__ out) {
-    const int x = blockIdx.x * 32 + (threadIdx.x & 31), k = threadIdx.x >> 5, y = blockIdx.y;
+                                                   int width, int rows, uint8_t *__restrict__ out) {
+    const int x = blockIdx.x * 32 + (threadIdx.x & 31), k = threadIdx.x >> 5;
     if (x >= width) return;
-    const uint8_t *src = planes + (int64_t)y * pitch + x;
-    uint32_t w[4];
+    for (int y = blockIdx.y; y < rows; y += gridDim.y) {
+        const uint8_t *src = planes + (int64_t)y * pitch + x;
+        uint32_t w[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        w[u] = 0u;
+        for (int u = 0; u < 4; ++u) {
+            w[u] = 0u;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int t = 16 * k + 4 * u + b;
-            if (t < kLbpBins) w[u] |= (uint32_t)__ldg(src + t * plane) << (8 * b);
+            for (int b = 0; b < 4; ++b) {
+                const int t = 16 * k + 4 * u + b;
+                if (t < kLbpBins) w[u] |= (uint32_t)__ldg(src + t * plane) << (8 * b);
+            }
         }
+        reinterpret_cast<uint4 *>(out)[((int64_t)y * width + x) * 4 + k] = make_uint4(w[0], w[1], w[2], w[3]);
     }
-    reinterpret_cast<uint4 *>(out)[((int64_t)y * width + x) * 4 + k] = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 }  // namespace
@@ -827,7 +831,8 @@ int encode_tc_maps(CUtensorMap *hog_map, CUtensorMap *lbp_map, const float *hog,
 cudaError_t launch_lbp_cells(cudaStream_t s, const uint8_t *planes, int64_t plane, int pitch, int width, int rows,
                              uint8_t *out) {
     if (width <= 0 || rows <= 0) return cudaSuccess;
-    k_lbp_cells<<<dim3((width + 31) / 32, rows), 128, 0, s>>>(planes, plane, pitch, width, out);
+    k_lbp_cells<<<dim3((width + 31) / 32, rows < kRowBlocks ? rows : kRowBlocks), 128, 0, s>>>(planes, plane, pitch,
+                                                                                              width, rows, out);
     return cudaGetLastError();
 }
 
