@@ -294,7 +294,11 @@ int pd_cell_features(pd_handle *h, void *stream, const uint8_t *d_level, int Wk,
  * d_scores float32 [cells_y-15][cells_x-7], row pitch cells_x-7. The
  * cell planes are read through TMA: d_hog and d_lbp must be 16-byte aligned,
  * cell_pitch a multiple of 16, hog_plane a multiple of 4 and lbp_plane a
- * multiple of 16 elements. Errors: PD_EINVAL, PD_ECUDA. */
+ * multiple of 16 elements. For the tensor cores the counts are first laid out
+ * cell by cell in the handle's own LBP cells (the next pd_detect writes them
+ * anew); a level of more cells than those takes 64 bytes per cell of scratch,
+ * allocated by the first such call (it synchronises the stream) and freed by
+ * pd_destroy. Errors: PD_EINVAL, PD_ENOMEM, PD_ECUDA. */
 int pd_window_scores(pd_handle *h, void *stream, const float *d_hog, int64_t hog_plane,
                      const uint8_t *d_lbp, int64_t lbp_plane, int cell_pitch, int cells_x,
                      int cells_y, float *d_scores);

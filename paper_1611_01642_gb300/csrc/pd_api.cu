@@ -1805,20 +1805,43 @@ int pd_window_scores(pd_handle *h, void *stream, const float *d_hog, int64_t hog
             return fail(h, PD_ECUDA, "pd_window_scores: tensor map encoding failed");
     }
     Packed o;
-    int r = upload_plan(h, s, p, o);
-    if (r != PD_OK) return r;
-    PD_CUDA(h, cudaMemsetAsync(h->d_err, 0, 2 * sizeof(int), s));  // and K4's item counter
-    h->err_stage = true;
     if (fp32) {
+        const int r = upload_plan(h, s, p, o);
+        if (r != PD_OK) return r;
+        PD_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(unsigned), s));
+        h->err_stage = true;
         PD_CUDA(h, launch_svm(s, hm, lm, dptr<LevelDesc>(h, o.levels), h->d_w, h->bias, h->p.l2hys_clip,
                               d_scores, dptr<SvmItem>(h, o.s_items), (int)p.s_items.size(), h->d_err));
-    } else {
-        PD_CUDA(h, launch_lbp_cells(s, d_lbp, lbp_plane, cell_pitch, cells_x, cells_y, cells));
+        return PD_OK;
+    }
+    // As many items per launch as the descriptor block holds: all of them, unless the level
+    // is far larger than the handle's own (a handle of 64x128 frames takes 16,000, 27 M windows).
+    const int64_t n = (int64_t)p.t_items.size(), item = (int64_t)sizeof(TcItem);
+    const int64_t fit = (h->desc_cap - (pack_layout(p).total - n * item)) / item - 4;  // (- 4: section alignment)
+    std::vector<TcItem> rest;
+    if (n > fit) {
+        if (fit < 1) return fail(h, PD_EINVAL, "plan descriptors exceed the arena");
+        rest.assign(p.t_items.begin() + fit, p.t_items.end());
+        p.t_items.resize((size_t)fit);
+    }
+    for (size_t at = 0;;) {
+        const int r = upload_plan(h, s, p, o);
+        if (r != PD_OK) return r;
+        if (at == 0) {
+            PD_CUDA(h, cudaMemsetAsync(h->d_err, 0, 2 * sizeof(int), s));  // and K4's item counter
+            h->err_stage = true;
+            PD_CUDA(h, launch_lbp_cells(s, d_lbp, lbp_plane, cell_pitch, cells_x, cells_y, cells));
+        } else {
+            PD_CUDA(h, cudaMemsetAsync(h->d_queue, 0, sizeof(int), s));
+        }
         PD_CUDA(h, launch_svm_tc(s, th, tl, dptr<LevelDesc>(h, o.levels), dptr<TcItem>(h, o.t_items),
                                  (int)p.t_items.size(), h->d_queue, h->sm_count, h->d_tc_consts, h->bias,
                                  h->p.l2hys_clip, d_scores, nullptr, h->d_err, hog_planes_of(h->p.flags)));
+        if (at == rest.size()) return PD_OK;
+        const size_t k = std::min(rest.size() - at, (size_t)fit);
+        p.t_items.assign(rest.begin() + at, rest.begin() + at + k);
+        at += k;
     }
-    return PD_OK;
 }
 
 int pd_nms_maps(pd_handle *h, void *stream, const float *d_scores, int n_levels, const int32_t *rows,

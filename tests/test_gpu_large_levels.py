@@ -48,3 +48,8 @@ def _check(cx, cy, parts):
 
 def test_taller_than_a_grid():
     _check(20, 65600, [(0, 0, 20, 90), (0, 65480, 20, 120), (0, 65520, 20, 80)])
+
+
+def test_more_items_than_the_descriptor_block_holds():
+    # 204 strips of 26 columns x 84 pieces of 64 rows: 17,136 work items at least
+    _check(5300, 5390, [(0, 0, 90, 80), (2608, 2650, 100, 100), (5216, 5280, 84, 110), (16, 5290, 60, 100)])
