@@ -75,6 +75,7 @@ struct Plan {
     int32_t max_wc = 0;
     bool tall = false;    // K1 tiles of 2 kResizeTH source rows
     int32_t c_tiles = 0;  // cell tiles of all levels (sparse path: one flag each)
+    int64_t frame_windows = 0;  // windows of the frame that has the most
     // frames of equal size share their Q11 tables: (W, H) -> first level index
     std::map<std::pair<int, int>, int> tab_owner;
 
@@ -91,6 +92,7 @@ struct Plan {
         tc_widths.clear();
         pyr_bytes = score_floats = 0;
         atlas_rows = max_wc = c_tiles = 0;
+        frame_windows = 0;
         tall = false;
     }
 };
@@ -712,6 +714,7 @@ int plan_frame(Plan &p, unsigned what, const pd_params &prm, const uint8_t *ptr,
     fd.ey = (float)H;
     fd.first_level = (int32_t)p.levels.size();
     fd.n_levels = n;
+    const int64_t first_score = p.score_floats;
     const int f = (int)p.frames.size();
     auto owner = p.tab_owner.find({W, H});
     const int first_shared = owner == p.tab_owner.end() ? -1 : owner->second;
@@ -734,6 +737,7 @@ int plan_frame(Plan &p, unsigned what, const pd_params &prm, const uint8_t *ptr,
                     for (int cx = 0; cx < L.Wc; cx += kCnnTile) p.cnn_items.push_back({li, cy, cx, 0});
         }
     }
+    p.frame_windows = std::max(p.frame_windows, p.score_floats - first_score);
     fd.rbw = staged_bytes(p, fd);
     if (n > 0)
         for (int y = 0; y < H; y += kResizeTH)
@@ -873,16 +877,6 @@ void invalidate_cache(pd_handle *h) {
 int max_pool_tiles(const Plan &p) {
     int m = 0;
     for (const LevelDesc &L : p.levels) m = std::max(m, pool_tiles_of(L.rows, L.cols));
-    return m;
-}
-
-int64_t max_windows(const Plan &p) {
-    int64_t m = 0;
-    for (const FrameDesc &f : p.frames) {
-        int64_t n = 0;
-        for (int k = 0; k < f.n_levels; ++k) n += (int64_t)p.levels[f.first_level + k].rows * p.levels[f.first_level + k].cols;
-        m = std::max(m, n);
-    }
     return m;
 }
 
@@ -1272,7 +1266,7 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
     auto record = [&](cudaEvent_t e, cudaStream_t q) {
         return capturing ? cudaEventRecordWithFlags(e, q, cudaEventRecordExternal) : cudaEventRecord(e, q);
     };
-    const int cluster = nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame, max_windows(p));
+    const int cluster = nms_cluster_for(n_frames, h->sm_count, h->p.max_candidates_per_frame, p.frame_windows);
     auto enqueue = [&](cudaStream_t q) -> int {
         if (n_frames)
             PD_CUDA(h, cudaMemcpyAsync(h->d_desc + o.frames, h->h_step_frames,
@@ -1884,7 +1878,7 @@ int pd_nms_maps(pd_handle *h, void *stream, const float *d_scores, int n_levels,
     PD_CUDA(h, launch_nms(s, dptr<FrameDesc>(h, o.frames), dptr<LevelDesc>(h, o.levels), 1, d_scores,
                           h->p.threshold, h->p.nms_iou, h->d_nms_scratch, h->p.max_candidates_per_frame,
                           d_boxes, max_boxes, d_counts,
-                          nms_cluster_for(1, h->sm_count, h->p.max_candidates_per_frame, max_windows(p))));
+                          nms_cluster_for(1, h->sm_count, h->p.max_candidates_per_frame, off)));
     return PD_OK;
 }
 

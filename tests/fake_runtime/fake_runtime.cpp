@@ -123,7 +123,10 @@ int encode_tc_maps(CUtensorMap *, CUtensorMap *, const float *, int64_t, int64_t
                    int64_t) {
     return PD_OK;
 }
-int nms_cluster_for(int, int, int, int64_t) { return 1; }
+int nms_cluster_for(int, int, int, int64_t windows) {
+    std::fprintf(stderr, "windows %ld\n", (long)windows);
+    return 1;
+}
 int nms_launches(int, int) { return 1; }
 size_t train_partial_floats() { return 0; }
 size_t scheme_cells_scratch(int, int) { return 0; }

@@ -36,3 +36,16 @@ def test_kernels_read_the_descriptors_of_their_own_call(program, calls):
     alone = {c: _log(program, c) for c in set(calls)}
     assert all(alone.values())
     assert _log(program, calls) == [line for c in calls for line in alone[c]]
+
+
+def test_the_plan_holds_the_largest_frames_windows(program):
+    """The NMS launch form follows from it; it comes with the plan, not from a walk over the levels per call."""
+    pd = pytest.importorskip("paper_1611_01642_gb300")
+
+    def windows(w, h):
+        return sum(max(b // 8 - 15, 0) * max(a // 8 - 7, 0) for a, b in pd.pd_pyramid(w, h, 1.05))
+
+    want = {"A": windows(320, 240), "B": max(windows(200, 180), windows(160, 150))}
+    calls = "ABBAA"
+    r = subprocess.run([program, *calls], capture_output=True, text=True, timeout=60)
+    assert r.stderr.split() == [x for c in calls for x in ("windows", str(want[c]))]
