@@ -287,13 +287,12 @@ struct pd_handle {
     cudaEvent_t stage_ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     bool timed = false;
     // learned proposal: parameters (fp32 master + Adam state + rounded copy),
-    // inference fragments, per-cell head values, window logits
+    // input table, per-cell head values, window logits
     float *cnn = nullptr;           // [5][kCnnParams]: master, m, v, grad, rounded
     float *in_tab = nullptr;        // [256]
-    uint32_t *w2frag = nullptr;     // [2304]
     float *hmap = nullptr;          // one f32 plane over the cell atlas
     float *logits = nullptr;        // window logits, score-map layout
-    bool cnn_loaded = false, frag_stale = false;
+    bool cnn_loaded = false, training = false;  // training: parameter updates not waited for yet
     bool proposal = false;          // sparse path on
     bool ran_proposal = false;      // the last pd_detect ran the sparse path
     float tau = 0.f;                // keep-logit threshold
@@ -847,24 +846,6 @@ float bf16_round_host(double a) {
     return (float)std::ldexp(std::nearbyint(m * 256.0) / 256.0, e);
 }
 
-uint32_t bf16_bits(float f) {  // f is already a bf16 value: its top 16 bits
-    uint32_t u;
-    std::memcpy(&u, &f, 4);
-    return u >> 16;
-}
-
-// mma.sync m16n8k16 B fragments (B = K x N): lane (g = lane/4, t = lane%4)
-// holds B[2t][g], B[2t+1][g] in register 0 and B[2t+8][g], B[2t+9][g] in
-// register 1 (first element in the low half).
-void pack_frag(const float *W, int cin, int ci0, int tap, int nt, uint32_t *out /* [32][2] */) {
-    for (int lane = 0; lane < 32; ++lane) {
-        const int g = lane >> 2, t = lane & 3, co = nt * 8 + g;
-        auto w = [&](int ci) { return bf16_bits(bf16_round_host(W[((size_t)co * cin + ci) * 9 + tap])); };
-        out[2 * lane] = w(ci0 + 2 * t) | (w(ci0 + 2 * t + 1) << 16);
-        out[2 * lane + 1] = w(ci0 + 2 * t + 8) | (w(ci0 + 2 * t + 9) << 16);
-    }
-}
-
 void invalidate_cache(pd_handle *h) {
     h->cache_valid = false;
     h->sig.clear();
@@ -903,7 +884,6 @@ CnnWeights cnn_weights(const pd_handle *h) {
     w.in_tab = h->in_tab;
     w.w1 = wr + kOffW1;
     w.b1 = wr + kOffB1;
-    w.w2frag = h->w2frag;
     w.w2 = wr + kOffW2;
     w.w3 = wr + kOffW3;
     w.b2 = wr + kOffB2;
@@ -915,20 +895,11 @@ CnnWeights cnn_weights(const pd_handle *h) {
     return w;
 }
 
-// Inference fragments from the master weights (after set_params or training).
-// Waits for the device first: training steps may still be writing the
-// master weights on a stream that the copy below does not order after.
-int refresh_fragments(pd_handle *h) {
+// Waits for training steps that may still be writing the parameters on a
+// stream that the caller's does not order after.
+int wait_training(pd_handle *h) {
     PD_CUDA(h, cudaDeviceSynchronize());
-    std::vector<float> p(kCnnParams);
-    PD_CUDA(h, cudaMemcpy(p.data(), h->cnn, kCnnParams * 4, cudaMemcpyDeviceToHost));
-    // layer 2's mma.sync B fragments (its edge positions); the tcgen05 operands
-    // are built by the kernel from the rounded weights
-    std::vector<uint32_t> f2(2304);
-    for (int tap = 0; tap < 9; ++tap)
-        for (int nt = 0; nt < 4; ++nt) pack_frag(p.data() + kOffW2, 16, 0, tap, nt, &f2[(tap * 4 + nt) * 64]);
-    PD_CUDA(h, cudaMemcpy(h->w2frag, f2.data(), f2.size() * 4, cudaMemcpyHostToDevice));
-    h->frag_stale = false;
+    h->training = false;
     return PD_OK;
 }
 
@@ -1096,7 +1067,7 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
         {h->frames_cap, 0},                                        // 9 host-input frames
         {(int64_t)params->max_frames * (int64_t)nms_scratch_float4s(params->max_candidates_per_frame) * 16,
          0},                                                                        // 10 NMS scratch
-        {(int64_t)5 * kCnnParams * 4 + 1024 + 2304 * 4, 0},                        // 11 CNN parameters
+        {(int64_t)5 * kCnnParams * 4 + 1024, 0},                                   // 11 CNN parameters, input table
         {(int64_t)rows * P * 4, 0},                                                 // 12 head values
         {h->score_cap * 4, 0},                                                      // 13 window logits
         {2 * h->flag_cap * 4, 0},                                                   // 14 tile flags
@@ -1127,7 +1098,6 @@ int pd_create(const pd_params *params, const float *svm_w, float svm_b, pd_handl
     h->d_nms_scratch = reinterpret_cast<float4 *>(h->arena + parts[10].off);
     h->cnn = reinterpret_cast<float *>(h->arena + parts[11].off);
     h->in_tab = h->cnn + 5 * kCnnParams;
-    h->w2frag = reinterpret_cast<uint32_t *>(h->in_tab + 256);
     h->hmap = reinterpret_cast<float *>(h->arena + parts[12].off);
     h->logits = reinterpret_cast<float *>(h->arena + parts[13].off);
     h->s_flag = reinterpret_cast<uint32_t *>(h->arena + parts[14].off);
@@ -1218,8 +1188,8 @@ int pd_detect(pd_handle *h, void *stream, int n_frames, const uint8_t *const *d_
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     h->stream = s;
     if (h->proposal && !h->cnn_loaded) return fail(h, PD_ESTATE, "proposal on but no parameters loaded");
-    if (h->proposal && h->frag_stale) {
-        int rr = refresh_fragments(h);
+    if (h->proposal && h->training) {
+        int rr = wait_training(h);
         if (rr != PD_OK) return rr;
     }
     Plan &p = h->plan;
@@ -1449,7 +1419,8 @@ int pd_cnn_set_params(pd_handle *h, const float *params, int n) {
     PD_CUDA(h, cudaDeviceSynchronize());
     h->adam_t = 0;
     h->cnn_loaded = true;
-    return refresh_fragments(h);
+    h->training = false;
+    return PD_OK;
 }
 
 int pd_cnn_get_params(pd_handle *h, float *params, float *grad, int n) {
@@ -1468,8 +1439,8 @@ int pd_cnn_forward(pd_handle *h, void *stream, const uint8_t *d_level, int Wk, i
     if (!d_level || !d_h || !d_logits || Wk < 1 || Hk < 1 || pitch < Wk || h_pitch < Wc)
         return fail(h, PD_EINVAL, "pd_cnn_forward: bad argument");
     if (!h->cnn_loaded) return fail(h, PD_ESTATE, "no proposal parameters (pd_cnn_set_params)");
-    if (h->frag_stale) {
-        int r = refresh_fragments(h);
+    if (h->training) {
+        int r = wait_training(h);
         if (r != PD_OK) return r;
     }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -1591,7 +1562,7 @@ int pd_cnn_train_step(pd_handle *h, void *stream, float pos_weight, float label_
         ++h->adam_t;
         a.c1 = 1.0f - (float)std::pow(0.9, h->adam_t);
         a.c2 = 1.0f - (float)std::pow(0.999, h->adam_t);
-        h->frag_stale = true;
+        h->training = true;
     }
     h->train_losses = (int)n_loss;
     h->train_loss_ptr = a.level_loss;
