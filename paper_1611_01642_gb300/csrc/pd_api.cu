@@ -537,11 +537,16 @@ void plan_strips(Plan &p, int resident_warps) {
     auto cost = [&](int rows) { return 4 * schedule(rows) + rows; };
     // Sparse path: one cell tile per strip. A tall strip whose tiles are partly
     // skipped leaves its warp with less than planned (8 x 1920x1080: cells
-    // 297 -> 283 us; two tiles 288 against 271 later). Two tiles, for less halo,
-    // from 12 tiles per warp on (16 frames, 17 tiles per warp: 499 -> 489; 8
-    // frames have 8).
+    // 272 us, 286 with two tiles). Two tiles, for less halo, from 20 tiles per
+    // warp on. Where two begin to pay follows from the share of tiles computed,
+    // which the plan does not know: at 13 to 16 tiles per warp with half of the
+    // windows scored (72 x 1242x375, 20: 643 against 619 us), at 15 to 18 with
+    // 0.3 of them (10 x 1920x1080, 13: 336 against 352; 16, 20: 497 against 487;
+    // 32, 41: 964 against 919), at 30 with 0.08 (4 x 3840x2160, 20: 232 against
+    // 245; 5, 25: 268 against 280; 8, 40: 409 against 401). At 20 no plan measured
+    // is more than 5% off the better of the two.
     const bool sparse = !p.cnn_items.empty();
-    int rows = !sparse ? kMaxRows : p.c_tiles >= 12 * R ? 2 * kCellTH : kCellTH;
+    int rows = !sparse ? kMaxRows : p.c_tiles >= 20 * R ? 2 * kCellTH : kCellTH;
     int64_t n32[kMaxRows + 1];
     if (!sparse && histogram(rows, n32) < 16 * R) {
         int64_t best = cost(rows);
