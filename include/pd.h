@@ -359,11 +359,12 @@ int pd_cnn_train_loss(pd_handle *h, void *stream, float *loss);
 
 /* Sparse path on (enable = 1) or off. When on, pd_detect also runs the
  * proposal network on every level after the pyramid. A window is kept when
- * its keep-logit exceeds keep_logit_threshold; the window tiles of the FP32
- * score kernel's plan that hold a kept window mark the cell tiles under them,
- * and only marked cell tiles are computed. The tensor-core score kernel then
- * scores every window whose cell tiles are all marked (a superset of the kept
- * windows: every window of a kept tile); the FP32 kernel scores the windows
+ * its keep-logit exceeds keep_logit_threshold. With the tensor-core score
+ * kernel every kept window marks the cell tiles (15 x 8 cells) under its own
+ * cells; with the FP32 one, every window tile of its plan that holds a kept
+ * window marks the cell tiles under the tile. Only marked cell tiles are
+ * computed. The tensor-core kernel then scores every window whose cell tiles
+ * are all marked (a superset of the kept windows), the FP32 kernel the windows
  * of kept tiles. Scored windows get exactly the plain path's score, the
  * others -inf. With the threshold at -inf every window is scored. Needs
  * parameters (pd_cnn_set_params) to enable. Affects the next pd_detect. */

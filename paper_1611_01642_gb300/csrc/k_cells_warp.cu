@@ -63,9 +63,9 @@
 // bands and are not walked (0.810 -> 0.785 ms). Each lane of a cell counts its
 // own 32 pixels of all bins and swaps half of them with the other (both lanes'
 // pixels for half of the bins took 80 instructions more per cell row: 0.785 ->
-// 0.766 ms). What bounds the kernel now:
-// issue (73% of cycles, about 77 instructions per pixel) with 16 warps per SM
-// at 128 registers; 20 warps at 96 registers measured slower (0.875 against
+// 0.766 ms). What bounds the kernel:
+// issue (72% of cycles, 75 thread instructions per pixel) with 16 warps per SM
+// at 125 registers; 20 warps at 96 registers measured slower (0.875 against
 // 0.828 ms), all of a row's slot loads before its stores no faster.
 // HOG epilogue of cell row r: each lane forms, per bin, the weighted sums of
 // its 4 columns for its own cell and for the neighbouring cell they reach;
@@ -172,7 +172,10 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // a time: the fitted coefficients scaled to 20-degree bins, doubled and negated
 // (exact: every step of the evaluation scales by -2). PREC: one degree more (15,
 // fitted to the least largest error), 3.3e-7 bin instead of 8.9e-7 in float32;
-// the histograms' error is 1.1e-7 of their norm with it and 2.9e-7 without.
+// the histograms' error is 1.1e-7 of their norm with it and 2.9e-7 without. The
+// scores' error, most of it from K4's split operands (5.2e-7 on exact histograms),
+// is 6.8e-7 of theirs (16 x 1242x375 frames); with the kernel before, whose
+// histograms were off by 2.8e-7 the other way, it was 6.1e-7.
 template <bool PREC>
 __device__ __forceinline__ f32x2 atan_bins2_poly(f32x2 s) {
     if constexpr (PREC) {
@@ -359,9 +362,9 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
         };
 
         // ---- one pixel row (rows a / b / c = y - 1, y, y + 1): HOG votes with
-        // weights wa, wb into the vote slots at float indices va[j] (cell row
-        // band - 1) and va[j] + dB (cell row band); LBP counts into the lane's counters
-        // (a row outside the cell grid votes with weight 0 and counts nothing)
+        // weights fa, fb into the vote slots at byte addresses va[j] (cell row
+        // band - 1; the rounded angle's bits are added) and va[j] + dB (cell row
+        // band); the LBP comparisons are shifted into the lane's bit planes
         auto pixel_row = [&](const Row &ra, const Row &rb, const Row &rc, float fa, float fb, const uint32_t (&va)[4],
                              uint32_t dB) {
             if (kHog) {
@@ -621,7 +624,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
         for (int band = 0; band <= nb; ++band) {
             const int yb = 8 * (cy0 + band) - 4;
             if (!(need(band - 1) || need(band))) {
-                if (walked_prev) {  // recycle row band - 1's slots and counters
+                if (walked_prev) {  // recycle row band - 1's slots
                     emit(band, false);
                 }
                 have = false;

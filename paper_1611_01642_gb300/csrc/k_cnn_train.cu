@@ -14,8 +14,10 @@
 // score-map offsets of the level.
 //
 // What bounds them: the convolutions are 3 x 468 multiply-adds per pyramid
-// pixel, and dz is fp32, so they run on the FP32 pipe, two multiply-adds per
-// instruction (fma.rn.f32x2 over pairs of channels or positions). Every kernel
+// pixel, all on the FP32 pipe, two multiply-adds per instruction
+// (fma.rn.f32x2 over pairs of channels or positions). In the gradients one
+// operand, dz, is fp32; the forward convolutions of layers 2 and 3 have bf16
+// operands and could run on the tensor cores as in inference. Every kernel
 // walks a contiguous share of the batch's tiles with persistent blocks; the
 // operands of a tile sit in shared memory, the next tile's arrive there
 // (cp.async) while this one is worked on, and a thread holds 4 to 16 positions

@@ -20,9 +20,9 @@
 //     warp) and decodes their boxes (exactly rounded float division);
 //  3. the leader walks this segment in batches of the next 64 not yet
 //     suppressed: all threads compute the batch's pairwise suppression bits,
-//     every warp resolves the batch (kept iff no kept earlier member
-//     suppresses it) and suppresses its share of the segment against the
-//     batch's kept members. This takes the same decisions as the
+//     warp 0 resolves the batch (kept iff no kept earlier member
+//     suppresses it) and all threads suppress the rest of the segment against
+//     the batch's kept members. This takes the same decisions as the
 //     one-at-a-time greedy walk (candidates between batch members are already
 //     suppressed);
 //  4. if candidates remain, every CTA drops from its list the segment's keys
@@ -31,12 +31,12 @@
 //     them, so the decisions stay those of the sequential walk.
 // What bounds it: the latency of the one frame with the most candidates: 3,000
 // to 10,000 cycles per batch of the walk, 15,000 to collect, 4,000 to 8,000 to sort.
-// A scan level by level, a bitonic sort of all candidates and a cluster-wide
-// pass over all of them after every batch took 80 us where this takes 31 (one
-// 1242x375 frame, 1,884 candidates), 317 against 137 (8 frames of 40 levels, up
-// to 10,363 candidates), 117 against 68 (64 frames of 1242x375). Of these 37, 152
-// and 76 had a batch's edges 32 bytes apart: 16 lanes on one bank group, and the
-// pairwise bits took 3,700 cycles per batch where they take about 1,200.
+// One 1242x375 frame (1,884 candidates) takes 31 us, 8 frames of 40 levels (up
+// to 10,363 candidates) 137, 64 frames of 1242x375 68; with a scan level by level,
+// a bitonic sort of all candidates and a cluster-wide pass over all of them after
+// every batch it was 80, 317 and 117. A batch's edges lie apart from its boxes: 32
+// bytes apart they put 16 lanes on one bank group (3,700 cycles per batch for the
+// pairwise bits, 1,200 so).
 // The IoU test first evaluates inter - thr * union in float. A coordinate sum or
 // difference is off by at most 3 float roundings of values up to m, the frame's
 // size or, for maps that reach beyond it, their farthest edge

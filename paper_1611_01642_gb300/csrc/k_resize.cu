@@ -8,10 +8,11 @@
 // writes, for every level of that frame, the output pixels it owns. The frame
 // is read from HBM once for all levels, and each level pixel is written once.
 //
-// What bounds it: instructions (issue 66% of cycles, the integer-multiply pipe
-// 68%), about 20 per output pixel. A warp's task (8 column groups of a level by
-// all its rows in the tile) costs some 60 instructions before its first row,
-// and rows go 4 at a time, so a taller tile pays less per pixel: 64 x 1242x375
+// What bounds it: instructions (issue 69% of cycles, the integer-multiply pipe
+// 71%, shared-memory data 72%), 15 thread instructions per output pixel. A
+// warp's task (kCG column groups of a level by all its rows in the tile) costs
+// some 60 instructions before its first row, and rows go kRS = 32 / kCG at a
+// time (8 and 4 by default), so a taller tile pays less per pixel: 64 x 1242x375
 // frames 234 us in 32-row tiles of 256 threads, 197 us in 64-row tiles of 512
 // (the divisions by the staged width as multiplications are 10 of these).
 // While the 32-row tiles of a plan fit the chip in one round the frame is as
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, kResizeCtas) k_resize(const FrameDes
     // of the level; a warp's first is its own, the others come off a shared
     // counter. Lane = (row slice j, group c):
     // it keeps its group's weights and quad addresses in registers and walks
-    // rows j, j + 4, ... (consecutive groups of a row store 32 contiguous bytes).
+    // rows j, j + kRS, ... (consecutive groups of a row store 32 contiguous bytes).
     const int total = s_pre[n];
     const uint32_t quad_base =
         (uint32_t)__cvta_generic_to_shared(quad) - (uint32_t)(it.y0 * kQP * 4);
